@@ -21,6 +21,7 @@
 //               convert                     -> out in the storage dtype
 #include <math_constants.h>
 
+#include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
 #include "tc_utils.cuh"
 #include "tma_map.cuh"
@@ -31,12 +32,11 @@ using namespace tc;
 
 namespace {
 
-constexpr int kInvTok = 1024;          // tokens per CTA in the inversion kernels
+constexpr int kInvTok = 1024;          // tokens per CTA in the inversion kernels, at most (window sizes are multiples of it)
+constexpr int kInvTokMin = 64;         // ... and at least
 constexpr int kWindowTok = 16384;      // tokens per window of the inverted lists
 constexpr int kBwdWindowTok = 32768;   // ... of the backward's lists (fewer, fuller lists: 2.3 ms of 55 at the headline shape)
 constexpr int kItemTiles = 32;         // a work item: at most this many consecutive tiles of one list
-constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLn2 = 0.6931471805599453f;
 
 // ------------------------------------------------------------------ list inversion
 
@@ -48,6 +48,7 @@ struct InvArgs {
   int K, fan, Mk, N, C, BH, tpt;
   int lgK, lgC;           // log2 of K and C when they are powers of two (shifts instead of divisions), else -1
   int W, NW;              // tokens per window (a multiple of kInvTok), windows per sequence
+  int tok;                // tokens per CTA of the counting and filling kernels (divides W)
   int32_t* count;         // [BH*Mk]
   int32_t* entry_off;     // [BH*Mk + 1]
   int32_t* tile_off;      // [nkeys + 1]  tiles of tpt tokens
@@ -76,7 +77,7 @@ __device__ __forceinline__ bool inv_valid(const InvArgs& a, int node, int t) {
 __global__ void __launch_bounds__(256) inv_count_kernel(InvArgs a, int use_smem) {
   extern __shared__ int s_hist[];
   const int bh = blockIdx.y;
-  const int t0 = blockIdx.x * kInvTok, t1 = min(t0 + kInvTok, a.N);
+  const int t0 = blockIdx.x * a.tok, t1 = min(t0 + a.tok, a.N);
   const long long kbase = ((long long)bh * a.NW + t0 / a.W) * a.Mk;
   if (use_smem) {
     for (int j = threadIdx.x; j < a.Mk; j += blockDim.x) s_hist[j] = 0;
@@ -187,12 +188,35 @@ __global__ void __launch_bounds__(1024) inv_scan_fix_kernel(InvArgs a) {
   }
 }
 
+// The three scans of a short key range by one CTA, 1024 lists at a time (each round trip of the three-launch form costs
+// about 4 us with its launch gap: 12 us against 3 to 5 for up to kOneScanKeys lists).
+constexpr int kOneScanKeys = 4096;
+__global__ void __launch_bounds__(1024) inv_scan_one_kernel(InvArgs a) {
+  __shared__ int3 s_w[32];
+  const int nkeys = a.BH * a.NW * a.Mk;
+  int3 carry = make_int3(0, 0, 0);
+  for (int i0 = 0; i0 < nkeys; i0 += 1024) {
+    const int i = i0 + threadIdx.x;
+    const int3 own = inv_key_counts(a, i, nkeys);
+    __syncthreads();                                       // s_w of the previous round has been read
+    const int3 inc = block_scan3(own, s_w);
+    if (i < nkeys) {
+      const int be = carry.x + inc.x - own.x, bi = carry.z + inc.z - own.z;
+      a.entry_off[i] = be; a.tile_off[i] = carry.y + inc.y - own.y; a.item_off[i] = bi; a.cursor[i] = be;
+      for (int x = 0; x < own.z; ++x) a.item_key[bi + x] = i;
+    }
+    const int3 tot = s_w[31];
+    carry.x += tot.x; carry.y += tot.y; carry.z += tot.z;
+  }
+  if (threadIdx.x == 0) { a.entry_off[nkeys] = carry.x; a.tile_off[nkeys] = carry.y; a.item_off[nkeys] = carry.z; }
+}
+
 __global__ void __launch_bounds__(256) inv_fill_kernel(InvArgs a, int use_smem) {
   extern __shared__ int s_mem[];
   int* s_hist = s_mem;
   int* s_base = s_mem + a.Mk;
   const int bh = blockIdx.y;
-  const int t0 = blockIdx.x * kInvTok, t1 = min(t0 + kInvTok, a.N);
+  const int t0 = blockIdx.x * a.tok, t1 = min(t0 + a.tok, a.N);
   const long long kbase = ((long long)bh * a.NW + t0 / a.W) * a.Mk;
   const int n = (t1 - t0) * a.K;
   const int32_t* nodes = a.nodes + ((long long)bh * a.N + t0) * a.K;
@@ -277,58 +301,6 @@ __device__ __noinline__ ItemInfo feed_get(ItemFeed& f, int k, volatile int* fail
   return r;
 }
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Online log-sum-exp (base 2) over one 32-column chunk of raw fp32 logits; (m, ssum) is the running
-// (max, sum of 2^(x - max)) with x = raw * sl2.  sl2 > 0, so the max commutes with the scaling.
-template <int NW>
-__device__ __forceinline__ void lse_chunk(const uint32_t (&rr)[NW], float sl2, float& m, float& ssum) {
-  float c0 = __uint_as_float(rr[0]), c1 = __uint_as_float(rr[1]);
-  float c2 = __uint_as_float(rr[2]), c3 = __uint_as_float(rr[3]);
-#pragma unroll
-  for (int j = 4; j < NW; j += 4) {
-    c0 = fmaxf(c0, __uint_as_float(rr[j]));
-    c1 = fmaxf(c1, __uint_as_float(rr[j + 1]));
-    c2 = fmaxf(c2, __uint_as_float(rr[j + 2]));
-    c3 = fmaxf(c3, __uint_as_float(rr[j + 3]));
-  }
-  const float mn = fmaxf(m, fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)) * sl2);
-  const float neg = -mn;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-  for (int j = 0; j < NW; j += 4) {
-    a0 += ex2_approx(fmaf(__uint_as_float(rr[j]), sl2, neg));
-    a1 += ex2_approx(fmaf(__uint_as_float(rr[j + 1]), sl2, neg));
-    a2 += ex2_approx(fmaf(__uint_as_float(rr[j + 2]), sl2, neg));
-    a3 += ex2_approx(fmaf(__uint_as_float(rr[j + 3]), sl2, neg));
-  }
-  ssum = ssum * ex2_approx(m - mn) + ((a0 + a1) + (a2 + a3));
-  m = mn;
-}
-// the same with only the first `nvalid` (>= 1) columns of the chunk taking part.  The sums associate
-// exactly as in lse_chunk (four interleaved accumulators), so a full row gives bit-identical results on
-// either path: which path a row takes depends on the other rows of its tile, and the composition of a
-// tile (the order of a list's entries) varies from run to run.
-template <int NW>
-__device__ __forceinline__ void lse_chunk_masked(const uint32_t (&rr)[NW], int nvalid, float sl2, float& m,
-                                                 float& ssum) {
-  float cm = -CUDART_INF_F;
-#pragma unroll
-  for (int j = 0; j < NW; ++j)
-    if (j < nvalid) cm = fmaxf(cm, __uint_as_float(rr[j]));
-  const float mn = fmaxf(m, cm * sl2);
-  const float neg = -mn;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int j = 0; j < NW; ++j)
-    if (j < nvalid) acc[j & 3] += ex2_approx(fmaf(__uint_as_float(rr[j]), sl2, neg));
-  ssum = ssum * ex2_approx(m - mn) + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
-  m = mn;
-}
 // first and second moments of the first `nvalid` of 32 logits about `shift` (score modes "mean" and
 // "mean + variance/2", Sec. 4.3)
 template <int NW>
@@ -1506,7 +1478,11 @@ int run_inversion(const Geometry& g, const int32_t* nodes, int fan, int Mk, char
   if (e != cudaSuccess) { record_cuda_error("inversion memset", e); return PISA_ERR_CUDA; }
   const int use_smem = (2 * (size_t)Mk * 4 <= 96 * 1024) ? 1 : 0;
   const size_t sm_count = use_smem ? (size_t)Mk * 4 : 0, sm_fill = use_smem ? 2 * (size_t)Mk * 4 : 0;
-  dim3 grid((g.N + kInvTok - 1) / kInvTok, a.BH);
+  // tokens per CTA: enough CTAs for four per SM (a CTA of 1024 tokens took 26 / 33 us to count / fill however short the
+  // problem was, on a handful of SMs), but no finer than the histogram's own size pays for
+  a.tok = kInvTok;
+  while (a.tok > kInvTokMin && (long long)((g.N + a.tok - 1) / a.tok) * a.BH < 4LL * num_sms() && a.tok * g.K > 2 * Mk) a.tok >>= 1;
+  dim3 grid((g.N + a.tok - 1) / a.tok, a.BH);
   if (sm_fill > 48 * 1024) {
     cudaFuncSetAttribute(inv_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_count);
     cudaFuncSetAttribute(inv_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_fill);
@@ -1514,16 +1490,22 @@ int run_inversion(const Geometry& g, const int32_t* nodes, int fan, int Mk, char
   inv_count_kernel<<<grid, 256, sm_count, s>>>(a, use_smem);
   int st = check_launch("inv_count");
   if (st != PISA_OK) return st;
-  const unsigned nblk = (unsigned)((nkeys + 1023) / 1024);
-  inv_scan_blocks_kernel<<<nblk, 1024, 0, s>>>(a);
-  st = check_launch("inv_scan_blocks");
-  if (st != PISA_OK) return st;
-  inv_scan_totals_kernel<<<1, 1024, 0, s>>>(a);
-  st = check_launch("inv_scan_totals");
-  if (st != PISA_OK) return st;
-  inv_scan_fix_kernel<<<nblk, 1024, 0, s>>>(a);
-  st = check_launch("inv_scan_fix");
-  if (st != PISA_OK) return st;
+  if (nkeys <= (size_t)kOneScanKeys) {
+    inv_scan_one_kernel<<<1, 1024, 0, s>>>(a);
+    st = check_launch("inv_scan_one");
+    if (st != PISA_OK) return st;
+  } else {
+    const unsigned nblk = (unsigned)((nkeys + 1023) / 1024);
+    inv_scan_blocks_kernel<<<nblk, 1024, 0, s>>>(a);
+    st = check_launch("inv_scan_blocks");
+    if (st != PISA_OK) return st;
+    inv_scan_totals_kernel<<<1, 1024, 0, s>>>(a);
+    st = check_launch("inv_scan_totals");
+    if (st != PISA_OK) return st;
+    inv_scan_fix_kernel<<<nblk, 1024, 0, s>>>(a);
+    st = check_launch("inv_scan_fix");
+    if (st != PISA_OK) return st;
+  }
   inv_fill_kernel<<<grid, 256, sm_fill, s>>>(a, use_smem);
   st = check_launch("inv_fill");
   *out = a;
