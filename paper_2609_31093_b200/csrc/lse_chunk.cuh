@@ -15,29 +15,56 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+// two fp32 lanes in one instruction (sm_100); the same roundings as the scalar forms
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 // Online log-sum-exp (base 2) over one 32-column chunk of raw fp32 logits; (m, ssum) is the running
 // (max, sum of 2^(x - max)) with x = raw * sl2.  sl2 > 0, so the max commutes with the scaling.
 template <int NW>
 __device__ __forceinline__ void lse_chunk(const uint32_t (&rr)[NW], float sl2, float& m, float& ssum) {
   float c0 = __uint_as_float(rr[0]), c1 = __uint_as_float(rr[1]);
-  float c2 = __uint_as_float(rr[2]), c3 = __uint_as_float(rr[3]);
 #pragma unroll
-  for (int j = 4; j < NW; j += 4) {
-    c0 = fmaxf(c0, __uint_as_float(rr[j]));
-    c1 = fmaxf(c1, __uint_as_float(rr[j + 1]));
-    c2 = fmaxf(c2, __uint_as_float(rr[j + 2]));
-    c3 = fmaxf(c3, __uint_as_float(rr[j + 3]));
+  for (int j = 2; j < NW - 2; j += 4) {
+    c0 = max3(c0, __uint_as_float(rr[j]), __uint_as_float(rr[j + 1]));
+    c1 = max3(c1, __uint_as_float(rr[j + 2]), __uint_as_float(rr[j + 3]));
   }
-  const float mn = fmaxf(m, fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)) * sl2);
-  const float neg = -mn;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+  c0 = max3(c0, __uint_as_float(rr[NW - 2]), __uint_as_float(rr[NW - 1]));
+  const float mn = fmaxf(m, fmaxf(c0, c1) * sl2);
+  const uint64_t neg = pack2(-mn, -mn), sc = pack2(sl2, sl2);
+  uint64_t a01 = pack2(0.f, 0.f), a23 = a01;
 #pragma unroll
   for (int j = 0; j < NW; j += 4) {
-    a0 += ex2_approx(fmaf(__uint_as_float(rr[j]), sl2, neg));
-    a1 += ex2_approx(fmaf(__uint_as_float(rr[j + 1]), sl2, neg));
-    a2 += ex2_approx(fmaf(__uint_as_float(rr[j + 2]), sl2, neg));
-    a3 += ex2_approx(fmaf(__uint_as_float(rr[j + 3]), sl2, neg));
+    float x0, x1, x2, x3;
+    unpack2(fma2(pack2(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1])), sc, neg), x0, x1);
+    unpack2(fma2(pack2(__uint_as_float(rr[j + 2]), __uint_as_float(rr[j + 3])), sc, neg), x2, x3);
+    a01 = add2(a01, pack2(ex2_approx(x0), ex2_approx(x1)));
+    a23 = add2(a23, pack2(ex2_approx(x2), ex2_approx(x3)));
   }
+  float a0, a1, a2, a3;
+  unpack2(a01, a0, a1);
+  unpack2(a23, a2, a3);
   ssum = ssum * ex2_approx(m - mn) + ((a0 + a1) + (a2 + a3));
   m = mn;
 }

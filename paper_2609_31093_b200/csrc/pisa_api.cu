@@ -159,6 +159,15 @@ static size_t route_ws_bytes(const pisa_params_t* p, const Geometry& g) {
   if (use_tensor(p, g)) b += tensor_route_workspace_bytes(g);
   return b;
 }
+// The query-major path for short sequences, wherever the caller's workspace holds its tables (one sized for another
+// length of the same problem may not: the list-driven path then runs).
+static bool prefers_dense(const pisa_params_t* p, const Geometry& g) {
+  return p->impl != PISA_IMPL_SIMT && qm_dense_preferred(g, p->dtype);
+}
+static size_t dense_ws_bytes(const Geometry& g) { return kStatusBytes + qm_workspace_bytes(g); }
+static bool use_dense(const pisa_params_t* p, const Geometry& g, size_t ws_bytes) {
+  return prefers_dense(p, g) && ws_bytes >= dense_ws_bytes(g);
+}
 static size_t bsa_ws_bytes(const pisa_params_t* p, const Geometry& g) {
   size_t b = kStatusBytes;
   if (use_tensor(p, g)) b += tensor_bsa_workspace_bytes(g);
@@ -187,6 +196,7 @@ static int host_arena(const pisa_params_t* p, HostArena* a) {
   const size_t es = elem_size(p->dtype);
   const size_t r = route_ws_bytes(&a->unit, g), b = bsa_ws_bytes(&a->unit, g);
   a->fwd = align_up(r > b ? r : b, 256);
+  if (prefers_dense(&a->unit, g)) a->fwd = std::max(a->fwd, align_up(dense_ws_bytes(g), 256));
   a->qb = align_up((size_t)g.B * g.N * g.Hq * g.d * es, 256);
   a->kb = align_up((size_t)g.B * g.N * g.d * es, 256);
   a->lb = align_up((size_t)g.B * g.Hq * g.N * sizeof(float), 256);
@@ -206,6 +216,8 @@ static int clear_status(void* ws, cudaStream_t s) {
 static int do_route(const pisa_params_t* p, const Geometry& g, const void* q, const void* k, const void* pyr,
                     int32_t* idx, float* sel_lse, float* margin, float* lse_out, void* ws, size_t ws_bytes,
                     cudaStream_t s) {
+  if (use_dense(p, g, ws_bytes))
+    return qm_route(g, q, k, pyr, idx, sel_lse, margin, lse_out, (char*)ws + kStatusBytes, (int32_t*)ws, s);
   if (ws_bytes < route_ws_bytes(p, g)) return PISA_ERR_WORKSPACE_TOO_SMALL;
   if (use_tensor(p, g))
     return tensor_route(g, p->dtype, q, k, pyr, idx, sel_lse, margin, lse_out, (char*)ws + kStatusBytes, (int32_t*)ws, s);
@@ -384,6 +396,11 @@ struct ChunkView {
 // Plans `ops` for (p, g), falls back to the unsplit plan when `ws_bytes` only covers that one, and
 // returns the bytes the plan needs.
 static int plan_for(const pisa_params_t* p, const Geometry& g, int ops, size_t ws_bytes, ForwardPlan* pl) {
+  if ((ops & kOpRoute) && use_dense(p, g, ws_bytes)) {       // query-major: one sequence of launches
+    pl->n = 1;
+    pl->streams = 1;
+    return PISA_OK;
+  }
   int st = forward_plan(p, g, ops, pl);
   if (st != PISA_OK) return st;
   if (pl->n > 1 && ws_bytes < pl->total) {   // a workspace sized for another length of the same problem: unsplit
@@ -521,7 +538,8 @@ static int do_forward(const pisa_params_t* p, const Geometry& g, const void* q, 
     if (ee == cudaSuccess && v_ready != nullptr) ee = cudaStreamWaitEvent(s, v_ready, 0);
     if (ee != cudaSuccess) { record_cuda_error("forward stage events", ee); return PISA_ERR_CUDA; }
     stage_mark(2, s);
-    st = do_bsa(p, g, q, k, v_, idx, nullptr, out, lse, use_tensor(p, g) && g.score_mode == PISA_SCORE_LSE, true, ws,
+    if (use_dense(p, g, ws_bytes)) st = qm_attend(g, q, k, v_, out, lse, (char*)ws + kStatusBytes, (int32_t*)ws, s);
+    else st = do_bsa(p, g, q, k, v_, idx, nullptr, out, lse, use_tensor(p, g) && g.score_mode == PISA_SCORE_LSE, true, ws,
                 ws_bytes, s);
   } else {
     st = run_chunks(p, g, pl, ws, s, [&](const ChunkView& v, int i) {
@@ -557,7 +575,7 @@ int route_unsplit(const pisa_params_t* p, const void* q, const void* k, const vo
   if (st != PISA_OK) return st;
   if (!q || !k || !pyramid || !idx || !ws || misaligned(q) || misaligned(k) || misaligned32(pyramid) || misaligned(ws))
     return PISA_ERR_INVALID_ARG;
-  if (ws_bytes < route_ws_bytes(p, g)) return PISA_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < route_ws_bytes(p, g) && !use_dense(p, g, ws_bytes)) return PISA_ERR_WORKSPACE_TOO_SMALL;
   st = clear_status(ws, s);
   if (st != PISA_OK) return st;
   return do_route(p, g, q, k, pyramid, idx, nullptr, margin, nullptr, ws, ws_bytes, s);
@@ -643,6 +661,7 @@ struct PackedArena {
 static size_t forward_ws_bytes(const pisa_params_t* p, const Geometry& g, int* st) {
   size_t r = route_ws_bytes(p, g), a = bsa_ws_bytes(p, g);
   size_t f = r > a ? r : a;
+  if (prefers_dense(p, g) && dense_ws_bytes(g) > f) f = dense_ws_bytes(g);
   ForwardPlan pl;
   *st = forward_plan(p, g, kOpRoute | kOpBsa, &pl);
   if (*st == PISA_OK && pl.total > f) f = pl.total;
@@ -797,6 +816,7 @@ int pisa_workspace_bytes(const pisa_params_t* p, int op, size_t* bytes) {
     if ((st = forward_plan(p, g, kOpBsa, &pl)) != PISA_OK) return st;
     if (pl.total > a) a = pl.total;
   }
+  if (prefers_dense(p, g) && dense_ws_bytes(g) > r) r = dense_ws_bytes(g);
   size_t f = r > a ? r : a;                  // one buffer sized for the forward also serves pisa_route and pisa_bsa_fwd
   {
     ForwardPlan pl;

@@ -22,6 +22,27 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
                const float* sel_lse, void* out, float* lse, bool lse_ready, bool forced_present, void* ws,
                int32_t* status, cudaStream_t s);
 
+// query-major path (query_major.cuh): dense scoring, one-thread-per-token selection, masked dense attention
+namespace qm { struct Args; }
+bool qm_supported(const Geometry& g, int dtype);
+// shapes for which the whole forward is cheaper query-major than through the lists
+bool qm_dense_preferred(const Geometry& g, int dtype);
+size_t qm_workspace_bytes(const Geometry& g);
+int qm_route(const Geometry& g, const void* q, const void* k, const void* pyramid, int32_t* idx, float* sel_lse,
+             float* margin, float* lse_out, void* ws, int32_t* status, cudaStream_t s);
+int qm_attend(const Geometry& g, const void* q, const void* k, const void* v, void* out, const float* lse, void* ws,
+              int32_t* status, cudaStream_t s);
+bool qm_map_rows(void* map, const void* base, int d, int H, long long tokens, int B, const long long* st, int heads, int rows);
+int launch_qm_score(const Geometry& g, const qm::Args& a, const void* q, const void* k, long long tokens, const void* pyramid,
+                    long long pyr_rows, cudaStream_t s);
+int launch_qm_select_full(const Geometry& g, const qm::Args& a, long long rows, int32_t* idx, float* margin, float* lse,
+                          float* sel_lse, cudaStream_t s);
+int launch_qm_select_stage1(const Geometry& g, const qm::Args& a, long long rows, int32_t* par, float* margin, cudaStream_t s);
+int launch_qm_select_final(const Geometry& g, const qm::Args& a, long long rows, const int32_t* par, const float* blk,
+                           int32_t* idx, float* margin, float* lse, float* sel_lse, cudaStream_t s);
+int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const void* k, const void* v, long long tokens,
+                     const float* row_lse, void* out, cudaStream_t s);
+
 // attention over the forced leaves, query-major (local_window.cu); stores the fp32 accumulator [B,Hkv,N,128,G]
 bool local_window_supported(const Geometry& g, int dtype);
 int launch_local_window(const Geometry& g, const void* q, const void* k, const void* v, const float* row_lse,
