@@ -146,15 +146,13 @@ local_window_kernel(Geometry geo, const __grid_constant__ CUtensorMap tm_q, cons
         if (ok && kvj >= 2) ok = mbar_wait_bounded(&s_empty[s], (uint32_t)(((kvj >> 1) - 1) & 1));
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        if (lane == 0) {
-          tcgen05_fence_after_sync();
-          const uint32_t q0 = smem_u32(sQ), k0 = smem_u32(sK + s * KV_BYTES);
+        tcgen05_fence_after_sync();
+        const uint32_t q0 = desc_lo(smem_u32(sQ), 0), k0 = desc_lo(smem_u32(sK) + (uint32_t)(s * KV_BYTES), 0);
+        if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t da = make_smem_desc(q0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-            const uint64_t db = make_smem_desc(k0 + (kk >> 2) * KV_SLAB + (kk & 3) * 32, 0, 1024);
-            umma_bf16(tmem + (uint32_t)(s * 128), da, db, idesc_s, kk > 0);
-          }
+          for (int kk = 0; kk < D / 16; ++kk)
+            umma_bf16(tmem + (uint32_t)(s * 128), desc64(q0 + ((uint32_t)((kk >> 2) * A_SLAB + (kk & 3) * 32) >> 4)),
+                      desc64(k0 + ((uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4)), idesc_s, kk > 0);
           umma_commit(&s_full[s]);
           umma_commit(&k_empty[s]);
           if (j == w.nb - 1) umma_commit(&q_empty);          // every S of this item has been issued
@@ -179,13 +177,12 @@ local_window_kernel(Geometry geo, const __grid_constant__ CUtensorMap tm_q, cons
         if (ok && j == 0 && it >= 1) ok = mbar_wait_bounded(&o_empty, (uint32_t)((it - 1) & 1));
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        if (lane == 0) {
-          tcgen05_fence_after_sync();
-          const uint32_t p0 = smem_u32(sP + s * P_BYTES), v0 = smem_u32(sV + s * KV_BYTES);
+        tcgen05_fence_after_sync();
+        const uint32_t p0 = desc_lo(smem_u32(sP) + (uint32_t)(s * P_BYTES), 0), v0 = desc_lo(smem_u32(sV) + (uint32_t)(s * KV_BYTES), KV_SLAB);
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < C / 16; ++kk) {
-            const uint64_t dp = make_smem_desc(p0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-            const uint64_t dv = make_smem_desc(v0 + kk * (16 * 128), KV_SLAB, 1024);
+            const uint64_t dp = desc64(p0 + ((uint32_t)((kk >> 2) * A_SLAB + (kk & 3) * 32) >> 4)), dv = desc64(v0 + kk * (2048 >> 4));
             if (kTransO) umma_bf16(tmem + 256u, dv, dp, idesc_ot, (j > 0 || kk > 0) ? 1u : 0u);
             else umma_bf16(tmem + 256u, dp, dv, idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
           }

@@ -32,6 +32,20 @@ int qm_route(const Geometry& g, const void* q, const void* k, const void* pyrami
              float* margin, float* lse_out, void* ws, int32_t* status, cudaStream_t s);
 int qm_attend(const Geometry& g, const void* q, const void* k, const void* v, void* out, const float* lse, void* ws,
               int32_t* status, cudaStream_t s);
+int qm_tiles_per_item(const Geometry& g, long long unit_tokens);
+// packed batches: workspace one sequence needs, and the forward of the sequences ids[0..n) (qm_packed.cu)
+size_t qm_packed_bytes(const Geometry& g, int len);
+int qm_forward_packed(const Geometry& g, const int32_t* cu, const int* ids, int n, long long total, const void* q, const void* k,
+                      const void* v, int32_t* idx, void* out, float* lse, void* ws, size_t ws_bytes, int32_t* status,
+                      cudaStream_t s);
+// levels L..2 for the list-driven path: scores of the nodes that can prune and the selection among them, a range of
+// tokens at a time through `scratch`
+bool qm_stage1_preferred(const Geometry& g, int dtype, size_t scratch_bytes);
+int qm_stage1(const Geometry& g, const void* q, const void* pyramid, int32_t* par, float* margin, float* scratch,
+              size_t scratch_bytes, int32_t* status, cudaStream_t s);
+// leaf level of the list-driven path: Select_K among the children of `par` by their scores `blk` (any score mode)
+int qm_select_final(const Geometry& g, const int32_t* par, const float* blk, int32_t* idx, float* margin, float* lse_out,
+                    float* sel_lse, int32_t* status, cudaStream_t s);
 bool qm_map_rows(void* map, const void* base, int d, int H, long long tokens, int B, const long long* st, int heads, int rows);
 int launch_qm_score(const Geometry& g, const qm::Args& a, const void* q, const void* k, long long tokens, const void* pyramid,
                     long long pyr_rows, cudaStream_t s);

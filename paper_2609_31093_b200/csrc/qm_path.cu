@@ -10,6 +10,11 @@ namespace {
 constexpr int kDenseMaxTokens = 32768;                 // 256 steps of 128 keys: the attention kernel's step lists
 constexpr size_t kDenseMaxBytes = (size_t)4 << 30;     // score tables (they grow with N * M1)
 
+constexpr int kStage1MaxG = 4;
+// node table of one range of tokens (list-driven path): the larger the better -- at the headline shape 48 MB, inside L2,
+// 7.5 ms for the stage, 256 MB 5.1, 1 GB 4.1 (each range is two launches that fill and drain the GPU)
+constexpr size_t kSlabBytes = (size_t)1 << 30;
+
 int log2i(int x) { return 31 - __builtin_clz((unsigned)x); }
 
 struct Layout { size_t ctr, leaf, up, bits, total; };
@@ -27,17 +32,11 @@ Layout layout(const Geometry& g) {
   return l;
 }
 
-// Two tiles per work item halve the key / value traffic, which bounds the dense kernels, once there are enough pairs for
-// four waves of one item per SM (4096 tokens x 16 heads still runs 5 % faster with one tile per item, 8192 5 % slower).
-int tiles_per_item(const Geometry& g, long long unit_tokens) {
-  return unit_tokens * g.G / 256 >= 4LL * num_sms() ? 2 : 1;
-}
-
 qm::Args uniform_args(const Geometry& g, char* ws, const Layout& l, int32_t* status) {
   qm::Args a = {};
   a.lgC = log2i(g.C); a.lgg = log2i(g.g); a.lgG = log2i(g.G);
   a.t0 = 0; a.t1 = g.N;
-  a.tiles = tiles_per_item(g, (long long)g.B * g.Hkv * g.N);
+  a.tiles = qm_tiles_per_item(g, (long long)g.B * g.Hkv * g.N);
   const int tpt = a.tiles * 128 / g.G;
   a.n_items = g.B * g.Hkv * ((g.N + tpt - 1) / tpt);
   a.want_leaf = 1;
@@ -48,6 +47,12 @@ qm::Args uniform_args(const Geometry& g, char* ws, const Layout& l, int32_t* sta
 }
 
 }  // namespace
+
+// Two tiles per work item halve the key / value traffic, which bounds the dense kernels, once there are enough pairs for
+// four waves of one item per SM (4096 tokens x 16 heads still runs 5 % faster with one tile per item, 8192 5 % slower).
+int qm_tiles_per_item(const Geometry& g, long long unit_tokens) {
+  return unit_tokens * g.G / 256 >= 4LL * num_sms() ? 2 : 1;
+}
 
 bool qm_supported(const Geometry& g, int dtype) {
   if (dtype != PISA_BF16 || g.score_mode != PISA_SCORE_LSE) return false;
@@ -89,6 +94,54 @@ int qm_attend(const Geometry& g, const void* q, const void* k, const void* v, vo
   const qm::Args a = uniform_args(g, ws, l, status);
   kernel_mark("qm_attend", s);
   return launch_qm_attend(g, a, q, k, v, g.N, lse, out, s);
+}
+
+// ---------------------------------------------------------------- upper levels and final selection of the list-driven path
+
+static long long stage1_slab(const Geometry& g, size_t scratch_bytes, int width) {
+  const size_t per_token = (size_t)g.B * g.Hkv * width * 4;
+  const size_t bytes = scratch_bytes < kSlabBytes ? scratch_bytes : kSlabBytes;
+  return (long long)(bytes / per_token) / 256 * 256;         // whole work items of two tiles
+}
+
+bool qm_stage1_preferred(const Geometry& g, int dtype, size_t scratch_bytes) {
+  // (groups of more than four heads: the per-token scoring shares its gathered summaries among them, 0.68 ms against 1.3
+  // at 65536 tokens, 2 KV heads of 16 query heads; beyond 2048 leaves it costs log N per token and this N)
+  if (!qm_supported(g, dtype) || g.L < 2 || g.M[1] > 2048 || g.G > kStage1MaxG) return false;
+  const int lgC = log2i(g.C), lgg = log2i(g.g), top = qm::top_level(g.N, lgC, lgg, g.K);
+  const int width = qm::table_width(g.N, lgC, lgg, top);
+  return width == 0 || stage1_slab(g, scratch_bytes, width) > 0;
+}
+
+int qm_stage1(const Geometry& g, const void* q, const void* pyramid, int32_t* par, float* margin, float* scratch,
+              size_t scratch_bytes, int32_t* status, cudaStream_t s) {
+  qm::Args a = {};
+  a.lgC = log2i(g.C); a.lgg = log2i(g.g); a.lgG = log2i(g.G);
+  a.up = scratch; a.status = status;
+  const int width = qm::table_width(g.N, a.lgC, a.lgg, qm::top_level(g.N, a.lgC, a.lgg, g.K));
+  const long long slab = width == 0 ? g.N : stage1_slab(g, scratch_bytes, width);
+  const long long pyr_rows = g.level_off[g.L] / g.d + (long long)g.B * g.Hkv * g.M[g.L];
+  for (long long t0 = 0; t0 < g.N; t0 += slab) {
+    a.t0 = (int)t0;
+    a.t1 = (int)(t0 + slab < g.N ? t0 + slab : g.N);
+    a.tiles = qm_tiles_per_item(g, (long long)g.B * g.Hkv * (a.t1 - a.t0));
+    const int tpt = a.tiles * 128 / g.G;
+    a.n_items = g.B * g.Hkv * ((a.t1 - a.t0 + tpt - 1) / tpt);
+    int st = PISA_OK;
+    if (width > 0) st = launch_qm_score(g, a, q, nullptr, g.N, pyramid, pyr_rows, s);
+    if (st == PISA_OK) st = launch_qm_select_stage1(g, a, (long long)g.B * (a.t1 - a.t0), par, margin, s);
+    if (st != PISA_OK) return st;
+  }
+  return PISA_OK;
+}
+
+int qm_select_final(const Geometry& g, const int32_t* par, const float* blk, int32_t* idx, float* margin, float* lse_out,
+                    float* sel_lse, int32_t* status, cudaStream_t s) {
+  qm::Args a = {};
+  a.lgC = log2i(g.C); a.lgg = log2i(g.g); a.lgG = log2i(g.G);
+  a.t0 = 0; a.t1 = g.N;
+  a.status = status;
+  return launch_qm_select_final(g, a, (long long)g.B * g.N, par, blk, idx, margin, lse_out, sel_lse, s);
 }
 
 }  // namespace pisa

@@ -28,11 +28,12 @@ __device__ __forceinline__ float lg2_approx(float x) {
   return y;
 }
 
-// group-summed natural scores of the 32 / FAN nodes whose children are these 32 columns; stored by the lanes of the group
-template <int FAN>
-__device__ __forceinline__ void score_nodes(const uint32_t (&r)[32], float sl2, int G, int head, float* dst, int node0,
-                                            int width, bool live) {
-  constexpr int NN = 32 / FAN;
+// group-summed natural scores of the 32 / FAN nodes whose children are these 32 columns.  The sum over the G lanes of a
+// token is a reduce-scatter (half of the live values per step: 12 shuffles for sixteen nodes and G = 4, 15 for G = 16,
+// where adding all of them in every lane takes 32 and 64), which leaves each lane the nodes it stores.
+template <int FAN, int G>
+__device__ __forceinline__ void score_nodes(const uint32_t (&r)[32], float sl2, int head, float* dst, int node0, int width, bool live) {
+  constexpr int NN = 32 / FAN, KEEP = NN / G > 0 ? NN / G : 1;
   float u[NN];
 #pragma unroll
   for (int i = 0; i < NN; ++i) {
@@ -50,18 +51,45 @@ __device__ __forceinline__ void score_nodes(const uint32_t (&r)[32], float sl2, 
       u[i] = m + lg2_approx(s);
     }
   }
-  for (int o = 1; o < G; o <<= 1)
+  int base = 0;                                                  // first node this lane keeps
 #pragma unroll
-    for (int i = 0; i < NN; ++i) u[i] += __shfl_xor_sync(0xffffffffu, u[i], o);
-  constexpr int N4 = NN / 4;
-  if (live)
+  for (int o = 1, cnt = NN; o < G; o <<= 1) {
+    if (cnt > 1) {
+      const bool up = (head & o) != 0;
+      cnt >>= 1;
 #pragma unroll
-    for (int i4 = 0; i4 < N4; ++i4) {
-      const int own = (G < N4) ? (i4 & (G - 1)) : i4;            // which head's lane stores this vector
-      if (head == own && node0 + 4 * i4 < width)
-        *reinterpret_cast<float4*>(dst + node0 + 4 * i4) =
-            make_float4(u[4 * i4] * kLn2, u[4 * i4 + 1] * kLn2, u[4 * i4 + 2] * kLn2, u[4 * i4 + 3] * kLn2);
+      for (int i = 0; i < NN / 2; ++i)
+        if (i < cnt) {
+          const float send = up ? u[i] : u[i + cnt], mine = up ? u[i + cnt] : u[i];
+          u[i] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      base += up ? cnt : 0;
+    } else {
+      u[0] += __shfl_xor_sync(0xffffffffu, u[0], o);
     }
+  }
+  if (!live || (G > NN && head >= NN)) return;
+  float* p = dst + node0 + base;
+  if constexpr (KEEP >= 4) {
+#pragma unroll
+    for (int i = 0; i < KEEP; i += 4)
+      if (node0 + base + i < width)
+        *reinterpret_cast<float4*>(p + i) = make_float4(u[i] * kLn2, u[i + 1] * kLn2, u[i + 2] * kLn2, u[i + 3] * kLn2);
+  } else if (node0 + base < width) {
+#pragma unroll
+    for (int i = 0; i < KEEP; ++i) p[i] = u[i] * kLn2;
+  }
+}
+template <int FAN>
+__device__ __forceinline__ void score_nodes_g(const uint32_t (&r)[32], float sl2, int G, int head, float* dst, int node0, int width,
+                                              bool live) {
+  switch (G) {
+    case 1: score_nodes<FAN, 1>(r, sl2, head, dst, node0, width, live); break;
+    case 2: score_nodes<FAN, 2>(r, sl2, head, dst, node0, width, live); break;
+    case 4: score_nodes<FAN, 4>(r, sl2, head, dst, node0, width, live); break;
+    case 8: score_nodes<FAN, 8>(r, sl2, head, dst, node0, width, live); break;
+    default: score_nodes<FAN, 16>(r, sl2, head, dst, node0, width, live); break;
+  }
 }
 
 // stages of the key ring: two CTAs per SM with one tile each, one CTA with two
@@ -218,8 +246,8 @@ qm_score_kernel(Geometry geo, qm::Args a, const __grid_constant__ CUtensorMap tm
           if (q == 3) handed_back();
           float* dst = up_row + st.z;
           const int node0 = st.y + ((q * 32) >> lgg);
-          if (lgg == 1) score_nodes<2>(rr, sl2, G, head, dst, node0, st.w, live);
-          else score_nodes<4>(rr, sl2, G, head, dst, node0, st.w, live);
+          if (lgg == 1) score_nodes_g<2>(rr, sl2, G, head, dst, node0, st.w, live);
+          else score_nodes_g<4>(rr, sl2, G, head, dst, node0, st.w, live);
         }
       }
     }

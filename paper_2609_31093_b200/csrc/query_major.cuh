@@ -27,6 +27,7 @@ struct Seq {
   int tok, batch;          // TMA coordinates of its first token
   int len;
   int pyr_row;             // packed: row of the pyramid scratch its levels start at, level l = [Hkv][M_l] rows
+  int row0, leaf0;         // packed: tokens / leaves of the launch's sequences before it
 };
 struct SeqOrder { int seq, item0; };   // work items of the packed launch: sequence, its first item (longest sequences first)
 
@@ -76,7 +77,7 @@ __device__ __forceinline__ Seq uniform_seq(const Geometry& geo, const Args& a, i
   q.leaf_off = (long long)b * geo.Hkv * geo.N * level_width(geo.M[1]) * geo.G;
   q.up_off = (long long)b * geo.Hkv * rows * width;
   q.bits_off = (long long)b * geo.Hkv * geo.N * ((geo.M[1] + 31) >> 5);
-  q.tok = 0; q.batch = b; q.len = geo.N; q.pyr_row = 0;
+  q.tok = 0; q.batch = b; q.len = geo.N; q.pyr_row = 0; q.row0 = 0; q.leaf0 = 0;
   return q;
 }
 

@@ -7,11 +7,11 @@
 // references, 128/G tokens x G heads are gathered into a 128-row A operand, and the block's keys
 // (and values) stay resident in shared memory as the B operand while the list is walked.
 //
-//   routing   : stage 1 (levels L..2, SIMT) -> kept level-2 nodes
+//   routing   : stage 1 (levels L..2)       -> kept level-2 nodes (qm_path.cu, route_mma.cu)
 //               invert by level-2 node      -> lists of (token, slot)
 //               lse_ws_kernel               -> per-head LSE of every child leaf (g*C keys per tile),
 //                                              causal mask inside the query's own leaf
-//               final_topk_kernel           -> grouped score = sum over heads, forced leaves, Top-K;
+//               qm_select / final_topk      -> grouped score = sum over heads, forced leaves, Top-K;
 //                                              also the softmax denominator of the kept leaves
 //   attention : invert idx by leaf          -> lists of (token, slot)
 //               [lse_ws + row_lse only when the denominators are not already known]
@@ -561,16 +561,14 @@ lse_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant
       if (ok && it >= 2) ok = mbar_wait_bounded(&t_empty[buf], (uint32_t)(((it >> 1) - 1) & 1));
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) { s_fail = 1; break; }
-      if (lane == 0) {
-        fence_proxy_async_smem();
-        tcgen05_fence_after_sync();
-        const uint32_t a0 = smem_u32(sA + s * A_STAGE), b0 = smem_u32(sB + pb * B_BUF);
+      fence_proxy_async_smem();
+      tcgen05_fence_after_sync();
+      const uint32_t a0 = desc_lo(smem_u32(sA) + (uint32_t)(s * A_STAGE), 0), b0 = desc_lo(smem_u32(sB) + (uint32_t)(pb * B_BUF), 0);
+      if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t da = make_smem_desc(a0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-          const uint64_t db = make_smem_desc(b0 + (kk >> 2) * B_SLAB + (kk & 3) * 32, 0, 1024);
-          umma_bf16(tmem + (uint32_t)(buf * NB), da, db, idesc, kk > 0);
-        }
+        for (int kk = 0; kk < D / 16; ++kk)
+          umma_bf16(tmem + (uint32_t)(buf * NB), desc64(a0 + ((uint32_t)((kk >> 2) * A_SLAB + (kk & 3) * 32) >> 4)),
+                    desc64(b0 + ((uint32_t)((kk >> 2) * B_SLAB + (kk & 3) * 32) >> 4)), idesc, kk > 0);
         umma_commit(&a_empty[s]);
         umma_commit(&t_full[buf]);
         if (flags & 2) umma_commit(&b_empty[pb]);    // last tile of the item: its MMAs release the keys
@@ -895,36 +893,36 @@ pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant_
       do_pv = __shfl_sync(0xffffffffu, do_pv, 0);
       if (do_pv) {
         const int ps = pv_it % NS, pb = pv_it & 1;
-        if (lane == 0) {
-          tcgen05_fence_after_sync();
-          const uint32_t p0 = smem_u32(sQ + ps * Q_STAGE), v0 = smem_u32(sV);
+        tcgen05_fence_after_sync();
+        const uint32_t p0 = desc_lo(smem_u32(sQ) + (uint32_t)(ps * Q_STAGE), 0), v0 = desc_lo(smem_u32(sV), KV_SLAB);
+        const bool closes = ((last_bits >> (pv_it & 31)) & 1u) != 0u;
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < C / 16; ++kk) {
-            const uint64_t dp = make_smem_desc(p0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-            const uint64_t dv = make_smem_desc(v0 + kk * (16 * 128), KV_SLAB, 1024);
+            const uint64_t dp = desc64(p0 + ((uint32_t)((kk >> 2) * A_SLAB + (kk & 3) * 32) >> 4)), dv = desc64(v0 + kk * (2048 >> 4));
             if (kTransO) umma_bf16(tmem + 256u + (uint32_t)(pb * 128), dv, dp, idesc_ot, kk > 0);
             else umma_bf16(tmem + 256u + (uint32_t)(pb * 128), dp, dv, idesc_o, kk > 0);
           }
           umma_commit(&o_full[pb]);
           if (kTransO) umma_commit(&q_empty[ps]);     // P has been consumed: the ring slot is free
-          if ((last_bits >> (pv_it & 31)) & 1u) umma_commit(&kv_empty);   // K/V of that item are free
+          if (closes) umma_commit(&kv_empty);         // K/V of that item are free
         }
+        __syncwarp();
         ++pv_it;
       }
       if (do_s) {
         const int s = s_it % NS, buf = s_it & 1;
-        if (lane == 0) {
-          fence_proxy_async_smem();
-          tcgen05_fence_after_sync();
-          const uint32_t q0 = smem_u32(sQ + s * Q_STAGE), k0 = smem_u32(sK);
+        fence_proxy_async_smem();
+        tcgen05_fence_after_sync();
+        const uint32_t q0 = desc_lo(smem_u32(sQ) + (uint32_t)(s * Q_STAGE), 0), k0 = desc_lo(smem_u32(sK), 0);
+        if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t da = make_smem_desc(q0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-            const uint64_t db = make_smem_desc(k0 + (kk >> 2) * KV_SLAB + (kk & 3) * 32, 0, 1024);
-            umma_bf16(tmem + (uint32_t)(buf * 128), da, db, idesc_s, kk > 0);
-          }
+          for (int kk = 0; kk < D / 16; ++kk)
+            umma_bf16(tmem + (uint32_t)(buf * 128), desc64(q0 + ((uint32_t)((kk >> 2) * A_SLAB + (kk & 3) * 32) >> 4)),
+                      desc64(k0 + ((uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4)), idesc_s, kk > 0);
           umma_commit(&s_full[buf]);
         }
+        __syncwarp();
         const bool last = (jt == inf.ntiles - 1);
         last_bits = (last_bits & ~(1u << (s_it & 31))) | ((last ? 1u : 0u) << (s_it & 31));
         ++s_it;
@@ -1137,7 +1135,9 @@ pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant_
 
 // ------------------------------------------------------------------ small SIMT stages
 
-// Final Select_K of the two-stage schedule (Algorithm 1): the candidates are the children of the
+// Final Select_K of the two-stage schedule (Algorithm 1) by a warp per token, for groups of more than four heads (a thread
+// per token, qm_select.cuh, would read its candidates' scores 64 bytes at a time from rows of a kilobyte: 0.35 ms against
+// 0.07 at 65536 tokens, 2 KV heads of 16 query heads, K = 8): the candidates are the children of the
 // kept level-2 nodes; grouped score = sum of the per-head leaf LSEs; forced leaves kept unscored.
 // Also emits the softmax denominator of the kept leaves per query head (their LSEs are known).
 __global__ void __launch_bounds__(128) final_topk_kernel(Geometry geo, const int32_t* __restrict__ par,
@@ -1630,8 +1630,11 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
   int32_t* par = (int32_t*)(ws + L.par);
   float* blk = (float*)(ws + L.blk);
   kernel_mark("route_stage1", s);
-  int st = route_stage1_mma_supported(g, dtype) ? launch_route_stage1_mma(g, q, pyramid, par, margin, s)
-                                                : launch_route_stage1_simt(g, dtype, q, pyramid, par, margin, s);
+  // the leaf scores' region is free until the leaf level: the node table of a range of tokens goes there
+  int st = qm_stage1_preferred(g, dtype, L.inv.count - L.blk)
+               ? qm_stage1(g, q, pyramid, par, margin, blk, L.inv.count - L.blk, status, s)
+           : route_stage1_mma_supported(g, dtype) ? launch_route_stage1_mma(g, q, pyramid, par, margin, s)
+                                                  : launch_route_stage1_simt(g, dtype, q, pyramid, par, margin, s);
   if (st != PISA_OK) return st;
   kernel_mark("invert_by_parent", s);
   InvArgs inv;
@@ -1648,9 +1651,13 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
   kernel_mark("final_topk", s);
   // only the LSE scores are also the per-leaf softmax denominators the attention stage can reuse
   const bool lse_scores = g.score_mode == PISA_SCORE_LSE;
-  final_topk_kernel<<<dim3((unsigned)((g.N + 3) / 4), (unsigned)(g.B * g.Hkv)), 128, 0, s>>>(
-      g, par, blk, idx, margin, lse_scores ? lse_out : nullptr, lse_scores ? sel_lse : nullptr, status);
-  st = check_launch("final_topk");
+  if (g.G <= 4) {
+    st = qm_select_final(g, par, blk, idx, margin, lse_scores ? lse_out : nullptr, lse_scores ? sel_lse : nullptr, status, s);
+  } else {
+    final_topk_kernel<<<dim3((unsigned)((g.N + 3) / 4), (unsigned)(g.B * g.Hkv)), 128, 0, s>>>(
+        g, par, blk, idx, margin, lse_scores ? lse_out : nullptr, lse_scores ? sel_lse : nullptr, status);
+    st = check_launch("final_topk");
+  }
   if (st != PISA_OK || sel_lse == nullptr || lse_scores) return st;
   // the other score modes rank by moments of the logits: the denominators take a pass of their own
   kernel_mark("sel_lse", s);
