@@ -192,7 +192,10 @@ int pisa_forward(const pisa_params_t* p, const void* q, const void* k, const voi
  *   lse         : device float, sequence-major: sequence i's [Hq, len_i] block starts at Hq * cu[i]
  *   ws          : device workspace sized for PISA_OP_FORWARD_PACKED with p (N = the longest sequence)
  *
- * Launches.  The method is causal (Sec. 3.2: a query only ever scores nodes that lie wholly in its
+ * Launches.  With a workspace sized for PISA_OP_FORWARD_PACKED all sequences short enough for the query-major kernels
+ * (bf16, LSE score, fan-in 2 or 4, C of 64 or 128; K * 704 .. 2048 tokens, by leaf size and heads per group) run unpadded
+ * through as few sets of launches as the workspace has room for their score tables.  For the others: the method is causal
+ * (Sec. 3.2: a query only ever scores nodes that lie wholly in its
  * past; the nodes on its own path are forced, not scored), so a sequence gives the same rows when it is
  * the head of a longer, zero-filled batch element.  Sequences of at most 8192 tokens are therefore
  * grouped by length (a group's members are no shorter than 3/4 of its padded length, padded lengths come
@@ -204,7 +207,8 @@ int pisa_forward(const pisa_params_t* p, const void* q, const void* k, const voi
  * the fp32 partial sums).
  */
 /*
- * The grouping pisa_forward_packed applies, as host arithmetic only (no GPU work, nothing allocated on the
+ * The grouping into padded batches (pisa_bsa_bwd_packed's, and pisa_forward_packed's for what the query-major kernels do
+ * not take), as host arithmetic only (no GPU work, nothing allocated on the
  * device): for sequence i, group[i] = the padded batch it runs in (0, 1, ... in launch order) and
  * padded[i] = that batch's padded length; group[i] = -1 (padded[i] = its own length) for a sequence that
  * runs alone -- longer than 8192 tokens, alone in its length class, or empty.

@@ -668,7 +668,29 @@ static size_t forward_ws_bytes(const pisa_params_t* p, const Geometry& g, int* s
   return f;
 }
 
+// The arena queries walk every padded length (a few hundred microseconds of host time), and a program asks with the
+// same parameters on every call: the last answers are kept, per host thread.
+extern "C++" {
+template <typename Arena>
+struct ArenaMemo {
+  static constexpr int kEntries = 4;
+  struct Entry { pisa_params_t p; int chunks; bool used; Arena a; } e[kEntries];
+  int next;
+  bool find(const pisa_params_t* p, int chunks, Arena* a) const {
+    for (int i = 0; i < kEntries; ++i)
+      if (e[i].used && e[i].chunks == chunks && memcmp(&e[i].p, p, sizeof(*p)) == 0) { *a = e[i].a; return true; }
+    return false;
+  }
+  void keep(const pisa_params_t* p, int chunks, const Arena& a) {
+    Entry& x = e[next++ % kEntries];
+    x.p = *p; x.chunks = chunks; x.a = a; x.used = true;
+  }
+};
+}
+static thread_local ArenaMemo<PackedArena> g_packed_memo = {};
+
 static int packed_arena(const pisa_params_t* p, PackedArena* a) {
+  if (g_packed_memo.find(p, g_chunk_limit, a)) return PISA_OK;
   Geometry g;
   int st = resolve(p, &g);
   if (st != PISA_OK) return st;
@@ -700,6 +722,7 @@ static int packed_arena(const pisa_params_t* p, PackedArena* a) {
   a->lb = align_up(tok * g.Hq * sizeof(float), 256);
   a->ib = align_up(tok * g.Hkv * g.K * sizeof(int32_t), 256);
   a->total = a->fwd + a->pyr + 2 * a->qb + 2 * a->kb + a->lb + a->ib;
+  g_packed_memo.keep(p, g_chunk_limit, *a);
   return PISA_OK;
 }
 
@@ -709,7 +732,10 @@ struct PackedBwdArena {
   long long tokens;
   size_t bwd, qb, kb, lb, ib, total;
 };
+static thread_local ArenaMemo<PackedBwdArena> g_packed_bwd_memo = {};
+
 static int packed_bwd_arena(const pisa_params_t* p, PackedBwdArena* a) {
+  if (g_packed_bwd_memo.find(p, g_chunk_limit, a)) return PISA_OK;
   Geometry g;
   int st = resolve(p, &g);
   if (st != PISA_OK) return st;
@@ -747,6 +773,7 @@ static int packed_bwd_arena(const pisa_params_t* p, PackedBwdArena* a) {
   a->lb = align_up(tok * g.Hq * sizeof(float), 256);
   a->ib = align_up(tok * g.Hkv * g.K * sizeof(int32_t), 256);
   a->total = a->bwd + 4 * a->qb + 4 * a->kb + a->lb + a->ib;
+  g_packed_bwd_memo.keep(p, g_chunk_limit, *a);
   return PISA_OK;
 }
 
@@ -754,14 +781,15 @@ static int packed_bwd_arena(const pisa_params_t* p, PackedBwdArena* a) {
 // longest first (nseq + 1 ints of scratch); group[i] / padded[i] for sequence i: its group (0, 1, ... in launch
 // order) and the group's padded length, or group -1 for a sequence that runs alone (longer than kPackDirectLen, the
 // only one of its length class, or empty: padded = its own length).  Returns the number of groups.
+// skip (nullable): sequences another path has taken; they are left out as empty ones are.
 static int packed_plan(const pisa_params_t* p, const int32_t* cu, int nseq, long long tokens, int* order,
-                       int32_t* group, int32_t* padded) {
+                       int32_t* group, int32_t* padded, const uint8_t* skip = nullptr) {
   size_t n_short = 0;
   for (int i = 0; i < nseq; ++i) {
     const int len = cu[i + 1] - cu[i];
     group[i] = -1;
     padded[i] = len;
-    if (len > 0 && len <= kPackDirectLen) order[n_short++] = i;
+    if (len > 0 && len <= kPackDirectLen && !(skip && skip[i])) order[n_short++] = i;
   }
   std::stable_sort(order, order + n_short, [&](int a, int b) { return cu[a + 1] - cu[a] > cu[b + 1] - cu[b]; });
   int n_groups = 0;
@@ -962,15 +990,36 @@ int pisa_forward_packed(const pisa_params_t* p, const int32_t* cu_seqlens, int32
   std::unique_ptr<int[]> order(new (std::nothrow) int[(size_t)nseq + 1]);
   std::unique_ptr<int32_t[]> group(new (std::nothrow) int32_t[(size_t)nseq + 1]);
   std::unique_ptr<int32_t[]> padded(new (std::nothrow) int32_t[(size_t)nseq + 1]);
-  if (!order || !group || !padded) return PISA_ERR_INVALID_ARG;
-  packed_plan(p, cu_seqlens, nseq, pa.tokens, order.get(), group.get(), padded.get());
+  std::unique_ptr<uint8_t[]> taken(new (std::nothrow) uint8_t[(size_t)nseq + 1]);
+  std::unique_ptr<int[]> ids(new (std::nothrow) int[(size_t)nseq + 1]);
+  if (!order || !group || !padded || !taken || !ids) return PISA_ERR_INVALID_ARG;
+  // sequences short enough for the query-major kernels: all of them in as few launches as the workspace has room for
+  int n_dense = 0;
+  for (int i = 0; i < nseq; ++i) {
+    const int len = cu_seqlens[i + 1] - cu_seqlens[i];
+    taken[i] = 0;
+    if (len == 0) continue;
+    pisa_params_t pi = *p;
+    pi.N = len;
+    Geometry gi;
+    if ((st = resolve(&pi, &gi)) != PISA_OK) return st;
+    if (!prefers_dense(&pi, gi) || kStatusBytes + qm_packed_bytes(gi, len) > ws_bytes) continue;
+    taken[i] = 1;
+    ids[n_dense++] = i;
+  }
+  if (n_dense > 0) {
+    st = qm_forward_packed(g, cu_seqlens, ids.get(), n_dense, cu_seqlens[nseq], q, k, v, idx, out, lse, base + kStatusBytes,
+                           ws_bytes - kStatusBytes, (int32_t*)ws, s);
+    if (st != PISA_OK || n_dense == nseq) return st;
+  }
+  packed_plan(p, cu_seqlens, nseq, pa.tokens, order.get(), group.get(), padded.get(), taken.get());
   for (int i = 0; i < nseq; ++i)
-    if (group[i] < 0 && (st = run_alone(i)) != PISA_OK) return st;
+    if (group[i] < 0 && !taken[i] && (st = run_alone(i)) != PISA_OK) return st;
   // `order` lists the grouped candidates longest first; the members of a group are consecutive in it
   size_t n_short = 0;
   for (int i = 0; i < nseq; ++i) {
     const int len = cu_seqlens[i + 1] - cu_seqlens[i];
-    if (len > 0 && len <= kPackDirectLen) ++n_short;
+    if (len > 0 && len <= kPackDirectLen && !taken[i]) ++n_short;
   }
   size_t at = 0;
   while (at < n_short) {

@@ -103,10 +103,10 @@ __global__ void __launch_bounds__(kSelThreads) qm_select_kernel(Geometry geo, qm
     int lo = 0, hi = a.nseq;                                      // sequences in order of their first token
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
-      if (a.seqs[mid].cu - a.seqs[0].cu <= r) lo = mid; else hi = mid;
+      if (a.seqs[mid].row0 <= r) lo = mid; else hi = mid;
     }
     q = a.seqs[lo];
-    t = (int)(r - (q.cu - a.seqs[0].cu));
+    t = (int)(r - q.row0);
     if (t >= q.len) return;
   }
   const int len = q.len, c = t >> lgC;

@@ -33,3 +33,40 @@ def test_forward_matches_the_oracle(shape):
     tri = S.sample_queries(w, 24, B=B)
     last = np.array([[b, h, p] for b in range(B) for h in range(Hkv) for p in {N - 1, max(N - 2, 0), 0}])
     T.check_forward_dev(dev, T.oracle_problem(w, t), np.concatenate([tri, last]))
+
+
+def test_packed_sequences_do_not_see_their_neighbours():
+    """Packed sequences share the TMA tiles of their last keys with the next sequence: whatever lies there, NaN and
+    infinities included, must not reach a row.  Lengths around tile and step edges, one set of launches for all."""
+    import torch
+    import paper_2609_31093_b200 as P
+    from paper_2609_31093_b200 import binding as PB
+    lens = [127, 1, 128, 129, 255, 64, 1000, 63, 31, 640]
+    Hq, Hkv, d, C, g, K = 8, 2, 128, 64, 2, 4
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    total = int(cu[-1])
+    w = S.Workload("qm_nan", 1, total, Hq, Hkv, d, C, g, K, "bf16", 1790, "iid")
+    t = S.make_inputs(w)
+    q, k, v = (T.to_torch(t[x][0], "bf16") for x in ("q", "k", "v"))
+    p = P.Params(1, max(lens), Hq, Hkv, d, C, g, K, dtype="bf16")
+    pyramid, ws = PB.alloc_pyramid(p), PB.alloc_workspace(p, PB.OP_FORWARD_PACKED)
+
+    def run():
+        idx = torch.full((Hkv * K * total,), -7, dtype=torch.int32, device="cuda")
+        out, lse = torch.zeros_like(q), torch.zeros((Hq * total,), dtype=torch.float32, device="cuda")
+        P.pisa_forward_packed(p, cu.tolist(), q, k, v, pyramid, idx, out, lse, ws)
+        torch.cuda.synchronize()
+        assert P.read_status(ws) == 0
+        return idx, out, lse
+
+    clean = run()
+    for i in range(1, len(lens), 2):                       # every second sequence turns into NaN and infinity
+        for x in (q, k, v):
+            x[cu[i]:cu[i + 1]] = float("nan")
+            x[cu[i]:cu[i] + 1] = float("inf")
+    dirty = run()
+    for i in range(0, len(lens), 2):
+        a, b = int(cu[i]), int(cu[i + 1])
+        assert torch.equal(dirty[0][Hkv * K * a:Hkv * K * b], clean[0][Hkv * K * a:Hkv * K * b]), i
+        assert torch.equal(dirty[1][a:b], clean[1][a:b]), i
+        assert torch.equal(dirty[2][Hq * a:Hq * b], clean[2][Hq * a:Hq * b]), i
