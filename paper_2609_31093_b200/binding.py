@@ -1,6 +1,7 @@
 """ctypes binding with the C ABI's names (include/pisa.h).  No arithmetic happens here."""
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
 from typing import Optional, Tuple
@@ -129,11 +130,26 @@ class Params:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# The current stream's handle without a Stream object per call (a decoding step's host side is about 10 us in all).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
+
+
+def _offsets(cu_seqlens):
+    """Host offsets as a C int32 array."""
+    try:
+        a = array.array("i", cu_seqlens)
+    except TypeError:                        # offsets that are not integers by type
+        a = array.array("i", [int(x) for x in cu_seqlens])
+    return (C.c_int32 * len(a)).from_buffer(a)
 
 
 def pyramid_layout(p: Params) -> Tuple[int, list, list, int]:
@@ -197,7 +213,7 @@ def pisa_forward(p: Params, q, k, v, pyramid, idx, out, lse, ws):
 
 def pisa_forward_packed(p: Params, cu_seqlens, q, k, v, pyramid, idx, out, lse, ws):
     """Packed variable-length batch; cu_seqlens is a host sequence of nseq + 1 offsets, p.N the longest length."""
-    cu = (C.c_int32 * len(cu_seqlens))(*[int(x) for x in cu_seqlens])
+    cu = _offsets(cu_seqlens)
     _check(lib().pisa_forward_packed(p.ref(), cu, len(cu_seqlens) - 1, _ptr(q), _ptr(k), _ptr(v), _ptr(pyramid),
                                      _ptr(idx), _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), _stream()),
            "pisa_forward_packed")
@@ -206,7 +222,7 @@ def pisa_forward_packed(p: Params, cu_seqlens, q, k, v, pyramid, idx, out, lse, 
 def packed_plan(p: Params, cu_seqlens):
     """Host-only: (group, padded, n_groups) of pisa_forward_packed's grouping; group -1 = the sequence runs alone."""
     n = len(cu_seqlens) - 1
-    cu = (C.c_int32 * len(cu_seqlens))(*[int(x) for x in cu_seqlens])
+    cu = _offsets(cu_seqlens)
     group, padded, ng = (C.c_int32 * max(n, 1))(), (C.c_int32 * max(n, 1))(), C.c_int32(0)
     _check(lib().pisa_packed_plan(p.ref(), cu, n, group, padded, C.byref(ng)), "pisa_packed_plan")
     return list(group)[:n], list(padded)[:n], int(ng.value)
@@ -229,7 +245,7 @@ def pisa_bsa_bwd(p: Params, q, k, v, idx, out, lse, dout, dq, dk, dv, ws):
 
 def pisa_bsa_bwd_packed(p: Params, cu_seqlens, q, k, v, idx, out, lse, dout, dq, dk, dv, ws):
     """pisa_bsa_bwd over a packed variable-length batch laid out as for pisa_forward_packed."""
-    cu = (C.c_int32 * len(cu_seqlens))(*[int(x) for x in cu_seqlens])
+    cu = _offsets(cu_seqlens)
     _check(lib().pisa_bsa_bwd_packed(p.ref(), cu, len(cu_seqlens) - 1, _ptr(q), _ptr(k), _ptr(v), _ptr(idx),
                                      _ptr(out), _ptr(lse), _ptr(dout), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(ws),
                                      ws.numel(), _stream()), "pisa_bsa_bwd_packed")

@@ -29,6 +29,7 @@
 
 #include <math_constants.h>
 
+#include "launch.cuh"
 #include "lse_chunk.cuh"
 #include "mma_frag.cuh"
 #include "pisa_common.cuh"
@@ -265,6 +266,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
   const int gid = lane >> 2, tig = lane & 3;
   const int rank = blockIdx.x;                            // cluster spans the x dimension
   const int bh = blockIdx.y;
+  grid_dependency();
   if (bh >= a.units) {                                    // a refreshing cluster: none of its CTAs meets a cluster barrier
     const int u = ((bh - a.units) * CLU + rank) * kDecWarps + warp;
     if (u < a.units) refresh_path<D>(geo, a, u / geo.Hkv, u % geo.Hkv, lane);
@@ -632,13 +634,13 @@ inline int refresh_clusters(long long units, int clu) { return (int)((units + kD
 
 template <int D, int NG, int MINB, int CLU, bool MOM>
 int launch_decode(const Geometry& g, const DecArgs& a, cudaStream_t s) {
-  auto kern = decode_step_kernel<D, NG, decode_piece(NG, MINB), MINB, CLU, MOM>;
-  const size_t smem = decode_smem<D, NG>();
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && CLU > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) { record_cuda_error("decode_step attr", e); return PISA_ERR_CUDA; }
-  kern<<<dim3(CLU, (unsigned)(a.units + refresh_clusters(a.units, CLU))), kDecThreads, smem, s>>>(g, a);
-  return check_launch("decode_step");
+  constexpr auto kern = decode_step_kernel<D, NG, decode_piece(NG, MINB), MINB, CLU, MOM>;
+  if (CLU > 8) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) { record_cuda_error("decode_step attr", e); return PISA_ERR_CUDA; }
+  }
+  return launch_dependent<kern>("decode_step", dim3(CLU, (unsigned)(a.units + refresh_clusters(a.units, CLU))), kDecThreads,
+                                decode_smem<D, NG>(), s, g, a);
 }
 // How many clusters of this instantiation the GPU holds at once (clusters are placed inside one GPC, so
 // this is less than SMs * MINB / CLU); asked of the driver once per instantiation.
@@ -647,8 +649,8 @@ int resident_clusters() {
   static int cached = -1;
   if (cached >= 0) return cached;
   const size_t smem = decode_smem<D, NG>();
-  auto kern = decode_step_kernel<D, NG, decode_piece(NG, 1), 1, CLU, false>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr auto kern = decode_step_kernel<D, NG, decode_piece(NG, 1), 1, CLU, false>;
+  allow_smem<kern>(smem);
   if (CLU > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     cached = 0;

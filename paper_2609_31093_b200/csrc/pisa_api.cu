@@ -520,12 +520,10 @@ static int do_forward(const pisa_params_t* p, const Geometry& g, const void* q, 
   ForwardPlan pl;
   int st = plan_for(p, g, kOpRoute | kOpBsa, ws_bytes, &pl);
   if (st != PISA_OK) return st;
-  st = clear ? clear_status(ws, s) : PISA_OK;
-  if (st != PISA_OK) return st;
   g_mark_n = 0;
   stage_mark(0, s);
   kernel_mark("pyramid", s);
-  st = launch_pyramid(g, p->dtype, k, pyr, (int32_t*)ws, s);
+  st = launch_pyramid(g, p->dtype, k, pyr, clear ? (int32_t*)ws : nullptr, s);
   if (st != PISA_OK) return st;
   stage_mark(1, s);
   if (pl.n == 1) {

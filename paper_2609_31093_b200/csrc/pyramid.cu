@@ -9,6 +9,7 @@
 // or by the first launch).  Tile loads by the TMA engine were measured for the level-1 slabs (one
 // 4-D tile of C rows x d*2 bytes per leaf, four 32 KB stages per SM) and were slower than plain
 // 16-byte loads: rows of 256 bytes cost the engine a request each.
+#include "launch.cuh"
 #include "pisa_common.cuh"
 
 namespace pisa {
@@ -19,7 +20,12 @@ constexpr int kSubMaxLeaves = 8;
 constexpr int kSubRowGroups = 16;
 template <typename T>
 __global__ void __launch_bounds__(256) pyramid_subtree_kernel(Geometry geo, const T* __restrict__ k,
-                                                              T* __restrict__ pyr, int s_levels, int span) {
+                                                              T* __restrict__ pyr, int s_levels, int span,
+                                                              int32_t* clear) {
+  grid_dependency();
+  // the first kernel of a forward clears the workspace's status word (a memset of its own costs 3 us)
+  if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < kStatusBytes / 16)
+    reinterpret_cast<uint4*>(clear)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
   constexpr int V = Elem<T>::kVec;
   __shared__ float red[kSubRowGroups][128];
   __shared__ float node[2][kSubMaxLeaves][128];      // stored values of the level being pooled / produced
@@ -96,6 +102,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) pyramid_upper_kernel(Geometry geo, T* __restrict__ pyr, int first_level) {
   constexpr int V = Elem<T>::kVec;
   extern __shared__ uint4 s_rows[];                  // [rows of the level below] | [rows of the level being pooled]
+  grid_dependency();
   const int cx = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int M0 = geo.M[first_level - 1];
   uint4* src = s_rows;
@@ -134,6 +141,7 @@ __global__ void __launch_bounds__(256) pyramid_upper_kernel(Geometry geo, T* __r
 // ... the same without the copy in shared memory, for levels that do not fit
 template <typename T>
 __global__ void __launch_bounds__(256) pyramid_upper_global_kernel(Geometry geo, T* __restrict__ pyr, int first_level) {
+  grid_dependency();
   constexpr int V = Elem<T>::kVec;
   const int cx = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   for (int l = first_level; l <= geo.L; ++l) {
@@ -159,7 +167,7 @@ __global__ void __launch_bounds__(256) pyramid_upper_global_kernel(Geometry geo,
 }
 
 template <typename T>
-static int launch_pyramid_t(const Geometry& g, const T* k, T* pyr, cudaStream_t s) {
+static int launch_pyramid_t(const Geometry& g, const T* k, T* pyr, int32_t* clear, cudaStream_t s) {
   constexpr int V = Elem<T>::kVec;
   const int chunks = g.d / V;
   if (g.d > 128 || chunks * 8 > 256) return PISA_ERR_UNSUPPORTED;
@@ -174,24 +182,22 @@ static int launch_pyramid_t(const Geometry& g, const T* k, T* pyr, cudaStream_t 
     ++s_levels;
   }
   dim3 grid1((g.M[1] + span - 1) / span, g.Hkv, g.B);
-  pyramid_subtree_kernel<T><<<grid1, threads, 0, s>>>(g, k, pyr, s_levels, span);
-  int st = check_launch("pyramid_subtree");
+  int st = launch_dependent<pyramid_subtree_kernel<T>>("pyramid_subtree", grid1, (unsigned)threads, 0, s, g, k, pyr, s_levels, span, clear);
   if (st != PISA_OK) return st;
   if (g.L >= 2 + s_levels) {
     dim3 grid2(chunks, g.Hkv, g.B);
     const int rows = g.M[1 + s_levels];
-    if (rows <= kUpperRows) pyramid_upper_kernel<T><<<grid2, 256, (size_t)(rows + g.M[2 + s_levels]) * 16, s>>>(g, pyr, 2 + s_levels);
-    else pyramid_upper_global_kernel<T><<<grid2, 256, 0, s>>>(g, pyr, 2 + s_levels);
-    st = check_launch("pyramid_upper");
+    st = rows <= kUpperRows
+             ? launch_dependent<pyramid_upper_kernel<T>>("pyramid_upper", grid2, 256u, (size_t)(rows + g.M[2 + s_levels]) * 16, s, g, pyr, 2 + s_levels)
+             : launch_dependent<pyramid_upper_global_kernel<T>>("pyramid_upper", grid2, 256u, 0, s, g, pyr, 2 + s_levels);
   }
   return st;
 }
 
-int launch_pyramid(const Geometry& g, int dtype, const void* k, void* pyramid, int32_t* status, cudaStream_t s) {
+int launch_pyramid(const Geometry& g, int dtype, const void* k, void* pyramid, int32_t* clear, cudaStream_t s) {
   if (dtype == PISA_BF16)
-    return launch_pyramid_t<__nv_bfloat16>(g, (const __nv_bfloat16*)k, (__nv_bfloat16*)pyramid, s);
-  (void)status;
-  return launch_pyramid_t<float>(g, (const float*)k, (float*)pyramid, s);
+    return launch_pyramid_t<__nv_bfloat16>(g, (const __nv_bfloat16*)k, (__nv_bfloat16*)pyramid, clear, s);
+  return launch_pyramid_t<float>(g, (const float*)k, (float*)pyramid, clear, s);
 }
 
 }  // namespace pisa

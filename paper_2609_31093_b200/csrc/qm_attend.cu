@@ -14,6 +14,7 @@
 // Measured at 8192 tokens, 16 KV heads, d = 128: P through shared memory with separate issuers took 2200 cycles per tile
 // and step with NT = 1 and NT = 2 alike (each product waited for the other's queue).
 // Every wait is bounded.
+#include "launch.cuh"
 #include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
 #include "query_major.cuh"
@@ -71,6 +72,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
   tcgen05_fence_before_sync();
   __syncthreads();
   tcgen05_fence_after_sync();
+  grid_dependency();
   const uint32_t tmem = tmem_slot;           // S / P buffers at columns 0 / 128, O buffers at 256 / 384
   const int lgC = a.lgC, lgG = a.lgG, G = geo.G, tpt = 128 >> lgG;
   constexpr int LPS = 128 / C;               // leaves per step
@@ -396,11 +398,8 @@ template <int D, int C, int NT>
 int launch_dcn(const Geometry& g, const qm::Args& a, const AttArgs& at, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                const CUtensorMap& tm_v, cudaStream_t s) {
   const size_t smem = (size_t)(D / 64) * (2 * NT + att_stages(D, NT)) * 128 * 128 + 1024;
-  cudaError_t e = cudaFuncSetAttribute(qm_attend_kernel<D, C, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) { record_cuda_error("qm_attend attr", e); return PISA_ERR_CUDA; }
   const int grid = a.n_items < num_sms() ? a.n_items : num_sms();
-  qm_attend_kernel<D, C, NT><<<grid, kAttThreads, smem, s>>>(g, a, at, tm_q, tm_k, tm_v);
-  return check_launch("qm_attend");
+  return launch_dependent<qm_attend_kernel<D, C, NT>>("qm_attend", dim3((unsigned)grid), kAttThreads, smem, s, g, a, at, tm_q, tm_k, tm_v);
 }
 template <int D, int C>
 int launch_dc(const Geometry& g, const qm::Args& a, const AttArgs& at, const CUtensorMap& tm_q, const CUtensorMap& tm_k,

@@ -6,6 +6,7 @@
 #include <memory>
 #include <new>
 
+#include "launch.cuh"
 #include "pisa_tensor.cuh"
 #include "query_major.cuh"
 
@@ -21,6 +22,7 @@ struct TableChunk {                       // a kernel parameter (16 KB): the tab
 };
 
 __global__ void __launch_bounds__(kChunkSeqs) qm_table_kernel(const __grid_constant__ TableChunk c, qm::Seq* seqs, qm::SeqOrder* order) {
+  grid_dependency();
   const int i = threadIdx.x;
   if (i < c.n) {
     seqs[c.first + i] = c.seq[i];
@@ -32,6 +34,7 @@ __global__ void __launch_bounds__(kChunkSeqs) qm_table_kernel(const __grid_const
 __global__ void __launch_bounds__(256) qm_packed_leaves_kernel(Geometry geo, const qm::Seq* seqs, int nseq, int lgC, int lgg,
                                                                const __nv_bfloat16* k, __nv_bfloat16* pyr) {
   __shared__ float red[16][128];
+  grid_dependency();
   const int h = blockIdx.y, d = geo.d, chunks = d / 8;
   int lo_s = 0, hi_s = nseq;
   while (hi_s - lo_s > 1) {
@@ -68,6 +71,7 @@ __global__ void __launch_bounds__(256) qm_packed_leaves_kernel(Geometry geo, con
 // the levels above, from shared memory: one CTA per (16-byte column chunk, KV head, sequence)
 __global__ void __launch_bounds__(128) qm_packed_levels_kernel(Geometry geo, const qm::Seq* seqs, int lgC, int lgg, __nv_bfloat16* pyr) {
   extern __shared__ uint4 s_rows[];
+  grid_dependency();
   const qm::Seq q = seqs[blockIdx.z];
   const int cx = blockIdx.x, h = blockIdx.y, d = geo.d;
   const int top = qm::top_level(q.len, lgC, lgg, geo.K);           // scores need the levels below it
@@ -207,18 +211,19 @@ int qm_forward_packed(const Geometry& g, const int32_t* cu, const int* ids, int 
         chunk->order[i].seq = by_len[i0 + i];
         chunk->order[i].item0 = item0[i0 + i];
       }
-      qm_table_kernel<<<1, kChunkSeqs, 0, s>>>(*chunk, d_seqs, d_order);
-      if ((st = check_launch("qm_table")) != PISA_OK) return st;
+      st = launch_dependent<qm_table_kernel>("qm_table", dim3(1), kChunkSeqs, 0, s, *chunk, d_seqs, d_order);
+      if (st != PISA_OK) return st;
     }
     // summaries of the levels that scores read (none when no sequence prunes above its leaves)
     if (deepest >= 2) {
       kernel_mark("qm_packed_pyramid", s);
-      qm_packed_leaves_kernel<<<dim3((unsigned)leaves, (unsigned)g.Hkv), 256, 0, s>>>(g, d_seqs, m, lgC, lgg, (const __nv_bfloat16*)k, d_pyr);
-      if ((st = check_launch("qm_packed_leaves")) != PISA_OK) return st;
+      st = launch_dependent<qm_packed_leaves_kernel>("qm_packed_leaves", dim3((unsigned)leaves, (unsigned)g.Hkv), 256u, 0, s, g,
+                                                     (const qm::Seq*)d_seqs, m, lgC, lgg, (const __nv_bfloat16*)k, d_pyr);
+      if (st != PISA_OK) return st;
       if (deepest >= 3) {
-        qm_packed_levels_kernel<<<dim3((unsigned)(g.d / 8), (unsigned)g.Hkv, (unsigned)m), 128, (size_t)most_leaves * 2 * 16, s>>>(
-            g, d_seqs, lgC, lgg, d_pyr);
-        if ((st = check_launch("qm_packed_levels")) != PISA_OK) return st;
+        st = launch_dependent<qm_packed_levels_kernel>("qm_packed_levels", dim3((unsigned)(g.d / 8), (unsigned)g.Hkv, (unsigned)m), 128u,
+                                                       (size_t)most_leaves * 2 * 16, s, g, (const qm::Seq*)d_seqs, lgC, lgg, d_pyr);
+        if (st != PISA_OK) return st;
       }
     }
     kernel_mark("qm_score", s);

@@ -8,6 +8,7 @@
 // pipe -- and the 32 KB (d = 128) of keys from L2, which an SM takes in at about 22 bytes per clock.  One tile per load
 // (two CTAs per SM) ran at that rate, 1470 cycles per tile and step with the epilogue switched off; two tiles share a
 // load, one CTA of 20 warps per SM.  Short batches, whose pairs of tiles would not fill the SMs, keep one tile per CTA.
+#include "launch.cuh"
 #include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
 #include "query_major.cuh"
@@ -113,6 +114,7 @@ qm_score_kernel(Geometry geo, qm::Args a, const __grid_constant__ CUtensorMap tm
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int lgC = a.lgC, lgg = a.lgg, lgG = a.lgG, tpt = 128 >> lgG, G = geo.G;
+  grid_dependency();
   const qm::Tile tl = qm::locate(geo, a, blockIdx.x, NT);
   const int len = tl.q.len, h = tl.h, tile0 = tl.tile * tpt * NT;
   const int t_last = min(len, tile0 + NT * tpt) - 1;
@@ -262,10 +264,7 @@ template <int D, int C, int NT>
 int launch_dcn(const Geometry& g, const qm::Args& a, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                const CUtensorMap& tm_p, int n_items, cudaStream_t s) {
   const size_t smem = (size_t)(D / 64) * 128 * 128 * (NT + score_stages(D, NT)) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(qm_score_kernel<D, C, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) { record_cuda_error("qm_score attr", e); return PISA_ERR_CUDA; }
-  qm_score_kernel<D, C, NT><<<(unsigned)n_items, 128 + 256 * NT, smem, s>>>(g, a, tm_q, tm_k, tm_p);
-  return check_launch("qm_score");
+  return launch_dependent<qm_score_kernel<D, C, NT>>("qm_score", dim3((unsigned)n_items), 128 + 256 * NT, smem, s, g, a, tm_q, tm_k, tm_p);
 }
 template <int D, int C>
 int launch_dc(const Geometry& g, const qm::Args& a, const CUtensorMap& tm_q, const CUtensorMap& tm_k,

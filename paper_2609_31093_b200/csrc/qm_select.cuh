@@ -9,6 +9,7 @@
 
 #include <math_constants.h>
 
+#include "launch.cuh"
 #include "pisa_tensor.cuh"
 #include "query_major.cuh"
 
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kSelThreads) qm_select_kernel(Geometry geo, qm
   const int tid = threadIdx.x, K = geo.K;
   float* s_u = s_mem + tid;                                       // [NC][threads] scores of the level, candidate order
   int* s_kept = reinterpret_cast<int*>(s_mem + NC * kSelThreads) + tid;   // [2][K][threads] kept nodes, ping-pong
+  grid_dependency();
   if (a.ctr != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *a.ctr = 0;
   const int lgC = a.lgC, h = blockIdx.y;
   long long r = (long long)blockIdx.x * kSelThreads + tid;
@@ -299,8 +301,7 @@ template <int NC, int FAN, int G, int MODE>
 int launch_sel(const Geometry& g, const qm::Args& a, const SelArgs& sa, long long rows, cudaStream_t s) {
   const size_t smem = (size_t)kSelThreads * (NC + 2 * g.K) * 4;
   dim3 grid((unsigned)((rows + kSelThreads - 1) / kSelThreads), (unsigned)g.Hkv);
-  qm_select_kernel<NC, FAN, G, MODE><<<grid, kSelThreads, smem, s>>>(g, a, sa);
-  return check_launch("qm_select");
+  return launch_dependent<qm_select_kernel<NC, FAN, G, MODE>>("qm_select", grid, kSelThreads, smem, s, g, a, sa);
 }
 template <int NC, int FAN, int MODE>
 int launch_sel_g(const Geometry& g, const qm::Args& a, const SelArgs& sa, long long rows, cudaStream_t s) {
