@@ -37,12 +37,14 @@ struct BwdArgs {
   float* dk_acc;                  // [B, N, Hkv, D] fp32
   float* dv_acc;
   int32_t* status;
+  Gate gate;
 };
 
 // delta[b, hq, t] = sum_d dO[b,t,hq,d] * O[b,t,hq,d]; one warp per row
 __global__ void __launch_bounds__(256) bwd_delta_kernel(Geometry geo, const __nv_bfloat16* __restrict__ out,
                                                         const __nv_bfloat16* __restrict__ dout,
-                                                        float* __restrict__ delta) {
+                                                        float* __restrict__ delta, Gate gate) {
+  if (gate.off_list()) return;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const long long rows = (long long)geo.B * geo.N * geo.Hq;
@@ -61,7 +63,8 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(Geometry geo, const __nv
 // fp32 accumulator rows of `row2` element pairs, dense -> bf16 rows `dst_pitch2` pairs apart (a chunk of
 // KV heads writes its columns of the caller's [B, N, Hkv, d] tensor)
 __global__ void __launch_bounds__(256) bwd_convert_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst,
-                                                          long long n2, int row2, long long dst_pitch2) {
+                                                          long long n2, int row2, long long dst_pitch2, Gate gate) {
+  if (gate.off_list()) return;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n2) return;
   const float2 x = reinterpret_cast<const float2*>(src)[i];
@@ -99,6 +102,7 @@ __device__ __forceinline__ ItemInfo item_info_keys(const int32_t* item_key, cons
 
 template <int C, int DIN>
 __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, BwdArgs a) {
+  if (a.gate.off_list()) return;
   extern __shared__ uint8_t smem_raw[];
   constexpr int D = 128;                                    // staged (padded) head dimension
   constexpr int CHV = DIN / 8;

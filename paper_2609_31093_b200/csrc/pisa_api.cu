@@ -234,7 +234,7 @@ static int do_bsa(const pisa_params_t* p, const Geometry& g, const void* q, cons
   if (ws_bytes < bsa_ws_bytes(p, g)) return PISA_ERR_WORKSPACE_TOO_SMALL;
   if (use_tensor(p, g))
     return tensor_bsa(g, p->dtype, q, k, v, idx, sel_lse, out, lse, lse_ready, forced_present,
-                      (char*)ws + kStatusBytes, (int32_t*)ws, s);
+                      (char*)ws + kStatusBytes, (int32_t*)ws, Gate{nullptr, 0u}, s);
   kernel_mark("bsa_simt", s);
   return launch_bsa_simt(g, p->dtype, q, k, v, idx, out, lse, s);
 }
@@ -483,7 +483,7 @@ static int do_bsa_chunked(const pisa_params_t* p, const Geometry& g, const void*
     st = run_chunks(p, g, pl, ws, s, [&](const ChunkView& v, int) {
       return tensor_bsa(v.g, p->dtype, (const char*)q + v.q_off, (const char*)k + v.k_off, (const char*)v_ + v.v_off,
                         idx + v.unit0 * g.N * g.K, sel_lse ? sel_lse + v.unit0 * g.G * g.N * g.K : nullptr,
-                        (char*)out + v.o_off, lse + v.unit0 * g.G * g.N, false, false, v.region, (int32_t*)ws, v.stream);
+                        (char*)out + v.o_off, lse + v.unit0 * g.G * g.N, false, false, v.region, (int32_t*)ws, Gate{nullptr, 0u}, v.stream);
     });
   kernel_mark("end", s);
   return st;
@@ -493,22 +493,32 @@ static int do_bsa_chunked(const pisa_params_t* p, const Geometry& g, const void*
 static int do_bwd(const pisa_params_t* p, const Geometry& g, const void* q, const void* k, const void* v_,
                   const int32_t* idx, const void* out, const float* lse, const void* dout, void* dq, void* dk,
                   void* dv, void* ws, size_t ws_bytes, cudaStream_t s) {
+  const bool dense = qm_bwd_supported(g, p->dtype);
+  if (dense && g.N <= qm_bwd_always(g) && ws_bytes >= kStatusBytes + qm_bwd_workspace_bytes(g))
+    return qm_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, (char*)ws + kStatusBytes, (int32_t*)ws, nullptr, s);
   ForwardPlan pl;
   int st = plan_for(p, g, kOpBwd, ws_bytes, &pl);
   if (st != PISA_OK) return st;
+  // longer sequences: the rows decide on the device (how many key blocks the tiles of neighbouring rows need in all)
+  Gate gate = {nullptr, 0u};
+  const size_t list_bytes = align_up(pl.total, 256);
+  if (dense && ws_bytes >= list_bytes + qm_bwd_workspace_bytes(g)) {
+    st = qm_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, (char*)ws + list_bytes, (int32_t*)ws, &gate, s);
+    if (st != PISA_OK) return st;
+  }
   const size_t es = elem_size(p->dtype);
   const long long dqs[3] = {(long long)g.N * g.Hq * g.d, (long long)g.Hq * g.d, g.d};
   const long long pitch = (long long)g.Hkv * g.d;
   if (pl.n == 1)
     return tensor_bsa_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, dqs, pitch, (char*)ws + kStatusBytes,
-                          (int32_t*)ws, s);
+                          (int32_t*)ws, gate, s);
   return run_chunks(p, g, pl, ws, s, [&](const ChunkView& v, int) {
     const size_t dq_off = (size_t)((long long)v.c.b0 * dqs[0] + (long long)v.c.h0 * g.G * dqs[2]) * es;
     const size_t dkv_off = (size_t)((long long)v.c.b0 * g.N * pitch + (long long)v.c.h0 * g.d) * es;
     return tensor_bsa_bwd(v.g, (const char*)q + v.q_off, (const char*)k + v.k_off, (const char*)v_ + v.v_off,
                           idx + v.unit0 * g.N * g.K, (const char*)out + v.o_off, lse + v.unit0 * g.G * g.N,
                           (const char*)dout + v.o_off, (char*)dq + dq_off, (char*)dk + dkv_off, (char*)dv + dkv_off, dqs,
-                          pitch, v.region, (int32_t*)ws, v.stream);
+                          pitch, v.region, (int32_t*)ws, gate, v.stream);
   });
 }
 
@@ -553,7 +563,7 @@ static int do_forward(const pisa_params_t* p, const Geometry& g, const void* q, 
       if (i == 0) stage_mark(2, s);
       return tensor_bsa(v.g, p->dtype, (const char*)q + v.q_off, (const char*)k + v.k_off, (const char*)v_ + v.v_off,
                         ic, nullptr, (char*)out + v.o_off, lc, g.score_mode == PISA_SCORE_LSE, true, v.region, (int32_t*)ws,
-                        v.stream);
+                        Gate{nullptr, 0u}, v.stream);
     });
     if (st == PISA_OK && routed != nullptr) {             // (chunks: the indices count as final when all chunks have ended)
       const cudaError_t ee = cudaEventRecord(routed, s);
@@ -724,6 +734,22 @@ static int packed_arena(const pisa_params_t* p, PackedArena* a) {
   return PISA_OK;
 }
 
+// the backward of one problem: the list-driven kernels (in chunks), the dense ones, or both where the rows decide
+static int bwd_ws_bytes(const pisa_params_t* p, const Geometry& g, size_t* out) {
+  if (!tensor_bwd_supported(g, p->dtype) || p->impl == PISA_IMPL_SIMT) return PISA_ERR_UNSUPPORTED;
+  size_t b = kStatusBytes + tensor_bwd_workspace_bytes(g);
+  ForwardPlan pl;
+  const int r = forward_plan(p, g, kOpBwd, &pl);
+  if (r != PISA_OK) return r;
+  if (pl.total > b) b = pl.total;
+  if (qm_bwd_supported(g, p->dtype)) {
+    const size_t d = qm_bwd_workspace_bytes(g);
+    b = g.N <= qm_bwd_always(g) ? std::max(b, kStatusBytes + d) : align_up(b, 256) + d;
+  }
+  *out = b;
+  return PISA_OK;
+}
+
 // ... and what pisa_bsa_bwd_packed needs to run the same groups: the backward's workspace for any group, padded q /
 // out / dout / dq, k / v / dk / dv, lse and idx
 struct PackedBwdArena {
@@ -739,14 +765,7 @@ static int packed_bwd_arena(const pisa_params_t* p, PackedBwdArena* a) {
   if (st != PISA_OK) return st;
   a->tokens = kPackTokens;
   auto need = [](const pisa_params_t* pp, const Geometry& gg, size_t* out) -> int {
-    if (!tensor_bwd_supported(gg, pp->dtype) || pp->impl == PISA_IMPL_SIMT) return PISA_ERR_UNSUPPORTED;
-    size_t b = kStatusBytes + tensor_bwd_workspace_bytes(gg);
-    ForwardPlan pl;
-    const int r = forward_plan(pp, gg, kOpBwd, &pl);
-    if (r != PISA_OK) return r;
-    if (pl.total > b) b = pl.total;
-    *out = b;
-    return PISA_OK;
+    return bwd_ws_bytes(pp, gg, out);
   };
   size_t bwd = 0;
   if ((st = need(p, g, &bwd)) != PISA_OK) return st;
@@ -855,13 +874,7 @@ int pisa_workspace_bytes(const pisa_params_t* p, int op, size_t* bytes) {
     case PISA_OP_FORWARD: *bytes = f; break;
     case PISA_OP_FLAT: *bytes = kStatusBytes; break;
     case PISA_OP_BSA_BWD:
-      if (!tensor_bwd_supported(g, p->dtype) || p->impl == PISA_IMPL_SIMT) return PISA_ERR_UNSUPPORTED;
-      *bytes = kStatusBytes + tensor_bwd_workspace_bytes(g);
-      {
-        ForwardPlan pl;
-        if ((st = forward_plan(p, g, kOpBwd, &pl)) != PISA_OK) return st;
-        if (pl.total > *bytes) *bytes = pl.total;
-      }
+      if ((st = bwd_ws_bytes(p, g, bytes)) != PISA_OK) return st;
       break;
     case PISA_OP_DECODE:
       if (!decode_supported(g, p->dtype)) return PISA_ERR_UNSUPPORTED;
@@ -1259,10 +1272,31 @@ int pisa_bsa_bwd_packed(const pisa_params_t* p, const int32_t* cu_seqlens, int32
   std::unique_ptr<int[]> order(new (std::nothrow) int[(size_t)nseq + 1]);
   std::unique_ptr<int32_t[]> group(new (std::nothrow) int32_t[(size_t)nseq + 1]);
   std::unique_ptr<int32_t[]> padded(new (std::nothrow) int32_t[(size_t)nseq + 1]);
-  if (!order || !group || !padded) return PISA_ERR_INVALID_ARG;
-  packed_plan(p, cu_seqlens, nseq, pa.tokens, order.get(), group.get(), padded.get());
+  std::unique_ptr<uint8_t[]> taken(new (std::nothrow) uint8_t[(size_t)nseq + 1]);
+  std::unique_ptr<int[]> ids(new (std::nothrow) int[(size_t)nseq + 1]);
+  if (!order || !group || !padded || !taken || !ids) return PISA_ERR_INVALID_ARG;
+  // sequences short enough for the dense kernels: all of them in as few launches as the workspace has room for
+  int n_dense = 0;
+  for (int i = 0; i < nseq; ++i) {
+    const int len = cu_seqlens[i + 1] - cu_seqlens[i];
+    taken[i] = 0;
+    if (len == 0) continue;
+    pisa_params_t pi = *p;
+    pi.N = len;
+    Geometry gi;
+    if ((st = resolve(&pi, &gi)) != PISA_OK) return st;
+    if (!qm_bwd_supported(gi, p->dtype) || len > qm_bwd_always(gi) || kStatusBytes + qm_bwd_packed_bytes(gi, len) > ws_bytes) continue;
+    taken[i] = 1;
+    ids[n_dense++] = i;
+  }
+  if (n_dense > 0) {
+    st = qm_bwd_packed(g, cu_seqlens, ids.get(), n_dense, cu_seqlens[nseq], q, k, v, idx, out, lse, dout, dq, dk, dv,
+                       (char*)ws + kStatusBytes, ws_bytes - kStatusBytes, (int32_t*)ws, s);
+    if (st != PISA_OK) return st;
+  }
+  packed_plan(p, cu_seqlens, nseq, pa.tokens, order.get(), group.get(), padded.get(), taken.get());
   for (int i = 0; i < nseq; ++i)
-    if (group[i] < 0 && (st = run_alone(i, pa.bwd)) != PISA_OK) return st;
+    if (group[i] < 0 && !taken[i] && (st = run_alone(i, pa.bwd)) != PISA_OK) return st;
   char* q_pad = (char*)ws + pa.bwd;
   char* o_pad = q_pad + pa.qb;
   char* do_pad = o_pad + pa.qb;
@@ -1276,7 +1310,7 @@ int pisa_bsa_bwd_packed(const pisa_params_t* p, const int32_t* cu_seqlens, int32
   size_t n_short = 0;
   for (int i = 0; i < nseq; ++i) {
     const int len = cu_seqlens[i + 1] - cu_seqlens[i];
-    if (len > 0 && len <= kPackDirectLen) ++n_short;
+    if (len > 0 && len <= kPackDirectLen && !taken[i]) ++n_short;
   }
   size_t at = 0;
   while (at < n_short) {

@@ -26,6 +26,16 @@ struct Geometry {
   long long qs[3], ks[3], vs[3], os[3];  // element strides (b, n, h)
 };
 
+// Two ways to the same result whose costs depend on the data: the preparation counts the dense one's steps, both are
+// launched, and each kernel looks at the count first: dense kernels go on if it is at most `limit`, list-driven ones if it is
+// above (a null count: no such choice, go on).
+struct Gate {
+  const uint32_t* count;
+  uint32_t limit;
+  __device__ __forceinline__ bool off_dense() const { return count != nullptr && *count > limit; }
+  __device__ __forceinline__ bool off_list() const { return count != nullptr && *count <= limit; }
+};
+
 // Status word at the start of every workspace (device int32[4]; [0] = pisa_status).
 constexpr size_t kStatusBytes = 256;
 

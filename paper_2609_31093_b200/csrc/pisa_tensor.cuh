@@ -20,7 +20,7 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
 // served by the query-major local-window kernel instead of the lists
 int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const void* v, const int32_t* idx,
                const float* sel_lse, void* out, float* lse, bool lse_ready, bool forced_present, void* ws,
-               int32_t* status, cudaStream_t s);
+               int32_t* status, const Gate& gate, cudaStream_t s);
 
 // query-major path (query_major.cuh): dense scoring, one-thread-per-token selection, masked dense attention
 namespace qm { struct Args; }
@@ -57,10 +57,27 @@ int launch_qm_select_final(const Geometry& g, const qm::Args& a, long long rows,
 int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const void* k, const void* v, long long tokens,
                      const float* row_lse, void* out, cudaStream_t s);
 
+// dense masked backward (qm_bwd.cuh).  gate (nullable): the choice is left to the data; receives what the list-driven kernels
+// have to look at
+bool qm_bwd_supported(const Geometry& g, int dtype);
+size_t qm_bwd_workspace_bytes(const Geometry& g);
+int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx, const void* out, const float* lse,
+           const void* dout, void* dq, void* dk, void* dv, void* ws, int32_t* status, Gate* gate, cudaStream_t s);
+// length up to which the dense backward is the better one whatever the rows selected
+int qm_bwd_always(const Geometry& g);
+// packed batches: workspace one sequence needs, and the backward of the sequences ids[0..n)
+size_t qm_bwd_packed_bytes(const Geometry& g, int len);
+int qm_bwd_packed(const Geometry& g, const int32_t* cu, const int* ids, int n, long long total, const void* q, const void* k,
+                  const void* v, const int32_t* idx, const void* out, const float* lse, const void* dout, void* dq, void* dk,
+                  void* dv, void* ws, size_t ws_bytes, int32_t* status, cudaStream_t s);
+namespace qm { struct Seq; struct SeqOrder; }
+// a packed launch's table -> device, as kernel parameters
+int qm_write_table(const qm::Seq* seqs, const qm::SeqOrder* order, int n, qm::Seq* d_seqs, qm::SeqOrder* d_order, cudaStream_t s);
+
 // attention over the forced leaves, query-major (local_window.cu); stores the fp32 accumulator [B,Hkv,N,128,G]
 bool local_window_supported(const Geometry& g, int dtype);
 int launch_local_window(const Geometry& g, const void* q, const void* k, const void* v, const float* row_lse,
-                        float* o_acc, int32_t* status, cudaStream_t s);
+                        float* o_acc, int32_t* status, const Gate& gate, cudaStream_t s);
 
 // backward of the block-sparse attention with frozen indices; dq [B,N,Hq,d], dk, dv [B,N,Hkv,d] dense
 bool tensor_bwd_supported(const Geometry& g, int dtype);
@@ -69,6 +86,6 @@ size_t tensor_bwd_workspace_bytes(const Geometry& g);
 // (both describe the caller's dense tensors, of which a chunk of units writes its part)
 int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx,
                    const void* out, const float* lse, const void* dout, void* dq, void* dk, void* dv,
-                   const long long* dq_strides, long long dkv_pitch, void* ws, int32_t* status, cudaStream_t s);
+                   const long long* dq_strides, long long dkv_pitch, void* ws, int32_t* status, const Gate& gate, cudaStream_t s);
 
 }  // namespace pisa

@@ -135,6 +135,20 @@ constexpr size_t kFixedBytes = 4096;                       // alignment of the r
 
 }  // namespace
 
+int qm_write_table(const qm::Seq* seqs, const qm::SeqOrder* order, int n, qm::Seq* d_seqs, qm::SeqOrder* d_order, cudaStream_t s) {
+  std::unique_ptr<TableChunk> chunk(new (std::nothrow) TableChunk);
+  if (!chunk) return PISA_ERR_INVALID_ARG;
+  for (int i0 = 0; i0 < n; i0 += kChunkSeqs) {
+    chunk->first = i0;
+    chunk->n = std::min(kChunkSeqs, n - i0);
+    std::copy(seqs + i0, seqs + i0 + chunk->n, chunk->seq);
+    std::copy(order + i0, order + i0 + chunk->n, chunk->order);
+    const int st = launch_dependent<qm_table_kernel>("qm_table", dim3(1), kChunkSeqs, 0, s, *chunk, d_seqs, d_order);
+    if (st != PISA_OK) return st;
+  }
+  return PISA_OK;
+}
+
 size_t qm_packed_bytes(const Geometry& g, int len) { return kFixedBytes + bytes_of(g, need_of(g, len)); }
 
 // The sequences ids[0..n) (ascending) of a packed batch; g: the geometry of the call (heads, strides); every one of them

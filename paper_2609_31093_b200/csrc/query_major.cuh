@@ -29,7 +29,9 @@ struct Seq {
   int pyr_row;             // packed: row of the pyramid scratch its levels start at, level l = [Hkv][M_l] rows
   int row0, leaf0;         // packed: tokens / leaves of the launch's sequences before it
 };
-struct SeqOrder { int seq, item0; };   // work items of the packed launch: sequence, its first item (longest sequences first)
+// work items of the packed launch: sequence, its first item (longest sequences first); the backward's: groups of tiles in
+// item0, tiles in item0t, 128-key blocks in item0k
+struct SeqOrder { int seq, item0, item0t, item0k; };
 
 struct Args {
   const Seq* seqs;         // null: uniform batch

@@ -60,6 +60,7 @@ struct InvArgs {
   int32_t* work_ctr;      // next-work-item counter of the attention kernel that walks these lists (zeroed with count)
   int32_t* status;        // the workspace's status word
   int debug;              // PISA_DEBUG_* bits
+  Gate gate;
   int skip_forced;        // leave the row's forced leaves (0, c-1, c) out of the lists: the local-window kernel serves them
 };
 
@@ -75,6 +76,7 @@ __device__ __forceinline__ bool inv_valid(const InvArgs& a, int node, int t) {
 }
 
 __global__ void __launch_bounds__(256) inv_count_kernel(InvArgs a, int use_smem) {
+  if (a.gate.off_list()) return;
   extern __shared__ int s_hist[];
   const int bh = blockIdx.y;
   const int t0 = blockIdx.x * a.tok, t1 = min(t0 + a.tok, a.N);
@@ -133,6 +135,7 @@ __device__ __forceinline__ int3 block_scan3(int3 v, int3* s_w /* [32] */) {
   return v;
 }
 __global__ void __launch_bounds__(1024) inv_scan_blocks_kernel(InvArgs a) {
+  if (a.gate.off_list()) return;
   __shared__ int3 s_w[32];
   const int nkeys = a.BH * a.NW * a.Mk;
   const int nblk = (nkeys + 1023) / 1024;
@@ -149,6 +152,7 @@ __global__ void __launch_bounds__(1024) inv_scan_blocks_kernel(InvArgs a) {
 }
 // block totals -> exclusive block offsets (entry [nblk] = grand total); one CTA walks them 1024 at a time
 __global__ void __launch_bounds__(1024) inv_scan_totals_kernel(InvArgs a) {
+  if (a.gate.off_list()) return;
   __shared__ int3 s_w[32];
   const int nkeys = a.BH * a.NW * a.Mk;
   const int nblk = (nkeys + 1023) / 1024;
@@ -171,6 +175,7 @@ __global__ void __launch_bounds__(1024) inv_scan_totals_kernel(InvArgs a) {
   }
 }
 __global__ void __launch_bounds__(1024) inv_scan_fix_kernel(InvArgs a) {
+  if (a.gate.off_list()) return;
   const int nkeys = a.BH * a.NW * a.Mk;
   const int nblk = (nkeys + 1023) / 1024;
   const int i = blockIdx.x * 1024 + threadIdx.x;
@@ -192,6 +197,7 @@ __global__ void __launch_bounds__(1024) inv_scan_fix_kernel(InvArgs a) {
 // about 4 us with its launch gap: 12 us against 3 to 5 for up to kOneScanKeys lists).
 constexpr int kOneScanKeys = 4096;
 __global__ void __launch_bounds__(1024) inv_scan_one_kernel(InvArgs a) {
+  if (a.gate.off_list()) return;
   __shared__ int3 s_w[32];
   const int nkeys = a.BH * a.NW * a.Mk;
   int3 carry = make_int3(0, 0, 0);
@@ -212,6 +218,7 @@ __global__ void __launch_bounds__(1024) inv_scan_one_kernel(InvArgs a) {
 }
 
 __global__ void __launch_bounds__(256) inv_fill_kernel(InvArgs a, int use_smem) {
+  if (a.gate.off_list()) return;
   extern __shared__ int s_mem[];
   int* s_hist = s_mem;
   int* s_base = s_mem + a.Mk;
@@ -270,6 +277,7 @@ struct TileArgs {
   float* o_acc;            // fp32 accumulator: [B, Hkv, N, D, G] when the second product is transposed, else [B, N, Hq, D]
   int32_t* status;
   int debug;               // PISA_DEBUG_* bits: list entries are range-checked before they are used
+  Gate gate;
 };
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
@@ -767,6 +775,7 @@ template <int D, int C>
 __global__ void __launch_bounds__(kPvThreads, 1)
 pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v) {
+  if (a.gate.off_list()) return;
   extern __shared__ uint8_t smem_raw[];
   constexpr int NS = 4;
   constexpr int KS = D / 64;
@@ -1366,7 +1375,8 @@ __global__ void __launch_bounds__(256) row_lse_from_sel_kernel(Geometry geo, con
 
 // fp32 accumulator [B,N,Hq,d] -> out in bf16 (strided)
 __global__ void __launch_bounds__(256) convert_out_kernel(Geometry geo, const float* __restrict__ acc,
-                                                           __nv_bfloat16* __restrict__ out) {
+                                                           __nv_bfloat16* __restrict__ out, Gate gate) {
+  if (gate.off_list()) return;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;     // one 8-element chunk
   const int ch = geo.d / 8;
   const long long total = (long long)geo.B * geo.N * geo.Hq * ch;
@@ -1390,7 +1400,8 @@ __global__ void __launch_bounds__(256) convert_out_kernel(Geometry geo, const fl
 // One thread takes two consecutive d of one (b, t, KV head): 2*G contiguous floats in, one bf16x2 per
 // head out; a warp reads 64*G contiguous floats and writes 128 contiguous bytes per head row.
 __global__ void __launch_bounds__(256) convert_out_heads_inner_kernel(Geometry geo, const float* __restrict__ acc,
-                                                                       __nv_bfloat16* __restrict__ out) {
+                                                                       __nv_bfloat16* __restrict__ out, Gate gate) {
+  if (gate.off_list()) return;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;     // one pair of d
   const int pairs = geo.d / 2, G = geo.G;
   const long long total = (long long)geo.B * geo.N * geo.Hkv * pairs;
@@ -1458,8 +1469,9 @@ BsaLayout bsa_layout(const Geometry& g) {
 }
 
 int run_inversion(const Geometry& g, const int32_t* nodes, int fan, int Mk, char* ws, const InvLayout& l,
-                  InvArgs* out, int32_t* status, cudaStream_t s, int win = kWindowTok, int skip_forced = 0) {
+                  InvArgs* out, int32_t* status, cudaStream_t s, int win = kWindowTok, int skip_forced = 0, Gate gate = Gate{nullptr, 0u}) {
   InvArgs a;
+  a.gate = gate;
   a.status = status; a.debug = g.debug; a.skip_forced = skip_forced;
   a.nodes = nodes; a.K = g.K; a.fan = fan; a.Mk = Mk; a.N = g.N; a.C = g.C; a.BH = g.B * g.Hkv;
   a.tpt = 128 / g.G;
@@ -1582,6 +1594,22 @@ int dispatch_tile_pv(const Geometry& g, const TileArgs& a, int32_t* work_ctr, cu
 
 #include "bsa_bwd_kernel.cuh"
 
+// zeroes `bytes` (a multiple of 256) unless the gate says the list-driven kernels are off
+__global__ void __launch_bounds__(256) zero_kernel(uint4* p, long long n, Gate gate) {
+  if (gate.off_list()) return;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+int launch_zero(void* p, size_t bytes, const Gate& gate, cudaStream_t s) {
+  if (gate.count == nullptr) {
+    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, s);
+    if (e != cudaSuccess) { record_cuda_error("accumulator memset", e); return PISA_ERR_CUDA; }
+    return PISA_OK;
+  }
+  const long long n = (long long)(bytes / 16), blocks = (n + 255) / 256, cap = 8LL * num_sms();
+  zero_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, s>>>((uint4*)p, n, gate);
+  return check_launch("zero");
+}
+
 struct BwdLayout { size_t delta, dq, dk, dv, total; InvLayout inv; };
 BwdLayout bwd_layout(const Geometry& g) {
   BwdLayout r;
@@ -1666,7 +1694,7 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
 
 int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const void* v, const int32_t* idx,
                const float* sel_lse, void* out, float* lse, bool lse_ready, bool forced_present, void* ws_,
-               int32_t* status, cudaStream_t s) {
+               int32_t* status, const Gate& gate, cudaStream_t s) {
   (void)dtype;
   char* ws = (char*)ws_;
   const BsaLayout L = bsa_layout(g);
@@ -1678,13 +1706,13 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   // local-window kernel, which also initialises the accumulator (it needs the rows' denominators, so only
   // when the routing handed them over: the block-LSE pass below walks the very lists they are left out of)
   const bool local = forced_present && lse_ready && local_window_supported(g, dtype);
-  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kWindowTok, local ? 1 : 0);
+  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kWindowTok, local ? 1 : 0, gate);
   if (st != PISA_OK) return st;
   TileArgs a = {};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
   a.entry_off = inv.entry_off; a.tile_off = inv.tile_off; a.item_off = inv.item_off; a.item_key = inv.item_key; a.entries = inv.entries;
   a.nkeys = g.B * g.Hkv * inv.NW * g.M[1]; a.Mk = g.M[1]; a.NW = inv.NW; a.fan = 1; a.slots = g.K;
-  a.blk_lse = blk; a.row_lse = lse; a.o_acc = acc; a.status = status; a.debug = g.debug;
+  a.blk_lse = blk; a.row_lse = lse; a.o_acc = acc; a.status = status; a.debug = g.debug; a.gate = gate;
   if (!lse_ready && sel_lse != nullptr) {
     kernel_mark("row_lse", s);
     const long long rows = (long long)g.B * g.Hq * g.N;
@@ -1702,7 +1730,7 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   }
   if (local) {
     kernel_mark("local_window", s);
-    st = launch_local_window(g, q, k, v, lse, acc, status, s);
+    st = launch_local_window(g, q, k, v, lse, acc, status, gate, s);
     if (st != PISA_OK) return st;
   } else {
     kernel_mark("accumulator_memset", s);
@@ -1715,10 +1743,10 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   kernel_mark("convert_out", s);
   if (g.d == 128) {
     const long long n = (long long)g.B * g.N * g.Hkv * (g.d / 2);
-    convert_out_heads_inner_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out);
+    convert_out_heads_inner_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out, gate);
   } else {
     const long long n = (long long)g.B * g.N * g.Hq * (g.d / 8);
-    convert_out_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out);
+    convert_out_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out, gate);
   }
   return check_launch("convert_out");
 }
@@ -1737,12 +1765,12 @@ size_t tensor_bwd_workspace_bytes(const Geometry& g) { return bwd_layout(g).tota
 
 int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx,
                    const void* out, const float* lse, const void* dout, void* dq, void* dk, void* dv,
-                   const long long* dq_strides, long long dkv_pitch, void* ws_, int32_t* status, cudaStream_t s) {
+                   const long long* dq_strides, long long dkv_pitch, void* ws_, int32_t* status, const Gate& gate, cudaStream_t s) {
   char* ws = (char*)ws_;
   const BwdLayout L = bwd_layout(g);
   kernel_mark("invert_by_leaf", s);
   InvArgs inv;
-  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kBwdWindowTok);
+  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kBwdWindowTok, 0, gate);
   if (st != PISA_OK) return st;
   BwdArgs a = {};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
@@ -1754,13 +1782,14 @@ int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* 
   a.dq_acc = (float*)(ws + L.dq); a.dk_acc = (float*)(ws + L.dk); a.dv_acc = (float*)(ws + L.dv);
   a.status = status;
   kernel_mark("gradient_memset", s);
-  cudaError_t e = cudaMemsetAsync(ws + L.dq, 0, L.inv.count - L.dq, s);     // dq, dk, dv accumulators are adjacent
-  if (e != cudaSuccess) { record_cuda_error("gradient memset", e); return PISA_ERR_CUDA; }
+  a.gate = gate;
+  st = launch_zero(ws + L.dq, L.inv.count - L.dq, gate, s);                // dq, dk, dv accumulators are adjacent
+  if (st != PISA_OK) return st;
   kernel_mark("delta", s);
   {
     const long long rows = (long long)g.B * g.N * g.Hq;
     bwd_delta_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(g, (const __nv_bfloat16*)out,
-                                                                        (const __nv_bfloat16*)dout, delta);
+                                                                        (const __nv_bfloat16*)dout, delta, gate);
     st = check_launch("bwd_delta");
     if (st != PISA_OK) return st;
   }
@@ -1773,13 +1802,13 @@ int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* 
     Geometry gd = g;                                   // dq: the caller's dense [B, N, Hq, d] (this chunk's heads of it)
     gd.os[0] = dq_strides[0]; gd.os[1] = dq_strides[1]; gd.os[2] = dq_strides[2];
     const long long n = (long long)g.B * g.N * g.Hkv * (g.d / 2);
-    convert_out_heads_inner_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(gd, a.dq_acc, (__nv_bfloat16*)dq);
+    convert_out_heads_inner_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(gd, a.dq_acc, (__nv_bfloat16*)dq, gate);
     st = check_launch("convert_dq");
     if (st != PISA_OK) return st;
     const long long n2 = (long long)g.B * g.N * g.Hkv * g.d / 2;
     const int row2 = g.Hkv * g.d / 2;                 // one token's pairs in the accumulator; dkv_pitch in the output
-    bwd_convert_kernel<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(a.dk_acc, (__nv_bfloat16*)dk, n2, row2, dkv_pitch / 2);
-    bwd_convert_kernel<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(a.dv_acc, (__nv_bfloat16*)dv, n2, row2, dkv_pitch / 2);
+    bwd_convert_kernel<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(a.dk_acc, (__nv_bfloat16*)dk, n2, row2, dkv_pitch / 2, gate);
+    bwd_convert_kernel<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(a.dv_acc, (__nv_bfloat16*)dv, n2, row2, dkv_pitch / 2, gate);
     st = check_launch("convert_dkv");
   }
   return st;
