@@ -40,7 +40,15 @@ Sizes uniform_sizes(const Geometry& g) {
   const Sizes z = seq_sizes(g, g.N);
   return {g.B * z.rows, g.B * z.words, g.B * z.twords};
 }
-int uniform_splits(const Geometry& g) { return qm_bwd_splits((long long)g.B * g.Hkv * ((g.N + 127) / 128)); }
+// splits, splits0 and the room for their sums
+struct Split { int all, first; long long acc; };
+Split uniform_split(const Geometry& g) {
+  Split x;
+  x.all = qm_bwd_splits((long long)g.B * g.Hkv * ((g.N + 127) / 128));
+  x.first = qm_bwd_splits0(((long long)g.N * g.G + 127) / 128, x.all);
+  x.acc = x.all > 1 ? (long long)kAccAll : x.first > 1 ? g.B : 0;
+  return x;
+}
 size_t table_bytes(size_t n) { return align_up(n * sizeof(qm::Seq), 256) + align_up(n * sizeof(qm::SeqOrder), 256); }
 
 // Steps (128-row tile x 128 keys) per tile and selected block up to which the dense kernels win, in eighths.  Measured SM
@@ -68,16 +76,17 @@ bool qm_bwd_supported(const Geometry& g, int dtype) {
 // (a tile has N / 256 steps on average when it needs all key blocks)
 int qm_bwd_always(const Geometry& g) { return 32 * g.K * steps_per_block8(g); }
 
-size_t qm_bwd_workspace_bytes(const Geometry& g) { return layout(g, uniform_sizes(g), uniform_splits(g) > 1 ? kAccAll : g.B).total; }
+size_t qm_bwd_workspace_bytes(const Geometry& g) { return layout(g, uniform_sizes(g), uniform_split(g).acc).total; }
 
 int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx, const void* out, const float* lse,
            const void* dout, void* dq, void* dk, void* dv, void* ws_, int32_t* status, Gate* gate, cudaStream_t s) {
   char* ws = (char*)ws_;
   const int tpt = 128 / g.G, units = g.B * g.Hkv;
   qmb::Args a = {};
-  a.splits = uniform_splits(g);
-  a.splits0 = qm_bwd_splits0((g.N + tpt - 1) / tpt, a.splits);
-  const Layout l = layout(g, uniform_sizes(g), a.splits > 1 ? kAccAll : a.splits0 > 1 ? g.B : 0);
+  const Split split = uniform_split(g);
+  a.splits = split.all;
+  a.splits0 = split.first;
+  const Layout l = layout(g, uniform_sizes(g), split.acc);
   a.lgC = log2i(g.C); a.lgG = log2i(g.G);
   a.n_tiles = units * ((g.N + tpt - 1) / tpt);
   a.per = qm_bwd_tiles_per_item(a.n_tiles);
