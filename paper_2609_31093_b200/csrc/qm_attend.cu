@@ -12,7 +12,9 @@
 // feed 256 rows.  The issuer walks the steps in order: the product with P that a buffer still owes, then the next S into
 // it -- no barrier guards the buffer, the tensor pipe runs one thread's instructions in order.
 // Measured at 8192 tokens, 16 KV heads, d = 128: P through shared memory with separate issuers took 2200 cycles per tile
-// and step with NT = 1 and NT = 2 alike (each product waited for the other's queue).
+// and step with NT = 1 and NT = 2 alike (each product waited for the other's queue).  An issuer per tile: 707 us against 653
+// (4 x 4 KV heads, G = 4), 583 against 485 (C = 128) -- the pipe loses more by changing chains than one issuer's loop does,
+// which is busy 1570 of 1855 cycles per tile and step, the chains' 1024 among them.
 // Every wait is bounded.
 #include "launch.cuh"
 #include "lse_chunk.cuh"
@@ -30,6 +32,8 @@ namespace {
 constexpr int kAttThreads = 640;
 constexpr int kMaxSteps = 256;                 // steps of one sequence: 32768 tokens
 constexpr int kRing = 2;
+
+template <bool V> struct Bool { static constexpr bool value = V; };
 
 struct AttArgs {
   const float* row_lse;      // [Hq, len] per sequence, natural log
@@ -309,36 +313,43 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
         ok = mbar_wait_bounded(&s_full[grp], (uint32_t)(c & 1));
         if (!ok) break;
         tcgen05_fence_after_sync();
+        // (two bodies: a warp whose rows see all of their leaves -- nearly every one -- does without two instructions per key)
+        const bool sel0 = live && ((mine >> ((half * 64) / C)) & 1u), sel1 = live && ((mine >> ((half * 64 + 32) / C)) & 1u);
+        const int nv0 = sel0 ? max(0, min(32, vis - 64 * half)) : 0, nv1 = sel1 ? max(0, min(32, vis - 64 * half - 32)) : 0;
+        auto probs = [&](int qq, bool sel, int nv, auto masked) {
+          const float bias = sel ? neg_lse2 : -CUDART_INF_F;                 // exp2(-inf) = 0: the row did not select the leaf
+          const uint64_t sc2 = pack2(sl2, sl2), bias2 = pack2(bias, bias);
+          uint32_t rr[32], pk[16];
+          tmem_ld_32x32(s_base + (uint32_t)(qq * 32), rr);
+          tmem_ld_wait();
 #pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
-          const int q = half * 2 + qq;
-          const bool sel = live && ((mine >> ((q * 32) / C)) & 1u);
-          const int nv = sel ? max(0, min(32, vis - 32 * q)) : 0;
-          uint32_t pk[16];
-          if (__any_sync(0xffffffffu, nv > 0)) {
-            uint32_t rr[32];
-            tmem_ld_32x32(s_base + (uint32_t)(qq * 32), rr);
-            const float bias = sel ? neg_lse2 : -CUDART_INF_F;               // exp2(-inf) = 0: the row did not select the leaf
-            const bool fast = __all_sync(0xffffffffu, nv == 32 || !sel);
-            const uint64_t sc2 = pack2(sl2, sl2), bias2 = pack2(bias, bias);
-            tmem_ld_wait();
-#pragma unroll
-            for (int x = 0; x < 16; ++x) {
-              float z0, z1;
-              unpack2(fma2(pack2(__uint_as_float(rr[2 * x]), __uint_as_float(rr[2 * x + 1])), sc2, bias2), z0, z1);
-              float p0 = ex2_approx(z0), p1 = ex2_approx(z1);
-              if (!fast) {
-                if (2 * x >= nv) p0 = 0.f;
-                if (2 * x + 1 >= nv) p1 = 0.f;
-              }
-              const __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
-              pk[x] = *reinterpret_cast<const uint32_t*>(&pp);
+          for (int x = 0; x < 16; ++x) {
+            float z0, z1;
+            unpack2(fma2(pack2(__uint_as_float(rr[2 * x]), __uint_as_float(rr[2 * x + 1])), sc2, bias2), z0, z1);
+            float p0 = ex2_approx(z0), p1 = ex2_approx(z1);
+            if (masked.value) {
+              if (2 * x >= nv) p0 = 0.f;
+              if (2 * x + 1 >= nv) p1 = 0.f;
             }
-          } else {
-#pragma unroll
-            for (int x = 0; x < 16; ++x) pk[x] = 0u;
+            const __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
+            pk[x] = *reinterpret_cast<const uint32_t*>(&pp);
           }
-          tmem_st_32x16(s_base + (uint32_t)(qq * 16), pk);       // over columns of S this warp has already read
+          tmem_st_32x16(s_base + (uint32_t)(qq * 16), pk);                   // over columns of S this warp has already read
+        };
+        if (__any_sync(0xffffffffu, nv0 > 0 || nv1 > 0)) {
+          if (__all_sync(0xffffffffu, (nv0 == 32 || !sel0) && (nv1 == 32 || !sel1))) {
+            probs(0, sel0, nv0, Bool<false>());
+            probs(1, sel1, nv1, Bool<false>());
+          } else {
+            probs(0, sel0, nv0, Bool<true>());
+            probs(1, sel1, nv1, Bool<true>());
+          }
+        } else {
+          uint32_t pk[16];
+#pragma unroll
+          for (int x = 0; x < 16; ++x) pk[x] = 0u;
+          tmem_st_32x16(s_base, pk);
+          tmem_st_32x16(s_base + 16u, pk);
         }
         tmem_st_wait();
         tcgen05_fence_before_sync();

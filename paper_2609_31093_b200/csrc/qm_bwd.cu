@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) qm_bwd_prep_kernel(Geometry geo, Args a) 
     for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (sub == 0 && t < len) {
       const float l = a.lse[(long long)geo.Hq * loc.q.cu + (long long)(h * G + hd) * len + t];
-      a.stat[loc.q.leaf_off + ((long long)h * len + t) * G + hd] = make_float2(l > -CUDART_INF_F ? -l * kLog2e : -CUDART_INF_F, -s);
+      a.stat[loc.q.leaf_off + ((long long)h * len + t) * G + hd] = make_float2(l > -CUDART_INF_F ? -l * kLog2e : -CUDART_INF_F, -s * geo.scale);
     }
   }
   __syncthreads();
@@ -86,27 +86,29 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&p);
 }
-// N floats of a row, scaled, -> bf16, 16 bytes at a time
+// N floats of a row -> bf16, 16 bytes at a time
 template <int N>
-__device__ __forceinline__ void store_row(__nv_bfloat16* dst, const uint32_t (&r)[N], float scale) {
+__device__ __forceinline__ void store_row(__nv_bfloat16* dst, const uint32_t (&r)[N]) {
 #pragma unroll
   for (int q4 = 0; q4 < N / 8; ++q4) {
     uint4 o;
     uint32_t* ow = &o.x;
 #pragma unroll
-    for (int x = 0; x < 4; ++x) ow[x] = pack_bf16(__uint_as_float(r[8 * q4 + 2 * x]) * scale, __uint_as_float(r[8 * q4 + 2 * x + 1]) * scale);
+    for (int x = 0; x < 4; ++x) ow[x] = pack_bf16(__uint_as_float(r[8 * q4 + 2 * x]), __uint_as_float(r[8 * q4 + 2 * x + 1]));
     *reinterpret_cast<uint4*>(dst + 8 * q4) = o;
   }
 }
-// Two probabilities and their dS / scale (the logit scale is applied to the sums at the end): p = 2^(s * sl2 + bias),
-// d = p * (dp - delta).  Packed arithmetic: seven instructions for two elements.
-__device__ __forceinline__ void prob_grad2(uint32_t s0, uint32_t s1, uint32_t dp0, uint32_t dp1, uint64_t sl2, uint64_t bias, uint64_t ndelta,
+// Two probabilities and their dS: p = 2^(s * sl2 + bias), d = p * (dp * scale - delta * scale).  The logit scale belongs in
+// front of the rounding to bf16, not behind the sums: the roundings are then those of the list-driven kernel, and where the
+// terms of a sum cancel (a key of large norm with most of a row's probability) they are what the result's error is made of.
+// Packed arithmetic: seven instructions for two elements.
+__device__ __forceinline__ void prob_grad2(uint32_t s0, uint32_t s1, uint32_t dp0, uint32_t dp1, uint64_t sl2, uint64_t bias, uint64_t sc, uint64_t ndelta,
                                            float& p0, float& p1, float& d0, float& d1) {
   float z0, z1;
   unpack2(fma2(pack2(__uint_as_float(s0), __uint_as_float(s1)), sl2, bias), z0, z1);
   p0 = ex2_approx(z0);
   p1 = ex2_approx(z1);
-  unpack2(mul2(pack2(p0, p1), add2(pack2(__uint_as_float(dp0), __uint_as_float(dp1)), ndelta)), d0, d1);
+  unpack2(mul2(pack2(p0, p1), fma2(pack2(__uint_as_float(dp0), __uint_as_float(dp1)), sc, ndelta)), d0, d1);
 }
 // rows [first, rows) of `slabs` swizzled 64-column slabs become zero (one warp)
 __device__ __forceinline__ void zero_rows(uint8_t* base, int slab_bytes, int slabs, int first, int rows) {
@@ -344,7 +346,7 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
     const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
     const int col0 = grp * 64 + part * 32;                    // first of this warp's query rows
     const uint32_t base = tmem + lane_sel + (uint32_t)col0;
-    const uint64_t sl2 = pack2(geo.scale * kLog2e, geo.scale * kLog2e);
+    const uint64_t sl2 = pack2(geo.scale * kLog2e, geo.scale * kLog2e), sc = pack2(geo.scale, geo.scale);
     int step = 0, items = 0;
     qmb::Loc loc;
     while (ring_pop(ring, n, e, &s_fail)) {
@@ -373,7 +375,7 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
             for (int x = 0; x < 16; ++x) {
               const float2 bi = *reinterpret_cast<const float2*>(bias + 2 * x), de = *reinterpret_cast<const float2*>(delta + 2 * x);
               float p0, p1, d0, d1;
-              prob_grad2(rs[2 * x], rs[2 * x + 1], rp[2 * x], rp[2 * x + 1], sl2, pack2(bi.x, bi.y), pack2(de.x, de.y), p0, p1, d0, d1);
+              prob_grad2(rs[2 * x], rs[2 * x + 1], rp[2 * x], rp[2 * x + 1], sl2, pack2(bi.x, bi.y), sc, pack2(de.x, de.y), p0, p1, d0, d1);
               if (masked.value) {
                 if (e.y * tpt + ((col0 + 2 * x) >> lgG) < key) p0 = d0 = 0.f;
                 if (e.y * tpt + ((col0 + 2 * x + 1) >> lgG) < key) p1 = d1 = 0.f;
@@ -412,7 +414,6 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
       }
       wait(&acc_full, (uint32_t)(items & 1));
       tcgen05_fence_after_sync();
-      const float f = which ? geo.scale : 1.f;
 #pragma unroll
       for (int x = 0; x < CPW; x += 32) {
         uint32_t r[32];
@@ -425,14 +426,14 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
         }
         if (!live) continue;
         if (direct) {
-          store_row<32>((which ? a.dk : a.dv) + orow + x, r, f);
+          store_row<32>((which ? a.dk : a.dv) + orow + x, r);
         } else {
           const long long arow = a.splits > 1 ? orow : (((long long)loc.q.pyr_row * geo.Hkv + loc.h) * 128 + row) * D + c0;
           float* dst = (which ? a.dk_acc : a.dv_acc) + arow + x;
 #pragma unroll
           for (int y = 0; y < 32; y += 4)
-            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + y), "f"(__uint_as_float(r[y]) * f),
-                         "f"(__uint_as_float(r[y + 1]) * f), "f"(__uint_as_float(r[y + 2]) * f), "f"(__uint_as_float(r[y + 3]) * f)
+            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + y), "f"(__uint_as_float(r[y])),
+                         "f"(__uint_as_float(r[y + 1])), "f"(__uint_as_float(r[y + 2])), "f"(__uint_as_float(r[y + 3]))
                          : "memory");
         }
       }
@@ -651,7 +652,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
     const int row = quarter * 32 + lane, head = row & (G - 1);
     const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
     const uint32_t base = tmem + lane_sel + (uint32_t)(x * 256 + part * 32);
-    const uint64_t sl2 = pack2(geo.scale * kLog2e, geo.scale * kLog2e);
+    const uint64_t sl2 = pack2(geo.scale * kLog2e, geo.scale * kLog2e), sc = pack2(geo.scale, geo.scale);
     int cnt = 0, outs = 0, t = 0, W = 0, wi = -1;
     bool live = false, any_step = false;
     float2 st = make_float2(-CUDART_INF_F, 0.f);
@@ -697,7 +698,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
 #pragma unroll
             for (int y = 0; y < 16; ++y) {
               float p0, p1, d0, d1;
-              prob_grad2(rs[2 * y], rs[2 * y + 1], rp[2 * y], rp[2 * y + 1], sl2, bias, nd, p0, p1, d0, d1);
+              prob_grad2(rs[2 * y], rs[2 * y + 1], rp[2 * y], rp[2 * y + 1], sl2, bias, sc, nd, p0, p1, d0, d1);
               if (masked.value) {
                 if (2 * y >= nv) d0 = 0.f;
                 if (2 * y + 1 >= nv) d1 = 0.f;
@@ -739,7 +740,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
           __syncwarp();
           if (lane == 0) mbar_arrive(&o_empty[x]);
         }
-        if (live) store_row<32>(dst + y, r, geo.scale);
+        if (live) store_row<32>(dst + y, r);
       }
     }
   }

@@ -49,9 +49,9 @@ qm::Args uniform_args(const Geometry& g, char* ws, const Layout& l, int32_t* sta
 }  // namespace
 
 // Two tiles per work item halve the key / value traffic, which bounds the dense kernels, once there are enough pairs for
-// four waves of one item per SM (4096 tokens x 16 heads still runs 5 % faster with one tile per item, 8192 5 % slower).
+// three waves of one item per SM (16 heads: 4096 tokens 206 us with one tile per item, 270 with two; 8192: 606 and 576).
 int qm_tiles_per_item(const Geometry& g, long long unit_tokens) {
-  return unit_tokens * g.G / 256 >= 4LL * num_sms() ? 2 : 1;
+  return unit_tokens * g.G / 256 >= 3LL * num_sms() ? 2 : 1;
 }
 
 bool qm_supported(const Geometry& g, int dtype) {
