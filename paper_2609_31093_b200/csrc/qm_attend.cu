@@ -43,7 +43,8 @@ struct AttArgs {
 // K / V tiles in flight (one ring: K, V, K, V, ...): what two items' query tiles leave of 227 KB
 __host__ __device__ constexpr int att_stages(int D, int NT) { return D == 128 ? (NT == 1 ? 5 : 3) : 8; }
 
-template <int D, int C, int NT>
+// LO: sequences of one leaf take P in two bf16 terms (an instantiation of its own: the registers would spill in the other)
+template <int D, int C, int NT, bool LO>
 __global__ void __launch_bounds__(kAttThreads, 1)
 qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ CUtensorMap tm_q,
                  const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v) {
@@ -180,7 +181,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
       if (!dead && !mbar_try_wait(bar, parity) && !mbar_wait_bounded(bar, parity)) { dead = true; s_fail = 1; }
     };
     // what a buffer owes: the product of its P with the values of a step (stage < 0: nothing)
-    struct Owed { int stage; uint32_t phase, p_phase, ob, o_wait; int rows; bool fresh, last; };
+    struct Owed { int stage; uint32_t phase, p_phase, ob, o_wait; int rows; bool fresh, last, lo; };
     Owed owed[2];
     owed[0].stage = owed[1].stage = -1;
     uint32_t p_phase[2] = {0u, 0u}, o_count[2] = {0u, 0u};          // products per P buffer (parity); outputs per O buffer
@@ -201,10 +202,19 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
       tcgen05_fence_after_sync();
       const uint32_t p0 = tmem + sb * 128u, d0 = tmem + 256u + w.ob * 128u, v0 = v_base + (uint32_t)(w.stage * (TILE >> 4));
       if (elect_one()) {
+        if (!LO || !w.lo) {
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk)                              // sixteen keys: eight columns of P, its halves 64 apart
-          umma_bf16_ts(d0, p0 + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 8), desc64(v0 + kk * (2048 >> 4)), idesc_o,
-                       (!w.fresh || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < 8; ++kk)                            // sixteen keys: eight columns of P, its halves 64 apart
+            umma_bf16_ts(d0, p0 + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 8), desc64(v0 + kk * (2048 >> 4)), idesc_o,
+                         (!w.fresh || kk > 0) ? 1u : 0u);
+        } else {
+#pragma unroll 1
+          for (int x = 0; x < 16; ++x) {                            // two terms of P
+            const int kk = x >> 1;
+            umma_bf16_ts(d0, p0 + (uint32_t)((kk >> 1) * 32 + (x & 1) * 16 + (kk & 1) * 8), desc64(v0 + (uint32_t)kk * (2048u >> 4)), idesc_o,
+                         x > 0 ? 1u : 0u);
+          }
+        }
         if (w.last) umma_commit(&o_full[w.ob]);
       }
       __syncwarp();
@@ -220,6 +230,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
       const int ny = __shfl_sync(0xffffffffu, e.y, 0), n0 = __shfl_sync(0xffffffffu, e.z, 0), n1 = __shfl_sync(0xffffffffu, e.w, 0);
       int len = 0x7fffffff;
       if (a.seqs != nullptr) len = qm::locate(geo, a, e.x, NT).q.len;
+      const bool one_leaf = (a.seqs != nullptr ? len : geo.N) <= C;
       int seen[2] = {0, 0};
       wait(&q_full[it & 1], (uint32_t)((it >> 1) & 1));
       const uint32_t q_item = q_base + (uint32_t)((it & 1) * NT * (TILE >> 4));
@@ -257,7 +268,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           }
           __syncwarp();
           Owed& w = owed[NT == 1 ? 1 : x];
-          w.stage = sv; w.phase = phv; w.rows = rows;
+          w.stage = sv; w.phase = phv; w.rows = rows; w.lo = one_leaf;
           const uint32_t pb = (NT == 1) ? par : (uint32_t)x;
           w.p_phase = (NT == 1) ? (p_phase[0] >> pb) & 1u : p_phase[x];
           if (NT == 1) p_phase[0] ^= 1u << pb; else p_phase[x] ^= 1u;
@@ -336,7 +347,29 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           }
           tmem_st_32x16(s_base + (uint32_t)(qq * 16), pk);                   // over columns of S this warp has already read
         };
-        if (__any_sync(0xffffffffu, nv0 > 0 || nv1 > 0)) {
+        if (LO && len <= C) {
+          // a sequence of one leaf: P in two bf16 terms, sixteen columns each for 32 keys (the product is a single step, and
+          // the fp32 path, which rounds no P, is the one such a sequence takes on its own)
+#pragma unroll 1
+          for (int qq = 0; qq < 2; ++qq) {
+            uint32_t rr[32], pk[16];
+            tmem_ld_32x32(s_base + (uint32_t)(qq * 32), rr);
+            tmem_ld_wait();
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+#pragma unroll
+              for (int x = 0; x < 16; ++x) {
+                const int nv = qq ? nv1 : nv0;
+                float p0 = 2 * x < nv ? ex2_approx(fmaf(__uint_as_float(rr[2 * x]), sl2, neg_lse2)) : 0.f;
+                float p1 = 2 * x + 1 < nv ? ex2_approx(fmaf(__uint_as_float(rr[2 * x + 1]), sl2, neg_lse2)) : 0.f;
+                __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
+                if (part) pp = __floats2bfloat162_rn(p0 - __low2float(pp), p1 - __high2float(pp));
+                pk[x] = *reinterpret_cast<const uint32_t*>(&pp);
+              }
+              tmem_st_32x16(s_base + (uint32_t)(qq * 32 + part * 16), pk);
+            }
+          }
+        } else if (__any_sync(0xffffffffu, nv0 > 0 || nv1 > 0)) {
           if (__all_sync(0xffffffffu, (nv0 == 32 || !sel0) && (nv1 == 32 || !sel1))) {
             probs(0, sel0, nv0, Bool<false>());
             probs(1, sel1, nv1, Bool<false>());
@@ -405,23 +438,24 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int D, int C, int NT>
+template <int D, int C, int NT, bool LO>
 int launch_dcn(const Geometry& g, const qm::Args& a, const AttArgs& at, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                const CUtensorMap& tm_v, cudaStream_t s) {
   const size_t smem = (size_t)(D / 64) * (2 * NT + att_stages(D, NT)) * 128 * 128 + 1024;
   const int grid = a.n_items < num_sms() ? a.n_items : num_sms();
-  return launch_dependent<qm_attend_kernel<D, C, NT>>("qm_attend", dim3((unsigned)grid), kAttThreads, smem, s, g, a, at, tm_q, tm_k, tm_v);
+  return launch_dependent<qm_attend_kernel<D, C, NT, LO>>("qm_attend", dim3((unsigned)grid), kAttThreads, smem, s, g, a, at, tm_q, tm_k, tm_v);
 }
 template <int D, int C>
 int launch_dc(const Geometry& g, const qm::Args& a, const AttArgs& at, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
-              const CUtensorMap& tm_v, cudaStream_t s) {
-  return a.tiles == 2 ? launch_dcn<D, C, 2>(g, a, at, tm_q, tm_k, tm_v, s) : launch_dcn<D, C, 1>(g, a, at, tm_q, tm_k, tm_v, s);
+              const CUtensorMap& tm_v, bool lo, cudaStream_t s) {
+  if (lo) return a.tiles == 2 ? launch_dcn<D, C, 2, true>(g, a, at, tm_q, tm_k, tm_v, s) : launch_dcn<D, C, 1, true>(g, a, at, tm_q, tm_k, tm_v, s);
+  return a.tiles == 2 ? launch_dcn<D, C, 2, false>(g, a, at, tm_q, tm_k, tm_v, s) : launch_dcn<D, C, 1, false>(g, a, at, tm_q, tm_k, tm_v, s);
 }
 
 }  // namespace
 
 int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const void* k, const void* v, long long tokens,
-                     const float* row_lse, void* out, cudaStream_t s) {
+                     const float* row_lse, void* out, bool one_leaf, cudaStream_t s) {
   CUtensorMap tm_q, tm_k, tm_v;
   if (!qm_map_rows(&tm_q, q, g.d, g.Hq, tokens, g.B, g.qs, g.G, 128 / g.G) ||
       !qm_map_rows(&tm_k, k, g.d, g.Hkv, tokens, g.B, g.ks, 1, 128) ||
@@ -431,8 +465,8 @@ int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const 
   }
   AttArgs at;
   at.row_lse = row_lse; at.out = (__nv_bfloat16*)out;
-  if (g.d == 128) return g.C == 128 ? launch_dc<128, 128>(g, a, at, tm_q, tm_k, tm_v, s) : launch_dc<128, 64>(g, a, at, tm_q, tm_k, tm_v, s);
-  return g.C == 128 ? launch_dc<64, 128>(g, a, at, tm_q, tm_k, tm_v, s) : launch_dc<64, 64>(g, a, at, tm_q, tm_k, tm_v, s);
+  if (g.d == 128) return g.C == 128 ? launch_dc<128, 128>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s) : launch_dc<128, 64>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s);
+  return g.C == 128 ? launch_dc<64, 128>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s) : launch_dc<64, 64>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s);
 }
 
 }  // namespace pisa

@@ -164,7 +164,7 @@ int qm_forward_packed(const Geometry& g, const int32_t* cu, const int* ids, int 
   for (int at = 0; at < n;) {
     size_t leaf = 0, up = 0, bits = 0, pyr = 0, used = kFixedBytes;
     long long rows = 0;
-    int end = at, leaves = 0, deepest = 0, most_leaves = 0;
+    int end = at, shortest = 0x7fffffff, leaves = 0, deepest = 0, most_leaves = 0;
     while (end < n) {                                      // as many sequences as the workspace takes
       const int len = cu[ids[end] + 1] - cu[ids[end]];
       const Need w = need_of(g, len);
@@ -172,6 +172,7 @@ int qm_forward_packed(const Geometry& g, const int32_t* cu, const int* ids, int 
       if (end > at && (used + b > ws_bytes || rows + len > (1LL << 24) || end - at >= 65535)) break;
       used += b; leaf += w.leaf; up += w.up; bits += w.bits; pyr += w.pyr;
       rows += len; leaves += w.leaves;
+      shortest = std::min(shortest, len);
       deepest = std::max(deepest, w.top);
       most_leaves = std::max(most_leaves, w.leaves);
       ++end;
@@ -245,7 +246,7 @@ int qm_forward_packed(const Geometry& g, const int32_t* cu, const int* ids, int 
     kernel_mark("qm_select", s);
     if ((st = launch_qm_select_full(g, a, rows, idx, nullptr, lse, nullptr, s)) != PISA_OK) return st;
     kernel_mark("qm_attend", s);
-    if ((st = launch_qm_attend(g, a, q, k, v, total, lse, out, s)) != PISA_OK) return st;
+    if ((st = launch_qm_attend(g, a, q, k, v, total, lse, out, shortest <= g.C, s)) != PISA_OK) return st;
     at = end;
   }
   return PISA_OK;

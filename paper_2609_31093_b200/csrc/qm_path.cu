@@ -93,7 +93,7 @@ int qm_attend(const Geometry& g, const void* q, const void* k, const void* v, vo
   const Layout l = layout(g);
   const qm::Args a = uniform_args(g, ws, l, status);
   kernel_mark("qm_attend", s);
-  return launch_qm_attend(g, a, q, k, v, g.N, lse, out, s);
+  return launch_qm_attend(g, a, q, k, v, g.N, lse, out, g.N <= g.C, s);
 }
 
 // ---------------------------------------------------------------- upper levels and final selection of the list-driven path
