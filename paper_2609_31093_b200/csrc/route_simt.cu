@@ -1,4 +1,4 @@
-// Coarse-to-fine Top-K routing, one warp per (b, KV head, query token), every level fused in one
+// Coarse-to-fine Top-K routing, one or four warps per (b, KV head, query token), every level fused in one
 // launch (Sec. 3.2 "Coarse-to-fine block selection"; the paper's "per-query" schedule, App. B).
 //
 // This is the exact-fp32 SIMT path: it serves the fp32 dtype, every shape the tensor-core path does
@@ -6,19 +6,24 @@
 // levels (LEAF = false), is stage 1 of the two-stage schedule (Algorithm 1): it then stores the
 // kept level-2 nodes, whose children are the leaf candidates, instead of scoring the leaves.
 //
-// Per warp state lives in shared memory: the G query vectors in fp32, the sorted candidate list
+// Where the tokens alone do not fill the GPU a token has WPT = 4 warps: the first walks the levels, all of them share the
+// scoring of the leaves, a leaf each; key rows are read by several lanes each (simt_dot.cuh; not for large groups).
+// 1024 tokens, one head, d = 64, K = 4: one warp per token and a lane per key 35 us.
+//
+// A token's state lives in shared memory: the G query vectors in fp32, the sorted candidate list
 // (at most g*K entries) and the candidates' grouped scores.  The query-summary score matrix is
 // never formed: each candidate's children are read, dotted with the G queries, reduced by the
 // block score and dropped.
 #include <math_constants.h>
 
 #include "pisa_common.cuh"
+#include "simt_dot.cuh"
 
 namespace pisa {
 
 namespace {
 
-constexpr int kWarpsPerCta = 4;
+constexpr int kTokensPerCta = 4;
 
 template <typename T, int D, int G>
 __device__ __forceinline__ void dot_row(const T* __restrict__ row, const float* __restrict__ qf,
@@ -26,7 +31,7 @@ __device__ __forceinline__ void dot_row(const T* __restrict__ row, const float* 
   constexpr int V = Elem<T>::kVec;
 #pragma unroll
   for (int h = 0; h < G; ++h) z[h] = 0.f;
-#pragma unroll 2
+#pragma unroll (G <= 2 ? 8 : 2)
   for (int c = 0; c < D / V; ++c) {
     float x[V];
     Elem<T>::load_chunk(row + c * V, x);
@@ -94,18 +99,25 @@ __device__ __forceinline__ float stat_warp_finish(Stat s, int mode) {
 
 }  // namespace
 
-template <typename T, int D, int G, bool LEAF>
-__global__ void __launch_bounds__(kWarpsPerCta * 32)
+template <typename T, int D, int G, bool LEAF, int WPT>
+__global__ void __launch_bounds__(kTokensPerCta * WPT * 32)
 route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k,
                   const T* __restrict__ pyr, int32_t* __restrict__ idx, float* __restrict__ margin,
                   int32_t* __restrict__ cand_out) {
-  __shared__ __align__(16) float s_q[kWarpsPerCta][G * D];
-  __shared__ int s_cand[kWarpsPerCta][2][kMaxCand];
-  __shared__ __align__(16) float s_u[kWarpsPerCta][kMaxCand];
-  __shared__ float s_cut[kWarpsPerCta][2];
+  static_assert(LEAF || WPT == 1, "only the leaf level is shared");
+  __shared__ __align__(16) float s_q[kTokensPerCta][G * D];
+  __shared__ int s_cand[kTokensPerCta][2][kMaxCand];
+  __shared__ __align__(16) float s_u[kTokensPerCta][kMaxCand];
+  __shared__ float s_cut[kTokensPerCta][2];
+  __shared__ int s_leaves[kTokensPerCta];           // leaf candidates to score
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long w = (long long)blockIdx.x * kWarpsPerCta + warp;
+  // (`warp`: the token of the CTA; `part`: the warp of the token)
+  const int warp = (threadIdx.x >> 5) / WPT, part = (threadIdx.x >> 5) % WPT, lane = threadIdx.x & 31;
+  auto group_sync = [&]() {
+    if (WPT == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + warp), "r"(WPT * 32) : "memory");
+  };
+  const long long w = (long long)blockIdx.x * kTokensPerCta + warp;
   const long long total = (long long)geo.B * geo.Hkv * geo.N;
   if (w >= total) return;
   const int t = (int)(w % geo.N);
@@ -119,13 +131,62 @@ route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k
   float* u = s_u[warp];
   for (int hh = 0; hh < G; ++hh) {
     const T* row = q + (long long)b * geo.qs[0] + (long long)t * geo.qs[1] + (long long)(h * G + hh) * geo.qs[2];
-    for (int e = lane; e < D; e += 32) qf[hh * D + e] = Elem<T>::to_float(row[e]);
+    for (int e = part * 32 + lane; e < D; e += WPT * 32) qf[hh * D + e] = Elem<T>::to_float(row[e]);
   }
   int cur = 0;
   int n = 1;
-  if (lane == 0) s_cand[warp][0][0] = 0;
+  if (lane == 0 && part == 0) s_cand[warp][0][0] = 0;
   float min_gap = CUDART_INF_F;
-  __syncwarp();
+  group_sync();
+
+  RowDots<T, D, G <= 2 ? G : 1> rows;
+  if constexpr (LEAF && G <= 2) rows.load(qf);
+  // leaf level: one candidate at a time and warp, one lane per raw key
+  auto score_leaves = [&](const int* cand, int nV) {
+    const int f1 = (c >= 1) ? c - 1 : 0;
+    const T* kb = k + (long long)b * geo.ks[0] + (long long)h * geo.ks[2];
+    int scored = 0;
+    for (int s = 0; s < nV; ++s) {
+      const int i = cand[s];
+      if (i == 0 || i == f1 || i == c) {             // forced leaves rank first and are never scored
+        if (lane == 0 && part == 0) u[s] = CUDART_INF_F;
+        continue;
+      }
+      if (WPT > 1 && scored++ % WPT != part) continue;
+      Stat st[G];
+#pragma unroll
+      for (int hh = 0; hh < G; ++hh) stat_init(st[hh], mode);
+      const int lo = i * C, hi = min(lo + C, geo.N);
+      if constexpr (G <= 2) {
+        for (int j0 = lo; j0 < hi; j0 += 32) {
+          float z[G];
+          rows.dots(kb + (long long)j0 * geo.ks[1], geo.ks[1], hi - j0, z);
+          if (j0 + lane < hi) {
+#pragma unroll
+            for (int hh = 0; hh < G; ++hh) stat_add(st[hh], z[hh] * geo.scale, mode);
+          }
+        }
+      } else {
+        for (int j = lo + lane; j < hi; j += 32) {
+          float z[G];
+          dot_row<T, D, G>(kb + (long long)j * geo.ks[1], qf, z);
+#pragma unroll
+          for (int hh = 0; hh < G; ++hh) stat_add(st[hh], z[hh] * geo.scale, mode);
+        }
+      }
+      float score = 0.f;
+#pragma unroll
+      for (int hh = 0; hh < G; ++hh) score += stat_warp_finish(st[hh], mode);
+      if (lane == 0) u[s] = score;
+    }
+  };
+  if (WPT > 1 && part > 0) {
+    group_sync();                                     // the first warp has the leaf candidates
+    const int nl = s_leaves[warp];
+    score_leaves(s_cand[warp][(geo.L - 1) & 1], nl);
+    group_sync();
+    return;
+  }
 
   for (int l = geo.L; l >= 1; --l) {
     int* cand = s_cand[warp][cur];
@@ -167,31 +228,18 @@ route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k
             u[s] = score;
           }
         } else {
-          // leaf level: one candidate at a time, one lane per raw key
-          const T* kb = k + (long long)b * geo.ks[0] + (long long)h * geo.ks[2];
-          for (int s = 0; s < nV; ++s) {
-            const int i = cand[s];
-            if (i == 0 || i == f1 || i == anc_c) {
-              if (lane == 0) u[s] = CUDART_INF_F;
-              continue;
-            }
-            Stat st[G];
-#pragma unroll
-            for (int hh = 0; hh < G; ++hh) stat_init(st[hh], mode);
-            const int lo = i * C, hi = min(lo + C, geo.N);
-            for (int j = lo + lane; j < hi; j += 32) {
-              float z[G];
-              dot_row<T, D, G>(kb + (long long)j * geo.ks[1], qf, z);
-#pragma unroll
-              for (int hh = 0; hh < G; ++hh) stat_add(st[hh], z[hh] * geo.scale, mode);
-            }
-            float score = 0.f;
-#pragma unroll
-            for (int hh = 0; hh < G; ++hh) score += stat_warp_finish(st[hh], mode);
-            if (lane == 0) u[s] = score;
+          if (WPT > 1) {
+            if (lane == 0) s_leaves[warp] = nV;
+            group_sync();
           }
+          score_leaves(cand, nV);
+          if (WPT > 1) group_sync();
         }
         __syncwarp();
+      } else if (WPT > 1 && l == 1) {                 // nothing to score: let the other warps go
+        if (lane == 0) s_leaves[warp] = 0;
+        group_sync();
+        group_sync();
       }
       // Select_K: rank by (score desc, position asc); keep rank < K.  Without pruning keep all.
       int base = 0;
@@ -250,13 +298,18 @@ template <typename T, int D, int G>
 static int launch_route_tdg(const Geometry& g, const void* q, const void* k, const void* pyr,
                             int32_t* idx, float* margin, int32_t* cand_out, bool leaf, cudaStream_t s) {
   const long long total = (long long)g.B * g.Hkv * g.N;
-  const long long ctas = (total + kWarpsPerCta - 1) / kWarpsPerCta;
+  const long long ctas = (total + kTokensPerCta - 1) / kTokensPerCta;
   if (ctas > 0x7fffffffLL) return PISA_ERR_UNSUPPORTED;
-  if (leaf)
-    route_simt_kernel<T, D, G, true><<<(unsigned)ctas, kWarpsPerCta * 32, 0, s>>>(
+  // four warps per token while that leaves no SM with more than its 64
+  constexpr int WPT = G <= 2 ? 4 : 1;
+  if (leaf && WPT > 1 && total <= 16LL * num_sms())
+    route_simt_kernel<T, D, G, true, WPT><<<(unsigned)ctas, kTokensPerCta * WPT * 32, 0, s>>>(
+        g, (const T*)q, (const T*)k, (const T*)pyr, idx, margin, nullptr);
+  else if (leaf)
+    route_simt_kernel<T, D, G, true, 1><<<(unsigned)ctas, kTokensPerCta * 32, 0, s>>>(
         g, (const T*)q, (const T*)k, (const T*)pyr, idx, margin, nullptr);
   else
-    route_simt_kernel<T, D, G, false><<<(unsigned)ctas, kWarpsPerCta * 32, 0, s>>>(
+    route_simt_kernel<T, D, G, false, 1><<<(unsigned)ctas, kTokensPerCta * 32, 0, s>>>(
         g, (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
   return check_launch("route_simt");
 }
