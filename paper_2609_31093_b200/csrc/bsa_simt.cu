@@ -124,8 +124,17 @@ bsa_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k, 
 #pragma unroll
         for (int u = 0; u < UV; ++u) {
           const T* vr = vb + (long long)(j0 + min(jj + u, cnt - 1)) * geo.vs[1] + lane * DV;
+          if constexpr (DV == 2 && sizeof(T) == 4) {
+            const float2 x = *reinterpret_cast<const float2*>(vr);
+            xv[u][0] = x.x;
+            xv[u][DV - 1] = x.y;
+          } else if constexpr (DV == 4 && sizeof(T) == 4) {
+            const float4 x = *reinterpret_cast<const float4*>(vr);
+            xv[u][0] = x.x; xv[u][DV - 3] = x.y; xv[u][DV - 2] = x.z; xv[u][DV - 1] = x.w;
+          } else {
 #pragma unroll
-          for (int e = 0; e < DV; ++e) xv[u][e] = Elem<T>::to_float(vr[e]);
+            for (int e = 0; e < DV; ++e) xv[u][e] = Elem<T>::to_float(vr[e]);
+          }
         }
 #pragma unroll
         for (int u = 0; u < UV; ++u) {
