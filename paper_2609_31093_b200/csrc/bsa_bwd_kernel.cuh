@@ -28,6 +28,7 @@ struct BwdArgs {
   const __nv_bfloat16* dout;      // [B, N, Hq, D], strides of `out`
   const float* lse;               // [B, Hq, N] natural log
   const float* delta;             // [B, Hq, N]
+  const float2* stat;             // or, instead of both: [B, Hkv, N, G] (-lse * log2 e, -delta), from the dense path's preparation
   const int32_t* entry_off;
   const int32_t* item_off;
   const int32_t* item_key;
@@ -43,8 +44,7 @@ struct BwdArgs {
 // delta[b, hq, t] = sum_d dO[b,t,hq,d] * O[b,t,hq,d]; one warp per row
 __global__ void __launch_bounds__(256) bwd_delta_kernel(Geometry geo, const __nv_bfloat16* __restrict__ out,
                                                         const __nv_bfloat16* __restrict__ dout,
-                                                        float* __restrict__ delta, Gate gate) {
-  if (gate.off_list()) return;
+                                                        float* __restrict__ delta) {
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const long long rows = (long long)geo.B * geo.N * geo.Hq;
@@ -178,9 +178,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       ent = (jt_ < inf.ntiles && e < inf.e_end) ? a.entries[e] : -1;
       nl = 0.f; dl = 0.f;
       if (ent >= 0) {
-        const long long li = ((long long)b * geo.Hq + h * G + (tid & (G - 1))) * geo.N + (ent & 0xFFFFFF);
-        nl = -a.lse[li] * kLog2e;
-        dl = a.delta[li];
+        if (a.stat != nullptr) {
+          const float2 st = a.stat[(((long long)b * geo.Hkv + h) * geo.N + (ent & 0xFFFFFF)) * G + (tid & (G - 1))];
+          nl = st.x; dl = -st.y;
+        } else {
+          const long long li = ((long long)b * geo.Hq + h * G + (tid & (G - 1))) * geo.N + (ent & 0xFFFFFF);
+          nl = -a.lse[li] * kLog2e;
+          dl = a.delta[li];
+        }
       }
     };
     auto gather_tile = [&](const int* ents, int buf) {

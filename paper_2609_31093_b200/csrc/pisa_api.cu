@@ -495,15 +495,16 @@ static int do_bwd(const pisa_params_t* p, const Geometry& g, const void* q, cons
                   void* dv, void* ws, size_t ws_bytes, cudaStream_t s) {
   const bool dense = qm_bwd_supported(g, p->dtype);
   if (dense && g.N <= qm_bwd_always(g) && ws_bytes >= kStatusBytes + qm_bwd_workspace_bytes(g))
-    return qm_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, (char*)ws + kStatusBytes, (int32_t*)ws, nullptr, s);
+    return qm_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, (char*)ws + kStatusBytes, (int32_t*)ws, nullptr, nullptr, s);
   ForwardPlan pl;
   int st = plan_for(p, g, kOpBwd, ws_bytes, &pl);
   if (st != PISA_OK) return st;
   // longer sequences: the rows decide on the device (how many key blocks the tiles of neighbouring rows need in all)
   Gate gate = {nullptr, 0u};
+  const float2* stat = nullptr;
   const size_t list_bytes = align_up(pl.total, 256);
   if (dense && ws_bytes >= list_bytes + qm_bwd_workspace_bytes(g)) {
-    st = qm_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, (char*)ws + list_bytes, (int32_t*)ws, &gate, s);
+    st = qm_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, (char*)ws + list_bytes, (int32_t*)ws, &gate, &stat, s);
     if (st != PISA_OK) return st;
   }
   const size_t es = elem_size(p->dtype);
@@ -511,14 +512,14 @@ static int do_bwd(const pisa_params_t* p, const Geometry& g, const void* q, cons
   const long long pitch = (long long)g.Hkv * g.d;
   if (pl.n == 1)
     return tensor_bsa_bwd(g, q, k, v_, idx, out, lse, dout, dq, dk, dv, dqs, pitch, (char*)ws + kStatusBytes,
-                          (int32_t*)ws, gate, s);
+                          (int32_t*)ws, gate, stat, s);
   return run_chunks(p, g, pl, ws, s, [&](const ChunkView& v, int) {
     const size_t dq_off = (size_t)((long long)v.c.b0 * dqs[0] + (long long)v.c.h0 * g.G * dqs[2]) * es;
     const size_t dkv_off = (size_t)((long long)v.c.b0 * g.N * pitch + (long long)v.c.h0 * g.d) * es;
     return tensor_bsa_bwd(v.g, (const char*)q + v.q_off, (const char*)k + v.k_off, (const char*)v_ + v.v_off,
                           idx + v.unit0 * g.N * g.K, (const char*)out + v.o_off, lse + v.unit0 * g.G * g.N,
                           (const char*)dout + v.o_off, (char*)dq + dq_off, (char*)dk + dkv_off, (char*)dv + dkv_off, dqs,
-                          pitch, v.region, (int32_t*)ws, gate, v.stream);
+                          pitch, v.region, (int32_t*)ws, gate, stat != nullptr ? stat + v.unit0 * g.G * g.N : nullptr, v.stream);
   });
 }
 

@@ -58,11 +58,11 @@ int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const 
                      const float* row_lse, void* out, bool one_leaf, cudaStream_t s);
 
 // dense masked backward (qm_bwd.cuh).  gate (nullable): the choice is left to the data; receives what the list-driven kernels
-// have to look at
+// have to look at; stat: where the preparation leaves the rows' (-lse * log2 e, -delta), [B, Hkv, N, G], for them too
 bool qm_bwd_supported(const Geometry& g, int dtype);
 size_t qm_bwd_workspace_bytes(const Geometry& g);
 int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx, const void* out, const float* lse,
-           const void* dout, void* dq, void* dk, void* dv, void* ws, int32_t* status, Gate* gate, cudaStream_t s);
+           const void* dout, void* dq, void* dk, void* dv, void* ws, int32_t* status, Gate* gate, const float2** stat, cudaStream_t s);
 // length up to which the dense backward is the better one whatever the rows selected
 int qm_bwd_always(const Geometry& g);
 // packed batches: workspace one sequence needs, and the backward of the sequences ids[0..n)
@@ -86,6 +86,7 @@ size_t tensor_bwd_workspace_bytes(const Geometry& g);
 // (both describe the caller's dense tensors, of which a chunk of units writes its part)
 int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx,
                    const void* out, const float* lse, const void* dout, void* dq, void* dk, void* dv,
-                   const long long* dq_strides, long long dkv_pitch, void* ws, int32_t* status, const Gate& gate, cudaStream_t s);
+                   const long long* dq_strides, long long dkv_pitch, void* ws, int32_t* status, const Gate& gate, const float2* stat,
+                   cudaStream_t s);
 
 }  // namespace pisa

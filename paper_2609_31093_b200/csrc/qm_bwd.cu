@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) qm_bwd_prep_kernel(Geometry geo, Args a) 
     for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (sub == 0 && t < len) {
       const float l = a.lse[(long long)geo.Hq * loc.q.cu + (long long)(h * G + hd) * len + t];
-      a.stat[loc.q.leaf_off + ((long long)h * len + t) * G + hd] = make_float2(l > -CUDART_INF_F ? -l * kLog2e : -CUDART_INF_F, -s * geo.scale);
+      a.stat[loc.q.leaf_off + ((long long)h * len + t) * G + hd] = make_float2(l > -CUDART_INF_F ? -l * kLog2e : -CUDART_INF_F, -s);
     }
   }
   __syncthreads();
@@ -252,7 +252,7 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
         const int r = lane + 32 * x;
 #pragma unroll
         for (int lf = 0; lf < LPS; ++lf) s_bias[s][lf][r] = ((wd[x] >> lf) & 1u) ? st[x].x : -CUDART_INF_F;
-        s_delta[s][r] = st[x].y;
+        s_delta[s][r] = st[x].y * geo.scale;
       }
       if (a.seqs != nullptr && (len - t0) * G < 128) {
         // packed: the rows past the sequence's end belong to its neighbour; their weight is zero, but a value that is not
@@ -691,7 +691,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
           uint32_t rs[32], rp[32];
           tmem_ld_32x32(base, rs);
           tmem_ld_32x32(base + 64u, rp);
-          const uint64_t bias = sel ? pack2(st.x, st.x) : pack2(-CUDART_INF_F, -CUDART_INF_F), nd = pack2(st.y, st.y);
+          const uint64_t bias = sel ? pack2(st.x, st.x) : pack2(-CUDART_INF_F, -CUDART_INF_F), nd = pack2(st.y * geo.scale, st.y * geo.scale);
           const bool fast = __all_sync(0xffffffffu, nv == 32 || !sel);
           tmem_ld_wait();
           auto run = [&](auto masked) {

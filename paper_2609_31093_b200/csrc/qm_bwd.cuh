@@ -3,7 +3,7 @@
 // one KV head) against 64- or 128-key steps, only those some row of the tile selected; everything by contiguous TMA tile
 // loads, no inverted lists, no fp32 accumulators in memory (but for split key blocks):
 //
-//   qm_bwd_prep_kernel  per row: -lse2 and -delta * scale = -dO . O * scale; selection bits per token and their union per 128-row tile
+//   qm_bwd_prep_kernel  per row: -lse2 and -delta = -dO . O; selection bits per token and their union per 128-row tile
 //   qm_bwd_kv_kernel    one item per 128 keys: S^T = K Q^T, dP^T = V dO^T -> P^T, dS^T over them in TMEM ->
 //                       dV += P^T dO, dK += dS^T Q in TMEM over the tiles that selected any of the keys
 //   qm_bwd_q_kernel     one item per one or two tiles: S = Q K^T, dP = dO V^T -> dS over S in TMEM -> dQ += dS K in TMEM
@@ -29,7 +29,7 @@ struct Args {
   int splits, splits0;
   uint32_t* bits;            // [Hkv][len][W] per sequence, W = ceil(M1 / 32)
   uint32_t* tbits;           // [Hkv][W][tiles] per sequence
-  float2* stat;              // [Hkv][len][G] per sequence: (-lse * log2 e, -inf for a row without keys; -delta * scale)
+  float2* stat;              // [Hkv][len][G] per sequence: (-lse * log2 e, -inf for a row without keys; -delta)
   const int32_t* idx;
   const float* lse;
   const __nv_bfloat16* out;

@@ -79,7 +79,8 @@ int qm_bwd_always(const Geometry& g) { return 32 * g.K * steps_per_block8(g); }
 size_t qm_bwd_workspace_bytes(const Geometry& g) { return layout(g, uniform_sizes(g), uniform_split(g).acc).total; }
 
 int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx, const void* out, const float* lse,
-           const void* dout, void* dq, void* dk, void* dv, void* ws_, int32_t* status, Gate* gate, cudaStream_t s) {
+           const void* dout, void* dq, void* dk, void* dv, void* ws_, int32_t* status, Gate* gate, const float2** stat,
+           cudaStream_t s) {
   char* ws = (char*)ws_;
   const int tpt = 128 / g.G, units = g.B * g.Hkv;
   qmb::Args a = {};
@@ -98,6 +99,7 @@ int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const
   a.dq_s[0] = (long long)g.N * g.Hq * g.d; a.dq_s[1] = (long long)g.Hq * g.d; a.dq_s[2] = g.d;
   a.ctr = (int32_t*)(ws + l.ctr); a.status = status;
   if (gate != nullptr) {
+    *stat = a.stat;
     a.count = (uint32_t*)a.ctr + 4;
     const long long limit = (long long)a.n_tiles * g.K * steps_per_block8(g) / 8;
     *gate = Gate{a.count, (uint32_t)std::min<long long>(limit, 0xfffffffeLL)};

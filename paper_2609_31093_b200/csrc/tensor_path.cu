@@ -1765,7 +1765,8 @@ size_t tensor_bwd_workspace_bytes(const Geometry& g) { return bwd_layout(g).tota
 
 int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* v, const int32_t* idx,
                    const void* out, const float* lse, const void* dout, void* dq, void* dk, void* dv,
-                   const long long* dq_strides, long long dkv_pitch, void* ws_, int32_t* status, const Gate& gate, cudaStream_t s) {
+                   const long long* dq_strides, long long dkv_pitch, void* ws_, int32_t* status, const Gate& gate, const float2* stat,
+                   cudaStream_t s) {
   char* ws = (char*)ws_;
   const BwdLayout L = bwd_layout(g);
   kernel_mark("invert_by_leaf", s);
@@ -1776,7 +1777,7 @@ int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* 
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
   a.dout = (const __nv_bfloat16*)dout; a.lse = lse;
   float* delta = (float*)(ws + L.delta);
-  a.delta = delta;
+  a.delta = delta; a.stat = stat;
   a.entry_off = inv.entry_off; a.item_off = inv.item_off; a.item_key = inv.item_key; a.entries = inv.entries;
   a.nkeys = g.B * g.Hkv * inv.NW * g.M[1]; a.Mk = g.M[1]; a.NW = inv.NW;
   a.dq_acc = (float*)(ws + L.dq); a.dk_acc = (float*)(ws + L.dk); a.dv_acc = (float*)(ws + L.dv);
@@ -1786,10 +1787,10 @@ int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* 
   st = launch_zero(ws + L.dq, L.inv.count - L.dq, gate, s);                // dq, dk, dv accumulators are adjacent
   if (st != PISA_OK) return st;
   kernel_mark("delta", s);
-  {
+  if (stat == nullptr) {
     const long long rows = (long long)g.B * g.N * g.Hq;
     bwd_delta_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(g, (const __nv_bfloat16*)out,
-                                                                        (const __nv_bfloat16*)dout, delta, gate);
+                                                                        (const __nv_bfloat16*)dout, delta);
     st = check_launch("bwd_delta");
     if (st != PISA_OK) return st;
   }
