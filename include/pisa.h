@@ -252,9 +252,11 @@ int pisa_forward_host(const pisa_params_t* p, const void* q_host, const void* k_
  *   dout           : gradient of the loss w.r.t. out, device, same dtype and strides as out
  *   dq             : device [B, N, Hq, d], dense, input dtype
  *   dk, dv         : device [B, N, Hkv, d], dense, input dtype; keys no query selected get zeros
- *   ws             : device workspace sized for PISA_OP_BSA_BWD (holds fp32 accumulators of all
- *                    three gradients; partial sums are added with fp32 reductions, so results are
- *                    reproducible to fp32 rounding, not bitwise)
+ *   ws             : device workspace sized for PISA_OP_BSA_BWD (holds fp32 partial sums, added with fp32
+ *                    reductions, so results are reproducible to fp32 rounding, not bitwise)
+ *
+ * A row names each block at most once, as the selection does.  Shorter sequences run on dense masked tiles, long ones on
+ * inverted lists; in between the rows' selection decides on the device which of the two does the work.
  *
  * bf16, d in {64, 128}, C in {64, 128}; other configurations return PISA_ERR_UNSUPPORTED.
  * Asynchronous on `stream`.
@@ -270,7 +272,8 @@ int pisa_bsa_bwd(const pisa_params_t* p, const void* q, const void* k, const voi
  *   p, cu_seqlens, nseq : as for pisa_forward_packed (B = 1, dense strides, p->N the longest sequence)
  *   q, out, dout, dq    : device [total, Hq, d];  k, v, dk, dv : device [total, Hkv, d]
  *   idx, lse            : sequence-major, as pisa_forward_packed wrote them
- *   ws                  : device workspace sized for PISA_OP_BSA_BWD_PACKED with p: the short sequences then run in
+ *   ws                  : device workspace sized for PISA_OP_BSA_BWD_PACKED with p: sequences short enough for the
+ *                         dense tiles then run unpadded in as few sets of launches as it has room for, other short ones in
  *                         the groups pisa_packed_plan reports, each group as one padded batch (a padded query row is
  *                         given idx = -1 and so contributes to no gradient); a workspace sized for PISA_OP_BSA_BWD
  *                         is accepted too and runs one backward per sequence

@@ -54,10 +54,10 @@ size_t table_bytes(size_t n) { return align_up(n * sizeof(qm::Seq), 256) + align
 // Steps (128-row tile x 128 keys) per tile and selected block up to which the dense kernels win, in eighths.  Measured SM
 // cycles: a dense step 7.2 K (d = 64) to 8.1 K, 8.7 K beyond L2; an entry of the lists 13.1 K (C = 128), 14 to 18 K (C = 64),
 // more without groups, where every entry of a tile is a row of its own to gather.  Where the queries, dout, keys and values are
-// more than twice L2 the line lies lower: 20000 tokens, 32 heads, fan-in 4 dense 4.31 ms, lists 4.08, but 16 heads 2.05 and
-// 2.40; 16 heads without groups 14000 tokens 2.26 and 2.54, twice that 4.77 and 4.06.
+// about twice L2 the line lies lower: 20000 tokens, 32 heads, fan-in 4 dense 4.31 ms, lists 4.08, but 16 heads 2.05 and 2.40;
+// 16 heads without groups 14000 tokens (229 MB) 2.26 and 2.54, 16000 (262 MB) 2.82 and 2.58, 2 x 14000 4.77 and 4.06.
 int steps_per_block8(const Geometry& g) {
-  const bool large = (long long)g.B * g.N * (g.Hq + g.Hkv) * g.d * 4 > (256LL << 20);
+  const bool large = (long long)g.B * g.N * (g.Hq + g.Hkv) * g.d * 4 > (230LL << 20);
   if (g.G == 1) return g.C == 128 ? (large ? 15 : 19) : (large ? 20 : 24);
   return g.C == 128 ? (large ? 11 : 12) : (large ? 14 : 15);
 }
