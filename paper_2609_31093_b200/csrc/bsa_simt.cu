@@ -11,6 +11,7 @@
 // blocks of 64: a lane per key and one value row at a time 49 us; four warps per token and eight rows 34.
 #include <math_constants.h>
 
+#include "launch.cuh"
 #include "pisa_common.cuh"
 #include "simt_dot.cuh"
 
@@ -59,6 +60,7 @@ bsa_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k, 
     if (WPT == 1) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + tok), "r"(WPT * 32) : "memory");
   };
+  grid_dependency();
   const long long w = (long long)blockIdx.x * TPC + tok;
   const long long total = (long long)geo.B * geo.Hkv * geo.N;
   if (w >= total) return;
@@ -194,12 +196,12 @@ static int launch_tdg(const Geometry& g, const void* q, const void* k, const voi
   // four warps per token while that leaves no SM with more than its 64 (larger groups have work for a warp's loads to hide behind)
   if constexpr (G <= 2) {
     if (total <= 16LL * num_sms()) {
-      bsa_simt_kernel<T, D, G, 4><<<(unsigned)ctas, 512, 0, s>>>(g, (const T*)q, (const T*)k, (const T*)v, idx, (T*)out, lse);
-      return check_launch("bsa_simt");
+      return launch_dependent<bsa_simt_kernel<T, D, G, 4>>("bsa_simt", dim3((unsigned)ctas), 512u, 0, s, g, (const T*)q, (const T*)k,
+                                                           (const T*)v, idx, (T*)out, lse);
     }
   }
-  bsa_simt_kernel<T, D, G, 1><<<(unsigned)ctas, 128, 0, s>>>(g, (const T*)q, (const T*)k, (const T*)v, idx, (T*)out, lse);
-  return check_launch("bsa_simt");
+  return launch_dependent<bsa_simt_kernel<T, D, G, 1>>("bsa_simt", dim3((unsigned)ctas), 128u, 0, s, g, (const T*)q, (const T*)k,
+                                                       (const T*)v, idx, (T*)out, lse);
 }
 
 template <typename T, int D>

@@ -16,6 +16,7 @@
 // block score and dropped.
 #include <math_constants.h>
 
+#include "launch.cuh"
 #include "pisa_common.cuh"
 #include "simt_dot.cuh"
 
@@ -117,6 +118,7 @@ route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k
     if (WPT == 1) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + warp), "r"(WPT * 32) : "memory");
   };
+  grid_dependency();
   const long long w = (long long)blockIdx.x * kTokensPerCta + warp;
   const long long total = (long long)geo.B * geo.Hkv * geo.N;
   if (w >= total) return;
@@ -303,15 +305,13 @@ static int launch_route_tdg(const Geometry& g, const void* q, const void* k, con
   // four warps per token while that leaves no SM with more than its 64
   constexpr int WPT = G <= 2 ? 4 : 1;
   if (leaf && WPT > 1 && total <= 16LL * num_sms())
-    route_simt_kernel<T, D, G, true, WPT><<<(unsigned)ctas, kTokensPerCta * WPT * 32, 0, s>>>(
-        g, (const T*)q, (const T*)k, (const T*)pyr, idx, margin, nullptr);
-  else if (leaf)
-    route_simt_kernel<T, D, G, true, 1><<<(unsigned)ctas, kTokensPerCta * 32, 0, s>>>(
-        g, (const T*)q, (const T*)k, (const T*)pyr, idx, margin, nullptr);
-  else
-    route_simt_kernel<T, D, G, false, 1><<<(unsigned)ctas, kTokensPerCta * 32, 0, s>>>(
-        g, (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
-  return check_launch("route_simt");
+    return launch_dependent<route_simt_kernel<T, D, G, true, WPT>>("route_simt", dim3((unsigned)ctas), kTokensPerCta * WPT * 32u, 0, s, g,
+                                                                   (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
+  if (leaf)
+    return launch_dependent<route_simt_kernel<T, D, G, true, 1>>("route_simt", dim3((unsigned)ctas), kTokensPerCta * 32u, 0, s, g,
+                                                                 (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
+  return launch_dependent<route_simt_kernel<T, D, G, false, 1>>("route_simt", dim3((unsigned)ctas), kTokensPerCta * 32u, 0, s, g,
+                                                                (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
 }
 
 template <typename T, int D>
