@@ -6,8 +6,8 @@
 // softmax over chunks of 32 keys, dealt out to the token's warps, whose sums are merged at the end.
 //
 // Bound by the wavefronts and the latency of a warp's loads: key rows are read by several lanes each (simt_dot.cuh; not for
-// large groups), value rows eight at a time, and where the tokens alone do not fill the GPU each gets four warps; the sixteen
-// warps of a CTA serve four neighbouring tokens then, which find one another's rows in L1.  1024 tokens, one head, d = 64, four
+// large groups), value rows eight at a time, and where the tokens alone do not fill the GPU each gets four or eight warps;
+// the sixteen warps of a CTA serve neighbouring tokens then, which find one another's rows in L1.  1024 tokens, one head, d = 64, four
 // blocks of 64: a lane per key and one value row at a time 49 us; four warps per token and eight rows 34.
 #include <math_constants.h>
 
@@ -46,11 +46,11 @@ __device__ __forceinline__ void dot_row(const T* __restrict__ row, const float* 
 }  // namespace
 
 template <typename T, int D, int G, int WPT>
-__global__ void __launch_bounds__(WPT * 128)
+__global__ void __launch_bounds__(WPT == 1 ? 128 : 512)
 bsa_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                 const int32_t* __restrict__ idx, T* __restrict__ out, float* __restrict__ lse) {
   constexpr int DV = D / 32;                  // output dims per lane
-  constexpr int TPC = 4;                      // tokens per CTA
+  constexpr int TPC = WPT == 1 ? 4 : 16 / WPT;   // tokens per CTA
   constexpr int UV = G <= 4 ? 8 : 4;          // value rows in flight
   __shared__ __align__(16) float s_q[TPC][G * D];
   __shared__ float s_acc[WPT > 1 ? TPC : 1][WPT > 1 ? WPT : 1][WPT > 1 ? G * D : 1], s_ml[WPT > 1 ? TPC : 1][WPT > 1 ? WPT : 1][2 * G];
@@ -193,8 +193,13 @@ static int launch_tdg(const Geometry& g, const void* q, const void* k, const voi
   const long long total = (long long)g.B * g.Hkv * g.N;
   const long long ctas = (total + 3) / 4;
   if (ctas > 0x7fffffffLL) return PISA_ERR_UNSUPPORTED;
-  // four warps per token while that leaves no SM with more than its 64 (larger groups have work for a warp's loads to hide behind)
+  // four warps per token while that leaves no SM with more than its 64, eight below a third of that (larger groups have work for
+  // a warp's loads to hide behind).  One head, d = 64: 300 tokens 36.7 us with four, 28.8 with eight (whole forward, the routing
+  // split alike), 600 tokens 44.7 and 41.2, 1024 tokens 47.0 and 53.9
   if constexpr (G <= 2) {
+    if (total <= 5LL * num_sms())
+      return launch_dependent<bsa_simt_kernel<T, D, G, 8>>("bsa_simt", dim3((unsigned)((total + 1) / 2)), 512u, 0, s, g, (const T*)q,
+                                                           (const T*)k, (const T*)v, idx, (T*)out, lse);
     if (total <= 16LL * num_sms()) {
       return launch_dependent<bsa_simt_kernel<T, D, G, 4>>("bsa_simt", dim3((unsigned)ctas), 512u, 0, s, g, (const T*)q, (const T*)k,
                                                            (const T*)v, idx, (T*)out, lse);

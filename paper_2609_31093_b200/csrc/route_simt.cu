@@ -1,4 +1,4 @@
-// Coarse-to-fine Top-K routing, one or four warps per (b, KV head, query token), every level fused in one
+// Coarse-to-fine Top-K routing, one, four or eight warps per (b, KV head, query token), every level fused in one
 // launch (Sec. 3.2 "Coarse-to-fine block selection"; the paper's "per-query" schedule, App. B).
 //
 // This is the exact-fp32 SIMT path: it serves the fp32 dtype, every shape the tensor-core path does
@@ -6,7 +6,7 @@
 // levels (LEAF = false), is stage 1 of the two-stage schedule (Algorithm 1): it then stores the
 // kept level-2 nodes, whose children are the leaf candidates, instead of scoring the leaves.
 //
-// Where the tokens alone do not fill the GPU a token has WPT = 4 warps: the first walks the levels, all of them share the
+// Where the tokens alone do not fill the GPU a token has WPT warps: the first walks the levels, all of them share the
 // scoring of the leaves, a leaf each; key rows are read by several lanes each (simt_dot.cuh; not for large groups).
 // 1024 tokens, one head, d = 64, K = 4: one warp per token and a lane per key 35 us.
 //
@@ -24,7 +24,7 @@ namespace pisa {
 
 namespace {
 
-constexpr int kTokensPerCta = 4;
+__host__ __device__ constexpr int simt_tokens(int wpt) { return wpt == 8 ? 2 : 4; }   // tokens per CTA
 
 template <typename T, int D, int G>
 __device__ __forceinline__ void dot_row(const T* __restrict__ row, const float* __restrict__ qf,
@@ -101,10 +101,11 @@ __device__ __forceinline__ float stat_warp_finish(Stat s, int mode) {
 }  // namespace
 
 template <typename T, int D, int G, bool LEAF, int WPT>
-__global__ void __launch_bounds__(kTokensPerCta * WPT * 32)
+__global__ void __launch_bounds__(simt_tokens(WPT) * WPT * 32)
 route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k,
                   const T* __restrict__ pyr, int32_t* __restrict__ idx, float* __restrict__ margin,
                   int32_t* __restrict__ cand_out) {
+  constexpr int kTokensPerCta = simt_tokens(WPT);
   static_assert(LEAF || WPT == 1, "only the leaf level is shared");
   __shared__ __align__(16) float s_q[kTokensPerCta][G * D];
   __shared__ int s_cand[kTokensPerCta][2][kMaxCand];
@@ -300,10 +301,17 @@ template <typename T, int D, int G>
 static int launch_route_tdg(const Geometry& g, const void* q, const void* k, const void* pyr,
                             int32_t* idx, float* margin, int32_t* cand_out, bool leaf, cudaStream_t s) {
   const long long total = (long long)g.B * g.Hkv * g.N;
+  constexpr int kTokensPerCta = 4;
   const long long ctas = (total + kTokensPerCta - 1) / kTokensPerCta;
   if (ctas > 0x7fffffffLL) return PISA_ERR_UNSUPPORTED;
-  // four warps per token while that leaves no SM with more than its 64
+  // four warps per token while that leaves no SM with more than its 64, eight below a third of that (times beside the same rule
+  // in bsa_simt.cu)
   constexpr int WPT = G <= 2 ? 4 : 1;
+  if constexpr (G <= 2) {
+    if (leaf && total <= 5LL * num_sms())
+      return launch_dependent<route_simt_kernel<T, D, G, true, 8>>("route_simt", dim3((unsigned)((total + 1) / 2)), 512u, 0, s, g,
+                                                                   (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
+  }
   if (leaf && WPT > 1 && total <= 16LL * num_sms())
     return launch_dependent<route_simt_kernel<T, D, G, true, WPT>>("route_simt", dim3((unsigned)ctas), kTokensPerCta * WPT * 32u, 0, s, g,
                                                                    (const T*)q, (const T*)k, (const T*)pyr, idx, margin, cand_out);
