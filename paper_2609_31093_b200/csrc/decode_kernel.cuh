@@ -128,7 +128,7 @@ __device__ __forceinline__ void heads_dot(const HeadFrag<D, WIDE>& q, const RowF
 
 // Select_K among n <= 128 candidates by all 256 threads: every candidate's rank under (score descending, position
 // ascending) is counted by four (n <= 64) or two threads, the kept ones (all of them when n <= K) are handed, in order, to
-// emit(position, candidate).  u: scores, 16-byte aligned, -inf from n to the next multiple of 64 when n > K.
+// emit(position, candidate).  u: scores (rankable), 16-byte aligned, -inf from n to the next multiple of 64 when n > K.
 // Returns the number kept.  Starts and ends with a barrier.
 template <typename Emit>
 __device__ __forceinline__ int block_select(const float* u, int n, int K, int* s_cnt, Emit&& emit) {
@@ -347,7 +347,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
     if (nV > K) {
       if (upfront) {
         if (tid < kMaxCand)
-          s_u[tid] = (tid >= nV) ? -CUDART_INF_F : (tid > 0 && tid < nEnd) ? s_tab[a.tile0[l] * 8 + cand[tid]] : forced_score(tid);
+          s_u[tid] = (tid >= nV) ? -CUDART_INF_F : (tid > 0 && tid < nEnd) ? rankable(s_tab[a.tile0[l] * 8 + cand[tid]]) : forced_score(tid);
       } else {
         for (int s = nV + tid; s < kMaxCand; s += kDecThreads) s_u[s] = -CUDART_INF_F;
         for (int k0 = warp * 8; k0 < nV; k0 += kDecThreads / 4) {
@@ -358,7 +358,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
 #pragma unroll
           for (int x = 0; x < 2; ++x) {
             const int s = k0 + 2 * tig + x;
-            if (gid == 0 && s < nV) s_u[s] = (s > 0 && s < nEnd) ? us[x] : forced_score(s);
+            if (gid == 0 && s < nV) s_u[s] = (s > 0 && s < nEnd) ? rankable(us[x]) : forced_score(s);
           }
         }
       }
@@ -451,7 +451,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
         us += __shfl_xor_sync(0xffffffffu, us, 4);
         us += __shfl_xor_sync(0xffffffffu, us, 8);
         us += __shfl_xor_sync(0xffffffffu, us, 16);
-        if (lane < CLU) st_remote(remote_smem(&s_leaf[ci], lane), us);
+        if (lane < CLU) st_remote(remote_smem(&s_leaf[ci], lane), rankable(us));
       }
     }
   }
@@ -469,7 +469,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
       lse_merge(m, ssum, p[2 * (NG + hh)], p[2 * (NG + hh) + 1]);
       us += m + __logf(ssum);
     }
-    s_leaf[tid] = us;
+    s_leaf[tid] = rankable(us);
   }
   const int nsel = block_select(s_leaf, nV, K, s_cnt, [&](int p, int s) { s_sel[p] = cand[s]; });
   if (rank == 0 && tid < K) a.idx[(long long)bh * K + tid] = (tid < nsel) ? s_sel[tid] : -1;

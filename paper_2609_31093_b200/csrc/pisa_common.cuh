@@ -150,6 +150,9 @@ __device__ inline float warp_sum(float v) {
 // position, so that they rank first.  A real score never comes near kForcedFloor.
 constexpr float kForcedFloor = 1.0e38f;
 __device__ __forceinline__ float forced_score(int pos) { return 3.0e38f - (float)pos * 1.0e34f; }
+// A score that is not a number (a key or a query that is not finite) ranks after every other one.  The selections count on
+// an order: left as it is, a NaN beats nothing and loses to nothing, and more than K candidates would be kept.
+__device__ __forceinline__ float rankable(float score) { return fmaxf(score, __int_as_float(0xff800000)); }
 
 // Rank of each candidate under (score descending, position ascending), for the candidates
 // s = lane + 32*k this lane owns.  `u` is the warp's score array in shared memory, 16-byte aligned,

@@ -194,7 +194,7 @@ route_stage1_mma_kernel(Geometry geo, const __nv_bfloat16* __restrict__ q, const
         }
         usum += __shfl_xor_sync(0xffffffffu, usum, 1);
         usum += __shfl_xor_sync(0xffffffffu, usum, 2);
-        if (has && tig == 0) u[kap] = (node == 0 || node == f1 || node == anc_c) ? forced_score(kap) : usum;
+        if (has && tig == 0) u[kap] = (node == 0 || node == f1 || node == anc_c) ? forced_score(kap) : rankable(usum);
       }
       if (lane < 4 && nV + lane < kMaxCand) u[nV + lane] = -CUDART_INF_F;     // padding read by the 16-byte loads
       __syncwarp();

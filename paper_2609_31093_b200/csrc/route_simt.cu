@@ -180,7 +180,7 @@ route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k
       float score = 0.f;
 #pragma unroll
       for (int hh = 0; hh < G; ++hh) score += stat_warp_finish(st[hh], mode);
-      if (lane == 0) u[s] = score;
+      if (lane == 0) u[s] = rankable(score);
     }
   };
   if (WPT > 1 && part > 0) {
@@ -228,7 +228,7 @@ route_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k
 #pragma unroll
               for (int hh = 0; hh < G; ++hh) score += stat_finish(st[hh], mode);
             }
-            u[s] = score;
+            u[s] = rankable(score);
           }
         } else {
           if (WPT > 1) {

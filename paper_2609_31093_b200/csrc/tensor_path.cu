@@ -1201,6 +1201,7 @@ __global__ void __launch_bounds__(128) final_topk_kernel(Geometry geo, const int
             sc = 0.f;
             for (int hh = 0; hh < G; ++hh) sc += bl[ci * G + hh];
           }
+          sc = rankable(sc);
         }
       }
       u[ci] = sc;

@@ -1,0 +1,111 @@
+"""Keys, queries, values and gradients that are not finite: what they reach and what they must not.
+
+Selection: a score that is not a number ranks after every other one, ties to the smaller index, on every path; a row always
+gets min(K, leaves before it) distinct blocks, the forced ones among them."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import pisa_synth as S
+from oracle import pisa_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+import pisa_testlib as T  # noqa: E402
+import paper_2609_31093_b200 as P  # noqa: E402
+from paper_2609_31093_b200 import binding as PB  # noqa: E402
+
+NAN = float("nan")
+
+
+def _walk(q, k, level, M, L, C, g, K, pos):
+    """Select_K of Sec. 3.2 for one row: q [G, d], k [N, d], level(l) [M_l, d] (device tensors).  Returns the leaves and the
+    smallest relative gap between a kept and a dropped score (rows inside the tie band may go either way)."""
+    q = q.double()
+    scale = 1.0 / math.sqrt(q.shape[1])
+    c = pos // C
+    A, gap = [0], math.inf
+    for l in range(L, 0, -1):
+        V = [i for i in A if i < M[l] and i <= c // g ** (l - 1)]
+        if len(V) > K:
+            F = O.forced_nodes(l, c, g)
+            rest = [i for i in V if i not in F]
+            u = {}
+            for i in rest:
+                x = (k[i * C:(i + 1) * C] if l == 1 else level(l - 1)[i * g:(i + 1) * g]).double()
+                s = float(torch.logsumexp(q @ x.T * scale, 1).sum())
+                u[i] = -math.inf if math.isnan(s) else s
+            order = sorted(rest, key=lambda i: (-u[i], i))
+            keep = K - len(F)
+            a, b = u[order[keep - 1]], u[order[keep]]
+            if a > -math.inf:
+                gap = min(gap, (a - b) / max(abs(a), 1.0))
+            V = sorted(set(F) | set(order[:keep]))
+        A = V if l == 1 else [r for i in V for r in range(i * g, i * g + g)]
+    return A, gap
+
+
+def _check_row(row, want, gap, K, c, what):
+    n = min(K, c + 1)
+    row = row.tolist()
+    assert row[n:] == [-1] * (K - n) and all(a < b for a, b in zip(row[:n], row[1:n])), (what, row)
+    assert {0, max(c - 1, 0), c} <= set(row[:n]) and 0 <= row[0] and row[n - 1] <= c, (what, row)
+    if gap > T.TIE_BAND:
+        assert row[:n] == want, (what, row, want)
+
+
+@pytest.mark.parametrize("C,g,K,G", [(64, 2, 16, 4), (32, 4, 32, 1), (64, 4, 32, 16), (64, 4, 3, 2)])
+def test_decoding_with_keys_that_are_not_numbers(C, g, K, G):
+    N, Hkv, d = 8192, 2, 64
+    w = S.Workload("nf_dec", 1, N, G * Hkv, Hkv, d, C, g, K, "bf16", 2100 + K, "iid")
+    t = S.make_inputs(w)
+    q, k, v = (T.to_torch(t[x], "bf16") for x in ("q", "k", "v"))
+    rng = np.random.default_rng(5)
+    M1 = N // C
+    for leaf in rng.choice(np.arange(1, M1 - 3), size=M1 // 2, replace=False):       # half of all leaves
+        k[0, int(leaf) * C + int(rng.integers(C)), 0] = NAN
+    k[0, (M1 // 2) * C + 5, 1] = NAN                                                 # head 1: one leaf
+    p = P.Params(1, N, G * Hkv, Hkv, d, C, g, K, dtype="bf16")
+    pyr = PB.alloc_pyramid(p)
+    P.pisa_build_pyramid(p, k, pyr)
+    L, M, off, _ = P.pyramid_layout(p)
+    ws = PB.alloc_workspace(p, PB.OP_DECODE)
+    idx = torch.full((1, Hkv, K), -7, dtype=torch.int32, device="cuda")
+    out, lse = torch.zeros((1, G * Hkv, d), dtype=torch.bfloat16, device="cuda"), torch.zeros((1, G * Hkv), device="cuda")
+    for pos in (N - 1, N - 100, N // 2 + 3):
+        P.pisa_decode_step(p, pos, q[:, pos].contiguous(), k, v, pyr, idx, out, lse, ws)
+        torch.cuda.synchronize()
+        assert P.read_status(ws) == 0
+        for h in range(Hkv):
+            level = lambda l: pyr[off[l]:off[l] + Hkv * M[l] * d].view(Hkv, M[l], d)[h]  # noqa: E731
+            want, gap = _walk(q[0, pos, h * G:(h + 1) * G], k[0, :, h], level, M, L, C, g, K, pos)
+            _check_row(idx[0, h], want, gap, K, pos // C, (pos, h))
+
+
+@pytest.mark.parametrize("dtype,impl,N,C,g,K,G", [("bf16", PB.IMPL_SIMT, 6000, 64, 2, 16, 2), ("fp32", PB.IMPL_AUTO, 3000, 32, 4, 32, 1),
+                                                  ("bf16", PB.IMPL_AUTO, 9000, 64, 2, 4, 16)])
+def test_ranked_selections_with_keys_that_are_not_numbers(dtype, impl, N, C, g, K, G):
+    """The kernels that select with a warp per token (SIMT; lists with large groups)."""
+    _selection(dtype, impl, N, C, g, K, G)
+
+
+def _selection(dtype, impl, N, C, g, K, G):
+    Hkv, d = 2, 64
+    w = S.Workload("nf_sel", 1, N, G * Hkv, Hkv, d, C, g, K, dtype, 2200 + K, "iid")
+    t = S.make_inputs(w)
+    dev = T.Device(w, t, impl=impl)
+    rng = np.random.default_rng(6)
+    M1 = -(-N // C)
+    for leaf in rng.choice(np.arange(1, M1 - 3), size=M1 // 2, replace=False):
+        dev.k[0, int(leaf) * C + int(rng.integers(C)), 0] = NAN
+    dev.k[0, (M1 // 2) * C + 5, 1] = NAN
+    dev.build_pyramid()
+    dev.route(with_margin=False)
+    assert dev.sync_status() == 0
+    rows = sorted({0, C, K * C, N // 2 + 3, N - 1} | {int(x) for x in rng.integers(0, N, 20)})
+    for h in range(Hkv):
+        for pos in rows:
+            want, gap = _walk(dev.q[0, pos, h * G:(h + 1) * G], dev.k[0, :, h], lambda l: dev.level(l)[0, h], dev.M, dev.L, C, g, K, pos)
+            _check_row(dev.idx[0, h, pos], want, gap, K, pos // C, (pos, h))
