@@ -81,6 +81,29 @@ __device__ __forceinline__ float sum_heads(const float* p) {
   return s;
 }
 
+// Select_K among nV > K scores by counting, a NaN last (the sorting network's results assume an order)
+struct Ranked { uint4 keep; float cut, next; };                   // one bit per candidate; the K-th largest score and the one after
+__device__ __noinline__ Ranked select_by_rank(const float* u, int nV, int K) {
+  Ranked r;
+  r.keep = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = 0; i < nV; ++i) {
+    const float ui = rankable(u[i * kSelThreads]);
+    int rank = 0;
+    for (int j = 0; j < nV; ++j) {
+      const float uj = rankable(u[j * kSelThreads]);
+      rank += uj > ui || (uj == ui && j < i);
+    }
+    const uint32_t bit = rank < K ? 1u << (i & 31) : 0u;
+    if (i < 32) r.keep.x |= bit;
+    else if (i < 64) r.keep.y |= bit;
+    else if (i < 96) r.keep.z |= bit;
+    else r.keep.w |= bit;
+    if (rank == K - 1) r.cut = ui;
+    if (rank == K) r.next = ui;
+  }
+  return r;
+}
+
 // NC: candidates a token can have at a level (g * K rounded up), FAN = g.
 // Bound by the latency of its loads, twelve warps per SM waiting; bounding the registers for more (10, 12, 14 CTAs per SM)
 // spills the sorting network: 575 us -> 576, 595, 600 for a forward of 8192 tokens, 16 heads.
@@ -193,12 +216,11 @@ __global__ void __launch_bounds__(kSelThreads) qm_select_kernel(Geometry geo, qm
 #pragma unroll
       for (int i = 0; i < NC; ++i)
         if (i == K - 1) T = v[i];
+      float T1 = 0.f;                                              // and the next one
       if (sa.margin != nullptr) {
-        float T1 = 0.f;
 #pragma unroll
         for (int i = 0; i < NC; ++i)
           if (i == K) T1 = v[i];
-        if (T < kForcedFloor) gap = fminf(gap, (T - T1) / fmaxf(fabsf(T), 1.f));
       }
       int cnt = 0;
 #pragma unroll
@@ -210,17 +232,29 @@ __global__ void __launch_bounds__(kSelThreads) qm_select_kernel(Geometry geo, qm
         keep[w] = (valid >= 32) ? m : (valid > 0 ? m & ((1u << valid) - 1u) : 0u);
         cnt += __popc(keep[w]);
       }
+      int room = K;                                                // less the candidates above the cut
       if (cnt > K) {                                               // equal scores at the cut: the smaller positions stay
-        int room = K;
         for (int w = 0; w < NW; ++w)
           for (uint32_t m = keep[w]; m != 0u; m &= m - 1u) room -= s_u[(w * 32 + __ffs(m) - 1) * kSelThreads] > T;
+        int eq = 0;
 #pragma unroll
         for (int w = 0; w < NW; ++w)
           for (uint32_t m = keep[w]; m != 0u; m &= m - 1u) {
             const int i = __ffs(m) - 1;
-            if (s_u[(w * 32 + i) * kSelThreads] == T && --room < 0) keep[w] &= ~(1u << i);
+            if (s_u[(w * 32 + i) * kSelThreads] == T && ++eq > room) keep[w] &= ~(1u << i);
           }
       }
+      // T is the K-th largest exactly if at least K candidates reach it and fewer than K exceed it.  A comparator replaces a
+      // NaN by a copy of its other input, so with scores that are not numbers it may be another one: then by rank, NaN last
+      // (clamping every score instead costs 3 us of the 530 of a forward of 8192 tokens, 16 heads)
+      if (cnt < K || room < 1) {
+        const Ranked r = select_by_rank(s_u, nV, K);
+        T = r.cut;
+        T1 = r.next;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) keep[w] = w == 0 ? r.keep.x : w == 1 ? r.keep.y : w == 2 ? r.keep.z : r.keep.w;
+      }
+      if (sa.margin != nullptr && T < kForcedFloor) gap = fminf(gap, (T - T1) / fmaxf(fabsf(T), 1.f));
     } else {
 #pragma unroll
       for (int w = 0; w < NW; ++w) {

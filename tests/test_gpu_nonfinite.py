@@ -91,6 +91,13 @@ def test_ranked_selections_with_keys_that_are_not_numbers(dtype, impl, N, C, g, 
     _selection(dtype, impl, N, C, g, K, G)
 
 
+@pytest.mark.parametrize("N,C,g,K,G", [(5000, 64, 2, 16, 4), (2500, 128, 4, 4, 2), (3000, 64, 4, 32, 1),   # query-major
+                                       (20000, 64, 2, 16, 4), (9000, 64, 4, 8, 2)])                    # lists
+def test_sorted_selections_with_keys_that_are_not_numbers(N, C, g, K, G):
+    """The kernels that select with a thread per token and a sorting network."""
+    _selection("bf16", PB.IMPL_AUTO, N, C, g, K, G)
+
+
 def _selection(dtype, impl, N, C, g, K, G):
     Hkv, d = 2, 64
     w = S.Workload("nf_sel", 1, N, G * Hkv, Hkv, d, C, g, K, dtype, 2200 + K, "iid")
