@@ -244,6 +244,15 @@ __device__ void refresh_path(const Geometry& geo, const DecArgs& a, int b, int h
   }
 }
 
+// the same as a launch of its own, for batches whose refreshing clusters do not fit into the step's grid (a third index
+// there, read by every CTA, cost 0.4 us of the 34 of a step of 32 sequences)
+template <int D>
+__global__ void __launch_bounds__(kDecThreads) decode_refresh_kernel(const __grid_constant__ Geometry geo, const __grid_constant__ DecArgs a) {
+  grid_dependency();
+  const int u = blockIdx.x * kDecWarps + (threadIdx.x >> 5);
+  if (u < a.units) refresh_path<D>(geo, a, u / geo.Hkv, u % geo.Hkv, threadIdx.x & 31);
+}
+
 // NG: query heads per KV head.  KT: keys per attention piece.  MINB = 1: all registers to one CTA per SM (lowest latency);
 // MINB = 2: two CTAs per SM so that the latency-bound phases of different clusters overlap once the grid exceeds the SM
 // count.  CLU: CTAs per cluster.  MOM: false = LSE score, true = the mean / mean + variance scores.
@@ -639,8 +648,14 @@ int launch_decode(const Geometry& g, const DecArgs& a, cudaStream_t s) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) { record_cuda_error("decode_step attr", e); return PISA_ERR_CUDA; }
   }
-  return launch_dependent<kern>("decode_step", dim3(CLU, (unsigned)(a.units + refresh_clusters(a.units, CLU))), kDecThreads,
-                                decode_smem<D, NG>(), s, g, a);
+  int refresh = refresh_clusters(a.units, CLU);
+  if (a.units + refresh > 65535) {                         // more clusters than a grid's y holds
+    refresh = 0;
+    const int st = launch_dependent<decode_refresh_kernel<D>>("decode_refresh", dim3((unsigned)((a.units + kDecWarps - 1) / kDecWarps)),
+                                                              kDecThreads, 0, s, g, a);
+    if (st != PISA_OK) return st;
+  }
+  return launch_dependent<kern>("decode_step", dim3(CLU, (unsigned)(a.units + refresh)), kDecThreads, decode_smem<D, NG>(), s, g, a);
 }
 // How many clusters of this instantiation the GPU holds at once (clusters are placed inside one GPC, so
 // this is less than SMs * MINB / CLU); asked of the driver once per instantiation.
