@@ -658,17 +658,21 @@ int launch_decode(const Geometry& g, const DecArgs& a, cudaStream_t s) {
   return launch_dependent<kern>("decode_step", dim3(CLU, (unsigned)(a.units + refresh)), kDecThreads, decode_smem<D, NG>(), s, g, a);
 }
 // How many clusters of this instantiation the GPU holds at once (clusters are placed inside one GPC, so
-// this is less than SMs * MINB / CLU); asked of the driver once per instantiation.
+// this is less than SMs * MINB / CLU); asked of the driver once per instantiation and device, again if it could not say.
 template <int D, int NG, int CLU>
 int resident_clusters() {
-  static int cached = -1;
-  if (cached >= 0) return cached;
+  constexpr int kMaxDev = 64;
+  static std::atomic<int> cached[kMaxDev] = {};           // clusters + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
+  const bool keep = dev >= 0 && dev < kMaxDev;
+  const int known = keep ? cached[dev].load(std::memory_order_relaxed) : 0;
+  if (known > 0) return known - 1;
   const size_t smem = decode_smem<D, NG>();
   constexpr auto kern = decode_step_kernel<D, NG, decode_piece(NG, 1), 1, CLU, false>;
   allow_smem<kern>(smem);
   if (CLU > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
-    cached = 0;
     return 0;
   }
   cudaLaunchConfig_t cfg = {};
@@ -681,8 +685,8 @@ int resident_clusters() {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-  cached = n;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  if (keep) cached[dev].store(n + 1, std::memory_order_relaxed);
   return n;
 }
 

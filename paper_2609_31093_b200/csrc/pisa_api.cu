@@ -678,21 +678,27 @@ static size_t forward_ws_bytes(const pisa_params_t* p, const Geometry& g, int* s
 }
 
 // The arena queries walk every padded length (a few hundred microseconds of host time), and a program asks with the
-// same parameters on every call: the last answers are kept, per host thread.
+// same parameters on every call: the last answers are kept, per host thread and device (sizes depend on its SM count).
 extern "C++" {
 template <typename Arena>
 struct ArenaMemo {
   static constexpr int kEntries = 4;
-  struct Entry { pisa_params_t p; int chunks; bool used; Arena a; } e[kEntries];
-  int next;
+  struct Entry { pisa_params_t p; int chunks, dev; bool used; Arena a; } e[kEntries];
+  unsigned next;
+  static int device() {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); dev = -1; }   // (sizes can be asked for without a device)
+    return dev;
+  }
   bool find(const pisa_params_t* p, int chunks, Arena* a) const {
+    const int dev = device();
     for (int i = 0; i < kEntries; ++i)
-      if (e[i].used && e[i].chunks == chunks && memcmp(&e[i].p, p, sizeof(*p)) == 0) { *a = e[i].a; return true; }
+      if (e[i].used && e[i].chunks == chunks && e[i].dev == dev && memcmp(&e[i].p, p, sizeof(*p)) == 0) { *a = e[i].a; return true; }
     return false;
   }
   void keep(const pisa_params_t* p, int chunks, const Arena& a) {
     Entry& x = e[next++ % kEntries];
-    x.p = *p; x.chunks = chunks; x.a = a; x.used = true;
+    x.p = *p; x.chunks = chunks; x.dev = device(); x.a = a; x.used = true;
   }
 };
 }
