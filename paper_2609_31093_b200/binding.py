@@ -145,11 +145,13 @@ def _stream():
 
 def _offsets(cu_seqlens):
     """Host offsets as a C int32 array."""
-    try:
-        a = array.array("i", cu_seqlens)
-    except TypeError:                        # offsets that are not integers by type
-        a = array.array("i", [int(x) for x in cu_seqlens])
-    return (C.c_int32 * len(a)).from_buffer(a)
+    if not isinstance(cu_seqlens, (bytes, bytearray)):    # (array() would take their bytes for the integers' memory)
+        try:
+            a = array.array("i", cu_seqlens)
+            return (C.c_int32 * len(a)).from_buffer(a)
+        except (TypeError, OverflowError):                # not integers by type, or wider than 32 bits: as ctypes takes them
+            pass
+    return (C.c_int32 * len(cu_seqlens))(*[int(x) for x in cu_seqlens])
 
 
 def pyramid_layout(p: Params) -> Tuple[int, list, list, int]:

@@ -88,3 +88,15 @@ def test_group_size_is_capped_by_the_kv_head_count():
         sizes = np.bincount(np.asarray(group))
         assert sizes.max() == cap and n_groups == -(-5000 // cap), (Hkv, sizes.max(), n_groups)
         assert set(padded) == {8}
+
+
+def test_offsets_of_every_kind_of_sequence():
+    p = P.Params(1, 64, 4, 2, 64, 64, 2, 3)
+    want = P.packed_plan(p, [0, 5, 9, 40])
+    import array
+    import torch
+    for cu in ((0, 5, 9, 40), np.array([0, 5, 9, 40], np.int64), [0.0, 5.0, 9.0, 40.0], torch.tensor([0, 5, 9, 40]), bytes([0, 5, 9, 40]),
+               bytearray([0, 5, 9, 40]), array.array("q", [0, 5, 9, 40]), range(0, 1)):
+        assert P.packed_plan(p, cu) == (want if len(cu) > 1 else ([], [], 0)), type(cu)
+    with pytest.raises(P.PisaError):
+        P.packed_plan(p, [0, 2 ** 31])                                      # wider than the C type: refused, as any bad length
