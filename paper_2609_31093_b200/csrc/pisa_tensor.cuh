@@ -46,6 +46,7 @@ int qm_stage1(const Geometry& g, const void* q, const void* pyramid, int32_t* pa
 // leaf level of the list-driven path: Select_K among the children of `par` by their scores `blk` (any score mode)
 int qm_select_final(const Geometry& g, const int32_t* par, const float* blk, int32_t* idx, float* margin, float* lse_out,
                     float* sel_lse, int32_t* status, cudaStream_t s);
+bool tma_strides(const long long* st);
 bool qm_map_rows(void* map, const void* base, int d, int H, long long tokens, int B, const long long* st, int heads, int rows);
 int launch_qm_score(const Geometry& g, const qm::Args& a, const void* q, const void* k, long long tokens, const void* pyramid,
                     long long pyr_rows, cudaStream_t s);

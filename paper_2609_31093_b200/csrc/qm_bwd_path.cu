@@ -78,7 +78,8 @@ int qm_bwd_splits0(long long tiles_of_longest, int splits) {
 int qm_bwd_tiles_per_item(long long tiles) { return tiles >= 2LL * num_sms() ? 2 : 1; }
 
 bool qm_bwd_supported(const Geometry& g, int dtype) {
-  return dtype == PISA_BF16 && (g.d == 64 || g.d == 128) && (g.C == 64 || g.C == 128) && g.M[1] <= 1024;
+  return dtype == PISA_BF16 && (g.d == 64 || g.d == 128) && (g.C == 64 || g.C == 128) && g.M[1] <= 1024 &&
+         tma_strides(g.qs) && tma_strides(g.os);                    // (keys and values are read through tensor maps on either path)
 }
 // (a tile has N / 256 steps on average when it needs all key blocks)
 int qm_bwd_always(const Geometry& g) { return 32 * g.K * steps_per_block8(g); }

@@ -54,8 +54,17 @@ int qm_tiles_per_item(const Geometry& g, long long unit_tokens) {
   return unit_tokens * g.G / 256 >= 3LL * num_sms() ? 2 : 1;
 }
 
+// Strides a tensor map can hold: below 2^40 bytes, not negative (the other kernels that read queries gather rows by pointer
+// and take any).
+bool tma_strides(const long long* st) {
+  for (int i = 0; i < 3; ++i)
+    if (st[i] < 0 || st[i] >= (1LL << 39)) return false;
+  return true;
+}
+
 bool qm_supported(const Geometry& g, int dtype) {
   if (dtype != PISA_BF16 || g.score_mode != PISA_SCORE_LSE) return false;
+  if (!tma_strides(g.qs) || !tma_strides(g.ks) || !tma_strides(g.vs)) return false;
   if ((g.d != 64 && g.d != 128) || (g.C != 64 && g.C != 128)) return false;
   return g.g == 2 || g.g == 4;
 }

@@ -66,3 +66,36 @@ def test_head_major_tensors_by_strides(name, impl):
         assert P.read_status(wsb) == 0 and P.read_status(wsd) == 0
         for a, b in zip(g_s, g_d):
             assert torch.allclose(a.float(), b.float(), rtol=0, atol=2.0 ** -6 * float(b.float().abs().max()))
+
+
+@pytest.mark.parametrize("N,g", [(1000, 2), (30000, 2), (700, 4)])        # short, long; the last one has C = 128 and no lists
+def test_queries_in_reverse_order(N, g):
+    """A negative token stride: no tensor map holds it, the kernels that gather rows by pointer take it."""
+    C = 128 if g == 4 else 64
+    w = S.Workload("strided_rev", 1, N, 4, 2, 64, C, g, 4, "bf16", 903, "iid")
+    dev = T.Device(w, S.make_inputs(w))
+    dev.build_pyramid()
+    dev.route(with_margin=False)
+    assert dev.sync_status() == 0
+    q = dev.q.flip(1).contiguous()
+    st = (N * w.Hq * w.d, -w.Hq * w.d, w.d)
+    p = P.Params(1, N, w.Hq, w.Hkv, w.d, C, g, w.K, dtype="bf16").set_strides(q=st)
+    idx, ws = torch.full_like(dev.idx, -7), PB.alloc_workspace(p, PB.OP_ROUTE)
+    P.pisa_route(p, q[:, N - 1:], dev.k, dev.pyramid, idx, None, ws)
+    torch.cuda.synchronize()
+    assert P.read_status(ws) == 0
+    assert float((idx != dev.idx).any(-1).float().mean()) <= 1e-3            # (ties)
+    if g == 4:
+        return
+    dev.bsa()
+    dout = torch.randn(dev.out.shape, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda").bfloat16()
+    got = []
+    for pp, qq in ((dev.p, dev.q), (p, q[:, N - 1:])):
+        g_ = [torch.zeros_like(x) for x in (dev.q, dev.k, dev.v)]
+        wsb = PB.alloc_workspace(pp, PB.OP_BSA_BWD)
+        P.pisa_bsa_bwd(pp, qq, dev.k, dev.v, dev.idx, dev.out, dev.lse, dout, *g_, wsb)
+        torch.cuda.synchronize()
+        assert P.read_status(wsb) == 0
+        got.append(g_)
+    for a, b in zip(*got):
+        assert torch.allclose(a.float(), b.float(), rtol=0, atol=2.0 ** -6 * float(b.float().abs().max()))
