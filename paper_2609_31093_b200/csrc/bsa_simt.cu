@@ -166,11 +166,11 @@ bsa_simt_kernel(Geometry geo, const T* __restrict__ q, const T* __restrict__ k, 
       for (int p = 0; p < WPT; ++p) mx = fmaxf(mx, s_ml[tok][p][2 * hh]);
 #pragma unroll
       for (int p = 0; p < WPT; ++p) {
-        const float lp = s_ml[tok][p][2 * hh + 1], f = lp > 0.f ? expf(s_ml[tok][p][2 * hh] - mx) : 0.f;   // (a warp without keys: m = -inf)
+        const float lp = s_ml[tok][p][2 * hh + 1], f = lp != 0.f ? expf(s_ml[tok][p][2 * hh] - mx) : 0.f;   // (a warp without keys: m = -inf; a NaN stays)
         sum = fmaf(lp, f, sum);
         o = fmaf(s_acc[tok][p][x], f, o);
       }
-      out[(long long)b * geo.os[0] + (long long)t * geo.os[1] + (long long)hq * geo.os[2] + x - hh * D] = Elem<T>::from_float(sum > 0.f ? o / sum : 0.f);
+      out[(long long)b * geo.os[0] + (long long)t * geo.os[1] + (long long)hq * geo.os[2] + x - hh * D] = Elem<T>::from_float(sum != 0.f ? o / sum : 0.f);
       if (x == hh * D) lse[((long long)b * geo.Hq + hq) * geo.N + t] = sum > 0.f ? mx + logf(sum) : -CUDART_INF_F;
     }
     return;

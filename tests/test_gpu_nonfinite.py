@@ -116,3 +116,29 @@ def _selection(dtype, impl, N, C, g, K, G):
         for pos in rows:
             want, gap = _walk(dev.q[0, pos, h * G:(h + 1) * G], dev.k[0, :, h], lambda l: dev.level(l)[0, h], dev.M, dev.L, C, g, K, pos)
             _check_row(dev.idx[0, h, pos], want, gap, K, pos // C, (pos, h))
+
+
+def _see(idx, N, C, key):
+    """Rows [B, Hkv, N] that selected the key's leaf and come no earlier than the key."""
+    t = torch.arange(N, device="cuda")
+    return (idx == key // C).any(-1) & (t >= key)
+
+
+@pytest.mark.parametrize("N,G", [(300, 1), (700, 2), (1500, 1), (3000, 1), (700, 4)])      # eight, four and one warp per token
+@pytest.mark.parametrize("what", ["k", "v"])
+def test_fp32_rows_show_what_they_attend_to(N, G, what):
+    """A NaN key or value reaches every row that selected and may see it, and no other one."""
+    C, K = 64, 4
+    w = S.Workload("nf_simt", 1, N, G, 1, 64, C, 2, K, "fp32", 2300 + N, "iid")
+    dev = T.Device(w, S.make_inputs(w))
+    dev.forward()
+    assert dev.sync_status() == 0
+    clean, idx = dev.out.clone(), dev.idx.clone()
+    for keys in ([70], list(range(64, 128)), list(range(N - 20, N))):          # one key; a whole leaf; the last ones
+        getattr(dev, what)[0, keys] = NAN
+        dev.bsa(idx)
+        assert dev.sync_status() == 0
+        see = torch.stack([_see(idx, N, C, k)[0, 0] for k in keys]).any(0)
+        assert bool(torch.isnan(dev.out[0, see]).all()), keys
+        assert torch.equal(dev.out[0, ~see], clean[0, ~see]), keys
+        dev = T.Device(w, S.make_inputs(w))
