@@ -489,7 +489,10 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
   for (int hh = 0; hh < NG; ++hh)
 #pragma unroll
     for (int j = 0; j < DV; ++j) o_acc[hh][j] = 0.f;
-  float m_run[2] = {-CUDART_INF_F, -CUDART_INF_F}, l_run[2] = {0.f, 0.f};   // heads gid, gid + 8 (base 2)
+  // heads gid, gid + 8 (base 2).  The maxima start at a finite value: parts without keys (sum 0) or with nothing but logits of
+  // -inf then merge with weight 0 and parts that hold a NaN with NaN, none of them a case of its own.
+  constexpr float kFloor = -3.0e38f;
+  float m_run[2] = {kFloor, kFloor}, l_run[2] = {0.f, 0.f};
   const float sl2 = geo.scale * kLog2e;
   const int ppb = C / KT;                                  // pieces per block
   for (int u = gw; u < nsel * ppb; u += CLU * kDecWarps) {
@@ -532,7 +535,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
       for (int x = 0; x < KT / 8; ++x) tm = fmaxf(tm, fmaxf(z[x][2 * y], z[x][2 * y + 1]));
       tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, 1));
       tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, 2));
-      const float mn = fmaxf(m_run[y], tm);                // finite: the piece's first key is visible
+      const float mn = fmaxf(m_run[y], tm);
       const float alpha = ex2_approx(m_run[y] - mn);
       float ps = 0.f;
 #pragma unroll
@@ -590,13 +593,13 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
   for (int e = tid; e < NG * D + NG; e += kDecThreads) {
     const bool is_o = e < NG * D;
     const int hh = is_o ? e / D : e - NG * D;
-    float mw[kDecWarps], M = -CUDART_INF_F;
+    float mw[kDecWarps], M = kFloor;
 #pragma unroll
     for (int w = 0; w < kDecWarps; ++w) { mw[w] = s_dyn[w * W + NG * D + hh]; M = fmaxf(M, mw[w]); }
     float acc = 0.f;
 #pragma unroll
     for (int w = 0; w < kDecWarps; ++w)
-      if (mw[w] > -CUDART_INF_F) acc += s_dyn[w * W + (is_o ? e : NG * D + NG + hh)] * ex2_approx(mw[w] - M);
+      acc += s_dyn[w * W + (is_o ? e : NG * D + NG + hh)] * ex2_approx(mw[w] - M);
     if (is_o) cta[e] = acc;
     else { cta[NG * D + hh] = M; cta[NG * D + NG + hh] = acc; }
   }
@@ -608,7 +611,7 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
     const int e = rank * SLICE + x;
     if (e >= NG * D) break;
     const int hh = e / D;
-    float mr[CLU], lr[CLU], orr[CLU], M = -CUDART_INF_F;
+    float mr[CLU], lr[CLU], orr[CLU], M = kFloor;
 #pragma unroll
     for (int r = 0; r < CLU; ++r) {
       const uint32_t p = remote_smem(cta, r);
@@ -621,11 +624,11 @@ decode_step_kernel(const __grid_constant__ Geometry geo, const __grid_constant__
     float acc = 0.f, den = 0.f;
 #pragma unroll
     for (int r = 0; r < CLU; ++r)
-      if (mr[r] > -CUDART_INF_F) {
-        const float f = ex2_approx(mr[r] - M);
-        acc += orr[r] * f;
-        den += lr[r] * f;
-      }
+    {
+      const float f = ex2_approx(mr[r] - M);
+      acc += orr[r] * f;
+      den += lr[r] * f;
+    }
     a.out[((long long)b * geo.Hq + (long long)h * NG + hh) * D + (e - hh * D)] = __float2bfloat16_rn(acc / den);
     if (e - hh * D == 0) a.lse[(long long)b * geo.Hq + (long long)h * NG + hh] = (M + log2f(den)) * kLn2;
   }

@@ -142,3 +142,49 @@ def test_fp32_rows_show_what_they_attend_to(N, G, what):
         assert bool(torch.isnan(dev.out[0, see]).all()), keys
         assert torch.equal(dev.out[0, ~see], clean[0, ~see]), keys
         dev = T.Device(w, S.make_inputs(w))
+
+
+@pytest.mark.parametrize("B,G,C", [(1, 4, 64), (1, 16, 128), (40, 1, 32), (3, 8, 64)])
+def test_decoding_shows_what_it_attends_to(B, G, C):
+    """A NaN key or value of a selected block reaches the output, also where all keys of a warp's share are NaN; keys with
+    logits of -inf weigh nothing."""
+    N, K, Hkv, d, pos = 16 * C, 16, 2, 64, 16 * C - 5
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    q, k, v = (torch.randn(s, generator=gen, device="cuda").bfloat16() for s in ((B, G * Hkv, d), (B, N, Hkv, d), (B, N, Hkv, d)))
+    p = P.Params(B, N, G * Hkv, Hkv, d, C, 2, K, dtype="bf16")
+    pyr, ws = PB.alloc_pyramid(p), PB.alloc_workspace(p, PB.OP_DECODE)
+    P.pisa_build_pyramid(p, k, pyr)
+
+    def step(kk, vv):
+        idx = torch.full((B, Hkv, K), -7, dtype=torch.int32, device="cuda")
+        out, lse = torch.zeros_like(q), torch.zeros((B, G * Hkv), device="cuda")
+        P.pisa_decode_step(p, pos, q, kk, vv, pyr.clone(), idx, out, lse, ws)
+        torch.cuda.synchronize()
+        assert P.read_status(ws) == 0 and bool((idx == torch.arange(K, device="cuda", dtype=torch.int32)).all())
+        return out, lse
+
+    clean = step(k, v)
+    for keys in (slice(7, 8), slice(3 * C, 4 * C), slice(0, N), slice(pos, pos + 1)):
+        kk, vv = k.clone(), v.clone()
+        kk[:, keys, 0] = NAN
+        vv[:, keys, 1, 3] = NAN
+        out, lse = step(kk, v)
+        assert bool(torch.isnan(out[:, :G]).all()) and bool(torch.isnan(lse[:, :G]).all()), keys
+        assert torch.equal(out[:, G:], clean[0][:, G:]) and torch.equal(lse[:, G:], clean[1][:, G:])
+        out, lse = step(k, vv)
+        assert bool(torch.isnan(out[:, G:, 3]).all()) and torch.equal(lse, clean[1])
+        out[:, G:, 3] = clean[0][:, G:, 3]
+        assert torch.equal(out, clean[0])
+    if G == 1:
+        kk = k.clone()
+        gone = torch.zeros(N, dtype=torch.bool, device="cuda")
+        gone[3 * C:5 * C] = True
+        gone[:9] = True
+        for h in range(Hkv):
+            kk[:, gone, h] = torch.where(q[:, None, h] > 0, -math.inf, math.inf).bfloat16().expand(-1, int(gone.sum()), -1)
+        out, lse = step(kk, v)
+        z = torch.einsum("bhd,bnhd->bhn", q.float(), k.float()) * d ** -0.5
+        z[:, :, gone] = -math.inf
+        z[:, :, pos + 1:] = -math.inf
+        want = torch.einsum("bhn,bnhd->bhd", torch.softmax(z, 2), v.float())
+        assert float((out.float() - want).abs().max()) <= T.BF16_MAX_ABS and torch.allclose(lse, torch.logsumexp(z, 2), atol=1e-3)
