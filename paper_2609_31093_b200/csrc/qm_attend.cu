@@ -15,7 +15,8 @@
 // and step with NT = 1 and NT = 2 alike (each product waited for the other's queue).  An issuer per tile: 707 us against 653
 // (4 x 4 KV heads, G = 4), 583 against 485 (C = 128) -- the pipe loses more by changing chains than one issuer's loop does,
 // which is busy 1570 of 1855 cycles per tile and step, the chains' 1024 among them.
-// Every wait is bounded.
+// Every wait is bounded.  What is not finite reaches only the rows that selected it (attend_row; finite inputs pay a test of
+// the sums as they are read out).
 #include "launch.cuh"
 #include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
@@ -37,8 +38,55 @@ template <bool V> struct Bool { static constexpr bool value = V; };
 
 struct AttArgs {
   const float* row_lse;      // [Hq, len] per sequence, natural log
+  const __nv_bfloat16 *q, *k, *v;   // for attend_row()
   __nv_bfloat16* out;        // strides of the geometry's `out`
 };
+
+// One row over its own leaves only, by one warp.  The tiles multiply every value of a step with every row, zero weights
+// included, so that a value (or a score) that is not finite reaches rows that did not select it or must not see it; rows that
+// came out not finite are computed again here, where only what they selected takes part.
+template <int D>
+__device__ __forceinline__ void attend_row(const __nv_bfloat16* q, const __nv_bfloat16* k, long long ks, const __nv_bfloat16* v, long long vs,
+                                           const uint32_t* bits, int t, int lgC, float sl2, float neg_lse2, bool round_p,
+                                           __nv_bfloat16* out) {
+  const int lane = threadIdx.x & 31;
+  float acc[D / 32];
+  bool gone = false;                             // every column is NaN, whatever follows
+#pragma unroll
+  for (int y = 0; y < D / 32; ++y) acc[y] = 0.f;
+  for (int leaf = 0; leaf <= (t >> lgC) && !gone; ++leaf) {
+    if (!((bits[leaf >> 5] >> (leaf & 31)) & 1u)) continue;
+    const int end = min((leaf + 1) << lgC, t + 1);
+    for (int j0 = leaf << lgC; j0 < end && !gone; j0 += 32) {
+      const int j = j0 + lane;
+      float p = 0.f;
+      if (j < end) {
+        float s = 0.f;
+#pragma unroll 4
+        for (int c = 0; c < D; c += 8) {
+          float x[8], y[8];
+          Elem<__nv_bfloat16>::load_chunk(q + c, x);
+          Elem<__nv_bfloat16>::load_chunk(k + j * ks + c, y);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) s = fmaf(x[e], y[e], s);
+        }
+        p = ex2_approx(fmaf(s, sl2, neg_lse2));
+        if (round_p) p = __bfloat162float(__float2bfloat16_rn(p));
+      }
+      for (int x = 0; x < min(32, end - j0); ++x) {
+        const float px = __shfl_sync(0xffffffffu, p, x);
+#pragma unroll
+        for (int y = 0; y < D / 32; ++y) acc[y] = fmaf(px, __bfloat162float(v[(long long)(j0 + x) * vs + lane + 32 * y]), acc[y]);
+      }
+      bool nan = true;
+#pragma unroll
+      for (int y = 0; y < D / 32; ++y) nan = nan && acc[y] != acc[y];
+      gone = __all_sync(0xffffffffu, nan);
+    }
+  }
+#pragma unroll
+  for (int y = 0; y < D / 32; ++y) out[lane + 32 * y] = __float2bfloat16_rn(acc[y]);
+}
 
 // K / V tiles in flight (one ring: K, V, K, V, ...): what two items' query tiles leave of 227 KB
 __host__ __device__ constexpr int att_stages(int D, int NT) { return D == 128 ? (NT == 1 ? 5 : 3) : 8; }
@@ -60,6 +108,10 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
   __shared__ int4 s_item[kRing];             // (work item or -1, steps, steps of the first tile, of the second)
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
+  __shared__ volatile int s_again;           // some row came out not finite
+  // this CTA's items: the last one + 1; the one before it stands in the score table (word `item`: nothing reads the scores any
+  // more, and there are four of them at least for every item)
+  __shared__ volatile int s_items;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -71,6 +123,8 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
     }
     for (int i = 0; i < NKV; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], 1); }
     s_fail = 0;
+    s_again = 0;
+    s_items = 0;
     mbar_fence_init();
   }
   if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
@@ -133,7 +187,13 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           n = min(n + __popc(bal), kMaxSteps);
         }
       }
-      if (lane == 0) s_item[r] = make_int4(item < a.n_items && ok ? item : -1, n, n0, n1);
+      if (lane == 0) {
+        s_item[r] = make_int4(item < a.n_items && ok ? item : -1, n, n0, n1);
+        if (item < a.n_items) {
+          reinterpret_cast<int*>(a.leaf)[item] = s_items;
+          s_items = item + 1;
+        }
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&l_full[r]);
       if (item >= a.n_items || !ok) break;
@@ -406,6 +466,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
       __nv_bfloat16* dst = at.out + (long long)tl.q.batch * geo.os[0] + (long long)(tl.q.tok + t) * geo.os[1] +
                            (long long)(tl.h * G + head) * geo.os[2] + col0;
       constexpr int LC = HC < 32 ? HC : 32;
+      uint64_t finite[2] = {0ull, 0ull};                                     // NaN once a value is infinite or NaN
 #pragma unroll
       for (int c0 = 0; c0 < HC; c0 += LC) {
         uint32_t rr[LC];
@@ -417,6 +478,9 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           __syncwarp();
           if (lane == 0) mbar_arrive(&o_empty[ob]);
         }
+#pragma unroll
+        for (int x = 0; x < LC / 2; ++x)
+          finite[x & 1] = fma2(pack2(__uint_as_float(rr[2 * x]), __uint_as_float(rr[2 * x + 1])), 0ull, finite[x & 1]);
         if (live)
 #pragma unroll
           for (int q4 = 0; q4 < LC / 8; ++q4) {
@@ -430,12 +494,34 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
             *reinterpret_cast<uint4*>(dst + c0 + 8 * q4) = o;
           }
       }
+      float f0, f1;
+      unpack2(add2(finite[0], finite[1]), f0, f1);
+      if (live && f0 + f1 != 0.f) s_again = 1;
     }
   }
   tcgen05_fence_before_sync();
   __syncthreads();
   if (s_fail && tid == 0) atomicExch(a.status, (int)PISA_ERR_TIMEOUT);
   if (warp == 0) tmem_dealloc(tmem, 512);
+  if (!s_again || s_fail) return;
+  for (int item = s_items - 1; item >= 0; item = reinterpret_cast<const int*>(a.leaf)[item] - 1) {
+    const qm::Tile tl = qm::locate(geo, a, item, NT);
+    const int len = tl.q.len, W = (((len + C - 1) >> lgC) + 31) >> 5;
+    const long long b = tl.q.batch, tok = tl.q.tok;
+    for (int row = warp; row < 128 * NT; row += kAttThreads / 32) {
+      const int t = tl.tile * NT * tpt + (row >> lgG), hq = tl.h * G + (row & (G - 1));
+      if (t >= len) break;
+      __nv_bfloat16* out = at.out + b * geo.os[0] + (tok + t) * geo.os[1] + hq * geo.os[2];
+      float finite = 0.f;
+#pragma unroll
+      for (int y = 0; y < D / 32; ++y) finite = fmaf(__bfloat162float(out[lane + 32 * y]), 0.f, finite);
+      if (!__any_sync(0xffffffffu, finite != finite)) continue;
+      attend_row<D>(at.q + b * geo.qs[0] + (tok + t) * geo.qs[1] + hq * geo.qs[2], at.k + b * geo.ks[0] + tok * geo.ks[1] + tl.h * geo.ks[2],
+                    geo.ks[1], at.v + b * geo.vs[0] + tok * geo.vs[1] + tl.h * geo.vs[2], geo.vs[1],
+                    a.bits + tl.q.bits_off + ((long long)tl.h * len + t) * W, t, lgC, geo.scale * kLog2e,
+                    -at.row_lse[(long long)geo.Hq * tl.q.cu + (long long)hq * len + t] * kLog2e, !(LO && len <= C), out);
+    }
+  }
 }
 
 template <int D, int C, int NT, bool LO>
@@ -465,6 +551,7 @@ int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const 
   }
   AttArgs at;
   at.row_lse = row_lse; at.out = (__nv_bfloat16*)out;
+  at.q = (const __nv_bfloat16*)q; at.k = (const __nv_bfloat16*)k; at.v = (const __nv_bfloat16*)v;
   if (g.d == 128) return g.C == 128 ? launch_dc<128, 128>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s) : launch_dc<128, 64>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s);
   return g.C == 128 ? launch_dc<64, 128>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s) : launch_dc<64, 64>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s);
 }

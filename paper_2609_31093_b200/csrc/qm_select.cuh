@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kSelThreads) qm_select_kernel(Geometry geo, qm
         float mn = m[hh];
 #pragma unroll
         for (int u = 0; u < U; ++u) mn = fmaxf(mn, x[u][hh]);
-        float sum = ssum[hh] > 0.f ? ssum[hh] * __expf(m[hh] - mn) : 0.f;
+        float sum = ssum[hh] != 0.f ? ssum[hh] * __expf(m[hh] - mn) : 0.f;     // (0: nothing yet, m = -inf)
 #pragma unroll
         for (int u = 0; u < U; ++u) sum += s0 + u < nk ? __expf(x[u][hh] - mn) : 0.f;
         m[hh] = mn;

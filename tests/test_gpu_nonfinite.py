@@ -188,3 +188,59 @@ def test_decoding_shows_what_it_attends_to(B, G, C):
         z[:, :, pos + 1:] = -math.inf
         want = torch.einsum("bhn,bnhd->bhd", torch.softmax(z, 2), v.float())
         assert float((out.float() - want).abs().max()) <= T.BF16_MAX_ABS and torch.allclose(lse, torch.logsumexp(z, 2), atol=1e-3)
+
+
+def _poison(x, what, N, C):
+    """x [B, N, H, d]"""
+    H = x.shape[2]
+    if what == "future":                          # everything from the middle of a leaf on
+        x[:, N // 2 + 9:] = NAN
+    elif what == "future_inf":                    # ... from a leaf's start on
+        x[:, N // 2 // C * C:] = math.inf
+    elif what == "key":                           # one key in the past of most rows, one column
+        x[:, N // 3, 0, 5] = NAN
+        x[:, N // 3 + C, H - 1, 7] = -math.inf
+    else:                                         # a whole leaf, and the first leaf of the last batch element
+        x[:, N // 3 // C * C:N // 3 // C * C + C] = NAN
+        x[-1, :C, 0] = math.inf
+
+
+def _same(got, want, what):
+    """NaN (or infinite) where the reference is, equal to bf16 rounding elsewhere."""
+    bad = ~torch.isfinite(want)
+    assert torch.equal(~torch.isfinite(got), bad), (what, int((~torch.isfinite(got) & ~bad).sum()), int((torch.isfinite(got) & bad).sum()))
+    g, w = got[~bad].double(), want[~bad].double()
+    assert bool(((g - w).abs() <= 2.0 ** -6 * w.abs() + T.BF16_MAX_ABS).all()), what
+
+
+FORWARD = [(2, 1500, 8, 2, 128, 64, 2, 4), (1, 700, 2, 2, 64, 64, 4, 4), (1, 900, 16, 1, 128, 128, 2, 3), (4, 2200, 32, 8, 64, 64, 2, 5),
+           (1, 600, 4, 1, 64, 128, 4, 3)]
+
+
+@pytest.mark.parametrize("shape", FORWARD, ids=lambda s: "b%d_n%d_h%d_%d_d%d_c%d_g%d_k%d" % s)
+@pytest.mark.parametrize("tensor", ["k", "v", "q"])
+@pytest.mark.parametrize("what", ["future", "future_inf", "key", "leaf"])
+def test_dense_forward_shows_what_its_rows_selected(shape, tensor, what):
+    """The dense tiles against the exact path (a warp per token, selected and visible keys only) on the same blocks."""
+    B, N, Hq, Hkv, d, C, g, K = shape
+    w = S.Workload("nf_fwd", B, N, Hq, Hkv, d, C, g, K, "bf16", 2400 + N, "iid")
+    dev = T.Device(w, S.make_inputs(w))
+    _poison(getattr(dev, tensor), what, N, C)
+    dev.forward()
+    assert dev.sync_status() == 0
+    ref = T.Device(w, S.make_inputs(w), impl=PB.IMPL_SIMT)
+    ref.q, ref.k, ref.v = dev.q, dev.k, dev.v
+    ref.bsa(dev.idx)
+    assert ref.sync_status() == 0
+    _same(dev.out, ref.out, (tensor, what))
+    ok = torch.isfinite(ref.lse)                  # (a NaN denominator reads -inf there)
+    assert torch.allclose(dev.lse[ok], ref.lse[ok], rtol=1e-4, atol=1e-3)
+    # a row whose past (up to its own token) is finite is what it was, and so are its blocks
+    dev2 = T.Device(w, S.make_inputs(w))
+    dev2.forward()
+    torch.cuda.synchronize()
+    first = N // 2 // C * C if what.startswith("future") else N // 3 // C * C
+    if what != "leaf":
+        assert torch.equal(dev.idx[:, :, :first], dev2.idx[:, :, :first])
+        assert torch.equal(dev.lse[:, :, :first], dev2.lse[:, :, :first])
+        _same(dev.out[:, :first], dev2.out[:, :first], (tensor, what))
