@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) qm_bwd_prep_kernel(Geometry geo, Args a) 
     for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (sub == 0 && t < len) {
       const float l = a.lse[(long long)geo.Hq * loc.q.cu + (long long)(h * G + hd) * len + t];
-      a.stat[loc.q.leaf_off + ((long long)h * len + t) * G + hd] = make_float2(l > -CUDART_INF_F ? -l * kLog2e : -CUDART_INF_F, -s);
+      a.stat[loc.q.leaf_off + ((long long)h * len + t) * G + hd] = make_float2(l == -CUDART_INF_F ? l : l < CUDART_INF_F ? -l * kLog2e : CUDART_NAN_F, -s);
     }
   }
   __syncthreads();
@@ -63,6 +63,12 @@ __global__ void __launch_bounds__(256) qm_bwd_prep_kernel(Geometry geo, Args a) 
     if (s_bits[i] != 0u) atomicOr(&s_bits[tpt * W + i % W], s_bits[i]);
   }
   __syncthreads();
+  for (int k = threadIdx.x; k < nt; k += blockDim.x) {      // a row without blocks counts for nothing, whatever it holds
+    uint32_t any = 0u;
+    for (int w = 0; w < W; ++w) any |= s_bits[k * W + w];
+    for (int hd = 0; hd < G && any == 0u; ++hd)
+      a.stat[loc.q.leaf_off + ((long long)h * len + t0 + k) * G + hd] = make_float2(-CUDART_INF_F, 0.f);
+  }
   uint32_t* tb = a.tbits + loc.q.up_off + (long long)h * tiles * W + loc.part;
   int steps = 0;                                            // 128-key blocks the tile needs
   for (int w = threadIdx.x; w < W; w += blockDim.x) {
@@ -85,6 +91,14 @@ template <bool V> struct Bool { static constexpr bool value = V; };
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&p);
+}
+__device__ __forceinline__ bool all_finite(const uint32_t (&r)[32]) {
+  uint64_t s[2] = {0ull, 0ull};                             // NaN once a value is infinite or NaN
+#pragma unroll
+  for (int x = 0; x < 16; ++x) s[x & 1] = fma2(pack2(__uint_as_float(r[2 * x]), __uint_as_float(r[2 * x + 1])), 0ull, s[x & 1]);
+  float a, b;
+  unpack2(add2(s[0], s[1]), a, b);
+  return a + b == 0.f;
 }
 // N floats of a row -> bf16, 16 bytes at a time
 template <int N>
@@ -247,19 +261,31 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
         }
       }
       if (step >= NS) wait(&st_empty[s], (uint32_t)((step / NS - 1) & 1));
+      // Rows that must not be multiplied as they are: those that count for nothing (past the sequence's end, where a packed
+      // neighbour's lie, or without blocks), and those that hold something not finite (their denominator is NaN or their
+      // delta not finite), unless only their dO does and they selected and see all of the step's keys
+      uint32_t off[4];
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
         const int r = lane + 32 * x;
+        constexpr uint32_t all = (1u << LPS) - 1u;
+        const bool none = st[x].x == -CUDART_INF_F, nan = st[x].x != st[x].x;
+        const bool whole = (wd[x] & all) == all && t0 + (r >> lgG) >= loc.part * 128 + 127;
+        const bool bad = none || nan || (!whole && !(fabsf(st[x].y) < CUDART_INF_F));
+        off[x] = __ballot_sync(0xffffffffu, bad);
 #pragma unroll
-        for (int lf = 0; lf < LPS; ++lf) s_bias[s][lf][r] = ((wd[x] >> lf) & 1u) ? st[x].x : -CUDART_INF_F;
-        s_delta[s][r] = st[x].y * geo.scale;
+        for (int lf = 0; lf < LPS; ++lf) s_bias[s][lf][r] = ((wd[x] >> lf) & 1u) ? (bad && !none ? CUDART_NAN_F : st[x].x) : -CUDART_INF_F;
+        s_delta[s][r] = bad ? 0.f : st[x].y * geo.scale;
       }
-      if (a.seqs != nullptr && (len - t0) * G < 128) {
-        // packed: the rows past the sequence's end belong to its neighbour; their weight is zero, but a value that is not
-        // finite would still reach the sums
+      if ((off[0] | off[1] | off[2] | off[3]) != 0u) {
         wait(&st_full[s], (uint32_t)((step / NS) & 1));
-        zero_rows(sQ + 2 * s * TILE, SLAB, KS, (len - t0) * G, 128);
-        zero_rows(sQ + (2 * s + 1) * TILE, SLAB, KS, (len - t0) * G, 128);
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          for (uint32_t m = off[x]; m != 0u; m &= m - 1u) {
+            const int r = 32 * x + __ffs(m) - 1;
+            if (lane < 16 * KS)                             // eight chunks of 16 bytes per 64 columns, Q and dO
+              st_shared_zero16(smem_u32(sQ + (2 * s + lane / (8 * KS)) * TILE + ((lane >> 3) % KS) * SLAB) + swz128(r, lane & 7));
+          }
         fence_proxy_async_smem();
       }
       __syncwarp();
@@ -325,7 +351,7 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
       const int s = step % NS;
       if (e.z & kFirst) wait(&kv_full, (uint32_t)(items & 1));
       wait(&st_full[s], (uint32_t)((step / NS) & 1));
-      if (a.seqs != nullptr) wait(&meta_full[s], (uint32_t)((step / NS) & 1));      // (rows past the sequence's end are zero)
+      wait(&meta_full[s], (uint32_t)((step / NS) & 1));       // (rows that count for nothing are zero)
       scores(0u, s);
       if (prev >= 0) owed();
       scores(1u, s);
@@ -360,7 +386,7 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
         // rows of this warp's columns whose token is not before the warp's last key need the causal comparison
         const int tok0 = e.y * tpt + (col0 >> lgG);
         const bool diag = tok0 < loc.part * 128 + quarter * 32 + 31;
-        const bool any = __any_sync(0xffffffffu, bias[lane] > -CUDART_INF_F) &&
+        const bool any = __any_sync(0xffffffffu, bias[lane] != -CUDART_INF_F) &&
                          (e.y * tpt + ((col0 + 31) >> lgG) >= loc.part * 128 + quarter * 32);
         wait(&s_full[grp], (uint32_t)(step & 1));
         tcgen05_fence_after_sync();
@@ -404,6 +430,14 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
       const bool live = key < loc.q.len;
       const long long orow = ((loc.q.cu + key) * geo.Hkv + loc.h) * D + c0;
       const bool direct = (loc.part == 0 ? a.splits0 : a.splits) == 1;
+      // does a row of this item select the key?  (asked only for sums that are not finite)
+      auto selected = [&]() -> bool {
+        const int len = loc.q.len, W = (((len + C - 1) >> lgC) + 31) >> 5, leaf = key >> lgC, sp = loc.part == 0 ? a.splits0 : a.splits;
+        for (int tile = (loc.part * 128) / tpt + loc.split; tile * tpt < len; tile += sp)
+          for (int t = max(key, tile * tpt); t < min(len, (tile + 1) * tpt); ++t)
+            if ((a.bits[loc.q.bits_off + ((long long)loc.h * len + t) * W + (leaf >> 5)] >> (leaf & 31)) & 1u) return true;
+        return false;
+      };
       if (e.z & kEmpty) {
         if (direct && live) {
           __nv_bfloat16* dst = (which ? a.dk : a.dv) + orow;
@@ -425,6 +459,10 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
           if (lane == 0) mbar_arrive(&acc_empty);
         }
         if (!live) continue;
+        if (!all_finite(r) && !selected()) {
+#pragma unroll
+          for (int y = 0; y < 32; ++y) r[y] = 0u;
+        }
         if (direct) {
           store_row<32>((which ? a.dk : a.dv) + orow + x, r);
         } else {
@@ -448,6 +486,54 @@ qm_bwd_kv_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q,
 
 // ------------------------------------------------------------------ dQ
 
+// One row of dQ over its own leaves only, by one warp (as attend_row in qm_attend.cu)
+template <int D>
+__device__ __forceinline__ void dq_row(const __nv_bfloat16* q, const __nv_bfloat16* dout, const __nv_bfloat16* k, long long ks,
+                                       const __nv_bfloat16* v, long long vs, const uint32_t* bits, int t, int lgC, float scale, float2 st,
+                                       __nv_bfloat16* dq) {
+  const int lane = threadIdx.x & 31;
+  float acc[D / 32];
+  bool gone = false;                                        // every column is NaN, whatever follows
+#pragma unroll
+  for (int y = 0; y < D / 32; ++y) acc[y] = 0.f;
+  for (int leaf = 0; leaf <= (t >> lgC) && !gone; ++leaf) {
+    if (!((bits[leaf >> 5] >> (leaf & 31)) & 1u)) continue;
+    const int end = min((leaf + 1) << lgC, t + 1);
+    for (int j0 = leaf << lgC; j0 < end && !gone; j0 += 32) {
+      const int j = j0 + lane;
+      float ds = 0.f;
+      if (j < end) {
+        float s = 0.f, dp = 0.f;
+#pragma unroll 2
+        for (int c = 0; c < D; c += 8) {
+          float x[8], y[8];
+          Elem<__nv_bfloat16>::load_chunk(q + c, x);
+          Elem<__nv_bfloat16>::load_chunk(k + j * ks + c, y);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) s = fmaf(x[e], y[e], s);
+          Elem<__nv_bfloat16>::load_chunk(dout + c, x);
+          Elem<__nv_bfloat16>::load_chunk(v + j * vs + c, y);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) dp = fmaf(x[e], y[e], dp);
+        }
+        ds = ex2_approx(fmaf(s, scale * kLog2e, st.x)) * fmaf(dp, scale, st.y * scale);
+        ds = __bfloat162float(__float2bfloat16_rn(ds));
+      }
+      for (int x = 0; x < min(32, end - j0); ++x) {
+        const float dx = __shfl_sync(0xffffffffu, ds, x);
+#pragma unroll
+        for (int y = 0; y < D / 32; ++y) acc[y] = fmaf(dx, __bfloat162float(k[(long long)(j0 + x) * ks + lane + 32 * y]), acc[y]);
+      }
+      bool nan = true;
+#pragma unroll
+      for (int y = 0; y < D / 32; ++y) nan = nan && acc[y] != acc[y];
+      gone = __all_sync(0xffffffffu, nan);
+    }
+  }
+#pragma unroll
+  for (int y = 0; y < D / 32; ++y) dq[lane + 32 * y] = __float2bfloat16_rn(acc[y]);
+}
+
 // Two tiles share every load of 64 keys and values.  TMEM, per tile: S at column 0, dP at 64, dQ at 128 (the second tile's
 // at 256 and on).  The issuer walks the steps: for either tile the product its dS still owes, then the next S and dP.
 // Floor per tile and 64 keys: 1 K cycles of the tensor pipe; measured 1.9 K.
@@ -463,7 +549,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
   __shared__ StepRing ring;
   __shared__ uint64_t q_full, q_empty, kv_full[NS], kv_empty[NS], s_full[2], p_full[2], o_full[2], o_empty[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ volatile int s_fail;
+  __shared__ volatile int s_fail, s_again, s_items;          // s_again: a row came out not finite; s_items: this CTA's last item + 1
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   grid_dependency();
@@ -473,7 +559,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
     for (int i = 0; i < NS; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], 1); }
     mbar_init(&q_full, 1); mbar_init(&q_empty, 1);
     for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 8); mbar_init(&o_full[i], 1); mbar_init(&o_empty[i], 8); }
-    s_fail = 0;
+    s_fail = s_again = s_items = 0;
     mbar_fence_init();
   }
   if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
@@ -496,6 +582,7 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
       if (lane == 0) item = atomicAdd(a.ctr + 1, 1);
       item = __shfl_sync(0xffffffffu, item, 0);
       if (item >= a.n_pairs) { ring_push(ring, n, make_int4(0, 0, kEnd, 0), &s_fail); break; }
+      if (lane == 0) { a.chain[item] = s_items; s_items = item + 1; }
       const qmb::Loc loc = qmb::locate<qmb::kPairs>(geo, a, item);
       const int len = loc.q.len, W = (((len + C - 1) >> lgC) + 31) >> 5, tiles = (len + tpt - 1) / tpt, tile0 = loc.part * a.per;
       const uint32_t* tb = a.tbits + loc.q.up_off + ((long long)loc.h * W + lane) * tiles + tile0;
@@ -740,7 +827,10 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
           __syncwarp();
           if (lane == 0) mbar_arrive(&o_empty[x]);
         }
-        if (live) store_row<32>(dst + y, r);
+        if (live) {
+          if (!all_finite(r)) s_again = 1;
+          store_row<32>(dst + y, r);
+        }
       }
     }
   }
@@ -748,6 +838,25 @@ qm_bwd_q_kernel(Geometry geo, Args a, const __grid_constant__ CUtensorMap tm_q, 
   __syncthreads();
   if (s_fail && tid == 0) atomicExch(a.status, (int)PISA_ERR_TIMEOUT);
   if (warp == 0) tmem_dealloc(tmem, 512);
+  if (!s_again || s_fail) return;
+  for (int item = s_items - 1; item >= 0; item = a.chain[item] - 1) {
+    const qmb::Loc loc = qmb::locate<qmb::kPairs>(geo, a, item);
+    const int len = loc.q.len, W = (((len + C - 1) >> lgC) + 31) >> 5;
+    const long long b = loc.q.batch, tok = loc.q.tok;
+    for (int row = warp; row < 128 * a.per; row += kBwdThreads2 / 32) {
+      const int t = loc.part * a.per * tpt + (row >> lgG), head = row & (G - 1), hq = loc.h * G + head;
+      if (t >= len) break;
+      __nv_bfloat16* dq = a.dq + b * a.dq_s[0] + (tok + t) * a.dq_s[1] + hq * a.dq_s[2];
+      float finite = 0.f;
+#pragma unroll
+      for (int y = 0; y < D / 32; ++y) finite = fmaf(__bfloat162float(dq[lane + 32 * y]), 0.f, finite);
+      if (!__any_sync(0xffffffffu, finite != finite)) continue;
+      const long long r0 = (long long)loc.h * len + t;
+      dq_row<D>(a.q + b * geo.qs[0] + (tok + t) * geo.qs[1] + hq * geo.qs[2], a.dout + b * geo.os[0] + (tok + t) * geo.os[1] + hq * geo.os[2],
+                a.k + b * geo.ks[0] + tok * geo.ks[1] + loc.h * geo.ks[2], geo.ks[1], a.v + b * geo.vs[0] + tok * geo.vs[1] + loc.h * geo.vs[2],
+                geo.vs[1], a.bits + loc.q.bits_off + r0 * W, t, lgC, geo.scale, a.stat[loc.q.leaf_off + r0 * G + head], dq);
+    }
+  }
 }
 
 // split sums -> bf16, dk and dv in one launch (blockIdx.y); n4: vectors of four

@@ -9,6 +9,11 @@
 //   qm_bwd_q_kernel     one item per one or two tiles: S = Q K^T, dP = dO V^T -> dS over S in TMEM -> dQ += dS K in TMEM
 //
 // Seven products instead of the list kernel's five, but no gathers and no reductions into memory.
+//
+// A product over a tile multiplies every row with every key, zero weights included, so what is not finite has to be kept from
+// what did not select it.  Rows (their denominator or delta shows it): their queries and gradients count as zero in a step, and
+// the keys they did select get NaN through the row's bias.  Keys: sums that are not finite become zero where no row selected
+// the key, and rows of dQ that are not finite are computed again from their own leaves.
 #pragma once
 
 #include "pisa_common.cuh"
@@ -29,7 +34,9 @@ struct Args {
   int splits, splits0;
   uint32_t* bits;            // [Hkv][len][W] per sequence, W = ceil(M1 / 32)
   uint32_t* tbits;           // [Hkv][W][tiles] per sequence
-  float2* stat;              // [Hkv][len][G] per sequence: (-lse * log2 e, -inf for a row without keys; -delta)
+  float2* stat;              // [Hkv][len][G] per sequence: (-lse * log2 e, -inf for a row without keys, NaN; -delta)
+  int32_t* chain;            // [n_pairs] the q kernel's items, per CTA (each holds the one before it + 1)
+  const __nv_bfloat16 *q, *k, *v;   // strides of the geometry, for rows that are computed again
   const int32_t* idx;
   const float* lse;
   const __nv_bfloat16* out;

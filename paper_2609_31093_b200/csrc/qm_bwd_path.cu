@@ -13,15 +13,16 @@ namespace {
 
 int log2i(int x) { return 31 - __builtin_clz((unsigned)x); }
 
-// tokens of all sequences, leaf-bit words and 128-row tiles' words summed over them (per KV head)
-struct Sizes { size_t rows, words, twords; };
-struct Layout { size_t ctr, bits, tbits, stat, acc, total; };
+// tokens of all sequences, leaf-bit words, 128-row tiles' words and tiles summed over them (per KV head)
+struct Sizes { size_t rows, words, twords, tiles; };
+struct Layout { size_t ctr, chain, bits, tbits, stat, acc, total; };
 // acc: room for the split sums, of all keys (kAccAll) or of the first blocks of `acc` sequences
 enum { kAccAll = -1 };
 Layout layout(const Geometry& g, const Sizes& z, long long acc) {
   Layout l;
   size_t o = 0;
   l.ctr = o; o += 256;
+  l.chain = o; o += align_up(z.tiles * g.Hkv * 4, 256);
   l.bits = o; o += align_up(z.words * g.Hkv * 4, 256);
   l.tbits = o; o += align_up(z.twords * g.Hkv * 4, 256);
   l.stat = o; o += align_up(z.rows * g.Hq * 8, 256);
@@ -33,12 +34,12 @@ Layout layout(const Geometry& g, const Sizes& z, long long acc) {
 }
 Sizes seq_sizes(const Geometry& g, int len) {
   const int tpt = 128 / g.G;
-  const size_t W = ((len + g.C - 1) / g.C + 31) / 32;
-  return {(size_t)len, (size_t)len * W, (size_t)((len + tpt - 1) / tpt) * W};
+  const size_t W = ((len + g.C - 1) / g.C + 31) / 32, tiles = (size_t)((len + tpt - 1) / tpt);
+  return {(size_t)len, (size_t)len * W, tiles * W, tiles};
 }
 Sizes uniform_sizes(const Geometry& g) {
   const Sizes z = seq_sizes(g, g.N);
-  return {g.B * z.rows, g.B * z.words, g.B * z.twords};
+  return {g.B * z.rows, g.B * z.words, g.B * z.twords, g.B * z.tiles};
 }
 // splits, splits0 and the room for their sums
 struct Split { int all, first; long long acc; };
@@ -102,6 +103,7 @@ int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const
   a.n_pairs = units * ((g.N + a.per * tpt - 1) / (a.per * tpt));
   a.n_keys = units * (a.splits0 + ((g.N + 127) / 128 - 1) * a.splits);
   a.bits = (uint32_t*)(ws + l.bits); a.tbits = (uint32_t*)(ws + l.tbits); a.stat = (float2*)(ws + l.stat);
+  a.chain = (int32_t*)(ws + l.chain); a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
   a.idx = idx; a.lse = lse; a.out = (const __nv_bfloat16*)out; a.dout = (const __nv_bfloat16*)dout;
   a.dq = (__nv_bfloat16*)dq; a.dk = (__nv_bfloat16*)dk; a.dv = (__nv_bfloat16*)dv;
   a.dq_s[0] = (long long)g.N * g.Hq * g.d; a.dq_s[1] = (long long)g.Hq * g.d; a.dq_s[2] = g.d;
@@ -137,12 +139,12 @@ int qm_bwd_packed(const Geometry& g, const int32_t* cu, const int* ids, int n, l
   if (!seqs || !order || !by_len) return PISA_ERR_INVALID_ARG;
   const int tpt = 128 / g.G;
   for (int at = 0; at < n;) {
-    Sizes z = {0, 0, 0};
+    Sizes z = {0, 0, 0, 0};
     int end = at, longest = 0;
     long long tiles = 0, key_items = 0;
     while (end < n) {                                       // as many sequences as the workspace takes
       const int len = cu[ids[end] + 1] - cu[ids[end]];
-      const Sizes w = seq_sizes(g, len), sum = {z.rows + w.rows, z.words + w.words, z.twords + w.twords};
+      const Sizes w = seq_sizes(g, len), sum = {z.rows + w.rows, z.words + w.words, z.twords + w.twords, z.tiles + w.tiles};
       if (end > at && (table_bytes((size_t)(end - at + 1)) + layout(g, sum, end - at + 1).total > ws_bytes ||
                        sum.rows * g.Hq > (1ull << 30) || end - at >= 65535)) break;
       z = sum;
@@ -192,6 +194,7 @@ int qm_bwd_packed(const Geometry& g, const int32_t* cu, const int* ids, int n, l
     a.lgC = log2i(g.C); a.lgG = log2i(g.G);
     a.n_pairs = i0; a.n_tiles = it; a.n_keys = ik;
     a.bits = (uint32_t*)(ws + l.bits); a.tbits = (uint32_t*)(ws + l.tbits); a.stat = (float2*)(ws + l.stat);
+    a.chain = (int32_t*)(ws + l.chain); a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
     a.idx = idx; a.lse = lse; a.out = (const __nv_bfloat16*)out; a.dout = (const __nv_bfloat16*)dout;
     a.dq = (__nv_bfloat16*)dq; a.dk = (__nv_bfloat16*)dk; a.dv = (__nv_bfloat16*)dv;
     a.dq_s[0] = 0; a.dq_s[1] = (long long)g.Hq * g.d; a.dq_s[2] = g.d;

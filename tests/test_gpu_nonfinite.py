@@ -244,3 +244,111 @@ def test_dense_forward_shows_what_its_rows_selected(shape, tensor, what):
         assert torch.equal(dev.idx[:, :, :first], dev2.idx[:, :, :first])
         assert torch.equal(dev.lse[:, :, :first], dev2.lse[:, :, :first])
         _same(dev.out[:, :first], dev2.out[:, :first], (tensor, what))
+
+
+def _check_backward(dev, idx, dout, got, C):
+    """Which gradients must, may and must not be finite, and the finite ones against float64: the bound of check_gradient_rows
+    with a tenth of the root mean square in place of its terms for the rounding of `out` inside delta (a wrong or a missing row
+    is an error of the order of a whole gradient)."""
+    B, N, Hq, d = dev.q.shape
+    Hkv, G = dev.k.shape[2], Hq // dev.k.shape[2]
+    leaf, t = torch.arange(N, device="cuda") // C, torch.arange(N, device="cuda")
+    fin = lambda x: torch.isfinite(x).all(-1)  # noqa: E731
+    dq, dk, dv = got
+    ref = [torch.zeros(x.shape, dtype=torch.float64, device="cuda") for x in got]
+    bad = [torch.zeros(x.shape[:3], dtype=torch.bool, device="cuda") for x in got]
+    num = lambda x: torch.nan_to_num(x.double(), 0.0, 0.0, 0.0)  # noqa: E731
+    for b in range(B):
+        for h in range(Hkv):
+            rows = idx[b, h].long()
+            kept = torch.zeros((N, int(leaf[-1]) + 2), dtype=torch.bool, device="cuda").scatter_(1, torch.where(rows < 0, int(leaf[-1]) + 1, rows), True)
+            see = kept[:, leaf] & (t[None, :] <= t[:, None])
+            k, v = dev.k[b, :, h], dev.v[b, :, h]
+            may_v = torch.zeros(N, dtype=torch.bool, device="cuda")
+            for hq in range(h * G, h * G + G):
+                has = see.any(1)
+                bl = has & (~fin(dev.q[b, :, hq]) | (see & ~fin(k)[None]).any(1))
+                bo = has & ~fin(dout[b, :, hq])
+                ba = bl | bo | (has & (see & ~fin(v)[None]).any(1))
+                bad[0][b, :, hq] = ba
+                bad[1][b, :, h] |= (see & ba[:, None]).any(0)
+                bad[2][b, :, h] |= (see & (bl | bo)[:, None]).any(0)
+                may_v |= (see & ba[:, None]).any(0)
+                good = (has & ~ba)[:, None]
+                known = (has & ~bl & ~bo)[:, None]           # (a NaN value leaves the weights alone)
+                s = (num(dev.q[b, :, hq]) @ num(k).T * d ** -0.5).masked_fill(~see, -math.inf)
+                p = torch.where(known, torch.nan_to_num(torch.softmax(s, 1), 0.0), 0.0)
+                do, o = num(dout[b, :, hq]), p @ num(v)
+                ds = torch.where(good, p, 0.0) * (do @ num(v).T - (o * do).sum(1, keepdim=True)) * d ** -0.5
+                ref[0][b, :, hq] = ds @ num(k)
+                ref[1][b, :, h] += ds.T @ num(dev.q[b, :, hq])
+                ref[2][b, :, h] += p.T @ do
+            gone = ~fin(dv[b, :, h])
+            assert bool((bad[2][b, :, h] <= gone).all()) and bool((gone <= may_v).all()), ("dv", b, h)
+            bad[2][b, :, h] = gone
+    assert torch.equal(~torch.isfinite(dq), bad[0][..., None].expand_as(dq)), "dq"
+    assert torch.equal(~torch.isfinite(dk), bad[1][..., None].expand_as(dk)), "dk"
+    for nm, x, r, m in zip(("dq", "dk", "dv"), got, ref, bad):
+        x, r = torch.where(m[..., None], 0.0, x.double()), torch.where(m[..., None], 0.0, r)
+        rms = float(r.square().mean().sqrt())
+        err, bound = (x - r).abs(), 2.0 ** -5 * r.abs().amax(-1, keepdim=True) + 0.1 * rms
+        assert bool((err <= bound).all()), (nm, float((err - bound).max()), rms)
+
+
+# uniform batches: every group size and block size, one and two tiles per item, split and unsplit key blocks
+BACKWARD = [(1, 700, 8, 2, 128, 64, 2, 4), (2, 500, 4, 1, 64, 128, 2, 3), (1, 1100, 2, 2, 64, 64, 2, 5), (1, 450, 16, 1, 128, 64, 4, 3),
+            (3, 900, 32, 8, 64, 128, 2, 3)]
+
+
+@pytest.mark.parametrize("shape", BACKWARD, ids=lambda s: "b%d_n%d_h%d_%d_d%d_c%d_g%d_k%d" % s)
+@pytest.mark.parametrize("tensor", ["q", "k", "v", "dout"])
+@pytest.mark.parametrize("what", ["future", "key", "leaf"])
+def test_dense_backward_shows_what_its_rows_selected(shape, tensor, what):
+    B, N, Hq, Hkv, d, C, g, K = shape
+    w = S.Workload("nf_bwd", B, N, Hq, Hkv, d, C, g, K, "bf16", 2500 + N, "iid")
+    dev = T.Device(w, S.make_inputs(w))
+    dout = torch.randn(dev.q.shape, generator=torch.Generator(device="cuda").manual_seed(4), device="cuda").bfloat16()
+    x = dout if tensor == "dout" else getattr(dev, tensor)
+    if what == "future":
+        x[:, N // 2 + 9:] = NAN
+    elif what == "key":
+        x[:, N // 3, 0, 5] = NAN
+        x[:, N // 3 + C, -1, 7] = math.inf if tensor in ("v", "dout") else NAN
+    else:
+        x[-1, N // 3 // C * C:N // 3 // C * C + C] = NAN
+    dev.forward()
+    assert dev.sync_status() == 0
+    got = [torch.full_like(y, 7.0) for y in (dev.q, dev.k, dev.v)]
+    ws = PB.alloc_workspace(dev.p, PB.OP_BSA_BWD)
+    P.pisa_bsa_bwd(dev.p, dev.q, dev.k, dev.v, dev.idx, dev.out, dev.lse, dout, *got, ws)
+    torch.cuda.synchronize()
+    assert P.read_status(ws) == 0
+    _check_backward(dev, dev.idx, dout, got, C)
+
+
+@pytest.mark.parametrize("shape", BACKWARD[:3], ids=lambda s: "b%d_n%d_h%d_%d_d%d_c%d_g%d_k%d" % s)
+def test_padded_rows_without_blocks_reach_no_gradient(shape):
+    """Rows whose blocks were set to -1 may hold anything: queries, gradients, outputs and denominators."""
+    B, N, Hq, Hkv, d, C, g, K = shape
+    w = S.Workload("nf_pad", B, N, Hq, Hkv, d, C, g, K, "bf16", 2600 + N, "iid")
+    dev = T.Device(w, S.make_inputs(w))
+    dev.forward()
+    assert dev.sync_status() == 0
+    dout = torch.randn(dev.q.shape, generator=torch.Generator(device="cuda").manual_seed(4), device="cuda").bfloat16()
+    end = N - 2 * C - 37                                    # inside a leaf and a tile
+    idx = dev.idx.clone()
+    idx[:, :, end:] = -1
+    for x in (dev.q, dout, dev.out):
+        x[:, end:] = NAN
+    for x in (dev.k, dev.v):
+        x[:, end:] = math.inf
+    for fill in (0.0, NAN, math.inf):
+        dev.lse[:, :, end:] = fill
+        got = [torch.full_like(y, 7.0) for y in (dev.q, dev.k, dev.v)]
+        ws = PB.alloc_workspace(dev.p, PB.OP_BSA_BWD)
+        P.pisa_bsa_bwd(dev.p, dev.q, dev.k, dev.v, idx, dev.out, dev.lse, dout, *got, ws)
+        torch.cuda.synchronize()
+        assert P.read_status(ws) == 0
+        _check_backward(dev, idx, dout, got, C)
+        for x in got:
+            assert bool((x[:, end:] == 0).all()), fill
