@@ -56,7 +56,7 @@ int launch_qm_select_stage1(const Geometry& g, const qm::Args& a, long long rows
 int launch_qm_select_final(const Geometry& g, const qm::Args& a, long long rows, const int32_t* par, const float* blk,
                            int32_t* idx, float* margin, float* lse, float* sel_lse, cudaStream_t s);
 int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const void* k, const void* v, long long tokens,
-                     const float* row_lse, void* out, bool one_leaf, cudaStream_t s);
+                     const float* row_lse, void* out, bool one_leaf, bool two_terms, cudaStream_t s);
 
 // dense masked backward (qm_bwd.cuh).  gate (nullable): the choice is left to the data; receives what the list-driven kernels
 // have to look at; stat: where the preparation leaves the rows' (-lse * log2 e, -delta), [B, Hkv, N, G], for them too

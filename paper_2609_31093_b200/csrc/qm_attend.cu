@@ -40,6 +40,7 @@ struct AttArgs {
   const float* row_lse;      // [Hq, len] per sequence, natural log
   const __nv_bfloat16 *q, *k, *v;   // for attend_row()
   __nv_bfloat16* out;        // strides of the geometry's `out`
+  int two_terms;             // every sequence takes P in two bf16 terms (LO), not only those of one leaf
 };
 
 // One row over its own leaves only, by one warp.  The tiles multiply every value of a step with every row, zero weights
@@ -91,7 +92,8 @@ __device__ __forceinline__ void attend_row(const __nv_bfloat16* q, const __nv_bf
 // K / V tiles in flight (one ring: K, V, K, V, ...): what two items' query tiles leave of 227 KB
 __host__ __device__ constexpr int att_stages(int D, int NT) { return D == 128 ? (NT == 1 ? 5 : 3) : 8; }
 
-// LO: sequences of one leaf take P in two bf16 terms (an instantiation of its own: the registers would spill in the other)
+// LO: P in two bf16 terms (an instantiation of its own: the registers would spill in the other) for sequences of one leaf, or
+// for all of them (two_terms): shapes whose alternative is the exact fp32 path, which rounds no P, keep its precision.
 template <int D, int C, int NT, bool LO>
 __global__ void __launch_bounds__(kAttThreads, 1)
 qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ CUtensorMap tm_q,
@@ -272,7 +274,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           for (int x = 0; x < 16; ++x) {                            // two terms of P
             const int kk = x >> 1;
             umma_bf16_ts(d0, p0 + (uint32_t)((kk >> 1) * 32 + (x & 1) * 16 + (kk & 1) * 8), desc64(v0 + (uint32_t)kk * (2048u >> 4)), idesc_o,
-                         x > 0 ? 1u : 0u);
+                         (!w.fresh || x > 0) ? 1u : 0u);
           }
         }
         if (w.last) umma_commit(&o_full[w.ob]);
@@ -290,7 +292,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
       const int ny = __shfl_sync(0xffffffffu, e.y, 0), n0 = __shfl_sync(0xffffffffu, e.z, 0), n1 = __shfl_sync(0xffffffffu, e.w, 0);
       int len = 0x7fffffff;
       if (a.seqs != nullptr) len = qm::locate(geo, a, e.x, NT).q.len;
-      const bool one_leaf = (a.seqs != nullptr ? len : geo.N) <= C;
+      const bool two_terms = at.two_terms || (a.seqs != nullptr ? len : geo.N) <= C;
       int seen[2] = {0, 0};
       wait(&q_full[it & 1], (uint32_t)((it >> 1) & 1));
       const uint32_t q_item = q_base + (uint32_t)((it & 1) * NT * (TILE >> 4));
@@ -328,7 +330,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           }
           __syncwarp();
           Owed& w = owed[NT == 1 ? 1 : x];
-          w.stage = sv; w.phase = phv; w.rows = rows; w.lo = one_leaf;
+          w.stage = sv; w.phase = phv; w.rows = rows; w.lo = two_terms;
           const uint32_t pb = (NT == 1) ? par : (uint32_t)x;
           w.p_phase = (NT == 1) ? (p_phase[0] >> pb) & 1u : p_phase[x];
           if (NT == 1) p_phase[0] ^= 1u << pb; else p_phase[x] ^= 1u;
@@ -407,9 +409,8 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
           }
           tmem_st_32x16(s_base + (uint32_t)(qq * 16), pk);                   // over columns of S this warp has already read
         };
-        if (LO && len <= C) {
-          // a sequence of one leaf: P in two bf16 terms, sixteen columns each for 32 keys (the product is a single step, and
-          // the fp32 path, which rounds no P, is the one such a sequence takes on its own)
+        if (LO && (at.two_terms || len <= C)) {
+          // P in two bf16 terms, sixteen columns each for 32 keys
 #pragma unroll 1
           for (int qq = 0; qq < 2; ++qq) {
             uint32_t rr[32], pk[16];
@@ -519,7 +520,7 @@ qm_attend_kernel(Geometry geo, qm::Args a, AttArgs at, const __grid_constant__ C
       attend_row<D>(at.q + b * geo.qs[0] + (tok + t) * geo.qs[1] + hq * geo.qs[2], at.k + b * geo.ks[0] + tok * geo.ks[1] + tl.h * geo.ks[2],
                     geo.ks[1], at.v + b * geo.vs[0] + tok * geo.vs[1] + tl.h * geo.vs[2], geo.vs[1],
                     a.bits + tl.q.bits_off + ((long long)tl.h * len + t) * W, t, lgC, geo.scale * kLog2e,
-                    -at.row_lse[(long long)geo.Hq * tl.q.cu + (long long)hq * len + t] * kLog2e, !(LO && len <= C), out);
+                    -at.row_lse[(long long)geo.Hq * tl.q.cu + (long long)hq * len + t] * kLog2e, !(LO && (at.two_terms || len <= C)), out);
     }
   }
 }
@@ -541,7 +542,7 @@ int launch_dc(const Geometry& g, const qm::Args& a, const AttArgs& at, const CUt
 }  // namespace
 
 int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const void* k, const void* v, long long tokens,
-                     const float* row_lse, void* out, bool one_leaf, cudaStream_t s) {
+                     const float* row_lse, void* out, bool one_leaf, bool two_terms, cudaStream_t s) {
   CUtensorMap tm_q, tm_k, tm_v;
   if (!qm_map_rows(&tm_q, q, g.d, g.Hq, tokens, g.B, g.qs, g.G, 128 / g.G) ||
       !qm_map_rows(&tm_k, k, g.d, g.Hkv, tokens, g.B, g.ks, 1, 128) ||
@@ -550,6 +551,8 @@ int launch_qm_attend(const Geometry& g, const qm::Args& a, const void* q, const 
     return PISA_ERR_CUDA;
   }
   AttArgs at;
+  at.two_terms = two_terms;
+  one_leaf |= two_terms;
   at.row_lse = row_lse; at.out = (__nv_bfloat16*)out;
   at.q = (const __nv_bfloat16*)q; at.k = (const __nv_bfloat16*)k; at.v = (const __nv_bfloat16*)v;
   if (g.d == 128) return g.C == 128 ? launch_dc<128, 128>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s) : launch_dc<128, 64>(g, a, at, tm_q, tm_k, tm_v, one_leaf, s);

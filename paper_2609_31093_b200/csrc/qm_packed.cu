@@ -246,7 +246,7 @@ int qm_forward_packed(const Geometry& g, const int32_t* cu, const int* ids, int 
     kernel_mark("qm_select", s);
     if ((st = launch_qm_select_full(g, a, rows, idx, nullptr, lse, nullptr, s)) != PISA_OK) return st;
     kernel_mark("qm_attend", s);
-    if ((st = launch_qm_attend(g, a, q, k, v, total, lse, out, shortest <= g.C, s)) != PISA_OK) return st;
+    if ((st = launch_qm_attend(g, a, q, k, v, total, lse, out, shortest <= g.C, !tensor_path_supported(g, PISA_BF16), s)) != PISA_OK) return st;
     at = end;
   }
   return PISA_OK;

@@ -102,7 +102,8 @@ int qm_attend(const Geometry& g, const void* q, const void* k, const void* v, vo
   const Layout l = layout(g);
   const qm::Args a = uniform_args(g, ws, l, status);
   kernel_mark("qm_attend", s);
-  return launch_qm_attend(g, a, q, k, v, g.N, lse, out, g.N <= g.C, s);
+  // (where the lists do not take the problem its alternative is the exact fp32 path)
+  return launch_qm_attend(g, a, q, k, v, g.N, lse, out, g.N <= g.C, !tensor_path_supported(g, PISA_BF16), s);
 }
 
 // ---------------------------------------------------------------- upper levels and final selection of the list-driven path

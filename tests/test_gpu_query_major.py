@@ -70,3 +70,43 @@ def test_packed_sequences_do_not_see_their_neighbours():
         assert torch.equal(dirty[0][Hkv * K * a:Hkv * K * b], clean[0][Hkv * K * a:Hkv * K * b]), i
         assert torch.equal(dirty[1][a:b], clean[1][a:b]), i
         assert torch.equal(dirty[2][Hq * a:Hq * b], clean[2][Hq * a:Hq * b]), i
+
+
+@pytest.mark.parametrize("shape", [(1, 3000, 32, 8, 128, 128, 4, 5), (2, 1500, 4, 4, 64, 128, 4, 3), (1, 60, 8, 2, 128, 64, 2, 4)],
+                         ids=lambda s: "b%d_n%d_h%d_%d_d%d_c%d_g%d_k%d" % s)
+@pytest.mark.parametrize("packed", [False, True])
+def test_shapes_without_lists_keep_the_exact_paths_precision(shape, packed):
+    """Shapes that the list-driven kernels do not take (fan-in 4 with C = 128; one leaf) ran on the exact fp32 path, which does
+    not round the probabilities: the dense kernels are no further from float64 (the rounding of the output, 2^-9, dominates;
+    one bf16 term per probability adds a quarter to the error)."""
+    import torch
+    import paper_2609_31093_b200 as P
+    from paper_2609_31093_b200 import binding as PB
+    B, N, Hq, Hkv, d, C, g, K = shape
+    w = S.Workload("qm_prec", B, N, Hq, Hkv, d, C, g, K, "bf16", 1795 + N, "iid")
+    dev = T.Device(w, S.make_inputs(w))
+    dev.forward()
+    if packed:
+        cu = [N * b for b in range(B + 1)]
+        p = P.Params(1, N, Hq, Hkv, d, C, g, K, dtype="bf16")
+        ws = PB.alloc_workspace(p, PB.OP_FORWARD_PACKED)
+        P.pisa_forward_packed(p, cu, dev.q, dev.k, dev.v, PB.alloc_pyramid(p), dev.idx, dev.out, dev.lse, ws)
+    assert dev.sync_status() == 0
+    ref = T.Device(w, S.make_inputs(w), impl=PB.IMPL_SIMT)
+    ref.bsa(dev.idx)
+    assert ref.sync_status() == 0
+    leaf, t = torch.arange(N, device="cuda") // C, torch.arange(N, device="cuda")
+    err = [0.0, 0.0]
+    for b in range(B):
+        for h in range(Hkv):
+            rows = dev.idx[b, h].long()
+            kept = torch.zeros((N, int(leaf[-1]) + 2), dtype=torch.bool, device="cuda").scatter_(1, torch.where(rows < 0, int(leaf[-1]) + 1, rows), True)
+            see = kept[:, leaf] & (t[None] <= t[:, None])
+            for hq in range(h * Hq // Hkv, (h + 1) * Hq // Hkv):
+                s = (dev.q[b, :, hq].double() @ dev.k[b, :, h].double().T * d ** -0.5).masked_fill(~see, float("-inf"))
+                o = torch.softmax(s, 1) @ dev.v[b, :, h].double()
+                for i, x in enumerate((dev.out, ref.out)):
+                    err[i] += float((x[b, :, hq].double() - o).square().sum())
+    err = [e ** 0.5 for e in err]
+    print("dense %.6e exact path %.6e ratio %.4f" % (err[0], err[1], err[0] / err[1]))
+    assert err[0] <= 1.002 * err[1]
