@@ -38,7 +38,6 @@ struct LocalArgs {
   int32_t* status;
   int tiles_per_leaf;      // C / (128 / G)
   int n_items;             // B * Hkv * M1 * tiles_per_leaf
-  Gate gate;
 };
 
 __device__ __forceinline__ float ex2l(float x) {
@@ -70,7 +69,6 @@ template <int C, int D>
 __global__ void __launch_bounds__(kLocalThreads, 1)
 local_window_kernel(Geometry geo, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, LocalArgs a) {
-  if (a.gate.off_list()) return;
   extern __shared__ uint8_t smem_raw[];
   constexpr int KS = D / 64;
   constexpr bool kTransO = (D == 128);
@@ -360,10 +358,10 @@ bool local_window_supported(const Geometry& g, int dtype) {
 
 template <int C, int D>
 static int launch_local_c(const Geometry& g, const void* q, const void* k, const void* v, const float* row_lse,
-                          float* o_acc, int32_t* status, const Gate& gate, cudaStream_t s) {
+                          float* o_acc, int32_t* status, cudaStream_t s) {
   const int tpt = 128 / g.G;
   LocalArgs a;
-  a.row_lse = row_lse; a.o_acc = o_acc; a.status = status; a.gate = gate;
+  a.row_lse = row_lse; a.o_acc = o_acc; a.status = status;
   a.tiles_per_leaf = g.C / tpt;
   const long long items = (long long)g.B * g.Hkv * g.M[1] * a.tiles_per_leaf;
   if (items > 0x7fffffffLL) return PISA_ERR_UNSUPPORTED;
@@ -392,13 +390,13 @@ static int launch_local_c(const Geometry& g, const void* q, const void* k, const
 }
 
 int launch_local_window(const Geometry& g, const void* q, const void* k, const void* v, const float* row_lse,
-                        float* o_acc, int32_t* status, const Gate& gate, cudaStream_t s) {
+                        float* o_acc, int32_t* status, cudaStream_t s) {
   if (g.d == 128) {
-    if (g.C == 128) return launch_local_c<128, 128>(g, q, k, v, row_lse, o_acc, status, gate, s);
-    return launch_local_c<64, 128>(g, q, k, v, row_lse, o_acc, status, gate, s);
+    if (g.C == 128) return launch_local_c<128, 128>(g, q, k, v, row_lse, o_acc, status, s);
+    return launch_local_c<64, 128>(g, q, k, v, row_lse, o_acc, status, s);
   }
-  if (g.C == 128) return launch_local_c<128, 64>(g, q, k, v, row_lse, o_acc, status, gate, s);
-  return launch_local_c<64, 64>(g, q, k, v, row_lse, o_acc, status, gate, s);
+  if (g.C == 128) return launch_local_c<128, 64>(g, q, k, v, row_lse, o_acc, status, s);
+  return launch_local_c<64, 64>(g, q, k, v, row_lse, o_acc, status, s);
 }
 
 }  // namespace pisa

@@ -234,7 +234,7 @@ static int do_bsa(const pisa_params_t* p, const Geometry& g, const void* q, cons
   if (ws_bytes < bsa_ws_bytes(p, g)) return PISA_ERR_WORKSPACE_TOO_SMALL;
   if (use_tensor(p, g))
     return tensor_bsa(g, p->dtype, q, k, v, idx, sel_lse, out, lse, lse_ready, forced_present,
-                      (char*)ws + kStatusBytes, (int32_t*)ws, Gate{nullptr, 0u}, s);
+                      (char*)ws + kStatusBytes, (int32_t*)ws, s);
   kernel_mark("bsa_simt", s);
   return launch_bsa_simt(g, p->dtype, q, k, v, idx, out, lse, s);
 }
@@ -483,7 +483,7 @@ static int do_bsa_chunked(const pisa_params_t* p, const Geometry& g, const void*
     st = run_chunks(p, g, pl, ws, s, [&](const ChunkView& v, int) {
       return tensor_bsa(v.g, p->dtype, (const char*)q + v.q_off, (const char*)k + v.k_off, (const char*)v_ + v.v_off,
                         idx + v.unit0 * g.N * g.K, sel_lse ? sel_lse + v.unit0 * g.G * g.N * g.K : nullptr,
-                        (char*)out + v.o_off, lse + v.unit0 * g.G * g.N, false, false, v.region, (int32_t*)ws, Gate{nullptr, 0u}, v.stream);
+                        (char*)out + v.o_off, lse + v.unit0 * g.G * g.N, false, false, v.region, (int32_t*)ws, v.stream);
     });
   kernel_mark("end", s);
   return st;
@@ -564,7 +564,7 @@ static int do_forward(const pisa_params_t* p, const Geometry& g, const void* q, 
       if (i == 0) stage_mark(2, s);
       return tensor_bsa(v.g, p->dtype, (const char*)q + v.q_off, (const char*)k + v.k_off, (const char*)v_ + v.v_off,
                         ic, nullptr, (char*)out + v.o_off, lc, g.score_mode == PISA_SCORE_LSE, true, v.region, (int32_t*)ws,
-                        Gate{nullptr, 0u}, v.stream);
+                        v.stream);
     });
     if (st == PISA_OK && routed != nullptr) {             // (chunks: the indices count as final when all chunks have ended)
       const cudaError_t ee = cudaEventRecord(routed, s);

@@ -20,7 +20,7 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
 // served by the query-major local-window kernel instead of the lists
 int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const void* v, const int32_t* idx,
                const float* sel_lse, void* out, float* lse, bool lse_ready, bool forced_present, void* ws,
-               int32_t* status, const Gate& gate, cudaStream_t s);
+               int32_t* status, cudaStream_t s);
 
 // query-major path (query_major.cuh): dense scoring, one-thread-per-token selection, masked dense attention
 namespace qm { struct Args; }
@@ -78,7 +78,7 @@ int qm_write_table(const qm::Seq* seqs, const qm::SeqOrder* order, int n, qm::Se
 // attention over the forced leaves, query-major (local_window.cu); stores the fp32 accumulator [B,Hkv,N,128,G]
 bool local_window_supported(const Geometry& g, int dtype);
 int launch_local_window(const Geometry& g, const void* q, const void* k, const void* v, const float* row_lse,
-                        float* o_acc, int32_t* status, const Gate& gate, cudaStream_t s);
+                        float* o_acc, int32_t* status, cudaStream_t s);
 
 // backward of the block-sparse attention with frozen indices; dq [B,N,Hq,d], dk, dv [B,N,Hkv,d] dense
 bool tensor_bwd_supported(const Geometry& g, int dtype);

@@ -277,7 +277,6 @@ struct TileArgs {
   float* o_acc;            // fp32 accumulator: [B, Hkv, N, D, G] when the second product is transposed, else [B, N, Hq, D]
   int32_t* status;
   int debug;               // PISA_DEBUG_* bits: list entries are range-checked before they are used
-  Gate gate;
 };
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
@@ -775,7 +774,6 @@ template <int D, int C>
 __global__ void __launch_bounds__(kPvThreads, 1)
 pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v) {
-  if (a.gate.off_list()) return;
   extern __shared__ uint8_t smem_raw[];
   constexpr int NS = 4;
   constexpr int KS = D / 64;
@@ -1376,8 +1374,7 @@ __global__ void __launch_bounds__(256) row_lse_from_sel_kernel(Geometry geo, con
 
 // fp32 accumulator [B,N,Hq,d] -> out in bf16 (strided)
 __global__ void __launch_bounds__(256) convert_out_kernel(Geometry geo, const float* __restrict__ acc,
-                                                           __nv_bfloat16* __restrict__ out, Gate gate) {
-  if (gate.off_list()) return;
+                                                           __nv_bfloat16* __restrict__ out) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;     // one 8-element chunk
   const int ch = geo.d / 8;
   const long long total = (long long)geo.B * geo.N * geo.Hq * ch;
@@ -1695,7 +1692,7 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
 
 int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const void* v, const int32_t* idx,
                const float* sel_lse, void* out, float* lse, bool lse_ready, bool forced_present, void* ws_,
-               int32_t* status, const Gate& gate, cudaStream_t s) {
+               int32_t* status, cudaStream_t s) {
   (void)dtype;
   char* ws = (char*)ws_;
   const BsaLayout L = bsa_layout(g);
@@ -1707,13 +1704,13 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   // local-window kernel, which also initialises the accumulator (it needs the rows' denominators, so only
   // when the routing handed them over: the block-LSE pass below walks the very lists they are left out of)
   const bool local = forced_present && lse_ready && local_window_supported(g, dtype);
-  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kWindowTok, local ? 1 : 0, gate);
+  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kWindowTok, local ? 1 : 0);
   if (st != PISA_OK) return st;
   TileArgs a = {};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
   a.entry_off = inv.entry_off; a.tile_off = inv.tile_off; a.item_off = inv.item_off; a.item_key = inv.item_key; a.entries = inv.entries;
   a.nkeys = g.B * g.Hkv * inv.NW * g.M[1]; a.Mk = g.M[1]; a.NW = inv.NW; a.fan = 1; a.slots = g.K;
-  a.blk_lse = blk; a.row_lse = lse; a.o_acc = acc; a.status = status; a.debug = g.debug; a.gate = gate;
+  a.blk_lse = blk; a.row_lse = lse; a.o_acc = acc; a.status = status; a.debug = g.debug;
   if (!lse_ready && sel_lse != nullptr) {
     kernel_mark("row_lse", s);
     const long long rows = (long long)g.B * g.Hq * g.N;
@@ -1731,7 +1728,7 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   }
   if (local) {
     kernel_mark("local_window", s);
-    st = launch_local_window(g, q, k, v, lse, acc, status, gate, s);
+    st = launch_local_window(g, q, k, v, lse, acc, status, s);
     if (st != PISA_OK) return st;
   } else {
     kernel_mark("accumulator_memset", s);
@@ -1744,10 +1741,10 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   kernel_mark("convert_out", s);
   if (g.d == 128) {
     const long long n = (long long)g.B * g.N * g.Hkv * (g.d / 2);
-    convert_out_heads_inner_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out, gate);
+    convert_out_heads_inner_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out, Gate{nullptr, 0u});
   } else {
     const long long n = (long long)g.B * g.N * g.Hq * (g.d / 8);
-    convert_out_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out, gate);
+    convert_out_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, acc, (__nv_bfloat16*)out);
   }
   return check_launch("convert_out");
 }
