@@ -20,6 +20,10 @@
  *   pyramid: levels 1..L back to back, level l = [B, Hkv, M_l, d] in the input dtype,
  *            at the element offsets pisa_pyramid_layout() reports.
  *
+ * Values that are not finite: a NaN score ranks after every other one; a NaN or an infinity in a key or value reaches the
+ * rows that selected it and may see it (where the list-driven kernels serve a long sequence, also earlier rows of its own
+ * leaf), one in a query or gradient its row and the gradients of the keys the row selected.  Rows whose idx is -1 reach nothing.
+ *
  * All functions return a pisa_status (0 = OK).  Nothing aborts, throws or traps the GPU.
  */
 #ifndef PISA_H_
@@ -95,7 +99,11 @@ const char* pisa_last_cuda_error(void);
  */
 int pisa_pyramid_layout(const pisa_params_t* p, int32_t* L, int32_t* M, int64_t* level_off, size_t* bytes);
 
-/* Host-only.  Bytes of device workspace `op` needs for these parameters (256-byte aligned base). */
+/*
+ * Host-only.  Bytes of device workspace `op` needs for these parameters (256-byte aligned base).  For shorter sequences
+ * PISA_OP_ROUTE and _FORWARD include the score tables of the dense kernels, a float per (token, leaf, query head), up to 4 GB
+ * (16 heads without groups, 32768 tokens: 2.1 GB); with a workspace that holds the list-driven kernels' scratch only, those run.
+ */
 int pisa_workspace_bytes(const pisa_params_t* p, int op, size_t* bytes);
 
 /*
@@ -148,8 +156,8 @@ int pisa_bsa_fwd(const pisa_params_t* p, const void* q, const void* k, const voi
  * Same arguments and results as pisa_route, without ws / ws_bytes: the scratch is a 32 MiB device
  * array built into the library (pisa_route_static_capacity()), present on every GPU that loads the
  * library until the process exits.  The call allocates nothing, on the host or on the device.
- *  - Problems whose PISA_OP_ROUTE workspace exceeds the capacity are refused with
- *    PISA_ERR_STATIC_SCRATCH_TOO_SMALL before anything is launched.
+ *  - Problems whose scratch exceeds the capacity (the list-driven kernels' part of the PISA_OP_ROUTE workspace) are refused
+ *    with PISA_ERR_STATIC_SCRATCH_TOO_SMALL before anything is launched.
  *  - The first call on each device looks up the array's device address (the device that is current
  *    at the call); make that first call outside any stream capture.
  *  - All calls on one device share the array, which keeps whatever the last call left in it; each

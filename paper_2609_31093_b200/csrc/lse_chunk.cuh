@@ -47,7 +47,7 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 
 // 2^z for two z on the FMA pipe, where the special-function unit (16 exponentials per clock and SM) is the limit: z = n + f
 // with n the nearest integer (Cody and Waite), a polynomial of degree five for 2^f on [-1/2, 1/2] with value 1 at 0 (relative
-// minimax by linear programming, 9.1e-8; 1.7e-7 with its fp32 roundings, what ex2.approx states), the exponent by integer
+// minimax by linear programming, 1.1e-7; 1.7e-7 with its fp32 roundings, what ex2.approx states), the exponent by integer
 // arithmetic.  z < -126 counts as -126; z < 128.
 __device__ __forceinline__ float max_nan(float a, float b) {
   float d;
@@ -102,7 +102,7 @@ __device__ __forceinline__ void lse_chunk(const uint32_t (&rr)[NW], float sl2, f
 }
 // the same with only the first `nvalid` (>= 1) columns of the chunk taking part.  The sums associate
 // exactly as in lse_chunk (four interleaved accumulators), so a full row gives bit-identical results on
-// either path: which path a row takes depends on the other rows of its tile, and the composition of a
+// either path where lse_chunk takes no polynomial (POLY = 0, the list-driven kernels): which path a row takes depends on the other rows of its tile, and the composition of a
 // tile (the order of a list's entries) varies from run to run.
 template <int NW>
 __device__ __forceinline__ void lse_chunk_masked(const uint32_t (&rr)[NW], int nvalid, float sl2, float& m,

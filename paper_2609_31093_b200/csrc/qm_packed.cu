@@ -15,7 +15,7 @@ namespace pisa {
 namespace {
 
 constexpr int kChunkSeqs = 256;
-struct TableChunk {                       // a kernel parameter (16 KB): the table travels without a copy from host memory
+struct TableChunk {                       // a kernel parameter (18 KB): the table travels without a copy from host memory
   int n, first;
   qm::Seq seq[kChunkSeqs];
   qm::SeqOrder order[kChunkSeqs];
