@@ -23,6 +23,7 @@
 
 #include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
+#include "shared_attend.cuh"
 #include "tc_utils.cuh"
 #include "tma_map.cuh"
 
@@ -61,17 +62,17 @@ struct InvArgs {
   int32_t* status;        // the workspace's status word
   int debug;              // PISA_DEBUG_* bits
   Gate gate;
-  int skip_forced;        // leave the row's forced leaves (0, c-1, c) out of the lists: the local-window kernel serves them
+  const uint32_t* taken;  // [BH, N] (or null) bit s: entry s of the row is served elsewhere (shared_attend.cu) and stays out of the lists
 };
 
 __device__ __forceinline__ int inv_token(const InvArgs& a, int e) { return a.lgK >= 0 ? (e >> a.lgK) : e / a.K; }
 __device__ __forceinline__ int inv_slot(const InvArgs& a, int e) { return a.lgK >= 0 ? (e & (a.K - 1)) : e % a.K; }
-__device__ __forceinline__ bool inv_valid(const InvArgs& a, int node, int t) {
+__device__ __forceinline__ bool inv_valid(const InvArgs& a, int bh, int node, int t, int slot) {
   const int leaf = a.lgC >= 0 ? (t >> a.lgC) : t / a.C;
   const bool ok = node >= 0 && node < a.Mk && (long long)node * a.fan <= (long long)leaf;
   // bounds-check mode: anything but the -1 padding that is not a usable node id is reported
   if ((a.debug & PISA_DEBUG_BOUNDS) && !ok && node != -1) atomicExch(a.status, (int)PISA_ERR_BOUNDS);
-  if (a.skip_forced && (node == 0 || node == leaf || node == leaf - 1)) return false;
+  if (a.taken != nullptr && ((a.taken[(long long)bh * a.N + t] >> slot) & 1u)) return false;
   return ok;
 }
 
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(256) inv_count_kernel(InvArgs a, int use_smem)
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int t = t0 + inv_token(a, e);
     const int node = a.nodes[((long long)bh * a.N + t0) * a.K + e];
-    if (inv_valid(a, node, t)) {
+    if (inv_valid(a, bh, node, t, inv_slot(a, e))) {
       if (use_smem) atomicAdd(&s_hist[node], 1);
       else atomicAdd(&a.count[kbase + node], 1);
     }
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(256) inv_fill_kernel(InvArgs a, int use_smem) 
   if (!use_smem) {
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
       const int t = t0 + inv_token(a, e), slot = inv_slot(a, e), node = nodes[e];
-      if (inv_valid(a, node, t)) {
+      if (inv_valid(a, bh, node, t, slot)) {
         const int pos = atomicAdd(&a.cursor[kbase + node], 1);
         a.entries[pos] = t | (slot << 24);
       }
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(256) inv_fill_kernel(InvArgs a, int use_smem) 
   __syncthreads();
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int node = nodes[e];
-    if (inv_valid(a, node, t0 + inv_token(a, e))) atomicAdd(&s_hist[node], 1);
+    if (inv_valid(a, bh, node, t0 + inv_token(a, e), inv_slot(a, e))) atomicAdd(&s_hist[node], 1);
   }
   __syncthreads();
   for (int j = threadIdx.x; j < a.Mk; j += blockDim.x) {
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(256) inv_fill_kernel(InvArgs a, int use_smem) 
   __syncthreads();
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int t = t0 + inv_token(a, e), slot = inv_slot(a, e), node = nodes[e];
-    if (inv_valid(a, node, t)) {
+    if (inv_valid(a, bh, node, t, slot)) {
       const int r = atomicAdd(&s_hist[node], 1);
       a.entries[s_base[node] + r] = t | (slot << 24);
     }
@@ -1467,10 +1468,10 @@ BsaLayout bsa_layout(const Geometry& g) {
 }
 
 int run_inversion(const Geometry& g, const int32_t* nodes, int fan, int Mk, char* ws, const InvLayout& l,
-                  InvArgs* out, int32_t* status, cudaStream_t s, int win = kWindowTok, int skip_forced = 0, Gate gate = Gate{nullptr, 0u}) {
+                  InvArgs* out, int32_t* status, cudaStream_t s, int win = kWindowTok, const uint32_t* taken = nullptr, Gate gate = Gate{nullptr, 0u}) {
   InvArgs a;
   a.gate = gate;
-  a.status = status; a.debug = g.debug; a.skip_forced = skip_forced;
+  a.status = status; a.debug = g.debug; a.taken = taken;
   a.nodes = nodes; a.K = g.K; a.fan = fan; a.Mk = Mk; a.N = g.N; a.C = g.C; a.BH = g.B * g.Hkv;
   a.tpt = 128 / g.G;
   a.lgK = (g.K & (g.K - 1)) == 0 ? 31 - __builtin_clz((unsigned)g.K) : -1;
@@ -1698,13 +1699,21 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   const BsaLayout L = bsa_layout(g);
   float* blk = (float*)(ws + L.blk);
   float* acc = (float*)(ws + L.acc);
+  // idx that came out of the routing (its denominators known): what neighbouring rows share, their forced leaves among it, goes
+  // to the query-major kernel, which also initialises the accumulator (with other denominators the block-LSE pass below walks
+  // lists of everything).  Its plan stands where that pass keeps its scores.
+  SharedPlan plan;
+  const bool shared = forced_present && lse_ready && shared_attend_supported(g, dtype) &&
+                      shared_plan_layout(g, (char*)blk, &plan) <= L.acc - L.blk;
+  int st = PISA_OK;
+  if (shared) {
+    kernel_mark("shared_plan", s);
+    st = launch_shared_plan(g, idx, plan, s);
+    if (st != PISA_OK) return st;
+  }
   kernel_mark("invert_by_leaf", s);
   InvArgs inv;
-  // idx that came out of the routing holds every row's forced leaves: those go to the query-major
-  // local-window kernel, which also initialises the accumulator (it needs the rows' denominators, so only
-  // when the routing handed them over: the block-LSE pass below walks the very lists they are left out of)
-  const bool local = forced_present && lse_ready && local_window_supported(g, dtype);
-  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kWindowTok, local ? 1 : 0);
+  st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kWindowTok, shared ? plan.taken : nullptr);
   if (st != PISA_OK) return st;
   TileArgs a = {};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
@@ -1726,9 +1735,9 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
     st = check_launch("row_lse");
     if (st != PISA_OK) return st;
   }
-  if (local) {
-    kernel_mark("local_window", s);
-    st = launch_local_window(g, q, k, v, lse, acc, status, s);
+  if (shared) {
+    kernel_mark("shared_attend", s);
+    st = launch_shared_attend(g, q, k, v, lse, acc, plan, inv.work_ctr + 2, status, s);
     if (st != PISA_OK) return st;
   } else {
     kernel_mark("accumulator_memset", s);
@@ -1769,7 +1778,7 @@ int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* 
   const BwdLayout L = bwd_layout(g);
   kernel_mark("invert_by_leaf", s);
   InvArgs inv;
-  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kBwdWindowTok, 0, gate);
+  int st = run_inversion(g, idx, 1, g.M[1], ws, L.inv, &inv, status, s, kBwdWindowTok, nullptr, gate);
   if (st != PISA_OK) return st;
   BwdArgs a = {};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
