@@ -201,7 +201,7 @@ int pisa_forward(const pisa_params_t* p, const void* q, const void* k, const voi
  *   ws          : device workspace sized for PISA_OP_FORWARD_PACKED with p (N = the longest sequence)
  *
  * Launches.  With a workspace sized for PISA_OP_FORWARD_PACKED all sequences short enough for the query-major kernels
- * (bf16, LSE score, fan-in 2 or 4, C of 64 or 128; K * 704 .. 2048 tokens, by leaf size and heads per group) run unpadded
+ * (bf16, LSE score, fan-in 2 or 4, C of 64 or 128; K * 480 .. 2048 tokens, by leaf size and heads per group) run unpadded
  * through as few sets of launches as the workspace has room for their score tables.  For the others: the method is causal
  * (Sec. 3.2: a query only ever scores nodes that lie wholly in its
  * past; the nodes on its own path are forced, not scored), so a sequence gives the same rows when it is

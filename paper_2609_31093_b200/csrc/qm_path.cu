@@ -69,13 +69,17 @@ bool qm_supported(const Geometry& g, int dtype) {
   return g.g == 2 || g.g == 4;
 }
 
-// Where the dense kernels win.  They cost a row N / 2 keys whatever it selects; the lists cost it K (token, block) pairs of
-// gathered query rows and fp32 reductions, so the line lies at a length proportional to K.  Measured crossovers of the
-// whole forward: 16 KV heads without groups (G = 1) beyond 32768 tokens at K = 16; G = 4, C = 64, K = 16 at 18 to 20
-// thousand; G = 4, C = 128, K = 32 (larger blocks per pair) at 24 thousand; G = 16, d = 64, K = 8 at 8 thousand.
+// Where the dense kernels win.  They cost a row N / 2 keys whatever it selects; the lists cost it K (token, block) pairs, so
+// the line lies at a length proportional to K.  Whole forwards in us, dense / lists, of passages on 32 topics (neighbours
+// select much the same leaves, which the lists' attention serves query-major: with queries that share nothing the lists take
+// a third longer and the lines lie 1.5 times higher): G = 4, C = 64, K = 16: 12288 tokens 745 / 748 (16 heads), 1402 / 1265
+// (32 heads, fan-in 4), 8192 763 / 838; G = 4, C = 128, K = 32: 12288 1744 / 2100, 16384 2964 / 2869; 16 KV heads without
+// groups, K = 16: 16384 1612 / 1740, 24000 3304 / 2846; G = 16, d = 64, K = 8: 6000 331 / 367, 8192 526 / 461.  Shapes that
+// the lists do not take stay dense further: their alternative is the exact fp32 path.
 bool qm_dense_preferred(const Geometry& g, int dtype) {
   if (!qm_supported(g, dtype) || g.M[1] > 512 || g.N > kDenseMaxTokens) return false;
-  const int per_block = g.G == 1 ? 2048 : (g.C == 128 ? 704 : 1024);
+  int per_block = g.G == 1 ? 1120 : g.C == 128 ? 480 : g.G == 16 ? 832 : 704;
+  if (!tensor_path_supported(g, dtype)) per_block = g.G == 1 ? 2048 : g.C == 128 ? 704 : 1024;
   return g.N <= g.K * per_block && layout(g).total <= kDenseMaxBytes;
 }
 

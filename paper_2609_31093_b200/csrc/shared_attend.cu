@@ -5,8 +5,8 @@
 // the same leaves -- the first, the previous and their own leaf by rule (App. B), others because they are about the same
 // thing -- and for those a dense product of the tile's 128 rows with the leaf costs a third, whoever selected it, and adds
 // nothing into memory:
-//   plan      one CTA per tile of 128 / G tokens: how many of them selected each leaf; a leaf that kShareNum / 8 of them
-//             selected (leaf 0 always) goes to the tile's list with a mask of who did, the rest to the inverted lists
+//   plan      one CTA per tile of 128 / G tokens: how many of them selected each leaf; a leaf that enough of them
+//             selected (share_threshold; leaf 0 always) goes to the tile's list with a mask of who did, the rest to the inverted lists
 //   attention one item per tile, drawn from a global counter: its queries stay in shared memory, the leaves of its list come
 //             by TMA tile loads, 128 keys a step (one leaf of 128 or two of 64 keys, wherever they lie); S = Q K^T -> P =
 //             exp(S - lse) in bf16 where selected and visible, zero elsewhere (the row's denominator is known from the
@@ -29,15 +29,22 @@ using namespace tc;
 
 namespace {
 
-constexpr int kShareNum = 3;                   // of every eight tokens of a tile, how many make a leaf shared
 constexpr int kShareMaxLeaves = 32768;         // a tile's counters: a byte per leaf in shared memory
 constexpr int kPlanThreads = 256;
 constexpr int kThreads = 640;
 constexpr int kRing = 4;                       // items listed ahead: reading an item out waits for products that go out two items later
 constexpr int kBufs = 3;                       // S / P buffers
-constexpr int kMaxShared = 96;                 // leaves of one tile: K * 8 / kShareNum and leaf 0, at most
+constexpr int kMaxShared = 176;                // leaves of one tile: at most K / the smallest share below, and leaf 0
 
-int share_threshold(int tpt) { return (tpt * kShareNum + 7) / 8; }
+// How many of a tile's tokens make a leaf shared.  A dense step takes about 1660 cycles of an SM (128 keys; 128 rows, d = 128)
+// whoever selected its leaves, 32 tokens' pairs with a leaf (G = 4) 5000 in the lists with C = 128 and 4300 with C = 64, and
+// without groups the lists' reductions are scalar.  Plan, shared and list attention in ms, by sixteenths: 131072 tokens,
+// C = 128: 4: 11.42, 6: 11.39, 8: 11.35; 2 x 32700, C = 64, G = 4: 4: 2.08, 6: 2.18, 8: 2.30; 40000, C = 64, G = 1: 4: 1.70,
+// 6: 1.88, 8: 2.08.
+int share_threshold(const Geometry& g) {
+  const int tpt = 128 / g.G, num = g.C == 128 ? 6 : (g.G == 1 ? 3 : 4);
+  return (tpt * num + 15) / 16;
+}
 
 template <bool V> struct Bool { static constexpr bool value = V; };
 
@@ -563,7 +570,7 @@ size_t shared_plan_layout(const Geometry& g, char* ws, SharedPlan* p) {
   const size_t bh = (size_t)g.B * g.Hkv;
   p->words = (tpt + 31) / 32;
   p->tiles = (g.N + tpt - 1) / tpt;
-  const int most = g.K * tpt / share_threshold(tpt) + 1;                   // ... and leaf 0
+  const int most = g.K * tpt / share_threshold(g) + 1;                   // ... and leaf 0
   p->max_leaves = most < kMaxShared ? most : kMaxShared;
   const size_t tiles = bh * p->tiles;
   size_t o = 0;
@@ -578,7 +585,7 @@ size_t shared_plan_layout(const Geometry& g, char* ws, SharedPlan* p) {
 
 int launch_shared_plan(const Geometry& g, const int32_t* idx, const SharedPlan& plan, cudaStream_t s) {
   const dim3 grid((unsigned)plan.tiles, (unsigned)(g.B * g.Hkv));
-  shared_plan_kernel<<<grid, kPlanThreads, (size_t)((g.M[1] + 3) / 4) * 4, s>>>(g, idx, plan, share_threshold(128 / g.G));
+  shared_plan_kernel<<<grid, kPlanThreads, (size_t)((g.M[1] + 3) / 4) * 4, s>>>(g, idx, plan, share_threshold(g));
   return check_launch("shared_plan");
 }
 

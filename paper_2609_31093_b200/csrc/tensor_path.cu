@@ -13,7 +13,8 @@
 //                                              causal mask inside the query's own leaf
 //               qm_select / final_topk      -> grouped score = sum over heads, forced leaves, Top-K;
 //                                              also the softmax denominator of the kept leaves
-//   attention : invert idx by leaf          -> lists of (token, slot)
+//   attention : shared_attend.cu            -> the leaves that a tile's rows share, query-major, into the accumulator
+//               invert idx by leaf          -> lists of (token, slot) of the others
 //               [lse_ws + row_lse only when the denominators are not already known]
 //               pv_ws_kernel                -> S = Q K^T, P = exp(S - lse_row) (already normalised),
 //                                              O_partial = P V, added into an fp32 accumulator with
