@@ -1,22 +1,20 @@
-// Attention over the leaves that a tile's rows share, query-major.
+// Attention over the leaves that a tile's rows share, query-major (shared.cuh).
 //
-// The list-driven attention (tensor_path.cu) pays about 5000 SM cycles per 128-row tile of gathered (token, leaf) pairs
-// (C = 128; 4300 with C = 64), most of it for the fp32 rows that each pair adds into memory.  Neighbouring tokens select much
-// the same leaves -- the first, the previous and their own leaf by rule (App. B), others because they are about the same
-// thing -- and for those a dense product of the tile's 128 rows with the leaf costs a third, whoever selected it, and adds
-// nothing into memory:
-//   plan      one CTA per tile of 128 / G tokens: how many of them selected each leaf; a leaf that enough of them
-//             selected (share_threshold; leaf 0 always) goes to the tile's list with a mask of who did, the rest to the inverted lists
-//   attention one item per tile, drawn from a global counter: its queries stay in shared memory, the leaves of its list come
-//             by TMA tile loads, 128 keys a step (one leaf of 128 or two of 64 keys, wherever they lie); S = Q K^T -> P =
-//             exp(S - lse) in bf16 where selected and visible, zero elsewhere (the row's denominator is known from the
-//             routing, so P is final), over S in TMEM -> O += P V.  The accumulator rows are STORED: nothing clears them first.
+// The lists cost about 5000 SM cycles per 128-row tile of gathered (token, leaf) pairs (C = 128; 4300 with C = 64), most of it
+// for the fp32 rows added into memory; a dense step here costs a third of that and adds nothing into memory.  One item per
+// tile, drawn from a global counter: its queries stay in shared memory, the leaves of its list come by TMA tile loads, 128 keys
+// a step (one leaf of 128 or two of 64 keys, wherever they lie); S = Q K^T -> P = exp(S - lse) in bf16 where selected and
+// visible, zero elsewhere (the row's denominator is known from the routing, so P is final), over S in TMEM -> O += P V.  The
+// accumulator rows are STORED: nothing clears them first, the list-driven kernel then adds to them.
 // Roles: warp 0 loads queries and keys, warp 2 values, warp 1 issues the products, warp 3 draws the items, warps 4-11 and
 // 12-19 are two softmax / read-out groups on alternate steps; inside a group two warps share a TMEM lane quarter, half of the
 // columns each.  Three S / P buffers, so that a step's softmax has the products of two others to run under.
+// Measured: 131072 tokens, 32 heads, C = 128: 6.6 ms for 77 % of the routed pairs and the forced leaves, 1660 cycles a step,
+// 1230 TFLOP/s executed (three quarters of the measured bf16 peak; the SM clock falls to 1.65 GHz); the lists take 16.8 ms for all
+// of the routed pairs.
 // Every wait is bounded.  What is not finite reaches only the rows that selected it: rows that came out not finite are
 // computed again from their own leaves (attend_shared_row).
-#include "shared_attend.cuh"
+#include "shared.cuh"
 
 #include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
@@ -29,13 +27,9 @@ using namespace tc;
 
 namespace {
 
-constexpr int kShareMaxLeaves = 32768;         // a tile's counters: a byte per leaf in shared memory
-constexpr int kPlanThreads = 256;
 constexpr int kThreads = 640;
 constexpr int kRing = 4;                       // items listed ahead: reading an item out waits for products that go out two items later
 constexpr int kBufs = 3;                       // S / P buffers
-constexpr int kMaxShared = 176;                // leaves of one tile: at most K / the smallest share below, and leaf 0
-
 // How many of a tile's tokens make a leaf shared.  A dense step takes about 1660 cycles of an SM (128 keys; 128 rows, d = 128)
 // whoever selected its leaves, 32 tokens' pairs with a leaf (G = 4) 5000 in the lists with C = 128 and 4300 with C = 64, and
 // without groups the lists' reductions are scalar.  Plan, shared and list attention in ms, by sixteenths: 131072 tokens,
@@ -47,62 +41,6 @@ int share_threshold(const Geometry& g) {
 }
 
 template <bool V> struct Bool { static constexpr bool value = V; };
-
-// ------------------------------------------------------------------ plan
-
-__global__ void __launch_bounds__(kPlanThreads) shared_plan_kernel(Geometry geo, const int32_t* __restrict__ idx, SharedPlan p, int thr) {
-  extern __shared__ uint32_t s_cnt[];                        // a byte per leaf: how many tokens selected it, then its place + 1
-  __shared__ uint32_t s_mask[kMaxShared * 4];
-  __shared__ uint32_t s_taken[128];
-  __shared__ int s_n, s_warp[kPlanThreads / 32];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tpt = 128 / geo.G, tile = blockIdx.x, bh = blockIdx.y, K = geo.K, C = geo.C;
-  const int t0 = tile * tpt, nt = min(tpt, geo.N - t0);
-  const int leaves = (t0 + nt - 1) / C + 1;                  // visible to the tile's last token
-  uint8_t* cnt8 = reinterpret_cast<uint8_t*>(s_cnt);
-  for (int i = tid; i < (leaves + 3) / 4; i += kPlanThreads) s_cnt[i] = 0u;
-  for (int i = tid; i < kMaxShared * 4; i += kPlanThreads) s_mask[i] = 0u;
-  if (tid < 128) s_taken[tid] = 0u;
-  if (tid == 0) s_n = 0;
-  __syncthreads();
-  const int32_t* rows = idx + ((long long)bh * geo.N + t0) * K;
-  for (int e = tid; e < nt * K; e += kPlanThreads) {
-    const int leaf = rows[e];
-    if (leaf >= 0 && leaf <= (t0 + e / K) / C) atomicAdd(&s_cnt[leaf >> 2], 1u << (8 * (leaf & 3)));
-  }
-  __syncthreads();
-  const long long slot0 = ((long long)bh * p.tiles + tile) * p.max_leaves;
-  for (int l0 = 0; l0 < leaves; l0 += kPlanThreads) {
-    const int leaf = l0 + tid;
-    const bool hot = leaf < leaves && (cnt8[leaf] >= thr || (leaf == 0 && cnt8[0] > 0));
-    const unsigned bal = __ballot_sync(0xffffffffu, hot);
-    if (lane == 0) s_warp[warp] = __popc(bal);
-    __syncthreads();
-    int place = s_n;
-    for (int w = 0; w < warp; ++w) place += s_warp[w];
-    place += __popc(bal & ((1u << lane) - 1u));
-    const bool fits = hot && place < p.max_leaves;
-    if (leaf < leaves) cnt8[leaf] = fits ? (uint8_t)(place + 1) : (uint8_t)0;
-    if (fits) p.leaf[slot0 + place] = (uint16_t)leaf;
-    __syncthreads();
-    if (tid == 0)
-      for (int w = 0; w < kPlanThreads / 32; ++w) s_n += s_warp[w];
-    __syncthreads();
-  }
-  for (int e = tid; e < nt * K; e += kPlanThreads) {
-    const int leaf = rows[e], tl = e / K;
-    if (leaf < 0 || leaf > (t0 + tl) / C) continue;
-    const int place = (int)cnt8[leaf] - 1;
-    if (place < 0) continue;
-    atomicOr(&s_mask[place * p.words + (tl >> 5)], 1u << (tl & 31));
-    atomicOr(&s_taken[tl], 1u << (e - tl * K));
-  }
-  __syncthreads();
-  const int n = min(s_n, p.max_leaves);
-  for (int i = tid; i < n * p.words; i += kPlanThreads) p.mask[slot0 * p.words + i] = s_mask[i];
-  if (tid < nt) p.taken[(long long)bh * geo.N + t0 + tid] = s_taken[tid];
-  if (tid == 0) p.count[(long long)bh * p.tiles + tile] = n;
-}
 
 // ------------------------------------------------------------------ attention
 
@@ -172,7 +110,7 @@ shared_attend_kernel(Geometry geo, AttArgs a, const __grid_constant__ CUtensorMa
   uint8_t* sV = sK + NK * TILE;              // [NV]
   __shared__ uint64_t q_full[2], q_empty[2], k_full[NK], k_empty[NK], v_full[NV], v_empty[NV], s_full[kBufs], p_full[kBufs],
       o_full, o_empty, l_full[kRing], l_empty[kRing];
-  __shared__ uint16_t s_leaf[kRing][kMaxShared];
+  __shared__ uint16_t s_leaf[kRing][kSharedMax];
   __shared__ int2 s_item[kRing];             // (work item or -1, its leaves)
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
@@ -224,8 +162,8 @@ shared_attend_kernel(Geometry geo, AttArgs a, const __grid_constant__ CUtensorMa
       const bool more = ok && item < a.n_items;
       int n = 0;
       if (more) {
-        n = min(a.plan.count[item], kMaxShared);
-        const uint16_t* src = a.plan.leaf + (long long)item * a.plan.max_leaves;
+        n = min(a.plan.count[item], kSharedMax);
+        const uint16_t* src = a.plan.node + (long long)item * a.plan.max_nodes;
         for (int i = lane; i < n; i += 32) s_leaf[r][i] = src[i];
       }
       if (lane == 0) {
@@ -442,7 +380,7 @@ shared_attend_kernel(Geometry geo, AttArgs a, const __grid_constant__ CUtensorMa
       const int t = tile * tpt + tl, ny = (e.y + LPS - 1) / LPS;
       const bool live = t < geo.N;
       const uint16_t* list = s_leaf[it % kRing];
-      const uint32_t* masks = a.plan.mask + (long long)e.x * a.plan.max_leaves * MW + (tl >> 5);
+      const uint32_t* masks = a.plan.mask + (long long)e.x * a.plan.max_nodes * MW + (tl >> 5);
       float neg_lse2 = 0.f;
       if (live) neg_lse2 = -a.row_lse[((long long)b * geo.Hq + h * G + head) * geo.N + t] * kLog2e;
       bool ok = true, owes = it > 0;             // owes: the item before this one is still to be read out
@@ -532,9 +470,9 @@ shared_attend_kernel(Geometry geo, AttArgs a, const __grid_constant__ CUtensorMa
 #pragma unroll
       for (int y = 0; y < D / 32; ++y) finite = fmaf(out[(long long)(lane + 32 * y) * stride], 0.f, finite);
       if (!__any_sync(0xffffffffu, finite != finite)) continue;
-      const uint32_t* masks = a.plan.mask + (long long)item * a.plan.max_leaves * a.plan.words + (tl >> 5);
+      const uint32_t* masks = a.plan.mask + (long long)item * a.plan.max_nodes * a.plan.words + (tl >> 5);
       attend_shared_row<D>(a.q + b * geo.qs[0] + t * geo.qs[1] + hq * geo.qs[2], a.k + b * geo.ks[0] + h * geo.ks[2], geo.ks[1],
-                           a.v + b * geo.vs[0] + h * geo.vs[2], geo.vs[1], a.plan.leaf + (long long)item * a.plan.max_leaves,
+                           a.v + b * geo.vs[0] + h * geo.vs[2], geo.vs[1], a.plan.node + (long long)item * a.plan.max_nodes,
                            a.plan.count[item], [&](int i) { return ((masks[i * a.plan.words] >> (tl & 31)) & 1u) != 0u; }, t, C,
                            geo.scale * kLog2e, -a.row_lse[(b * geo.Hq + hq) * geo.N + t] * kLog2e, out, stride);
     }
@@ -554,39 +492,25 @@ int launch_dc(const Geometry& g, const AttArgs& a, const CUtensorMap& tm_q, cons
 
 }  // namespace
 
-bool shared_attend_supported(const Geometry& g, int dtype) {
-  if (dtype != PISA_BF16 || (g.d != 128 && g.d != 64) || (g.C != 64 && g.C != 128)) return false;
-  if (g.G > 16 || (g.G & (g.G - 1)) != 0 || g.K > kMaxK || g.M[1] > kShareMaxLeaves) return false;
-  for (int i = 0; i < 3; ++i)
-    if ((g.qs[i] * 2) % 16 || (g.ks[i] * 2) % 16 || (g.vs[i] * 2) % 16) return false;
-  if (!tma_strides(g.qs) || !tma_strides(g.ks) || !tma_strides(g.vs)) return false;
-  const int tpt = 128 / g.G;
-  if ((long long)g.B * g.Hkv > 65535 || (long long)g.B * g.Hkv * ((g.N + tpt - 1) / tpt) > 0x7fffffffLL) return false;
-  return tma::encoder() != nullptr;
-}
-
-size_t shared_plan_layout(const Geometry& g, char* ws, SharedPlan* p) {
+size_t shared_attend_layout(const Geometry& g, char* ws, SharedPlan* p) {
   const int tpt = 128 / g.G;
   const size_t bh = (size_t)g.B * g.Hkv;
+  p->threshold = share_threshold(g);
+  p->span = g.C;
   p->words = (tpt + 31) / 32;
   p->tiles = (g.N + tpt - 1) / tpt;
-  const int most = g.K * tpt / share_threshold(g) + 1;                   // ... and leaf 0
-  p->max_leaves = most < kMaxShared ? most : kMaxShared;
+  const int most = g.K * tpt / p->threshold + 1;                           // ... and leaf 0
+  p->max_nodes = most < kSharedMax ? most : kSharedMax;
   const size_t tiles = bh * p->tiles;
   size_t o = 0;
   auto take = [&](size_t bytes) { char* r = ws + o; o += align_up(bytes, 256); return r; };
-  p->leaf = (uint16_t*)take(tiles * p->max_leaves * 2);
-  p->mask = (uint32_t*)take(tiles * p->max_leaves * p->words * 4);
+  p->node = (uint16_t*)take(tiles * p->max_nodes * 2);
+  p->mask = (uint32_t*)take(tiles * p->max_nodes * p->words * 4);
+  p->slot = nullptr;
   p->count = (int32_t*)take(tiles * 4);
   p->taken = (uint32_t*)take(bh * g.N * 4);
   p->chain = (int32_t*)take(tiles * 4);
   return o;
-}
-
-int launch_shared_plan(const Geometry& g, const int32_t* idx, const SharedPlan& plan, cudaStream_t s) {
-  const dim3 grid((unsigned)plan.tiles, (unsigned)(g.B * g.Hkv));
-  shared_plan_kernel<<<grid, kPlanThreads, (size_t)((g.M[1] + 3) / 4) * 4, s>>>(g, idx, plan, share_threshold(g));
-  return check_launch("shared_plan");
 }
 
 int launch_shared_attend(const Geometry& g, const void* q, const void* k, const void* v, const float* row_lse, float* o_acc,

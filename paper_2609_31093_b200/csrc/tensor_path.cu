@@ -24,7 +24,7 @@
 
 #include "lse_chunk.cuh"
 #include "pisa_tensor.cuh"
-#include "shared_attend.cuh"
+#include "shared.cuh"
 #include "tc_utils.cuh"
 #include "tma_map.cuh"
 
@@ -1664,15 +1664,30 @@ int tensor_route(const Geometry& g, int dtype, const void* q, const void* k, con
            : route_stage1_mma_supported(g, dtype) ? launch_route_stage1_mma(g, q, pyramid, par, margin, s)
                                                   : launch_route_stage1_simt(g, dtype, q, pyramid, par, margin, s);
   if (st != PISA_OK) return st;
+  // nodes that neighbouring rows share are scored query-major; the plan stands where the indices will (nothing else of the
+  // workspace is free for it)
+  SharedPlan plan;
+  const bool shared = g.score_mode == PISA_SCORE_LSE && shared_supported(g, dtype, g.M[2]) &&
+                      shared_score_layout(g, (char*)idx, &plan) <= (size_t)g.B * g.Hkv * g.N * g.K * 4;
+  if (shared) {
+    kernel_mark("shared_plan_nodes", s);
+    st = launch_shared_plan(g, par, plan, false, s);
+    if (st != PISA_OK) return st;
+  }
   kernel_mark("invert_by_parent", s);
   InvArgs inv;
-  st = run_inversion(g, par, g.g, g.M[2], ws, L.inv, &inv, status, s);
+  st = run_inversion(g, par, g.g, g.M[2], ws, L.inv, &inv, status, s, kWindowTok, shared ? plan.taken : nullptr);
   if (st != PISA_OK) return st;
   TileArgs a = {};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = nullptr;
   a.entry_off = inv.entry_off; a.tile_off = inv.tile_off; a.item_off = inv.item_off; a.item_key = inv.item_key; a.entries = inv.entries;
   a.nkeys = g.B * g.Hkv * inv.NW * g.M[2]; a.Mk = g.M[2]; a.NW = inv.NW; a.fan = g.g; a.slots = g.K;
   a.blk_lse = blk; a.status = status; a.mode = g.score_mode; a.debug = g.debug;
+  if (shared) {
+    kernel_mark("shared_score", s);
+    st = launch_shared_score(g, q, k, blk, plan, inv.work_ctr + 2, status, s);
+    if (st != PISA_OK) return st;
+  }
   kernel_mark("leaf_lse_tiles", s);
   st = dispatch_tile_lse(g, g.g * g.C, a, inv.work_ctr, s);
   if (st != PISA_OK) return st;
@@ -1704,12 +1719,12 @@ int tensor_bsa(const Geometry& g, int dtype, const void* q, const void* k, const
   // to the query-major kernel, which also initialises the accumulator (with other denominators the block-LSE pass below walks
   // lists of everything).  Its plan stands where that pass keeps its scores.
   SharedPlan plan;
-  const bool shared = forced_present && lse_ready && shared_attend_supported(g, dtype) &&
-                      shared_plan_layout(g, (char*)blk, &plan) <= L.acc - L.blk;
+  const bool shared = forced_present && lse_ready && shared_supported(g, dtype, g.M[1]) &&
+                      shared_attend_layout(g, (char*)blk, &plan) <= L.acc - L.blk;
   int st = PISA_OK;
   if (shared) {
     kernel_mark("shared_plan", s);
-    st = launch_shared_plan(g, idx, plan, s);
+    st = launch_shared_plan(g, idx, plan, true, s);
     if (st != PISA_OK) return st;
   }
   kernel_mark("invert_by_leaf", s);
