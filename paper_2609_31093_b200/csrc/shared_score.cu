@@ -4,8 +4,9 @@
 // come by TMA tile loads, 256 keys a step (one node of 256 or two of 128 keys).  S = Q K^T as one chain of N = 256 UMMAs into
 // one of two TMEM accumulators; two groups of eight epilogue warps take alternate steps, a warp 32 rows x 128 columns: the
 // log-sum-exp of its leaf (C = 128) or two leaves (C = 64), written to the place the node has in the token's row.
-// What bounds it: the exponentials (128 x 256 a step: 2048 cycles of the special-function units, less what kPoly moves to the
-// FMA pipe), and the tensor pipe under the power cap (1024).  N = 256 because a chain of N = 128 instructions reads as many
+// What bounds it: the exponentials, 128 x 256 a step = 2048 cycles of the special-function units, 85 % busy (a quarter of them on
+// the FMA pipe: 4.96 ms instead of 4.80 at 65536 tokens, C = 128, 32 heads, half of a tile's tokens making a node shared); the
+// tensor pipe's 1024 come second.  N = 256 because a chain of N = 128 instructions reads as many
 // bytes of shared memory per clock as there are (operand A again for every instruction): 710 cycles instead of 512 a chain
 // measured beside the loads.  The issuer looks at the next step's barriers before the last instructions of this one: it stands
 // still while the pipe works, and the pipe while it does anything else.
@@ -26,10 +27,14 @@ namespace {
 constexpr int kThreads = 640;
 constexpr int kRing = 4;                       // items listed ahead
 constexpr int kKeys = 256;                     // keys of a step
-constexpr int kPoly = 2;                       // of every eight pairs of exponentials, how many take the FMA pipe
 
-// How many of a tile's tokens make a node shared.
-int share_threshold(const Geometry& g) { return (128 / g.G * 3 + 7) / 8; }
+// How many of a tile's tokens make a node shared.  A step takes about 2450 cycles here (256 keys, 128 rows) at an SM clock of
+// 1.7 GHz, in the lists a tile of gathered rows 3700 at 1.9 with nodes of 256 keys and 2840 with nodes of 128 (two of which are a
+// step here).  Plan, inversion and both kernels in ms, lists alone and with 4 / 5 / 6 / 7 eighths of the tokens:
+// 65536 tokens, C = 128, 32 heads: 6.78, 6.28 / 6.17 / 6.11 / 6.22; 32700, C = 64, fan-in 4, 32 heads: 1.72, 1.71 / 1.65 / 1.64 /
+// 1.71; 40000, C = 64, fan-in 2, 16 heads: 0.99, 0.77 / 0.75 / 0.77 / 0.78; 65536, d = 64, 16 heads per group: 1.35, 1.19 / 1.19 /
+// 1.19 / 1.19.
+int share_threshold(const Geometry& g) { return (128 / g.G * (g.g * g.C == kKeys ? 6 : 5) + 7) / 8; }
 
 struct ScoreArgs {
   SharedPlan plan;
@@ -64,8 +69,8 @@ __device__ __forceinline__ void lse_64(const uint32_t (&a)[32], const uint32_t (
     float x0, x1, y0, y1;
     unpack2(fma2(pack2(__uint_as_float(a[j]), __uint_as_float(a[j + 1])), sc, neg), x0, x1);
     unpack2(fma2(pack2(__uint_as_float(b[j]), __uint_as_float(b[j + 1])), sc, neg), y0, y1);
-    s0 = add2(s0, exp_poly_pair(j / 2, kPoly) ? exp2_fma2(x0, x1) : pack2(ex2_approx(x0), ex2_approx(x1)));
-    s1 = add2(s1, exp_poly_pair(j / 2, kPoly) ? exp2_fma2(y0, y1) : pack2(ex2_approx(y0), ex2_approx(y1)));
+    s0 = add2(s0, pack2(ex2_approx(x0), ex2_approx(x1)));
+    s1 = add2(s1, pack2(ex2_approx(y0), ex2_approx(y1)));
   }
   float p0, p1;
   unpack2(add2(s0, s1), p0, p1);

@@ -99,3 +99,31 @@ def test_a_value_that_is_not_finite_reaches_only_rows_that_selected_it(shape):
             assert float((rows - clean[0, :, h * G:(h + 1) * G].float())[~has].abs().max()) <= 2 ** -7 * max(1.0, float(clean.abs().max()))
             after = has & (torch.arange(N, device="cuda") >= (leaf + 1) * C)
             assert not torch.isfinite(rows[after][:, :, ::3]).any()
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "n%d_h%d_%d_d%d_c%d_g%d_k%d" % s)
+def test_leaf_scores_of_shared_and_listed_nodes(shape):
+    """The routing's per-leaf denominators (whichever kernel scored the leaf, in whichever place of the row) against float64:
+    2e-6 relative for ex2.approx and the sums of up to 128 terms, 2^-22 of the logits' size for their fp32 accumulation."""
+    N, Hq, Hkv, d, C, g, K = shape
+    q, k, _ = _tensors(N, Hq, Hkv, d, 91 + N)
+    p = P.Params(1, N, Hq, Hkv, d, C, g, K)
+    pyramid, ws = PB.alloc_pyramid(p), PB.alloc_workspace(p, PB.OP_ROUTE)
+    ws.fill_(0x5a)
+    P.pisa_build_pyramid(p, k, pyramid)
+    idx = torch.full((1, Hkv, N, K), -7, dtype=torch.int32, device="cuda")
+    sel = torch.full((1, Hq, N, K), 7.0, dtype=torch.float32, device="cuda")
+    P.pisa_route(p, q, k, pyramid, idx, None, ws, sel_lse=sel)
+    torch.cuda.synchronize()
+    assert P.read_status(ws) == 0
+    t, G = torch.arange(N, device="cuda"), Hq // Hkv
+    M1 = (N + C - 1) // C
+    for h in range(Hkv):
+        rows = idx[0, h].long()
+        for hq in range(h * G, (h + 1) * G):
+            s = (q[0, :, hq].double() @ k[0, :, h].double().T / math.sqrt(d)).masked_fill(t[None] > t[:, None], -math.inf)
+            s = torch.nn.functional.pad(s, (0, M1 * C - N), value=-math.inf).view(N, M1, C)
+            ref = torch.logsumexp(s, 2).gather(1, rows.clamp(min=0))
+            got = sel[0, hq].double()
+            assert bool((got[rows < 0] == -math.inf).all())
+            assert float((got - ref).abs()[rows >= 0].max()) <= 2e-6 + 2 ** -22 * float(s[s > -math.inf].abs().max())
