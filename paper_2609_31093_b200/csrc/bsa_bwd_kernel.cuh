@@ -1,25 +1,28 @@
 // Backward of the block-sparse attention with the selected indices held fixed (App. B), d = 128 or 64.
 // Included by tensor_path.cu inside its unnamed namespace: it works on the same inverted
-// (key block -> tokens) lists, work items and operand layouts as the forward attention kernel.
+// (key block -> tokens) lists and work items as the forward attention kernel.
 //
-// One CTA per SM, eight warps, no role specialisation: the five products of a tile depend on one
-// another through the element-wise step, so a tile is walked in order
-//   gather Q, dO rows (cp.async)  ->  S = Q K^T,  dP = dO V^T           (two UMMA chains)
-//   P = 2^(S*scale*log2e - lse2),  dS = P o (dP - delta) * scale        (TMEM -> registers -> bf16 in smem)
-//   dV^T += dO^T P,  dK^T += Q^T dS,  dQ^T = K^T dS^T                   (three UMMA chains)
-//   dQ^T -> fp32 accumulator (vector reductions, heads innermost)
-// with dV^T and dK^T ([d lanes] x [C columns] each) staying in TMEM over all the tiles of a work
-// item and added to the fp32 key/value gradient accumulators once per item.  All three gradient
-// products are issued transposed (M = d = 128) so that C = 64 needs no 64-row UMMA shape and every
-// read-out has d along the TMEM lanes: a warp's reduction covers 32 consecutive floats.
-// TMEM: S / dQ^T at columns 0..127 (dQ^T reuses S once P and dS are in shared memory), dP at
-// 128.., dV^T at 256.., dK^T at 384...  delta = rowsum(dO o O) comes from a small kernel of its own.
-// d = 64 runs on the same M = 128 shapes: rows are staged as 128 columns with the upper 64 zero, and only
-// the first 64 TMEM lanes of the gradients are read out (half of the tensor work is padding; the kernel is
-// bound by its gathers and reductions, not by the tensor pipe).
+// A tile is 64 gathered rows (64 / G tokens) against one key block; scores and their gradients are held transposed, a TMEM lane
+// per key, so that P and dS are operands of the key and value gradients where they lie:
+//   S^T = K Q^T,  dP^T = V dO^T                                            (UMMA, 128 x 64)
+//   P = 2^(S*scale*log2e - lse2),  dS = P o (dP - delta) * scale           (TMEM -> bf16: both over S^T in TMEM, dS also to
+//                                                                           shared memory)
+//   dV += P^T dO,  dK += dS^T Q      (A from TMEM; kept there over all tiles of a work item, then added to fp32 in memory)
+//   dQ^T = K^T dS^T                  (-> fp32 accumulator by vector reductions, heads innermost)
+// Warps: 8 gather the Q and dO rows (cp.async, three pairs of tiles in flight), one loads an item's K and V, one draws items and
+// lays out tiles ahead of everybody, one issues the products, 8 do the element-wise step and the dV / dK read-out, 4 reduce dQ.
+// TMEM: dV at columns 0..127, dK at 128.., two buffers of 128 from 256 on: S, over which P and dS are written, and dP, whose
+// columns are free once both are there and take dQ.  The next tile's S and dP go out before this tile's other products, so that
+// its element-wise step runs under them, as do the gathers and the reductions (32 KB a tile, 16 bytes per clock and SM at best).
+// C = 64: the upper 64 key rows are zero (so are their scores and gradients) and never read out; d = 64: the rows are one
+// 64-column slab, and the upper lanes of dQ^T, fed from the neighbouring slab, are not read out.
+// delta = rowsum(dO o O) comes from a small kernel of its own or from the dense way's preparation.
 #pragma once
 
-constexpr int kBwdThreads = 256;
+constexpr int kBwdThreads = 736;
+constexpr int kBwdRows = 64;           // rows of a tile
+constexpr int kBwdStages = 3;          // pairs of Q / dO tiles
+constexpr int kBwdRing = 8;            // tiles the scheduler may run ahead
 
 struct BwdArgs {
   const __nv_bfloat16* q;
@@ -37,6 +40,8 @@ struct BwdArgs {
   float* dq_acc;                  // [B, Hkv, N, D, G] fp32
   float* dk_acc;                  // [B, N, Hkv, D] fp32
   float* dv_acc;
+  int32_t* work_ctr;              // next work item (zero on entry)
+  int kv_tma;                     // keys and values through the tensor maps
   int32_t* status;
   Gate gate;
 };
@@ -72,20 +77,6 @@ __global__ void __launch_bounds__(256) bwd_convert_kernel(const float* __restric
   reinterpret_cast<__nv_bfloat162*>(dst)[row * dst_pitch2 + (i - row * row2)] = __floats2bfloat162_rn(x.x, x.y);
 }
 
-// 256 threads copy `nrows` rows of 256 bytes ([row][128 bf16]) into two swizzled K-major slabs of
-// `slab_bytes` each; src_of(row) returns the row's address or nullptr (zero fill).
-template <int CHV, typename F>                              // CHV: 16-byte chunks a source row really has (d / 8)
-__device__ __forceinline__ void bwd_load_rows(uint8_t* dst, int slab_bytes, int nrows, int p, F src_of) {
-  const int ck = p & 15, rb = p >> 4;                       // 16-byte chunk of the row, first row
-  uint32_t d = smem_u32(dst + (ck >> 3) * slab_bytes) + swz128(rb, ck & 7);
-  for (int row = rb; row < nrows; row += 16) {              // row % 8 is the same for all of a thread's rows
-    const __nv_bfloat16* src = (ck < CHV) ? src_of(row) : nullptr;
-    if (src != nullptr) cp_async16(d, src + ck * 8);
-    else st_shared_zero16(d);
-    d += 16 * 128;
-  }
-}
-
 __device__ __forceinline__ ItemInfo item_info_keys(const int32_t* item_key, const int32_t* item_off,
                                                    const int32_t* entry_off, int item, int tpt) {
   ItemInfo r;
@@ -100,305 +91,419 @@ __device__ __forceinline__ ItemInfo item_info_keys(const int32_t* item_key, cons
   return r;
 }
 
-template <int C, int DIN>
-__global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, BwdArgs a) {
+template <bool V> struct BwdOwn { static constexpr bool value = V; };
+
+template <int C, int D>
+__global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, BwdArgs a, const __grid_constant__ CUtensorMap tm_k,
+                                                                 const __grid_constant__ CUtensorMap tm_v) {
   if (a.gate.off_list()) return;
   extern __shared__ uint8_t smem_raw[];
-  constexpr int D = 128;                                    // staged (padded) head dimension
-  constexpr int CHV = DIN / 8;
-  constexpr int A_SLAB = 128 * 128;                         // one 64-column slab of a 128-row tile
-  constexpr int KV_SLAB = C * 128;
-  constexpr int P_BYTES = (C / 64) * A_SLAB;
+  constexpr int KS = D / 64, CH = D / 8;                    // 64-column slabs, 16-byte chunks of a row
+  constexpr int R_SLAB = kBwdRows * 128, R_TILE = KS * R_SLAB, KV_SLAB = 128 * 128, KV_TILE = KS * KV_SLAB, DS_TILE = 128 * 128;
+  constexpr int NS = kBwdStages, R = kBwdRing;
   uint8_t* smem = align1024(smem_raw);
-  uint8_t* sQ = smem;
-  uint8_t* sdO = sQ + 2 * A_SLAB;
-  uint8_t* sP = sdO + 2 * A_SLAB;
-  uint8_t* sdS = sP + P_BYTES;
-  uint8_t* sK = sdS + P_BYTES;
-  uint8_t* sV = sK + 2 * KV_SLAB;
-  // C = 64 leaves room for a second pair of Q / dO tiles: the next tile is then gathered under the whole
-  // of the current one instead of only under its dQ^T reduction
-  constexpr bool DB = (C == 64);
-  constexpr int NM = DB ? 3 : 2;                            // metadata buffers: tiles jt, jt+1 (and jt+2)
-  uint8_t* sQ1 = sV + 2 * KV_SLAB;
-  uint8_t* sdO1 = sQ1 + 2 * A_SLAB;
-  __shared__ uint64_t bar_mma;
+  uint8_t* sK = smem;
+  uint8_t* sV = sK + KV_TILE;                               // (right behind K: d = 64 reads past K's only slab)
+  uint8_t* sdS = sV + KV_TILE;                              // [2]
+  uint8_t* sQ = sdS + 2 * DS_TILE;                          // [NS]
+  uint8_t* sdO = sQ + NS * R_TILE;                          // [NS]
+  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, s_full[2], e_done[2], dq_full[2], dq_empty[2],
+      acc_full, acc_empty;
+  __shared__ int s_ent[R][kBwdRows];                        // a tile's entries (token | slot << 24, -1 = none)
+  __shared__ int4 s_tkey[R];                                // its (unit, leaf, flags: 1 / 2 = first / last of its item, 4 = own-leaf rows)
+  __shared__ __align__(16) float2 s_stat[NS][kBwdRows];     // per row (-lse * log2 e, -delta); (-inf, 0) where there is no row
+  __shared__ volatile int s_total;                          // number of tiles of this CTA, known once the walk has ended
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
-  __shared__ int s_ent2[NM][128];                           // per-tile metadata
-  __shared__ float s_nlse22[NM][128], s_delta2[NM][128];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    mbar_init(&bar_mma, 1);
+    for (int i = 0; i < R; ++i) { mbar_init(&m_full[i], 1); mbar_init(&m_empty[i], 22); }
+    for (int i = 0; i < NS; ++i) { mbar_init(&qd_full[i], 256); mbar_init(&qd_empty[i], 1); }
+    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&s_full[i], 1); mbar_init(&e_done[i], 8);
+      mbar_init(&dq_full[i], 1); mbar_init(&dq_empty[i], 4);
+    }
+    mbar_init(&acc_full, 1); mbar_init(&acc_empty, 8);
+    s_total = 0x7fffffff;
     s_fail = 0;
     mbar_fence_init();
   }
   if (warp == 0) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
+  if (C == 64)                                              // key rows beyond the block: zero for good
+    for (int i = tid; i < 2 * KS * 64 * 8; i += kBwdThreads) {
+      const int slab = i / (64 * 8), x = i - slab * (64 * 8);
+      st_shared_zero16(smem_u32(sK + slab * KV_SLAB) + 64 * 128 + x * 16);
+    }
+  fence_proxy_async_smem();
   tcgen05_fence_before_sync();
   __syncthreads();
   tcgen05_fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  constexpr uint32_t T_DV = 0u, T_DK = 128u, T_BUF = 256u;         // buffer b at T_BUF + 128 b: S (then P, dS), dP (then dQ) 64 further
 
-  const int G = geo.G, lgG = 31 - __clz(G), tpt = 128 >> lgG;
+  const int G = geo.G, lgG = 31 - __clz(G), tpt = kBwdRows >> lgG;
   const float sl2 = geo.scale * kLog2e;
-  const int n_items = a.item_off[a.nkeys];
-  // descriptors: S/dP chains contract over d (K-major operands); the gradient chains contract over the
-  // tile rows or the keys with both "row-of-memory = contraction index" operands MN-major
-  const uint32_t idesc_s = make_idesc_bf16(128, C, 0, 0);
-  const uint32_t idesc_g = make_idesc_bf16(128, C, 1, 1);     // dV^T = dO^T P, dK^T = Q^T dS
-  const uint32_t idesc_q = make_idesc_bf16(128, 128, 1, 0);   // dQ^T = K^T dS^T
-  uint32_t phase = 0;                                          // completed phases of bar_mma
+  // a tile's ring entry, or false when the walk has ended before it (every role walks the CTA's tiles; bounded as in lse_ws_kernel)
+  auto wait_tile = [&](int it) -> bool {
+    for (uint32_t i = 0; i < (1u << 24); ++i) {
+      if (mbar_try_wait(&m_full[it % R], (uint32_t)((it / R) & 1))) return true;
+      if (it >= s_total || s_fail) return false;
+    }
+    s_fail = 1;
+    return false;
+  };
+  auto done_tile = [&](int it) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&m_empty[it % R]);
+  };
+  // (the loops of all roles are rolled as far as the registers allow: unrolled, their code did not fit the instruction cache --
+  // 62 % hits, and more stalls for instructions than for anything else)
 
-  const int q4r = warp & 3;                                    // TMEM lane quarter of this warp
-  const int row = q4r * 32 + lane;                             // tile row (S, dP) or output column d (gradients)
-  const int chalf = warp >> 2;                                 // which half of the columns this warp takes
-  const uint32_t lane_sel = (uint32_t)(q4r * 32) << 16;
-
-  bool dead = false;
-  for (int item = blockIdx.x; item < n_items && !dead; item += gridDim.x) {
-    const ItemInfo inf = item_info_keys(a.item_key, a.item_off, a.entry_off, item, tpt);
-    const int bh = inf.key / (a.NW * a.Mk), leaf = inf.key % a.Mk;
-    const int b = bh / geo.Hkv, h = bh % geo.Hkv;
-    const __nv_bfloat16* kb = a.k + (long long)b * geo.ks[0] + (long long)h * geo.ks[2];
-    const __nv_bfloat16* vb = a.v + (long long)b * geo.vs[0] + (long long)h * geo.vs[2];
-    bwd_load_rows<CHV>(sK, KV_SLAB, C, tid, [&](int r) {
-      const int t = leaf * C + r;
-      return (t < geo.N) ? kb + (long long)t * geo.ks[1] : (const __nv_bfloat16*)nullptr;
-    });
-    bwd_load_rows<CHV>(sV, KV_SLAB, C, tid, [&](int r) {
-      const int t = leaf * C + r;
-      return (t < geo.N) ? vb + (long long)t * geo.vs[1] : (const __nv_bfloat16*)nullptr;
-    });
-    const __nv_bfloat16* qb = a.q + (long long)b * geo.qs[0] + (long long)(h * G) * geo.qs[2];
-    const __nv_bfloat16* dob = a.dout + (long long)b * geo.os[0] + (long long)(h * G) * geo.os[2];
-    // rows of a tile: entry, -lse*log2e and delta per row (threads 0..127, one row each)
-    auto load_meta = [&](int jt_, int& ent, float& nl, float& dl) {
-      const int e = inf.e_begin + jt_ * tpt + (tid >> lgG);
-      ent = (jt_ < inf.ntiles && e < inf.e_end) ? a.entries[e] : -1;
-      nl = 0.f; dl = 0.f;
-      if (ent >= 0) {
-        if (a.stat != nullptr) {
-          const float2 st = a.stat[(((long long)b * geo.Hkv + h) * geo.N + (ent & 0xFFFFFF)) * G + (tid & (G - 1))];
-          nl = st.x; dl = -st.y;
+  if (warp < 8) {
+    // ------------------------------------------------ gather: a tile's Q and dO rows and their statistics
+    constexpr int RPP = 256 / CH;                           // rows per pass
+    const int ck = tid % CH, rb = tid / CH;
+    for (int it = 0; wait_tile(it); ++it) {
+      const int st = it % NS, mr = it % R;
+      if (it >= NS && !mbar_wait_bounded(&qd_empty[st], (uint32_t)((it / NS - 1) & 1))) { s_fail = 1; break; }
+      const int bh = s_tkey[mr].x, b = bh / geo.Hkv, h = bh % geo.Hkv;
+      const int* ents = s_ent[mr];
+      const __nv_bfloat16* qb = a.q + (long long)b * geo.qs[0] + (long long)(h * G) * geo.qs[2] + ck * 8;
+      const __nv_bfloat16* ob = a.dout + (long long)b * geo.os[0] + (long long)(h * G) * geo.os[2] + ck * 8;
+      const uint32_t off = (uint32_t)(st * R_TILE + (ck >> 3) * R_SLAB);
+      const uint32_t dq0 = smem_u32(sQ) + off, do0 = smem_u32(sdO) + off;
+#pragma unroll 1
+      for (int row = rb; row < kBwdRows; row += RPP) {
+        const int ent = ents[row >> lgG];
+        const uint32_t d = swz128(row, ck & 7);
+        if (ent >= 0) {
+          cp_async16(dq0 + d, qb + (long long)(ent & 0xFFFFFF) * geo.qs[1] + (long long)(row & (G - 1)) * geo.qs[2]);
+          cp_async16(do0 + d, ob + (long long)(ent & 0xFFFFFF) * geo.os[1] + (long long)(row & (G - 1)) * geo.os[2]);
         } else {
-          const long long li = ((long long)b * geo.Hq + h * G + (tid & (G - 1))) * geo.N + (ent & 0xFFFFFF);
-          nl = -a.lse[li] * kLog2e;
-          dl = a.delta[li];
+          st_shared_zero16(dq0 + d);
+          st_shared_zero16(do0 + d);
         }
       }
-    };
-    auto gather_tile = [&](const int* ents, int buf) {
-      bwd_load_rows<CHV>((DB && buf) ? sQ1 : sQ, A_SLAB, 128, tid, [&](int r) {
-        const int ent = ents[r];
-        return (ent >= 0) ? qb + (long long)(ent & 0xFFFFFF) * geo.qs[1] + (long long)(r & (G - 1)) * geo.qs[2]
-                          : (const __nv_bfloat16*)nullptr;
-      });
-      bwd_load_rows<CHV>((DB && buf) ? sdO1 : sdO, A_SLAB, 128, tid, [&](int r) {
-        const int ent = ents[r];
-        return (ent >= 0) ? dob + (long long)(ent & 0xFFFFFF) * geo.os[1] + (long long)(r & (G - 1)) * geo.os[2]
-                          : (const __nv_bfloat16*)nullptr;
-      });
-    };
-    // first tile of the item: metadata and gathers up front; later tiles are fetched while the previous
-    // tile's dQ^T is being reduced
-    if (tid < 128) {
-      int ent; float nl, dl;
-      load_meta(0, ent, nl, dl);
-      s_ent2[0][tid] = ent; s_nlse22[0][tid] = nl; s_delta2[0][tid] = dl;
-      if (DB) {
-        load_meta(1, ent, nl, dl);
-        s_ent2[1][tid] = ent; s_nlse22[1][tid] = nl; s_delta2[1][tid] = dl;
+      if (tid < kBwdRows) {
+        const int ent = ents[tid >> lgG];
+        float2 x = make_float2(-CUDART_INF_F, 0.f);
+        if (ent >= 0) {
+          const int t = ent & 0xFFFFFF, head = tid & (G - 1);
+          if (a.stat != nullptr) {
+            x = a.stat[((long long)bh * geo.N + t) * G + head];
+          } else {
+            const long long li = ((long long)b * geo.Hq + h * G + head) * geo.N + t;
+            x = make_float2(-a.lse[li] * kLog2e, -a.delta[li]);
+          }
+        }
+        s_stat[st][tid] = x;
+      }
+      fence_proxy_async_smem();                             // zero-filled rows (plain stores) -> async proxy
+      cp_async_arrive_noinc(&qd_full[st]);                  // fires when this thread's copies have landed
+      done_tile(it);
+    }
+    cp_async_wait_all();
+  } else if (warp == 8) {
+    // ------------------------------------------------ an item's keys and values
+    int n_item = 0;
+    for (int it = 0; wait_tile(it); ++it) {
+      const int4 key = s_tkey[it % R];
+      if (key.z & 1) {
+        if (n_item >= 1 && !mbar_wait_bounded(&kv_empty, (uint32_t)((n_item - 1) & 1))) { s_fail = 1; break; }
+        ++n_item;
+        const int b = key.x / geo.Hkv, h = key.x % geo.Hkv;
+        if (a.kv_tma) {                                     // (own memory, no multicast; rows past N read as zero)
+          if (lane == 0) {
+            mbar_arrive_expect_tx(&kv_full, (uint32_t)(2 * KS * C * 128));
+            for (int ks = 0; ks < KS; ++ks) {
+              tma_load_4d(smem_u32(sK + ks * KV_SLAB), &tm_k, &kv_full, ks * 64, h, key.y * C, b);
+              tma_load_4d(smem_u32(sV + ks * KV_SLAB), &tm_v, &kv_full, ks * 64, h, key.y * C, b);
+            }
+          }
+        } else {                                            // strides a tensor map cannot hold
+          const int ck = lane % CH;
+          const __nv_bfloat16* kb = a.k + (long long)b * geo.ks[0] + (long long)h * geo.ks[2] + ck * 8;
+          const __nv_bfloat16* vb = a.v + (long long)b * geo.vs[0] + (long long)h * geo.vs[2] + ck * 8;
+          const uint32_t k0 = smem_u32(sK + (ck >> 3) * KV_SLAB), v0 = smem_u32(sV + (ck >> 3) * KV_SLAB);
+#pragma unroll 1
+          for (int row = lane / CH; row < C; row += 32 / CH) {
+            const long long t = (long long)key.y * C + row;
+            const uint32_t d = swz128(row, ck & 7);
+            if (t < geo.N) {
+              cp_async16(k0 + d, kb + t * geo.ks[1]);
+              cp_async16(v0 + d, vb + t * geo.vs[1]);
+            } else {
+              st_shared_zero16(k0 + d);
+              st_shared_zero16(v0 + d);
+            }
+          }
+          cp_async_wait_all();
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&kv_full);
+        }
+      }
+      done_tile(it);
+    }
+  } else if (warp == 9) {
+    // ------------------------------------------------ scheduler: draws work items, lays out their tiles
+    const int n_items = a.item_off[a.nkeys], tpt128 = 128 >> lgG;
+    int it = 0;
+    bool ok = true;
+    while (ok) {
+      int item = 0;
+      if (lane == 0) item = atomicAdd(a.work_ctr, 1);
+      item = __shfl_sync(0xffffffffu, item, 0);
+      if (item >= n_items) break;
+      const ItemInfo inf = item_info_keys(a.item_key, a.item_off, a.entry_off, item, tpt128);
+      const int bh = inf.key / (a.NW * a.Mk), leaf = inf.key % a.Mk;
+      const int e_end = min(inf.e_end, inf.e_begin + inf.ntiles * tpt128), n = (e_end - inf.e_begin + tpt - 1) / tpt;
+      auto fetch = [&](int j, int x) -> int {               // the tile's entry x
+        const int e = inf.e_begin + j * tpt + x;
+        return (j < n && x < tpt && e < e_end) ? a.entries[e] : -1;
+      };
+      int nx0 = fetch(0, lane), nx1 = fetch(0, lane + 32);
+      for (int j = 0; j < n && ok; ++j, ++it) {
+        const int e0 = nx0, e1 = nx1, mr = it % R;
+        nx0 = fetch(j + 1, lane);
+        nx1 = fetch(j + 1, lane + 32);
+        if (it >= R) ok = mbar_wait_bounded(&m_empty[mr], (uint32_t)((it / R - 1) & 1));
+        ok = __all_sync(0xffffffffu, ok && !s_fail);
+        if (!ok) break;
+        s_ent[mr][lane] = e0;
+        s_ent[mr][lane + 32] = e1;
+        const bool own = __any_sync(0xffffffffu, (e0 >= 0 && (e0 & 0xFFFFFF) / C == leaf) || (e1 >= 0 && (e1 & 0xFFFFFF) / C == leaf));
+        if (lane == 0) s_tkey[mr] = make_int4(bh, leaf, (j == 0 ? 1 : 0) | (j == n - 1 ? 2 : 0) | (own ? 4 : 0), 0);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&m_full[mr]);            // release: the ring entry is complete
       }
     }
-    __syncthreads();
-    gather_tile(s_ent2[0], 0);
-    for (int jt = 0; jt < inf.ntiles && !dead; ++jt) {
-      const int cb = jt % NM;                                // this tile's metadata buffer
-      const int nb = (jt + NM - 1) % NM;                     // where the metadata fetched during this tile goes
-      const int qb_i = DB ? (jt & 1) : 0;                    // this tile's Q / dO pair
-      const int* s_ent = s_ent2[cb];
-      const float* s_nlse2 = s_nlse22[cb];
-      const float* s_delta = s_delta2[cb];
-      // metadata of the tile after the one already known: loads issued now, stored once this tile's
-      // products are under way
-      int n_ent = -1; float n_nl = 0.f, n_dl = 0.f;
-      if (tid < 128) load_meta(jt + NM - 1, n_ent, n_nl, n_dl);
-      cp_async_wait_all();
-      fence_proxy_async_smem();
-      __syncthreads();
-      // the other Q / dO pair was last read by the previous tile's products, which have completed
-      if (DB && jt + 1 < inf.ntiles) gather_tile(s_ent2[(jt + 1) % NM], qb_i ^ 1);
-      // ---- S = Q K^T, dP = dO V^T
-      if (tid == 0) {
-        tcgen05_fence_after_sync();
-        const uint32_t q0 = smem_u32(qb_i ? sQ1 : sQ), o0 = smem_u32(qb_i ? sdO1 : sdO), k0 = smem_u32(sK),
-                       v0 = smem_u32(sV);
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t da = make_smem_desc(q0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-          const uint64_t db = make_smem_desc(k0 + (kk >> 2) * KV_SLAB + (kk & 3) * 32, 0, 1024);
-          umma_bf16(tmem, da, db, idesc_s, kk > 0);
-        }
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t da = make_smem_desc(o0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-          const uint64_t db = make_smem_desc(v0 + (kk >> 2) * KV_SLAB + (kk & 3) * 32, 0, 1024);
-          umma_bf16(tmem + 128u, da, db, idesc_s, kk > 0);
-        }
-        umma_commit(&bar_mma);
-      }
-      {
-        const bool ok = mbar_wait_bounded(&bar_mma, phase & 1u);
-        ++phase;
-        if (__syncthreads_or(!ok)) { s_fail = 1; dead = true; break; }
-      }
+    if (!ok) s_fail = 1;
+    if (lane == 0) s_total = it;
+  } else if (warp == 10) {
+    // ------------------------------------------------ UMMA issuer (after a wait that gave up it runs through without waiting)
+    const uint32_t idesc_s = make_idesc_bf16(128, kBwdRows, 0, 0);   // keys x rows, both K-major over d
+    const uint32_t idesc_g = make_idesc_bf16(128, D, 0, 1);          // keys (TMEM) x d, over the rows
+    const uint32_t idesc_q = make_idesc_bf16(128, kBwdRows, 1, 1);   // d x rows, over the keys
+    const uint32_t k0 = desc_lo(smem_u32(sK), 0), v0 = desc_lo(smem_u32(sV), 0), kt0 = desc_lo(smem_u32(sK), KV_SLAB);
+    bool dead = false;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      if (!dead && !mbar_try_wait(bar, parity) && !mbar_wait_bounded(bar, parity)) { dead = true; s_fail = 1; }
+    };
+    int n_item = 0;                                         // items begun
+    // a tile's gradients: dV, dK and dQ^T once its P and dS are there
+    auto gradients = [&](int it, uint32_t flags) {
+      const int st = it % NS, buf = it & 1;
+      if ((flags & 1u) && n_item >= 2) wait(&acc_empty, (uint32_t)((n_item - 2) & 1));
+      wait(&e_done[buf], (uint32_t)((it >> 1) & 1));
       tcgen05_fence_after_sync();
-      // ---- P and dS: this warp's 32 rows x C/2 columns, bf16 into the swizzled [row][key] tiles
-      {
-        const int ent = s_ent[row];
-        int ncols = 0;                                        // visible keys of the block for this row
-        if (ent >= 0) {
-          const int t = ent & 0xFFFFFF, c_t = t / C;
-          if (leaf < c_t) ncols = min(C, geo.N - leaf * C);
-          else if (leaf == c_t) ncols = t - leaf * C + 1;
-        }
-        const float nl2 = (ent >= 0) ? s_nlse2[row] : 0.f;
-        const float dl = (ent >= 0) ? s_delta[row] : 0.f;
+      const uint32_t qm = desc_lo(smem_u32(sQ) + (uint32_t)(st * R_TILE), R_SLAB), om = desc_lo(smem_u32(sdO) + (uint32_t)(st * R_TILE), R_SLAB);
+      const uint32_t s0 = desc_lo(smem_u32(sdS) + (uint32_t)(buf * DS_TILE), DS_TILE), tb = tmem + T_BUF + (uint32_t)(buf * 128);
+      const uint32_t acc = (flags & 1u) ? 0u : 1u;
+      if (elect_one()) {
 #pragma unroll
-        for (int cc = 0; cc < C / 2; cc += 32) {
-          const int c0 = chalf * (C / 2) + cc;
-          uint32_t rs[32], rp[32];
-          tmem_ld_32x32(tmem + lane_sel + (uint32_t)c0, rs);
-          tmem_ld_32x32(tmem + lane_sel + 128u + (uint32_t)c0, rp);
-          tmem_ld_wait();
-          uint32_t pk[16], dk[16];
+        for (int kk = 0; kk < kBwdRows / 16; ++kk)
+          umma_bf16_ts(tmem + T_DV, tb + (uint32_t)(kk * 16), desc64(om + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
 #pragma unroll
-          for (int jx = 0; jx < 16; ++jx) {
-            float p0 = (c0 + 2 * jx < ncols) ? ex2_approx(fmaf(__uint_as_float(rs[2 * jx]), sl2, nl2)) : 0.f;
-            float p1 = (c0 + 2 * jx + 1 < ncols) ? ex2_approx(fmaf(__uint_as_float(rs[2 * jx + 1]), sl2, nl2)) : 0.f;
-            const float d0 = p0 * (__uint_as_float(rp[2 * jx]) - dl) * geo.scale;
-            const float d1 = p1 * (__uint_as_float(rp[2 * jx + 1]) - dl) * geo.scale;
-            const __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
-            const __nv_bfloat162 dd = __floats2bfloat162_rn(d0, d1);
-            pk[jx] = *reinterpret_cast<const uint32_t*>(&pp);
-            dk[jx] = *reinterpret_cast<const uint32_t*>(&dd);
-          }
+        for (int kk = 0; kk < kBwdRows / 16; ++kk)
+          umma_bf16_ts(tmem + T_DK, tb + (uint32_t)(kk * 16 + 8), desc64(qm + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
+        umma_commit(&qd_empty[st]);
+        if (flags & 2u) umma_commit(&acc_full);
 #pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            const int ck = c0 / 8 + q4;
-            const uint32_t off = (uint32_t)((ck >> 3) * A_SLAB) + swz128(row, ck & 7);
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(sP) + off), "r"(pk[4 * q4]),
-                         "r"(pk[4 * q4 + 1]), "r"(pk[4 * q4 + 2]), "r"(pk[4 * q4 + 3])
-                         : "memory");
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(sdS) + off), "r"(dk[4 * q4]),
-                         "r"(dk[4 * q4 + 1]), "r"(dk[4 * q4 + 2]), "r"(dk[4 * q4 + 3])
-                         : "memory");
-          }
-        }
+        for (int kk = 0; kk < C / 16; ++kk)
+          umma_bf16(tb + 64u, desc64(kt0 + kk * (2048 >> 4)), desc64(s0 + kk * (2048 >> 4)), idesc_q, kk > 0);
+        umma_commit(&dq_full[buf]);
+        if (flags & 2u) umma_commit(&kv_empty);
       }
+      __syncwarp();
+    };
+    uint32_t prev = 0u;                                     // flags of the tile before, whose gradients are owed (8: there is one)
+    int it = 0;
+    for (; wait_tile(it); ++it) {
+      const int st = it % NS, buf = it & 1;
+      const uint32_t flags = (uint32_t)__shfl_sync(0xffffffffu, s_tkey[it % R].z, 0);
+      done_tile(it);
+      const bool flush = (flags & 1u) && (prev & 8u);       // the keys of the item before go with its last gradients
+      if (!flush) {
+        if (flags & 1u) { wait(&kv_full, (uint32_t)(n_item & 1)); ++n_item; }
+      } else {
+        gradients(it - 1, prev);
+        prev = 0u;
+        wait(&kv_full, (uint32_t)(n_item & 1));
+        ++n_item;
+      }
+      wait(&qd_full[st], (uint32_t)((it / NS) & 1));
+      if (it >= 2) wait(&dq_empty[buf], (uint32_t)(((it >> 1) - 1) & 1));
       fence_proxy_async_smem();
+      tcgen05_fence_after_sync();
+      const uint32_t q0 = desc_lo(smem_u32(sQ) + (uint32_t)(st * R_TILE), 0), o0 = desc_lo(smem_u32(sdO) + (uint32_t)(st * R_TILE), 0);
+      const uint32_t tb = tmem + T_BUF + (uint32_t)(buf * 128);
+      if (elect_one()) {
+#pragma unroll
+        for (int kk = 0; kk < D / 16; ++kk) {
+          const uint32_t ko = (uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4, ro = (uint32_t)((kk >> 2) * R_SLAB + (kk & 3) * 32) >> 4;
+          umma_bf16(tb, desc64(k0 + ko), desc64(q0 + ro), idesc_s, kk > 0);
+        }
+#pragma unroll
+        for (int kk = 0; kk < D / 16; ++kk) {
+          const uint32_t ko = (uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4, ro = (uint32_t)((kk >> 2) * R_SLAB + (kk & 3) * 32) >> 4;
+          umma_bf16(tb + 64u, desc64(v0 + ko), desc64(o0 + ro), idesc_s, kk > 0);
+        }
+        umma_commit(&s_full[buf]);
+      }
+      __syncwarp();
+      if (prev & 8u) gradients(it - 1, prev);
+      prev = flags | 8u;
+    }
+    if (prev & 8u) gradients(it - 1, prev);
+  } else if (warp >= 11 && warp < 19) {
+    // ------------------------------------------------ element-wise step (lane = key), dV / dK read-out
+    const int quarter = warp & 3, half = (warp - 11) >> 2;            // TMEM lane quarter; half of the tile's rows
+    const int key = quarter * 32 + lane;
+    const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
+    const bool active = quarter * 32 < C;                             // C = 64: the upper lanes stay zero
+    int n_item = 0;
+    for (int it = 0; wait_tile(it); ++it) {
+      const int4 tk = s_tkey[it % R];
+      const float4* stat = reinterpret_cast<const float4*>(s_stat[it % NS] + half * 32);
+      uint8_t* ds = sdS + (it & 1) * DS_TILE;
+      // (s_full says that the rows had landed; their statistics were written by then)
+      if (!mbar_wait_bounded(&qd_full[it % NS], (uint32_t)((it / NS) & 1)) ||
+          !mbar_wait_bounded(&s_full[it & 1], (uint32_t)((it >> 1) & 1))) { s_fail = 1; break; }
+      tcgen05_fence_after_sync();
+      if (active) {
+        // sixteen rows at a time, P and dS over their own columns of S (two bodies: a branch inside would cut the unrolled
+        // chains into blocks that wait for one another, 3000 cycles a tile)
+        auto step = [&](auto own) {
+#pragma unroll 1
+          for (int cc = 0; cc < 2; ++cc) {
+            const uint32_t s_base = tmem + lane_sel + T_BUF + (uint32_t)((it & 1) * 128 + half * 32 + cc * 16);
+            uint32_t rs[16], rp[16], pk[8], dk[8];
+            tmem_ld_32x16(s_base, rs);
+            tmem_ld_32x16(s_base + 64u, rp);
+            tmem_ld_wait();
+#pragma unroll
+            for (int jx = 0; jx < 8; ++jx) {
+              const float4 x = stat[cc * 8 + jx];                     // two rows
+              float p0 = ex2_approx(fmaf(__uint_as_float(rs[2 * jx]), sl2, x.x));
+              float p1 = ex2_approx(fmaf(__uint_as_float(rs[2 * jx + 1]), sl2, x.z));
+              float d0 = p0 * (__uint_as_float(rp[2 * jx]) + x.y) * geo.scale;
+              float d1 = p1 * (__uint_as_float(rp[2 * jx + 1]) + x.w) * geo.scale;
+              if (own.value) {                                        // rows of the block's own leaf see keys up to themselves
+                const int r = half * 32 + cc * 16 + 2 * jx, j = tk.y * C + key;
+                const int e0 = s_ent[it % R][r >> lgG], e1 = s_ent[it % R][(r + 1) >> lgG];
+                const bool off0 = e0 < 0 || j > (e0 & 0xFFFFFF), off1 = e1 < 0 || j > (e1 & 0xFFFFFF);
+                p0 = off0 ? 0.f : p0; d0 = off0 ? 0.f : d0;
+                p1 = off1 ? 0.f : p1; d1 = off1 ? 0.f : d1;
+              }
+              const __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1), dd = __floats2bfloat162_rn(d0, d1);
+              pk[jx] = *reinterpret_cast<const uint32_t*>(&pp);
+              dk[jx] = *reinterpret_cast<const uint32_t*>(&dd);
+            }
+            tmem_st_32x8(s_base, pk);
+            tmem_st_32x8(s_base + 8u, dk);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(ds) + swz128(key, half * 4 + cc * 2 + q)), "r"(dk[4 * q]),
+                           "r"(dk[4 * q + 1]), "r"(dk[4 * q + 2]), "r"(dk[4 * q + 3])
+                           : "memory");
+          }
+        };
+        if (tk.z & 4) step(BwdOwn<true>());
+        else step(BwdOwn<false>());
+        tmem_st_wait();
+        fence_proxy_async_smem();
+      }
       tcgen05_fence_before_sync();
-      __syncthreads();
-      // ---- dV^T += dO^T P,  dK^T += Q^T dS,  dQ^T = K^T dS^T
-      if (tid == 0) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&e_done[it & 1]);
+      done_tile(it);
+      if (tk.z & 2) {
+        // the item's dV (half 0) or dK (half 1): lane = key, TMEM column = d
+        if (!mbar_wait_bounded(&acc_full, (uint32_t)(n_item & 1))) { s_fail = 1; break; }
+        ++n_item;
         tcgen05_fence_after_sync();
-        const uint32_t q0 = smem_u32(qb_i ? sQ1 : sQ), o0 = smem_u32(qb_i ? sdO1 : sdO), k0 = smem_u32(sK);
-        const uint32_t p0 = smem_u32(sP), s0 = smem_u32(sdS);
+        const int b = tk.x / geo.Hkv, h = tk.x % geo.Hkv;
+        const long long t = (long long)tk.y * C + key;
+        float* dst = (half == 0 ? a.dv_acc : a.dk_acc) + (((long long)b * geo.N + t) * geo.Hkv + h) * D;
+        if (active) {
+#pragma unroll 1
+          for (int c0 = 0; c0 < D; c0 += 16) {
+            uint32_t r[16];
+            tmem_ld_32x16(tmem + lane_sel + (half == 0 ? T_DV : T_DK) + (uint32_t)c0, r);
+            tmem_ld_wait();
+            if (t < geo.N)
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {                       // contraction over the 128 tile rows
-          const uint64_t da = make_smem_desc(o0 + kk * 2048, A_SLAB, 1024);
-          const uint64_t db = make_smem_desc(p0 + kk * 2048, A_SLAB, 1024);
-          umma_bf16(tmem + 256u, da, db, idesc_g, (jt > 0) || (kk > 0));
-        }
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t da = make_smem_desc(q0 + kk * 2048, A_SLAB, 1024);
-          const uint64_t db = make_smem_desc(s0 + kk * 2048, A_SLAB, 1024);
-          umma_bf16(tmem + 384u, da, db, idesc_g, (jt > 0) || (kk > 0));
-        }
-#pragma unroll
-        for (int kk = 0; kk < C / 16; ++kk) {                  // contraction over the block's keys
-          const uint64_t da = make_smem_desc(k0 + kk * 2048, KV_SLAB, 1024);
-          const uint64_t db = make_smem_desc(s0 + (kk >> 2) * A_SLAB + (kk & 3) * 32, 0, 1024);
-          umma_bf16(tmem, da, db, idesc_q, kk > 0);
-        }
-        umma_commit(&bar_mma);
-      }
-      {
-        const bool ok = mbar_wait_bounded(&bar_mma, phase & 1u);
-        ++phase;
-        if (__syncthreads_or(!ok)) { s_fail = 1; dead = true; break; }
-      }
-      tcgen05_fence_after_sync();
-      // Q, dO, P, dS tiles are free: (single pair) bring in the next tile while this one's dQ^T is reduced
-      if (tid < 128) { s_ent2[nb][tid] = n_ent; s_nlse22[nb][tid] = n_nl; s_delta2[nb][tid] = n_dl; }
-      __syncthreads();
-      if (!DB && jt + 1 < inf.ntiles) gather_tile(s_ent2[nb], 0);
-      // ---- dQ^T out of TMEM: lane = column d, TMEM column = tile row (entry*G + head); this warp's 64 rows
-      {
-        float* acc_d = a.dq_acc + (((long long)b * geo.Hkv + h) * geo.N) * (long long)(DIN * G) + (long long)row * G;
-        const long long tok_stride = (long long)DIN * G;
-        const bool live = row < DIN;                          // lanes beyond d hold padding
-#pragma unroll
-        for (int cc = 0; cc < 64; cc += 32) {
-          const int c0 = chalf * 64 + cc;
-          uint32_t r[32];
-          tmem_ld_32x32(tmem + lane_sel + (uint32_t)c0, r);
-          tmem_ld_wait();
-          if (G >= 4) {
-#pragma unroll
-            for (int q4 = 0; q4 < 8; ++q4) {
-              const int col = c0 + 4 * q4;
-              const int ent_c = s_ent[col];
-              if (ent_c >= 0 && live) {
-                float* dst = acc_d + (long long)(ent_c & 0xFFFFFF) * tok_stride + (col & (G - 1));
-                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst),
+              for (int q4 = 0; q4 < 4; ++q4)
+                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + c0 + 4 * q4),
                              "f"(__uint_as_float(r[4 * q4])), "f"(__uint_as_float(r[4 * q4 + 1])),
                              "f"(__uint_as_float(r[4 * q4 + 2])), "f"(__uint_as_float(r[4 * q4 + 3]))
                              : "memory");
-              }
+          }
+        }
+        tcgen05_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty);
+      }
+    }
+  } else if (warp >= 19) {
+    // ------------------------------------------------ reducer: dQ^T (lane = column d, TMEM column = tile row) -> fp32 accumulator
+    const int quarter = warp & 3, row = quarter * 32 + lane;
+    const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
+    for (int it = 0; wait_tile(it); ++it) {
+      const int buf = it & 1, bh = s_tkey[it % R].x;
+      const int* ents = s_ent[it % R];
+      float* acc_d = a.dq_acc + (long long)bh * geo.N * (long long)(D * G) + (long long)row * G;
+      const long long tok_stride = (long long)D * G;
+      if (!mbar_wait_bounded(&dq_full[buf], (uint32_t)((it >> 1) & 1))) { s_fail = 1; break; }
+      tcgen05_fence_after_sync();
+      if (quarter * 32 < D) {                               // lanes beyond d hold nothing of use
+#pragma unroll 1
+        for (int c0 = 0; c0 < kBwdRows; c0 += 16) {
+          uint32_t r[16];
+          tmem_ld_32x16(tmem + lane_sel + T_BUF + (uint32_t)(buf * 128 + 64 + c0), r);
+          tmem_ld_wait();
+          if (c0 + 16 == kBwdRows) {
+            tcgen05_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&dq_empty[buf]);
+          }
+          if (G >= 4) {
+#pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4) {
+              const int col = c0 + 4 * q4, ent = ents[col >> lgG];
+              if (ent >= 0)
+                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                                 acc_d + (long long)(ent & 0xFFFFFF) * tok_stride + (col & (G - 1))),
+                             "f"(__uint_as_float(r[4 * q4])), "f"(__uint_as_float(r[4 * q4 + 1])),
+                             "f"(__uint_as_float(r[4 * q4 + 2])), "f"(__uint_as_float(r[4 * q4 + 3]))
+                             : "memory");
+            }
+          } else if (G == 2) {
+#pragma unroll
+            for (int q2 = 0; q2 < 8; ++q2) {
+              const int ent = ents[(c0 + 2 * q2) >> 1];
+              if (ent >= 0)
+                asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(acc_d + (long long)(ent & 0xFFFFFF) * tok_stride),
+                             "f"(__uint_as_float(r[2 * q2])), "f"(__uint_as_float(r[2 * q2 + 1]))
+                             : "memory");
             }
           } else {
 #pragma unroll
-            for (int q1 = 0; q1 < 32; ++q1) {
-              const int col = c0 + q1;
-              const int ent_c = s_ent[col];
-              if (ent_c >= 0 && live)
-                atomicAdd(acc_d + (long long)(ent_c & 0xFFFFFF) * tok_stride + (col & (G - 1)), __uint_as_float(r[q1]));
+            for (int q1 = 0; q1 < 16; ++q1) {
+              const int ent = ents[c0 + q1];
+              if (ent >= 0) atomicAdd(acc_d + (long long)(ent & 0xFFFFFF) * tok_stride, __uint_as_float(r[q1]));
             }
           }
         }
+      } else if (lane == 0) {
+        mbar_arrive(&dq_empty[buf]);
       }
-      tcgen05_fence_before_sync();
-      __syncthreads();                                       // tiles and the S / dQ^T columns are free again
-    }
-    if (dead) break;
-    // ---- the item's dV^T and dK^T: lane = column d, TMEM column = key of the block
-    {
-      tcgen05_fence_after_sync();
-#pragma unroll
-      for (int cc = 0; cc < C / 2; cc += 32) {
-        const int c0 = chalf * (C / 2) + cc;
-        uint32_t rv[32], rk[32];
-        tmem_ld_32x32(tmem + lane_sel + 256u + (uint32_t)c0, rv);
-        tmem_ld_32x32(tmem + lane_sel + 384u + (uint32_t)c0, rk);
-        tmem_ld_wait();
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int t = leaf * C + c0 + j;
-          if (t < geo.N && row < DIN) {
-            const long long o = (((long long)b * geo.N + t) * geo.Hkv + h) * DIN + row;
-            atomicAdd(a.dv_acc + o, __uint_as_float(rv[j]));
-            atomicAdd(a.dk_acc + o, __uint_as_float(rk[j]));
-          }
-        }
-      }
-      tcgen05_fence_before_sync();
-      __syncthreads();                                       // K, V tiles and the accumulators are free again
+      done_tile(it);
     }
   }
-  cp_async_wait_all();                                      // nothing of this CTA's copies may outlive it
   tcgen05_fence_before_sync();
   __syncthreads();
   if (s_fail && tid == 0) atomicExch(a.status, (int)PISA_ERR_TIMEOUT);

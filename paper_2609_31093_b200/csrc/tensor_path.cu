@@ -1624,13 +1624,15 @@ BwdLayout bwd_layout(const Geometry& g) {
 }
 
 template <int C, int DIN>
-int launch_bwd(const Geometry& g, const BwdArgs& a, cudaStream_t s) {
-  // Q, dO (two pairs when C = 64), P, dS, K, V
-  const size_t smem = (C == 64 ? 8 : 4) * (size_t)(128 * 128) + 2 * (size_t)(C / 64) * (128 * 128) +
-                      4 * (size_t)(C * 128) + 1024;
+int launch_bwd(const Geometry& g, BwdArgs a, cudaStream_t s) {
+  // K, V, two dS, pairs of Q and dO
+  const size_t smem = (size_t)(DIN / 64) * 2 * (128 * 128) + 2 * (128 * 128) + (size_t)(DIN / 64) * 2 * kBwdStages * (kBwdRows * 128) + 1024;
   cudaError_t e = cudaFuncSetAttribute(bsa_bwd_kernel<C, DIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) { record_cuda_error("bsa_bwd attr", e); return PISA_ERR_CUDA; }
-  bsa_bwd_kernel<C, DIN><<<num_sms(), kBwdThreads, smem, s>>>(g, a);
+  CUtensorMap tm_k = {}, tm_v = {};
+  a.kv_tma = tma_strides(g.ks) && tma_strides(g.vs) && qm_map_rows(&tm_k, a.k, g.d, g.Hkv, g.N, g.B, g.ks, 1, C) &&
+             qm_map_rows(&tm_v, a.v, g.d, g.Hkv, g.N, g.B, g.vs, 1, C);
+  bsa_bwd_kernel<C, DIN><<<num_sms(), kBwdThreads, smem, s>>>(g, a, tm_k, tm_v);
   return check_launch("bsa_bwd");
 }
 
@@ -1805,6 +1807,7 @@ int tensor_bsa_bwd(const Geometry& g, const void* q, const void* k, const void* 
   a.nkeys = g.B * g.Hkv * inv.NW * g.M[1]; a.Mk = g.M[1]; a.NW = inv.NW;
   a.dq_acc = (float*)(ws + L.dq); a.dk_acc = (float*)(ws + L.dk); a.dv_acc = (float*)(ws + L.dv);
   a.status = status;
+  a.work_ctr = inv.work_ctr;
   kernel_mark("gradient_memset", s);
   a.gate = gate;
   st = launch_zero(ws + L.dq, L.inv.count - L.dq, gate, s);                // dq, dk, dv accumulators are adjacent
