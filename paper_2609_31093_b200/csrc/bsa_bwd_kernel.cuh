@@ -284,80 +284,119 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
     if (lane == 0) s_total = it;
   } else if (warp == 10) {
     // ------------------------------------------------ UMMA issuer (after a wait that gave up it runs through without waiting)
+    // The warp stands still while the pipe works, and the pipe while the warp does anything else: what the next run of
+    // instructions waits for is looked at before the last ones of this run.
     const uint32_t idesc_s = make_idesc_bf16(128, kBwdRows, 0, 0);   // keys x rows, both K-major over d
     const uint32_t idesc_g = make_idesc_bf16(128, D, 0, 1);          // keys (TMEM) x d, over the rows
     const uint32_t idesc_q = make_idesc_bf16(128, kBwdRows, 1, 1);   // d x rows, over the keys
     const uint32_t k0 = desc_lo(smem_u32(sK), 0), v0 = desc_lo(smem_u32(sV), 0), kt0 = desc_lo(smem_u32(sK), KV_SLAB);
+    const uint32_t q_base = desc_lo(smem_u32(sQ), 0), o_base = desc_lo(smem_u32(sdO), 0), ds_base = desc_lo(smem_u32(sdS), DS_TILE);
+    constexpr uint32_t R_LBO = (uint32_t)(R_SLAB >> 4) << 16;        // the row tiles as MN-major operands
+    constexpr int HOLD = 2;                                 // instructions still to go out when the next run is looked at
     bool dead = false;
     auto wait = [&](uint64_t* bar, uint32_t parity) {
       if (!dead && !mbar_try_wait(bar, parity) && !mbar_wait_bounded(bar, parity)) { dead = true; s_fail = 1; }
     };
-    int n_item = 0;                                         // items begun
-    // a tile's gradients: dV, dK and dQ^T once its P and dS are there
-    auto gradients = [&](int it, uint32_t flags) {
-      const int st = it % NS, buf = it & 1;
-      if ((flags & 1u) && n_item >= 2) wait(&acc_empty, (uint32_t)((n_item - 2) & 1));
-      wait(&e_done[buf], (uint32_t)((it >> 1) & 1));
+    int n_item = 0, it = 0;                                 // items begun; the tile whose S and dP are next
+    uint32_t st = 0u, st_ph = 0u, st_prev = 0u;             // its stage and phase; stage of the tile before
+    uint32_t flags = 0u, prev = 0u;                         // its flags; those of the tile before, whose gradients are owed (8: there is one)
+    bool known = false, rows_ready = false, e_ready = false;
+    // gradients of tile it - 1 once its P and dS are there: dQ^T first, so that the reducers have it by the time the tile after
+    // next wants its columns.  look: see to tile it + 1 meanwhile
+    auto gradients = [&](bool look) {
+      const uint32_t buf = (uint32_t)((it - 1) & 1);
+      if ((prev & 1u) && n_item >= 2) wait(&acc_empty, (uint32_t)((n_item - 2) & 1));
+      if (!e_ready) wait(&e_done[buf], (uint32_t)(((it - 1) >> 1) & 1));
+      e_ready = false;
       tcgen05_fence_after_sync();
-      const uint32_t qm = desc_lo(smem_u32(sQ) + (uint32_t)(st * R_TILE), R_SLAB), om = desc_lo(smem_u32(sdO) + (uint32_t)(st * R_TILE), R_SLAB);
-      const uint32_t s0 = desc_lo(smem_u32(sdS) + (uint32_t)(buf * DS_TILE), DS_TILE), tb = tmem + T_BUF + (uint32_t)(buf * 128);
-      const uint32_t acc = (flags & 1u) ? 0u : 1u;
+      const uint32_t off = st_prev * (uint32_t)(R_TILE >> 4);
+      const uint32_t qm = q_base + R_LBO + off, om = o_base + R_LBO + off, s0 = ds_base + buf * (uint32_t)(DS_TILE >> 4);
+      const uint32_t tb = tmem + T_BUF + buf * 128u, acc = (prev & 1u) ? 0u : 1u;
       if (elect_one()) {
-#pragma unroll
-        for (int kk = 0; kk < kBwdRows / 16; ++kk)
-          umma_bf16_ts(tmem + T_DV, tb + (uint32_t)(kk * 16), desc64(om + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
-#pragma unroll
-        for (int kk = 0; kk < kBwdRows / 16; ++kk)
-          umma_bf16_ts(tmem + T_DK, tb + (uint32_t)(kk * 16 + 8), desc64(qm + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
-        umma_commit(&qd_empty[st]);
-        if (flags & 2u) umma_commit(&acc_full);
 #pragma unroll
         for (int kk = 0; kk < C / 16; ++kk)
           umma_bf16(tb + 64u, desc64(kt0 + kk * (2048 >> 4)), desc64(s0 + kk * (2048 >> 4)), idesc_q, kk > 0);
         umma_commit(&dq_full[buf]);
-        if (flags & 2u) umma_commit(&kv_empty);
+#pragma unroll
+        for (int kk = 0; kk < kBwdRows / 16; ++kk)
+          umma_bf16_ts(tmem + T_DV, tb + (uint32_t)(kk * 16), desc64(om + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
+#pragma unroll
+        for (int kk = 0; kk < kBwdRows / 16 - HOLD; ++kk)
+          umma_bf16_ts(tmem + T_DK, tb + (uint32_t)(kk * 16 + 8), desc64(qm + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
+      }
+      __syncwarp();
+      if (look) {
+        const int nx = it + 1;
+        const uint32_t ns = (st + 1u == (uint32_t)NS) ? 0u : st + 1u;
+        const bool m = mbar_test(&m_full[nx % R], (uint32_t)((nx / R) & 1)), r = mbar_test(&qd_full[ns], st_ph ^ (ns == 0u ? 1u : 0u));
+        const uint32_t word = (m ? 256u : 0u) | (r ? 512u : 0u) | (uint32_t)s_tkey[nx % R].z;
+        const uint32_t w0 = __shfl_sync(0xffffffffu, word, 0);
+        known = (w0 & 256u) != 0u;
+        rows_ready = known && (w0 & 512u) != 0u;
+        flags = w0 & 255u;
+      }
+      if (elect_one()) {
+#pragma unroll
+        for (int kk = kBwdRows / 16 - HOLD; kk < kBwdRows / 16; ++kk)
+          umma_bf16_ts(tmem + T_DK, tb + (uint32_t)(kk * 16 + 8), desc64(qm + kk * (2048 >> 4)), idesc_g, kk > 0 ? 1u : acc);
+        umma_commit(&qd_empty[st_prev]);
+        if (prev & 2u) {
+          umma_commit(&acc_full);
+          umma_commit(&kv_empty);
+        }
       }
       __syncwarp();
     };
-    uint32_t prev = 0u;                                     // flags of the tile before, whose gradients are owed (8: there is one)
-    int it = 0;
-    for (; wait_tile(it); ++it) {
-      const int st = it % NS, buf = it & 1;
-      const uint32_t flags = (uint32_t)__shfl_sync(0xffffffffu, s_tkey[it % R].z, 0);
-      done_tile(it);
-      const bool flush = (flags & 1u) && (prev & 8u);       // the keys of the item before go with its last gradients
-      if (!flush) {
-        if (flags & 1u) { wait(&kv_full, (uint32_t)(n_item & 1)); ++n_item; }
-      } else {
-        gradients(it - 1, prev);
-        prev = 0u;
+    for (;; ++it) {
+      if (!known) {
+        if (!wait_tile(it)) break;
+        flags = (uint32_t)__shfl_sync(0xffffffffu, s_tkey[it % R].z, 0);
+      }
+      known = false;
+      if (flags & 1u) {
+        if (prev & 8u) {                                    // the keys of the item before go with its last gradients
+          gradients(false);
+          prev = 0u;
+        }
         wait(&kv_full, (uint32_t)(n_item & 1));
         ++n_item;
       }
-      wait(&qd_full[st], (uint32_t)((it / NS) & 1));
-      if (it >= 2) wait(&dq_empty[buf], (uint32_t)(((it >> 1) - 1) & 1));
+      const uint32_t buf = (uint32_t)(it & 1), own = flags;
+      if (!rows_ready) wait(&qd_full[st], st_ph);
+      rows_ready = false;
       fence_proxy_async_smem();
       tcgen05_fence_after_sync();
-      const uint32_t q0 = desc_lo(smem_u32(sQ) + (uint32_t)(st * R_TILE), 0), o0 = desc_lo(smem_u32(sdO) + (uint32_t)(st * R_TILE), 0);
-      const uint32_t tb = tmem + T_BUF + (uint32_t)(buf * 128);
+      const uint32_t q0 = q_base + st * (uint32_t)(R_TILE >> 4), o0 = o_base + st * (uint32_t)(R_TILE >> 4), tb = tmem + T_BUF + buf * 128u;
+      auto mma_s = [&](int kk, uint32_t d, uint32_t a0, uint32_t b0) {
+        const uint32_t ko = (uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4, ro = (uint32_t)((kk >> 2) * R_SLAB + (kk & 3) * 32) >> 4;
+        umma_bf16(d, desc64(a0 + ko), desc64(b0 + ro), idesc_s, kk > 0);
+      };
       if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t ko = (uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4, ro = (uint32_t)((kk >> 2) * R_SLAB + (kk & 3) * 32) >> 4;
-          umma_bf16(tb, desc64(k0 + ko), desc64(q0 + ro), idesc_s, kk > 0);
-        }
+        for (int kk = 0; kk < D / 16; ++kk) mma_s(kk, tb, k0, q0);
+      }
+      __syncwarp();
+      done_tile(it);
+      if (it >= 2) wait(&dq_empty[buf], (uint32_t)(((it >> 1) - 1) & 1));    // dP goes where the dQ^T of the tile before last was
+      tcgen05_fence_after_sync();
+      if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t ko = (uint32_t)((kk >> 2) * KV_SLAB + (kk & 3) * 32) >> 4, ro = (uint32_t)((kk >> 2) * R_SLAB + (kk & 3) * 32) >> 4;
-          umma_bf16(tb + 64u, desc64(v0 + ko), desc64(o0 + ro), idesc_s, kk > 0);
-        }
+        for (int kk = 0; kk < D / 16 - HOLD; ++kk) mma_s(kk, tb + 64u, v0, o0);
+      }
+      __syncwarp();
+      if (prev & 8u) e_ready = __all_sync(0xffffffffu, mbar_test(&e_done[buf ^ 1u], (uint32_t)(((it - 1) >> 1) & 1)));
+      if (elect_one()) {
+#pragma unroll
+        for (int kk = D / 16 - HOLD; kk < D / 16; ++kk) mma_s(kk, tb + 64u, v0, o0);
         umma_commit(&s_full[buf]);
       }
       __syncwarp();
-      if (prev & 8u) gradients(it - 1, prev);
-      prev = flags | 8u;
+      if (prev & 8u) gradients(true);
+      prev = own | 8u;
+      st_prev = st;
+      if (++st == (uint32_t)NS) { st = 0u; st_ph ^= 1u; }
     }
-    if (prev & 8u) gradients(it - 1, prev);
+    if (prev & 8u) gradients(false);
   } else if (warp >= 11 && warp < 19) {
     // ------------------------------------------------ element-wise step (lane = key), dV / dK read-out
     const int quarter = warp & 3, half = (warp - 11) >> 2;            // TMEM lane quarter; half of the tile's rows
@@ -460,19 +499,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       if (!mbar_wait_bounded(&dq_full[buf], (uint32_t)((it >> 1) & 1))) { s_fail = 1; break; }
       tcgen05_fence_after_sync();
       if (quarter * 32 < D) {                               // lanes beyond d hold nothing of use
-#pragma unroll 1
-        for (int c0 = 0; c0 < kBwdRows; c0 += 16) {
-          uint32_t r[16];
-          tmem_ld_32x16(tmem + lane_sel + T_BUF + (uint32_t)(buf * 128 + 64 + c0), r);
-          tmem_ld_wait();
-          if (c0 + 16 == kBwdRows) {
-            tcgen05_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&dq_empty[buf]);
-          }
+        uint32_t ra[32], rb[32];                            // all of them at once: dP of the tile after next waits for the columns
+        tmem_ld_32x32(tmem + lane_sel + T_BUF + (uint32_t)(buf * 128 + 64), ra);
+        tmem_ld_32x32(tmem + lane_sel + T_BUF + (uint32_t)(buf * 128 + 96), rb);
+        tmem_ld_wait();
+        tcgen05_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&dq_empty[buf]);
+        auto add = [&](const uint32_t (&r)[32], int c0) {
           if (G >= 4) {
 #pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
+            for (int q4 = 0; q4 < 8; ++q4) {
               const int col = c0 + 4 * q4, ent = ents[col >> lgG];
               if (ent >= 0)
                 asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
@@ -483,7 +520,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
             }
           } else if (G == 2) {
 #pragma unroll
-            for (int q2 = 0; q2 < 8; ++q2) {
+            for (int q2 = 0; q2 < 16; ++q2) {
               const int ent = ents[(c0 + 2 * q2) >> 1];
               if (ent >= 0)
                 asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(acc_d + (long long)(ent & 0xFFFFFF) * tok_stride),
@@ -492,12 +529,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
             }
           } else {
 #pragma unroll
-            for (int q1 = 0; q1 < 16; ++q1) {
+            for (int q1 = 0; q1 < 32; ++q1) {
               const int ent = ents[c0 + q1];
               if (ent >= 0) atomicAdd(acc_d + (long long)(ent & 0xFFFFFF) * tok_stride, __uint_as_float(r[q1]));
             }
           }
-        }
+        };
+        add(ra, 0);
+        add(rb, 32);
       } else if (lane == 0) {
         mbar_arrive(&dq_empty[buf]);
       }
