@@ -495,7 +495,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       const int buf = it & 1, bh = s_tkey[it % R].x;
       const int* ents = s_ent[it % R];
       float* acc_d = a.dq_acc + (long long)bh * geo.N * (long long)(D * G) + (long long)row * G;
-      const long long tok_stride = (long long)D * G;
+      const uint32_t tok_bytes = (uint32_t)(D * G * 4);
+      auto at = [&](int ent) -> float* { return reinterpret_cast<float*>(reinterpret_cast<char*>(acc_d) + (uint64_t)(uint32_t)(ent & 0xFFFFFF) * tok_bytes); };
       if (!mbar_wait_bounded(&dq_full[buf], (uint32_t)((it >> 1) & 1))) { s_fail = 1; break; }
       tcgen05_fence_after_sync();
       if (quarter * 32 < D) {                               // lanes beyond d hold nothing of use
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
               const int col = c0 + 4 * q4, ent = ents[col >> lgG];
               if (ent >= 0)
                 asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
-                                 acc_d + (long long)(ent & 0xFFFFFF) * tok_stride + (col & (G - 1))),
+                                 at(ent) + (col & (G - 1))),
                              "f"(__uint_as_float(r[4 * q4])), "f"(__uint_as_float(r[4 * q4 + 1])),
                              "f"(__uint_as_float(r[4 * q4 + 2])), "f"(__uint_as_float(r[4 * q4 + 3]))
                              : "memory");
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
             for (int q2 = 0; q2 < 16; ++q2) {
               const int ent = ents[(c0 + 2 * q2) >> 1];
               if (ent >= 0)
-                asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(acc_d + (long long)(ent & 0xFFFFFF) * tok_stride),
+                asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(at(ent)),
                              "f"(__uint_as_float(r[2 * q2])), "f"(__uint_as_float(r[2 * q2 + 1]))
                              : "memory");
             }
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
 #pragma unroll
             for (int q1 = 0; q1 < 32; ++q1) {
               const int ent = ents[c0 + q1];
-              if (ent >= 0) atomicAdd(acc_d + (long long)(ent & 0xFFFFFF) * tok_stride, __uint_as_float(r[q1]));
+              if (ent >= 0) atomicAdd(at(ent), __uint_as_float(r[q1]));
             }
           }
         };
