@@ -496,7 +496,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       const int* ents = s_ent[it % R];
       float* acc_d = a.dq_acc + (long long)bh * geo.N * (long long)(D * G) + (long long)row * G;
       const uint32_t tok_bytes = (uint32_t)(D * G * 4);
-      auto at = [&](int ent) -> float* { return reinterpret_cast<float*>(reinterpret_cast<char*>(acc_d) + (uint64_t)(uint32_t)(ent & 0xFFFFFF) * tok_bytes); };
       if (!mbar_wait_bounded(&dq_full[buf], (uint32_t)((it >> 1) & 1))) { s_fail = 1; break; }
       tcgen05_fence_after_sync();
       if (quarter * 32 < D) {                               // lanes beyond d hold nothing of use
@@ -507,37 +506,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
         tcgen05_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&dq_empty[buf]);
-        auto add = [&](const uint32_t (&r)[32], int c0) {
-          if (G >= 4) {
-#pragma unroll
-            for (int q4 = 0; q4 < 8; ++q4) {
-              const int col = c0 + 4 * q4, ent = ents[col >> lgG];
-              if (ent >= 0)
-                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
-                                 at(ent) + (col & (G - 1))),
-                             "f"(__uint_as_float(r[4 * q4])), "f"(__uint_as_float(r[4 * q4 + 1])),
-                             "f"(__uint_as_float(r[4 * q4 + 2])), "f"(__uint_as_float(r[4 * q4 + 3]))
-                             : "memory");
-            }
-          } else if (G == 2) {
-#pragma unroll
-            for (int q2 = 0; q2 < 16; ++q2) {
-              const int ent = ents[(c0 + 2 * q2) >> 1];
-              if (ent >= 0)
-                asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(at(ent)),
-                             "f"(__uint_as_float(r[2 * q2])), "f"(__uint_as_float(r[2 * q2 + 1]))
-                             : "memory");
-            }
-          } else {
-#pragma unroll
-            for (int q1 = 0; q1 < 32; ++q1) {
-              const int ent = ents[c0 + q1];
-              if (ent >= 0) atomicAdd(at(ent), __uint_as_float(r[q1]));
-            }
-          }
+        auto at = [&](int r, int cols) -> float* {
+          const int ent = ents[r >> lgG];
+          return ent >= 0 ? reinterpret_cast<float*>(reinterpret_cast<char*>(acc_d) + (uint64_t)(uint32_t)(ent & 0xFFFFFF) * tok_bytes) + cols * G
+                          : nullptr;
         };
-        add(ra, 0);
-        add(rb, 32);
+        reduce_columns(ra, G, lane, at);
+        reduce_columns(rb, G, lane, [&](int r, int cols) { return at(32 + r, cols); });
       } else if (lane == 0) {
         mbar_arrive(&dq_empty[buf]);
       }
