@@ -52,15 +52,16 @@ Split uniform_split(const Geometry& g) {
 }
 size_t table_bytes(size_t n) { return align_up(n * sizeof(qm::Seq), 256) + align_up(n * sizeof(qm::SeqOrder), 256); }
 
-// Steps (128-row tile x 128 keys) per tile and selected block up to which the dense kernels win, in eighths.  Measured SM
-// cycles: a dense step 7.2 K (d = 64) to 8.1 K, 8.7 K beyond L2; an entry of the lists 13.1 K (C = 128), 14 to 18 K (C = 64),
-// more without groups, where every entry of a tile is a row of its own to gather.  Where the queries, dout, keys and values are
-// about twice L2 the line lies lower: 20000 tokens, 32 heads, fan-in 4 dense 4.31 ms, lists 4.08, but 16 heads 2.05 and 2.40;
-// 16 heads without groups 14000 tokens (229 MB) 2.26 and 2.54, 16000 (262 MB) 2.82 and 2.58, 2 x 14000 4.77 and 4.06.
+// Steps (128-row tile x 128 keys) per tile and selected block up to which the dense kernels win, in eighths: a dense step takes
+// 7.2 K (d = 64) to 8.1 K SM cycles, 128 rows of the lists 7 to 7.5 K and 0.15 ms of preparation, inversion and conversions at
+// 6000 tokens.  Whole calls in us, dense / lists (steps per tile and block in parentheses): 16 heads, G = 4, C = 64, K = 16: 3000
+// tokens 213 / 291, 6000 483 / 471 (1.1), 12288 1097 / 879 (1.35); 32 heads, fan-in 4: 6000 891 / 836; C = 128, K = 32, 32 heads:
+// 6000 1135 / 1143 (0.7), 12288 3961 / 2617 (1.25); 16 heads without groups: 6000 570 / 801, 12288 1749 / 1485 (2.2); 16 heads
+// per group, d = 64, K = 8: 16384 919 / 1172, 32768 1943 / 2233 (1.0).
 int steps_per_block8(const Geometry& g) {
-  const bool large = (long long)g.B * g.N * (g.Hq + g.Hkv) * g.d * 4 > (230LL << 20);
-  if (g.G == 1) return g.C == 128 ? (large ? 15 : 19) : (large ? 20 : 24);
-  return g.C == 128 ? (large ? 11 : 12) : (large ? 14 : 15);
+  if (g.G == 1) return g.C == 128 ? 9 : 13;
+  if (g.G == 16) return g.C == 128 ? 8 : 10;
+  return g.C == 128 ? 6 : 8;
 }
 
 }  // namespace
