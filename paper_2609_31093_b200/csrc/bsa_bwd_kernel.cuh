@@ -17,6 +17,9 @@
 // C = 64: the upper 64 key rows are zero (so are their scores and gradients) and never read out; d = 64: the rows are one
 // 64-column slab, and the upper lanes of dQ^T, fed from the neighbouring slab, are not read out.
 // delta = rowsum(dO o O) comes from a small kernel of its own or from the dense way's preparation.
+// What is not finite reaches only what it belongs to: where a row sees a part of its own block only, the products multiply the
+// rest by zero.  So keys that are not finite count as zero and their scores as NaN, and so do, in tiles with rows of the block's
+// own leaf, rows whose denominator or delta shows that they are not finite.
 #pragma once
 
 constexpr int kBwdThreads = 736;
@@ -107,11 +110,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
   uint8_t* sdS = sV + KV_TILE;                              // [2]
   uint8_t* sQ = sdS + 2 * DS_TILE;                          // [NS]
   uint8_t* sdO = sQ + NS * R_TILE;                          // [NS]
-  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, s_full[2], e_done[2], dq_full[2], dq_empty[2],
+  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, k_seen, s_full[2], e_done[2], dq_full[2], dq_empty[2],
       acc_full, acc_empty;
   __shared__ int s_ent[R][kBwdRows];                        // a tile's entries (token | slot << 24, -1 = none)
   __shared__ int4 s_tkey[R];                                // its (unit, leaf, flags: 1 / 2 = first / last of its item, 4 = own-leaf rows)
   __shared__ __align__(16) float2 s_stat[NS][kBwdRows];     // per row (-lse * log2 e, -delta); (-inf, 0) where there is no row
+  __shared__ float s_kscale[128];                           // per key scale * log2 e, NaN where the key is not finite
   __shared__ volatile int s_total;                          // number of tiles of this CTA, known once the walk has ended
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
@@ -120,7 +124,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
   if (tid == 0) {
     for (int i = 0; i < R; ++i) { mbar_init(&m_full[i], 1); mbar_init(&m_empty[i], 22); }
     for (int i = 0; i < NS; ++i) { mbar_init(&qd_full[i], 256); mbar_init(&qd_empty[i], 1); }
-    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1);
+    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1); mbar_init(&k_seen, C / 32);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1); mbar_init(&e_done[i], 8);
       mbar_init(&dq_full[i], 1); mbar_init(&dq_empty[i], 4);
@@ -358,12 +362,29 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
           gradients(false);
           prev = 0u;
         }
-        wait(&kv_full, (uint32_t)(n_item & 1));
+        wait(&k_seen, (uint32_t)(n_item & 1));
         ++n_item;
       }
       const uint32_t buf = (uint32_t)(it & 1), own = flags;
       if (!rows_ready) wait(&qd_full[st], st_ph);
       rows_ready = false;
+      if (own & 4u) {                                       // rows that are not finite (see the head of this file)
+#pragma unroll 1
+        for (int r0 = 0; r0 < kBwdRows; r0 += 32) {
+          const float2 x = s_stat[st][r0 + lane];
+          const bool bad = !(fabsf(x.y) < CUDART_INF_F) || !(x.x < CUDART_INF_F);
+          if (bad) s_stat[st][r0 + lane].x = CUDART_NAN_F;
+          for (unsigned m = __ballot_sync(0xffffffffu, bad); m != 0u; m &= m - 1u) {
+            const int row = r0 + __ffs(m) - 1;
+            if (lane < KS * 8) {
+              const uint32_t d = st * (uint32_t)R_TILE + (uint32_t)((lane >> 3) * R_SLAB) + swz128(row, lane & 7);
+              st_shared_zero16(smem_u32(sQ) + d);
+              st_shared_zero16(smem_u32(sdO) + d);
+            }
+          }
+        }
+        __syncwarp();
+      }
       fence_proxy_async_smem();
       tcgen05_fence_after_sync();
       const uint32_t q0 = q_base + st * (uint32_t)(R_TILE >> 4), o0 = o_base + st * (uint32_t)(R_TILE >> 4), tb = tmem + T_BUF + buf * 128u;
@@ -408,6 +429,28 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       const int4 tk = s_tkey[it % R];
       const float4* stat = reinterpret_cast<const float4*>(s_stat[it % NS] + half * 32);
       uint8_t* ds = sdS + (it & 1) * DS_TILE;
+      if ((tk.z & 1) && half == 0 && active) {
+        // the item's keys: one that is not finite counts as zero (see the head of this file)
+        if (!mbar_wait_bounded(&kv_full, (uint32_t)(n_item & 1))) { s_fail = 1; break; }
+        const uint32_t k_row = smem_u32(sK);
+        float f = 0.f;
+#pragma unroll 1
+        for (int ck = 0; ck < CH; ++ck) {
+          const uint32_t d = k_row + (uint32_t)((ck >> 3) * KV_SLAB) + swz128(key, ck & 7);
+          uint32_t w[4];
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(d));
+#pragma unroll
+          for (int x = 0; x < 4; ++x) f = fmaf(__uint_as_float(w[x] << 16), 0.f, fmaf(__uint_as_float(w[x] & 0xFFFF0000u), 0.f, f));
+        }
+        if (f != 0.f) {                                               // (0 or NaN)
+#pragma unroll 1
+          for (int ck = 0; ck < CH; ++ck) st_shared_zero16(k_row + (uint32_t)((ck >> 3) * KV_SLAB) + swz128(key, ck & 7));
+        }
+        s_kscale[key] = f != 0.f ? CUDART_NAN_F : sl2;
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&k_seen);
+      }
       // (s_full says that the rows had landed; their statistics were written by then)
       if (!mbar_wait_bounded(&qd_full[it % NS], (uint32_t)((it / NS) & 1)) ||
           !mbar_wait_bounded(&s_full[it & 1], (uint32_t)((it >> 1) & 1))) { s_fail = 1; break; }
@@ -415,6 +458,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       if (active) {
         // sixteen rows at a time, P and dS over their own columns of S (two bodies: a branch inside would cut the unrolled
         // chains into blocks that wait for one another, 3000 cycles a tile)
+        const float ks = s_kscale[key];
         auto step = [&](auto own) {
 #pragma unroll 1
           for (int cc = 0; cc < 2; ++cc) {
@@ -426,8 +470,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
 #pragma unroll
             for (int jx = 0; jx < 8; ++jx) {
               const float4 x = stat[cc * 8 + jx];                     // two rows
-              float p0 = ex2_approx(fmaf(__uint_as_float(rs[2 * jx]), sl2, x.x));
-              float p1 = ex2_approx(fmaf(__uint_as_float(rs[2 * jx + 1]), sl2, x.z));
+              float p0 = ex2_approx(fmaf(__uint_as_float(rs[2 * jx]), ks, x.x));
+              float p1 = ex2_approx(fmaf(__uint_as_float(rs[2 * jx + 1]), ks, x.z));
               float d0 = p0 * (__uint_as_float(rp[2 * jx]) + x.y) * geo.scale;
               float d1 = p1 * (__uint_as_float(rp[2 * jx + 1]) + x.w) * geo.scale;
               if (own.value) {                                        // rows of the block's own leaf see keys up to themselves
