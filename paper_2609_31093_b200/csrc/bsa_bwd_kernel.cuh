@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
         const int nx = it + 1;
         const uint32_t ns = (st + 1u == (uint32_t)NS) ? 0u : st + 1u;
         const bool m = mbar_test(&m_full[nx % R], (uint32_t)((nx / R) & 1)), r = mbar_test(&qd_full[ns], st_ph ^ (ns == 0u ? 1u : 0u));
-        const uint32_t word = (m ? 256u : 0u) | (r ? 512u : 0u) | (uint32_t)s_tkey[nx % R].z;
+        const uint32_t word = (m ? 256u : 0u) | (r ? 512u : 0u) | ((uint32_t)s_tkey[nx % R].z & 7u);   // (no such tile yet: whatever stands there)
         const uint32_t w0 = __shfl_sync(0xffffffffu, word, 0);
         known = (w0 & 256u) != 0u;
         rows_ready = known && (w0 & 512u) != 0u;
