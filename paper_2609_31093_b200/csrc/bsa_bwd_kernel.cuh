@@ -96,7 +96,7 @@ __device__ __forceinline__ ItemInfo item_info_keys(const int32_t* item_key, cons
 
 template <bool V> struct BwdOwn { static constexpr bool value = V; };
 
-template <int C, int D>
+template <int C, int D, bool WIDE>
 __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, BwdArgs a, const __grid_constant__ CUtensorMap tm_k,
                                                                  const __grid_constant__ CUtensorMap tm_v) {
   if (a.gate.off_list()) return;
@@ -550,13 +550,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
         tcgen05_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&dq_empty[buf]);
-        auto at = [&](int r, int cols) -> float* {
-          const int ent = ents[r >> lgG];
-          return ent >= 0 ? reinterpret_cast<float*>(reinterpret_cast<char*>(acc_d) + (uint64_t)(uint32_t)(ent & 0xFFFFFF) * tok_bytes) + cols * G
-                          : nullptr;
-        };
-        reduce_columns(ra, G, lane, at);
-        reduce_columns(rb, G, lane, [&](int r, int cols) { return at(32 + r, cols); });
+        auto at = [&](int e) { return reinterpret_cast<float*>(reinterpret_cast<char*>(acc_d) + (uint64_t)(uint32_t)(e & 0xFFFFFF) * tok_bytes); };
+        reduce_columns<WIDE>(ra, G, lane, [&](int r) { return ents[r >> lgG]; }, at);
+        reduce_columns<WIDE>(rb, G, lane, [&](int r) { return ents[(32 + r) >> lgG]; }, at);
       } else if (lane == 0) {
         mbar_arrive(&dq_empty[buf]);
       }

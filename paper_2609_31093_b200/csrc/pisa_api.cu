@@ -1293,7 +1293,7 @@ int pisa_bsa_bwd_packed(const pisa_params_t* p, const int32_t* cu_seqlens, int32
     pi.N = len;
     Geometry gi;
     if ((st = resolve(&pi, &gi)) != PISA_OK) return st;
-    if (!qm_bwd_supported(gi, p->dtype) || len > qm_bwd_always(gi) || kStatusBytes + qm_bwd_packed_bytes(gi, len) > ws_bytes) continue;
+    if (!qm_bwd_supported(gi, p->dtype) || len > qm_bwd_packed_longest(gi) || kStatusBytes + qm_bwd_packed_bytes(gi, len) > ws_bytes) continue;
     taken[i] = 1;
     ids[n_dense++] = i;
   }

@@ -66,6 +66,7 @@ int qm_bwd(const Geometry& g, const void* q, const void* k, const void* v, const
            const void* dout, void* dq, void* dk, void* dv, void* ws, int32_t* status, Gate* gate, const float2** stat, cudaStream_t s);
 // length up to which the dense backward is the better one whatever the rows selected
 int qm_bwd_always(const Geometry& g);
+int qm_bwd_packed_longest(const Geometry& g);
 // packed batches: workspace one sequence needs, and the backward of the sequences ids[0..n)
 size_t qm_bwd_packed_bytes(const Geometry& g, int len);
 int qm_bwd_packed(const Geometry& g, const int32_t* cu, const int* ids, int n, long long total, const void* q, const void* k,

@@ -317,23 +317,24 @@ __device__ __forceinline__ void red_add_v4(float* dst, uint32_t x, uint32_t y, u
 }
 // Reductions of 32 TMEM columns (tile rows) by one warp whose lanes are output columns, into an accumulator whose G heads of a
 // column are adjacent.  An SM hands about one lane's request per clock to L2 whatever its size, so that requests are made 16
-// bytes wide: with fewer than four heads neighbouring lanes exchange columns (scalar adds without groups took 2.2 times as
-// long: attention of 40000 tokens, 16 KV heads).  at(r): accumulator of tile row r's token, at this lane's column; null: no row.
-template <typename AT>
-__device__ __forceinline__ void reduce_columns(const uint32_t (&r)[32], int G, int lane, AT at) {
-  if (G >= 4) {
+// bytes wide: with fewer than four heads (WIDE = false) neighbouring lanes exchange columns.  (Scalar adds without groups: 1.5
+// instead of 1.1 ms for the listed leaves of 40000 tokens, 16 KV heads; their backward 4.5 instead of 3.7 ms.)
+// ent(r): list entry of tile row r, negative: no row; at(e): accumulator of the entry's token, at this lane's column.
+template <bool WIDE, typename ENT, typename AT>
+__device__ __forceinline__ void reduce_columns(const uint32_t (&r)[32], int G, int lane, ENT ent, AT at) {
+  if (WIDE) {
 #pragma unroll
     for (int q4 = 0; q4 < 8; ++q4) {
-      float* dst = at(4 * q4, 0);
-      if (dst != nullptr) red_add_v4(dst + ((4 * q4) & (G - 1)), r[4 * q4], r[4 * q4 + 1], r[4 * q4 + 2], r[4 * q4 + 3]);
+      const int e = ent(4 * q4);
+      if (e >= 0) red_add_v4(at(e) + ((4 * q4) & (G - 1)), r[4 * q4], r[4 * q4 + 1], r[4 * q4 + 2], r[4 * q4 + 3]);
     }
   } else if (G == 2) {
     const bool up = (lane & 1) != 0;                        // the odd lane takes the second of two tokens, both columns
 #pragma unroll
     for (int i = 0; i < 32; i += 4) {
       const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? r[i] : r[i + 2], 1), g1 = __shfl_xor_sync(0xffffffffu, up ? r[i + 1] : r[i + 3], 1);
-      float* dst = at(i + (up ? 2 : 0), up ? -1 : 0);
-      if (dst != nullptr) red_add_v4(dst, up ? g0 : r[i], up ? g1 : r[i + 1], up ? r[i + 2] : g0, up ? r[i + 3] : g1);
+      const int e = ent(i + (up ? 2 : 0));
+      if (e >= 0) red_add_v4(at(e) - (lane & 1) * 2, up ? g0 : r[i], up ? g1 : r[i + 1], up ? r[i + 2] : g0, up ? r[i + 3] : g1);
     }
   } else {
     const bool u1 = (lane & 1) != 0, u2 = (lane & 2) != 0;  // lane l takes the (l mod 4)-th of four tokens, four columns
@@ -342,8 +343,8 @@ __device__ __forceinline__ void reduce_columns(const uint32_t (&r)[32], int G, i
       const uint32_t g0 = __shfl_xor_sync(0xffffffffu, u1 ? r[i] : r[i + 1], 1), g1 = __shfl_xor_sync(0xffffffffu, u1 ? r[i + 2] : r[i + 3], 1);
       const uint32_t n0 = u1 ? g0 : r[i], n1 = u1 ? r[i + 1] : g0, n2 = u1 ? g1 : r[i + 2], n3 = u1 ? r[i + 3] : g1;
       const uint32_t h0 = __shfl_xor_sync(0xffffffffu, u2 ? n0 : n2, 2), h1 = __shfl_xor_sync(0xffffffffu, u2 ? n1 : n3, 2);
-      float* dst = at(i + (lane & 3), -(lane & 3));
-      if (dst != nullptr) red_add_v4(dst, u2 ? h0 : n0, u2 ? h1 : n1, u2 ? n2 : h0, u2 ? n3 : h1);
+      const int e = ent(i + (lane & 3));
+      if (e >= 0) red_add_v4(at(e) - (lane & 3), u2 ? h0 : n0, u2 ? h1 : n1, u2 ? n2 : h0, u2 ? n3 : h1);
     }
   }
 }
@@ -810,7 +811,8 @@ lse_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant
 // per tile), so it gets warps of its own and is never stalled by the exponentials.
 constexpr int kPvThreads = 544;
 
-template <int D, int C>
+// WIDE: groups of four heads or more (what the reducer does with fewer would not fit its registers)
+template <int D, int C, bool WIDE>
 __global__ void __launch_bounds__(kPvThreads, 1)
 pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v) {
@@ -1084,7 +1086,7 @@ pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant_
           // lane = output column d (= `row` of this thread), TMEM column = tile row = entry*G + head
           const int* ents = s_ent[it % kMetaRing];
           float* acc_d = a.o_acc + (((long long)b * geo.Hkv + h) * geo.N) * (long long)(D * G) + (long long)row * G;
-          const long long tok_stride = (long long)D * G;
+          const uint32_t tok_bytes = (uint32_t)(D * G * 4);
           uint32_t ra[32], rb[32];
           tmem_ld_32x32(o_base, ra);
 #pragma unroll
@@ -1098,10 +1100,8 @@ pv_ws_kernel(Geometry geo, TileArgs a, int32_t* work_ctr, const __grid_constant_
               tcgen05_fence_before_sync();
               mbar_arrive(&o_empty[ob]);          // O has been read out of TMEM
             }
-            reduce_columns(cur, G, lane, [&](int r, int cols) -> float* {
-              const int ent_c = ents[(c0 + r) >> lgG];
-              return ent_c >= 0 ? acc_d + (long long)(ent_c & 0xFFFFFF) * tok_stride + cols * G : nullptr;
-            });
+            reduce_columns<WIDE>(cur, G, lane, [&](int r) { return ents[(c0 + r) >> lgG]; },
+                                 [&](int e) { return reinterpret_cast<float*>(reinterpret_cast<char*>(acc_d) + (uint64_t)(uint32_t)(e & 0xFFFFFF) * tok_bytes); });
           }
         } else {
 #pragma unroll
@@ -1589,9 +1589,13 @@ int launch_tile_pv(const Geometry& g, const TileArgs& a, int32_t* work_ctr, cuda
   }
   constexpr int QP = (KS * 128 * 128 > 128 * 272) ? KS * 128 * 128 : 128 * 272;
   const size_t smem = 4 * (size_t)((QP + 1023) / 1024 * 1024) + 2 * (size_t)KS * C * 128 + 1024;
-  cudaError_t e = cudaFuncSetAttribute(pv_ws_kernel<D, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr bool kBoth = D == 128;           // (the d = 64 read-out has no such case)
+  const bool wide = !kBoth || g.G >= 4;
+  cudaError_t e = wide ? cudaFuncSetAttribute(pv_ws_kernel<D, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                       : cudaFuncSetAttribute(pv_ws_kernel<D, C, !kBoth>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) { record_cuda_error("pv_ws attr", e); return PISA_ERR_CUDA; }
-  pv_ws_kernel<D, C><<<num_sms(), kPvThreads, smem, s>>>(g, a, work_ctr, tm_k, tm_v);
+  if (wide) pv_ws_kernel<D, C, true><<<num_sms(), kPvThreads, smem, s>>>(g, a, work_ctr, tm_k, tm_v);
+  else pv_ws_kernel<D, C, !kBoth><<<num_sms(), kPvThreads, smem, s>>>(g, a, work_ctr, tm_k, tm_v);
   return check_launch("pv_ws");
 }
 
@@ -1634,17 +1638,21 @@ BwdLayout bwd_layout(const Geometry& g) {
   return r;
 }
 
-template <int C, int DIN>
-int launch_bwd(const Geometry& g, BwdArgs a, cudaStream_t s) {
+template <int C, int DIN, bool WIDE>
+int launch_bwd_w(const Geometry& g, BwdArgs a, cudaStream_t s) {
   // K, V, two dS, pairs of Q and dO
   const size_t smem = (size_t)(DIN / 64) * 2 * (128 * 128) + 2 * (128 * 128) + (size_t)(DIN / 64) * 2 * kBwdStages * (kBwdRows * 128) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(bsa_bwd_kernel<C, DIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(bsa_bwd_kernel<C, DIN, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) { record_cuda_error("bsa_bwd attr", e); return PISA_ERR_CUDA; }
   CUtensorMap tm_k = {}, tm_v = {};
   a.kv_tma = tma_strides(g.ks) && tma_strides(g.vs) && qm_map_rows(&tm_k, a.k, g.d, g.Hkv, g.N, g.B, g.ks, 1, C) &&
              qm_map_rows(&tm_v, a.v, g.d, g.Hkv, g.N, g.B, g.vs, 1, C);
-  bsa_bwd_kernel<C, DIN><<<num_sms(), kBwdThreads, smem, s>>>(g, a, tm_k, tm_v);
+  bsa_bwd_kernel<C, DIN, WIDE><<<num_sms(), kBwdThreads, smem, s>>>(g, a, tm_k, tm_v);
   return check_launch("bsa_bwd");
+}
+template <int C, int DIN>
+int launch_bwd(const Geometry& g, const BwdArgs& a, cudaStream_t s) {
+  return g.G >= 4 ? launch_bwd_w<C, DIN, true>(g, a, s) : launch_bwd_w<C, DIN, false>(g, a, s);
 }
 
 }  // namespace
