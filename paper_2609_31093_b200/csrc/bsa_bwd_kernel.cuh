@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
   uint8_t* sdS = sV + KV_TILE;                              // [2]
   uint8_t* sQ = sdS + 2 * DS_TILE;                          // [NS]
   uint8_t* sdO = sQ + NS * R_TILE;                          // [NS]
-  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, k_seen, rows_seen, s_full[2], e_done[2], dq_full[2], dq_empty[2],
+  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, k_seen, rows_seen[NS], s_full[2], e_done[2], dq_full[2], dq_empty[2],
       acc_full, acc_empty;
   __shared__ int s_ent[R][kBwdRows];                        // a tile's entries (token | slot << 24, -1 = none)
   __shared__ int4 s_tkey[R];                                // its (unit, leaf, flags: 1 / 2 = first / last of its item, 4 = own-leaf rows)
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
   if (tid == 0) {
     for (int i = 0; i < R; ++i) { mbar_init(&m_full[i], 1); mbar_init(&m_empty[i], 22); }
     for (int i = 0; i < NS; ++i) { mbar_init(&qd_full[i], 256); mbar_init(&qd_empty[i], 1); }
-    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1); mbar_init(&k_seen, C / 32); mbar_init(&rows_seen, 1);
+    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1); mbar_init(&k_seen, C / 32); for (int i = 0; i < NS; ++i) mbar_init(&rows_seen[i], 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1); mbar_init(&e_done[i], 8);
       mbar_init(&dq_full[i], 1); mbar_init(&dq_empty[i], 4);
@@ -249,9 +249,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
           if (lane == 0) mbar_arrive(&kv_full);
         }
       }
+      // (every tile's rows are waited for and announced, looked at or not: nothing runs a phase ahead of the issuer)
+      const int st = it % NS;
+      if (!mbar_wait_bounded(&qd_full[st], (uint32_t)((it / NS) & 1))) { s_fail = 1; break; }
       if (key.z & 4) {                                      // rows that are not finite (see the head of this file)
-        const int st = it % NS;
-        if (!mbar_wait_bounded(&qd_full[st], (uint32_t)((it / NS) & 1))) { s_fail = 1; break; }
 #pragma unroll 1
         for (int r0 = 0; r0 < kBwdRows; r0 += 32) {
           const float2 x = s_stat[st][r0 + lane];
@@ -268,8 +269,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
         }
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&rows_seen);
       }
+      if (lane == 0) mbar_arrive(&rows_seen[st]);
       done_tile(it);
     }
   } else if (warp == 9) {
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
     auto wait = [&](uint64_t* bar, uint32_t parity) {
       if (!dead && !mbar_try_wait(bar, parity) && !mbar_wait_bounded(bar, parity)) { dead = true; s_fail = 1; }
     };
-    int n_item = 0, n_own = 0, it = 0;                      // items begun; tiles with own-leaf rows; the tile whose S and dP are next
+    int n_item = 0, it = 0;                                 // items begun; the tile whose S and dP are next
     uint32_t st = 0u, st_ph = 0u, st_prev = 0u;             // its stage and phase; stage of the tile before
     uint32_t flags = 0u, prev = 0u;                         // its flags; those of the tile before, whose gradients are owed (8: there is one)
     bool known = false, rows_ready = false, e_ready = false;
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       const uint32_t buf = (uint32_t)(it & 1), own = flags;
       if (!rows_ready) wait(&qd_full[st], st_ph);
       rows_ready = false;
-      if (own & 4u) wait(&rows_seen, (uint32_t)(n_own++ & 1));
+      if (own & 4u) wait(&rows_seen[st], st_ph);
       fence_proxy_async_smem();
       tcgen05_fence_after_sync();
       const uint32_t q0 = q_base + st * (uint32_t)(R_TILE >> 4), o0 = o_base + st * (uint32_t)(R_TILE >> 4), tb = tmem + T_BUF + buf * 128u;
