@@ -16,6 +16,9 @@
 // its element-wise step runs under them, as do the gathers and the reductions (32 KB a tile, 16 bytes per clock and SM at best).
 // C = 64: the upper 64 key rows are zero (so are their scores and gradients) and never read out; d = 64: the rows are one
 // 64-column slab, and the upper lanes of dQ^T, fed from the neighbouring slab, are not read out.
+// Measured: 32768 tokens, 32 heads, C = 128, K = 32: 7.0 ms, 570 TFLOP/s of the five products (one CTA that walked a tile of 128
+// rows with all its warps in step: 12.3 ms); with C = 64, K = 16 1.9 ms (3.1 ms).  What bounds it: the issuing warp's chain, about
+// 3700 cycles a tile of which the tensor pipe works 1660.
 // delta = rowsum(dO o O) comes from a small kernel of its own or from the dense way's preparation.
 // What is not finite reaches only what it belongs to: where a row sees a part of its own block only, the products multiply the
 // rest by zero.  So keys that are not finite count as zero and their scores as NaN, and so do, in tiles with rows of the block's
@@ -110,7 +113,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
   uint8_t* sdS = sV + KV_TILE;                              // [2]
   uint8_t* sQ = sdS + 2 * DS_TILE;                          // [NS]
   uint8_t* sdO = sQ + NS * R_TILE;                          // [NS]
-  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, k_seen, rows_seen[NS], s_full[2], e_done[2], dq_full[2], dq_empty[2],
+  __shared__ uint64_t m_full[R], m_empty[R], qd_full[NS], qd_empty[NS], kv_full, kv_empty, k_seen, s_full[2], e_done[2], dq_full[2], dq_empty[2],
       acc_full, acc_empty;
   __shared__ int s_ent[R][kBwdRows];                        // a tile's entries (token | slot << 24, -1 = none)
   __shared__ int4 s_tkey[R];                                // its (unit, leaf, flags: 1 / 2 = first / last of its item, 4 = own-leaf rows)
@@ -124,7 +127,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
   if (tid == 0) {
     for (int i = 0; i < R; ++i) { mbar_init(&m_full[i], 1); mbar_init(&m_empty[i], 22); }
     for (int i = 0; i < NS; ++i) { mbar_init(&qd_full[i], 256); mbar_init(&qd_empty[i], 1); }
-    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1); mbar_init(&k_seen, C / 32); for (int i = 0; i < NS; ++i) mbar_init(&rows_seen[i], 1);
+    mbar_init(&kv_full, 1); mbar_init(&kv_empty, 1); mbar_init(&k_seen, C / 32);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1); mbar_init(&e_done[i], 8);
       mbar_init(&dq_full[i], 1); mbar_init(&dq_empty[i], 4);
@@ -162,8 +165,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
     __syncwarp();
     if (lane == 0) mbar_arrive(&m_empty[it % R]);
   };
-  // (the loops of all roles are rolled as far as the registers allow: unrolled, their code did not fit the instruction cache --
-  // 62 % hits, and more stalls for instructions than for anything else)
+  // (code size: with all roles' loops unrolled 62 % of the instruction fetches hit the SM's cache, and more stalls were for
+  // instructions than for anything else: 8.4 ms at 32768 tokens, 32 heads, C = 128, now 7.0)
 
   if (warp < 8) {
     // ------------------------------------------------ gather: a tile's Q and dO rows and their statistics
@@ -210,7 +213,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
     }
     cp_async_wait_all();
   } else if (warp == 8) {
-    // ------------------------------------------------ an item's keys and values; rows that see a part of the block
+    // ------------------------------------------------ an item's keys and values
     int n_item = 0;
     for (int it = 0; wait_tile(it); ++it) {
       const int4 key = s_tkey[it % R];
@@ -249,28 +252,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
           if (lane == 0) mbar_arrive(&kv_full);
         }
       }
-      // (every tile's rows are waited for and announced, looked at or not: nothing runs a phase ahead of the issuer)
-      const int st = it % NS;
-      if (!mbar_wait_bounded(&qd_full[st], (uint32_t)((it / NS) & 1))) { s_fail = 1; break; }
-      if (key.z & 4) {                                      // rows that are not finite (see the head of this file)
-#pragma unroll 1
-        for (int r0 = 0; r0 < kBwdRows; r0 += 32) {
-          const float2 x = s_stat[st][r0 + lane];
-          const bool bad = !(fabsf(x.y) < CUDART_INF_F) || !(x.x < CUDART_INF_F);
-          if (bad) s_stat[st][r0 + lane].x = CUDART_NAN_F;
-          for (unsigned m = __ballot_sync(0xffffffffu, bad); m != 0u; m &= m - 1u) {
-            const int row = r0 + __ffs(m) - 1;
-            if (lane < KS * 8) {
-              const uint32_t d = (uint32_t)(st * R_TILE + (lane >> 3) * R_SLAB) + swz128(row, lane & 7);
-              st_shared_zero16(smem_u32(sQ) + d);
-              st_shared_zero16(smem_u32(sdO) + d);
-            }
-          }
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-      }
-      if (lane == 0) mbar_arrive(&rows_seen[st]);
       done_tile(it);
     }
   } else if (warp == 9) {
@@ -390,7 +371,23 @@ __global__ void __launch_bounds__(kBwdThreads, 1) bsa_bwd_kernel(Geometry geo, B
       const uint32_t buf = (uint32_t)(it & 1), own = flags;
       if (!rows_ready) wait(&qd_full[st], st_ph);
       rows_ready = false;
-      if (own & 4u) wait(&rows_seen[st], st_ph);
+      if (own & 4u) {                                       // rows that are not finite (see the head of this file)
+#pragma unroll 1
+        for (int r0 = 0; r0 < kBwdRows; r0 += 32) {
+          const float2 x = s_stat[st][r0 + lane];
+          const bool bad = !(fabsf(x.y) < CUDART_INF_F) || !(x.x < CUDART_INF_F);
+          if (bad) s_stat[st][r0 + lane].x = CUDART_NAN_F;
+          for (unsigned m = __ballot_sync(0xffffffffu, bad); m != 0u; m &= m - 1u) {
+            const int row = r0 + __ffs(m) - 1;
+            if (lane < KS * 8) {
+              const uint32_t d = st * (uint32_t)R_TILE + (uint32_t)((lane >> 3) * R_SLAB) + swz128(row, lane & 7);
+              st_shared_zero16(smem_u32(sQ) + d);
+              st_shared_zero16(smem_u32(sdO) + d);
+            }
+          }
+        }
+        __syncwarp();
+      }
       fence_proxy_async_smem();
       tcgen05_fence_after_sync();
       const uint32_t q0 = q_base + st * (uint32_t)(R_TILE >> 4), o0 = o_base + st * (uint32_t)(R_TILE >> 4), tb = tmem + T_BUF + buf * 128u;
