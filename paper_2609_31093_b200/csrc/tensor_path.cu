@@ -417,24 +417,9 @@ __device__ __forceinline__ ItemInfo feed_publish(ItemFeed& f, const TileArgs& a,
   return r;
 }
 
-// The 128 producer threads copy rows [row0, row0+nrows) of a [tokens][D] matrix into swizzled K-major
-// slabs.  Thread p always moves 16-byte chunk (p % (D/8)) of rows (p / (D/8)) + i * (1024/D): the row
-// index modulo 8 -- hence the swizzle -- is the same for every i, so the destination just advances.
-template <int D>
-__device__ __forceinline__ void prod_load_rows(uint8_t* dst, int slab_bytes, const __nv_bfloat16* base,
-                                               long long row_stride, int row0, int nrows, int limit, int p) {
-  constexpr int CH = D / 8, RPP = kProdThreads / CH;
-  const int ck = p % CH, rb = p / CH;
-  uint32_t d = smem_u32(dst + (ck >> 3) * slab_bytes) + swz128(rb, ck & 7);
-  const __nv_bfloat16* src = base + (long long)(row0 + rb) * row_stride + ck * 8;
-  for (int row = rb; row < nrows; row += RPP) {
-    if (row0 + row < limit) cp_async16(d, src);
-    else st_shared_zero16(d);
-    d += RPP * 128;
-    src += (long long)RPP * row_stride;
-  }
-}
-// ... and gather the 128 query rows of a tile: row r = (entry r >> lgG, head r & (G-1)); the tile's
+// The 128 producer threads gather the 128 query rows of a tile into swizzled K-major slabs.  Thread p always moves 16-byte chunk
+// (p % (D/8)) of rows (p / (D/8)) + i * (1024/D): the row index modulo 8 -- hence the swizzle -- is the same for every i, so the
+// destination just advances.  Row r = (entry r >> lgG, head r & (G-1)); the tile's
 // entries sit in shared memory (-1 = no entry)
 template <int D>
 __device__ __forceinline__ void prod_gather_q(uint8_t* dst, const Geometry& geo, const __nv_bfloat16* qb,
@@ -449,25 +434,6 @@ __device__ __forceinline__ void prod_gather_q(uint8_t* dst, const Geometry& geo,
   for (int row = rb; row < 128; row += RPP) {
     const int ent = s_ent[row >> lgG];
     if (ent >= 0) cp_async16(d, src0 + (long long)(ent & 0xFFFFFF) * s1 + (long long)(row & (G - 1)) * s2);
-    else st_shared_zero16(d);
-    d += RPP * 128;
-  }
-}
-// ... the same gather with the tile's entries already in the thread's registers (ent[i] belongs to row
-// rb + i * RPP; -1 = no entry): no shared-memory round trip and no barrier among the producer warps
-template <int D>
-__device__ __forceinline__ void prod_gather_q_regs(uint8_t* dst, const Geometry& geo, const __nv_bfloat16* qb,
-                                                   const int (&ent)[128 / (kProdThreads / (D / 8))], int p) {
-  constexpr int CH = D / 8, RPP = kProdThreads / CH, RPT = 128 / RPP;
-  const int ck = p % CH, rb = p / CH;
-  const int G = geo.G;
-  uint32_t d = smem_u32(dst + (ck >> 3) * (128 * 128)) + swz128(rb, ck & 7);
-  const __nv_bfloat16* src0 = qb + ck * 8;
-  const long long s1 = geo.qs[1], s2 = geo.qs[2];
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const int row = rb + i * RPP;
-    if (ent[i] >= 0) cp_async16(d, src0 + (long long)(ent[i] & 0xFFFFFF) * s1 + (long long)(row & (G - 1)) * s2);
     else st_shared_zero16(d);
     d += RPP * 128;
   }
