@@ -75,11 +75,12 @@ bool qm_supported(const Geometry& g, int dtype) {
 // a third longer and the lines lie 1.5 times higher): G = 4, C = 64, K = 16: 12288 tokens 745 / 748 (16 heads), 1402 / 1265
 // (32 heads, fan-in 4), 8192 763 / 838; G = 4, C = 128, K = 32: 12288 1744 / 2100, 16384 2964 / 2869; 16 KV heads without
 // groups, K = 16: 16384 1612 / 1740, 24000 3304 / 2846; G = 16, d = 64, K = 8: 6000 331 / 367, 8192 526 / 461.  Shapes that
-// the lists do not take stay dense further: their alternative is the exact fp32 path.
+// the lists do not take stay dense further: their alternative is the exact fp32 path.  So do small problems, which the lists'
+// eighteen launches weigh on (host tensors, 16384 tokens, one KV head of four query heads at a time: 3.13 ms dense, 3.21 lists).
 bool qm_dense_preferred(const Geometry& g, int dtype) {
   if (!qm_supported(g, dtype) || g.M[1] > 512 || g.N > kDenseMaxTokens) return false;
   int per_block = g.G == 1 ? 1120 : g.C == 128 ? 480 : g.G == 16 ? 832 : 704;
-  if (!tensor_path_supported(g, dtype)) per_block = g.G == 1 ? 2048 : g.C == 128 ? 704 : 1024;
+  if (!tensor_path_supported(g, dtype) || (long long)g.B * g.Hq * g.N < (1 << 17)) per_block = g.G == 1 ? 2048 : g.C == 128 ? 704 : 1024;
   return g.N <= g.K * per_block && layout(g).total <= kDenseMaxBytes;
 }
 
